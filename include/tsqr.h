@@ -81,7 +81,9 @@ typedef enum {
     TSQR_TREE_PANELS = 4
 } tsqr_tree_t;
 
-/* Leaf (tile) factorization of the MIXED path (TSQR_PREC_MIXED; the FP64 path has one leaf).
+/* How the row tiles are reduced: the leaf (tile) factorization of the MIXED path
+ * (TSQR_PREC_MIXED), and GRAM, the FP64 reduction AUTO takes where it serves (the FP64 path has
+ * one Householder leaf beside it, 0).
  * FOLD:   the fused fold R <- R([R; chunk]) one reflector at a time, every reflector applied to
  *         every later column by the CUDA cores (FP32 bulk arithmetic, FP64 R and scalars); any
  *         n <= TSQR_MAX_N.
@@ -92,9 +94,20 @@ typedef enum {
  *         (each as accurate as an FP32 dot product); R in double-FP32 in the leaf, FP64 in the
  *         tree.  n <= 112; chunks of 256, 384, 512, 640, 768 or 1024 rows (tile_rows; AUTO:
  *         the tallest the width's shared and tensor memory allow).
- * AUTO picks PANELS for n <= 112 (FP32 from n = 9, BF16 from n = 3), where it measured
- * faster, else FOLD. */
-typedef enum { TSQR_LEAF_AUTO = 0, TSQR_LEAF_FOLD = 1, TSQR_LEAF_PANELS = 2 } tsqr_leaf_t;
+ * GRAM:   (FP64, HYBRID) R as the Cholesky factor of A^T A, without the digits that route loses
+ *         in floating point: every column is written in fixed point against its largest entry
+ *         (62 bits, in eight 8-bit digits), the digits' products are summed on the tensor cores
+ *         (exact: whole numbers below 2^24 in FP32 accumulators), put together in 128-bit
+ *         integers, added over the row blocks, and the sum is factored in 122-bit fixed point.
+ *         m >= 1024, m >= 16 n, n <= 32.  A matrix it cannot serve (a NaN or Inf, entries
+ *         outside 2^-400 .. 2^400, a pivot below 2^-64 of its column's square: zero or dependent
+ *         columns) is found in the same launch, which then runs the Householder leaves and tree
+ *         that the plan's other fields describe.
+ * AUTO picks, FP64: GRAM where it serves; MIXED: PANELS for n <= 112 (FP32 from n = 9, BF16 from
+ * n = 3), where it measured faster, else FOLD. */
+typedef enum {
+    TSQR_LEAF_AUTO = 0, TSQR_LEAF_FOLD = 1, TSQR_LEAF_PANELS = 2, TSQR_LEAF_GRAM = 3
+} tsqr_leaf_t;
 
 /* Optional plan override.  Zero fields mean "choose".  The chosen plan fixes the arithmetic
  * order, so two calls with equal plans and inputs return identical bytes. */
@@ -108,7 +121,8 @@ typedef struct {
                            in one sweep (the R factor of [R_1; ...; R_c], equal to a sequence of
                            binary operators by associativity, Section 2).  0 = as many as the
                            kernel's shared memory holds.                                     */
-    int32_t leaf;       /* tsqr_leaf_t (mixed path only; 0 elsewhere).  With PANELS,
+    int32_t leaf;       /* tsqr_leaf_t (FP64: 0 or GRAM, whose plan is AUTO's whatever the other
+                           fields say).  With PANELS,
                            tile_rows is the chunk height (256, 384, 512, 640, 768 or 1024) of a HYBRID
                            plan, warps is 8 (or 0).                                          */
 } tsqr_plan_t;

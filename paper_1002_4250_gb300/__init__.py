@@ -26,7 +26,7 @@ SUCCESS, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_CUDA, ERR_ALLOC, ERR_TIMEOUT, STA
 F64, F32, BF16 = 0, 1, 2
 PREC_F64, PREC_MIXED = 0, 1
 TREE_AUTO, TREE_BINARY, TREE_FLAT, TREE_HYBRID, TREE_PANELS = 0, 1, 2, 3, 4
-LEAF_AUTO, LEAF_FOLD, LEAF_PANELS = 0, 1, 2
+LEAF_AUTO, LEAF_FOLD, LEAF_PANELS, LEAF_GRAM = 0, 1, 2, 3
 MAX_N = 128
 _TREES = {"auto": TREE_AUTO, "binary": TREE_BINARY, "flat": TREE_FLAT, "hybrid": TREE_HYBRID,
           "panels": TREE_PANELS}
@@ -53,7 +53,7 @@ def make_batch_plan(warps=0, ctas_per_sm=0, leaves_per_cta=0, arity=(0, 0, 0, 0)
                     leaf="auto") -> BatchPlan:
     """Knobs of a varlen batch call; arity per width bucket (n <= 8, <= 16, <= 32, > 32); leaf
     "auto", "fold" or "panels" (mixed precision)."""
-    lf = {"auto": LEAF_AUTO, "fold": LEAF_FOLD, "panels": LEAF_PANELS}[leaf] \
+    lf = {"auto": LEAF_AUTO, "fold": LEAF_FOLD, "panels": LEAF_PANELS, "gram": LEAF_GRAM}[leaf] \
         if isinstance(leaf, str) else int(leaf)
     return BatchPlan(int(warps), int(ctas_per_sm), int(leaves_per_cta),
                      (ctypes.c_int32 * 4)(*[int(a) for a in arity]), lf)
@@ -186,7 +186,7 @@ def empty_r(n: int, device=None):
     return torch.empty((n, n), dtype=torch.float64, device=device).T
 
 
-_LEAVES = {"auto": LEAF_AUTO, "fold": LEAF_FOLD, "panels": LEAF_PANELS}
+_LEAVES = {"auto": LEAF_AUTO, "fold": LEAF_FOLD, "panels": LEAF_PANELS, "gram": LEAF_GRAM}
 
 
 def make_plan(tree="auto", tile_rows=0, ctas=0, warps=0, arity=0, leaf="auto") -> Plan:

@@ -11,6 +11,7 @@
 #include <cmath>
 
 #include "tsqr.h"
+#include "tsqr_gram.cuh"
 #include "tsqr_internal.h"
 #include "tsqr_qr.cuh"
 
@@ -88,6 +89,7 @@ struct F64Plan {
     size_t smem = 0;
     TreeShape shape{};
     int64_t nodes = 0;
+    int gram_ctas = 0;             // TSQR_LEAF_GRAM: leaves of the Gram sum (0: no Gram)
 };
 
 // Arguments of the Q^T apply for a factorization with storage `q` under plan p: B (m x ktot,
@@ -385,7 +387,7 @@ tsqr_status_t plan_leaf(int64_t m, int n, const tsqr_plan_t *over, bool mixed, F
     if (di.sms <= 0) return TSQR_ERR_CUDA;
     tsqr_plan_t tuned;
     if (plan_is_auto(over) && tuned_plan(dev, m, n, mixed, &tuned) &&
-        tuned.tree != TSQR_TREE_PANELS)
+        tuned.tree != TSQR_TREE_PANELS && tuned.leaf != TSQR_LEAF_GRAM)
         over = &tuned;
     p->tree = (over && over->tree) ? over->tree : TSQR_TREE_HYBRID;
     if (p->tree < TSQR_TREE_BINARY || p->tree > TSQR_TREE_HYBRID) return TSQR_ERR_INVALID_ARG;
@@ -468,6 +470,123 @@ tsqr_status_t zero_r(double *R, int64_t n, int64_t ldr, cudaStream_t stream) {
     return TSQR_SUCCESS;
 }
 
+// The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to kGramMaxN columns.
+constexpr int64_t kGramMinRows = 1024;
+bool gram_fits(int64_t m, int64_t n) {
+    return n >= 1 && n <= kGramMaxN && m >= kGramMinRows && m >= 16 * n;
+}
+
+// Plan of an FP64 R by one reduction: the exact-Gram reduction where it serves (AUTO, or a plan
+// that asks for TSQR_LEAF_GRAM), else the Householder leaves.  The Gram plan's other fields are
+// those of the Householder reduction the same launch falls back to: one CTA of 12 bulk warps
+// per SM, an even number of rows per lane (the kernel's inner block is two rows).
+tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
+    tsqr_plan_t tuned;
+    if (plan_is_auto(over) && tuned_plan(dev, m, n, false, &tuned) &&
+        tuned.tree != TSQR_TREE_PANELS)
+        over = &tuned;
+    const bool asked = over && over->leaf == TSQR_LEAF_GRAM;
+    if (asked && (over->tree > TSQR_TREE_HYBRID || over->tree == TSQR_TREE_BINARY ||
+                  over->tree == TSQR_TREE_FLAT || !gram_fits(m, n)))
+        return TSQR_ERR_INVALID_ARG;
+    if (!asked && !(plan_is_auto(over) && gram_fits(m, n))) return plan_f64(m, n, over, p);
+    const DeviceInfo di = device_info(dev);
+    if (di.sms <= 0) return TSQR_ERR_CUDA;
+    p->tree = TSQR_TREE_HYBRID;
+    p->leaf = TSQR_LEAF_GRAM;
+    p->warps = kGramFoldWarps;
+    const size_t budget = std::min(di.smem_block_optin, di.smem_sm - 1024);
+    int r = max_rows_per_lane_p(n, p->warps, budget, false);
+    while (r > 0 && (r % 2 || good_r(r) != r)) --r;
+    tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, di.sms, p->warps, 0, 0};
+    const tsqr_status_t st = plan_with_r(m, n, &fold, false, r, di, p);
+    if (st != TSQR_SUCCESS) return st;
+    if (p->blk % 2) {  // a matrix of few rows: two rows per lane all the same
+        fold.tile_rows = 64 * p->warps;
+        const tsqr_status_t st2 = plan_with_r(m, n, &fold, false, r, di, p);
+        if (st2 != TSQR_SUCCESS) return st2;
+    }
+    const int64_t kb = gram_round_rows(n) / 64, nkb = (m + 63) / 64;
+    p->gram_ctas = (int)std::min<int64_t>(di.sms, (nkb + kb - 1) / kb);
+    p->smem = std::max(p->smem, gram_smem_bytes(n));
+    return TSQR_SUCCESS;
+}
+
+// Inner nodes of the Gram sum's tree over `ctas` leaves.
+int64_t gram_inner_nodes(int64_t ctas) {
+    int64_t inner = 0;
+    for (int64_t c = ctas; c > 1;) {
+        c = (c + kGramArity - 1) / kGramArity;
+        inner += c;
+    }
+    return inner;
+}
+
+// Workspace of one reduction under plan p: counters (zeroed per call), then tree slots.
+struct RLayout {
+    size_t cnt_words = 0, cnt_bytes = 0, bytes = 0;
+};
+RLayout r_layout(const F64Plan &p, int64_t n) {
+    RLayout w;
+    const size_t inner = p.gram_ctas ? (size_t)gram_inner_nodes(p.gram_ctas) : 0;
+    w.cnt_words = (size_t)p.nodes + (p.gram_ctas ? inner + 1 : 0);
+    w.cnt_bytes = align_up(w.cnt_words * sizeof(unsigned int), 256);
+    w.bytes = w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double);
+    if (p.gram_ctas)
+        w.bytes = align_up(w.bytes, 256) + (inner + p.gram_ctas) * gram_slot_bytes((int)n);
+    return w;
+}
+
+// One reduction of [A | B] (B: columns na .. n-1, or none) under plan p in the workspace at base
+// (r_layout(p, n).bytes), R to device memory.  Only the Gram plan takes a second matrix.
+tsqr_status_t enqueue_r(const F64Plan &p, const double *A, int64_t lda, const double *B,
+                        int64_t ldb, int64_t na, int64_t m, int64_t n, void *base, double *R,
+                        int64_t ldr, int *status, cudaStream_t stream) {
+    const RLayout w = r_layout(p, n);
+    F64Args a = plan_args(p, A, m, n, lda);
+    a.counters = (unsigned int *)base;
+    a.slots = (double *)((char *)base + w.cnt_bytes);
+    a.R = R;
+    a.ldr = ldr;
+    a.status = status;
+    if ((p.gram_ctas ? gram_prepare((int)n, p.smem) : f64_prepare(p.smem)) != cudaSuccess)
+        return TSQR_ERR_CUDA;
+    if (cudaMemsetAsync(a.counters, 0, w.cnt_words * sizeof(unsigned int), stream) != cudaSuccess)
+        return TSQR_ERR_CUDA;
+    if (!p.gram_ctas)
+        return f64_launch(a, p.warps, p.smem, stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
+    GramArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.A = A;
+    g.B = B;
+    g.lda = lda;
+    g.ldb = ldb;
+    g.m = m;
+    g.n = (int)n;
+    g.na = (int)na;
+    g.ctas = p.gram_ctas;
+    g.nkb = (m + 63) / 64;
+    g.counters = a.counters + p.nodes;
+    g.verdict = g.counters + gram_inner_nodes(p.gram_ctas);
+    g.slots = (unsigned char *)base +
+              align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
+    g.slot_bytes = gram_slot_bytes((int)n);
+    g.R = R;
+    g.ldr = ldr;
+    g.status = status;
+    g.fold = a;
+    cudaError_t e = gram_launch(g, p.smem, stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // a context that owns only part of the device: the plan's Householder reduction
+        cudaGetLastError();
+        if (f64_prepare(p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
+        e = f64_launch(a, p.warps, p.smem, stream);
+    }
+    return e == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
+}
+
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
                        int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream);
 
@@ -514,24 +633,14 @@ tsqr_status_t run_f64(const double *A, int64_t m, int64_t n, int64_t lda, double
     }
     if (n > TSQR_MAX_N) return TSQR_ERR_UNSUPPORTED;
     F64Plan p;
-    tsqr_status_t st = plan_f64(m, (int)n, over, &p);
+    tsqr_status_t st = plan_r(m, (int)n, over, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
-    if (f64_prepare(p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
-    const size_t cnt_bytes = align_up((size_t)p.nodes * sizeof(unsigned int), 256);
-    const size_t slot_bytes = (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double);
     Workspace *ws = nullptr;
-    st = get_workspace(stream, cnt_bytes + slot_bytes, &ws);
+    st = get_workspace(stream, r_layout(p, n).bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
-    F64Args a = plan_args(p, A, m, n, lda);
-    a.counters = (unsigned int *)ws->base;
-    a.slots = (double *)((char *)ws->base + cnt_bytes);
-    a.R = R;
-    a.ldr = ldr;
-    a.status = ws->status;
-    if (cudaMemsetAsync(a.counters, 0, (size_t)p.nodes * sizeof(unsigned int), stream) != cudaSuccess)
-        return TSQR_ERR_CUDA;
-    if (f64_launch(a, p.warps, p.smem, stream) != cudaSuccess) return TSQR_ERR_CUDA;
+    st = enqueue_r(p, A, lda, nullptr, 0, n, m, n, ws->base, R, ldr, ws->status, stream);
+    if (st != TSQR_SUCCESS) return st;
     g_last_launches = 1;
     return TSQR_SUCCESS;
 }
@@ -771,23 +880,21 @@ tsqr_status_t run_f64_host(const double *A, int64_t m, int64_t n, int64_t lda, d
     }
     const double *Amapped = mapped_device_ptr(A);
     F64Plan p;
-    tsqr_status_t st = plan_f64(m, (int)n, nullptr, &p);
+    tsqr_status_t st = plan_r(m, (int)n, nullptr, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
-    if (f64_prepare(p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
-    const size_t cnt_bytes = align_up((size_t)p.nodes * sizeof(unsigned int), 256);
-    const size_t slot_bytes = align_up((size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
+    const size_t r_off = align_up(r_layout(p, n).bytes, 256);
     const size_t r_bytes = align_up((size_t)n * (size_t)n * sizeof(double), 256);
     const size_t a_bytes = Amapped ? 0 : (size_t)m * (size_t)n * sizeof(double);
     Workspace *ws = nullptr;
-    st = get_workspace(stream, cnt_bytes + slot_bytes + r_bytes + a_bytes, &ws);
+    st = get_workspace(stream, r_off + r_bytes + a_bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
     char *base = (char *)ws->base;
-    double *Rd = (double *)(base + cnt_bytes + slot_bytes);
+    double *Rd = (double *)(base + r_off);
     const double *Ain = Amapped;
     int64_t ld_in = lda;
     if (!Amapped) {
-        double *Ad = (double *)(base + cnt_bytes + slot_bytes + r_bytes);
+        double *Ad = (double *)(base + r_off + r_bytes);
         if (cudaMemcpy2DAsync(Ad, (size_t)m * sizeof(double), A, (size_t)lda * sizeof(double),
                               (size_t)m * sizeof(double), (size_t)n, cudaMemcpyHostToDevice,
                               stream) != cudaSuccess)
@@ -795,16 +902,8 @@ tsqr_status_t run_f64_host(const double *A, int64_t m, int64_t n, int64_t lda, d
         Ain = Ad;
         ld_in = m;
     }
-    F64Args a = plan_args(p, Ain, m, n, ld_in);
-    a.counters = (unsigned int *)base;
-    a.slots = (double *)(base + cnt_bytes);
-    a.R = Rd;
-    a.ldr = n;
-    a.status = ws->status;
-    if (cudaMemsetAsync(a.counters, 0, (size_t)p.nodes * sizeof(unsigned int), stream) !=
-            cudaSuccess ||
-        f64_launch(a, p.warps, p.smem, stream) != cudaSuccess)
-        return TSQR_ERR_CUDA;
+    st = enqueue_r(p, Ain, ld_in, nullptr, 0, n, m, n, base, Rd, n, ws->status, stream);
+    if (st != TSQR_SUCCESS) return st;
     if (cudaMemcpy2DAsync(R, (size_t)ldr * sizeof(double), Rd, (size_t)n * sizeof(double),
                           (size_t)n * sizeof(double), (size_t)n, cudaMemcpyDeviceToHost,
                           stream) != cudaSuccess)
@@ -883,6 +982,8 @@ bool plan_wy(int w, const F64Plan &p, const DeviceInfo &di, int *ldX, size_t *wy
 // n where the AUTO plan takes 8 or 12 bulk warps); then the four-warp plan.  tsqr_last_plan
 // reports which.
 tsqr_status_t plan_store(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
+    // the exact-Gram reduction keeps no reflectors: those calls' own plan
+    if (over && over->leaf == TSQR_LEAF_GRAM) over = nullptr;
     // the passes that keep and apply the reflectors run 4, 8 or 12 bulk warps
     if (over && over->warps % 4 != 0) return TSQR_ERR_INVALID_ARG;
     tsqr_status_t st = plan_f64(m, n, over, p);
@@ -1144,6 +1245,19 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
     const DeviceInfo di = device_info(dev);
+    if (N <= nb && plan_is_auto(over) && gram_fits(m, N)) {  // one panel: tsqr_r's reduction
+        F64Plan p;
+        tsqr_status_t st = plan_r(m, (int)N, over, &p);
+        if (st != TSQR_SUCCESS) return st;
+        Workspace *ws = nullptr;
+        st = get_workspace(stream, r_layout(p, N).bytes, &ws);
+        if (st != TSQR_SUCCESS) return st;
+        st = enqueue_r(p, A, lda, nullptr, 0, N, m, N, ws->base, R, ldr, ws->status, stream);
+        if (st != TSQR_SUCCESS) return st;
+        g_last_plan = public_plan(p);
+        g_last_launches = 1;
+        return TSQR_SUCCESS;
+    }
     std::vector<CaqrPanel> panels;
     int64_t M = m;
     size_t max_fsmem = 0, max_qt = 0;
@@ -2156,7 +2270,7 @@ tsqr_status_t tsqr_resolve_plan(int64_t m, int64_t n, int32_t dtype, int32_t pre
     }
     F64Plan p;
     tsqr_status_t st = mixed ? plan_mixed(m, (int)n, dtype == TSQR_BF16, plan, &p)
-                             : plan_leaf(m, (int)n, plan, false, &p);
+                             : plan_r(m, (int)n, plan, &p);
     if (st != TSQR_SUCCESS) return st;
     *out = public_plan(p);
     return TSQR_SUCCESS;
@@ -2202,6 +2316,11 @@ tsqr_status_t tsqr_autotune(const void *A, int32_t dtype, int32_t prec, int64_t 
                 if (!dup) cands.push_back(c);
             }
         }
+    }
+    if (f64 && gram_fits(m, n)) {
+        F64Plan g;
+        const tsqr_plan_t ask{TSQR_TREE_HYBRID, 0, 0, 0, 0, TSQR_LEAF_GRAM};
+        if (plan_r(m, (int)n, &ask, &g) == TSQR_SUCCESS) cands.push_back(public_plan(g));
     }
     if (f64 && n >= 48 && m >= 8 * n)
         for (int32_t nb : {16, 32}) cands.push_back(tsqr_plan_t{TSQR_TREE_PANELS, nb, 0, 0, 0, 0});
@@ -2250,7 +2369,8 @@ tsqr_status_t tsqr_autotune(const void *A, int32_t dtype, int32_t prec, int64_t 
         }
     }
     // then the tree arity of the fastest one-reduction plan: 2 (the paper's binary tree) to 8
-    if (st == TSQR_SUCCESS && best_ms >= 0.0f && best_plan.tree == TSQR_TREE_HYBRID) {
+    if (st == TSQR_SUCCESS && best_ms >= 0.0f && best_plan.tree == TSQR_TREE_HYBRID &&
+        best_plan.leaf != TSQR_LEAF_GRAM) {
         const tsqr_plan_t base = best_plan;
         for (int32_t k : {2, 3, 4, 6, 8}) {
             tsqr_plan_t c = base;

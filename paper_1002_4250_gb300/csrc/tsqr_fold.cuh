@@ -19,6 +19,12 @@
 #include "tsqr_f64.cuh"
 #include "tsqr_internal.h"
 
+// Threads that run the fold and the tree: the CTA's, or fewer where a kernel lets the others
+// exit first (it defines this before including the header).
+#ifndef TSQR_FOLD_THREADS
+#define TSQR_FOLD_THREADS blockDim.x
+#endif
+
 namespace tsqr {
 
 // ------------------------------------------------------------------------------------------
@@ -38,6 +44,12 @@ __device__ __forceinline__ void cp_async4(void *smem_dst, const void *gsrc, int 
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// At most `kPending` of the thread's newest groups still on their way.
+template <int kPending>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kPending) : "memory");
+}
 
 // A chunk of rows of A (src == nullptr: none).
 template <typename Tin>
@@ -65,7 +77,7 @@ __device__ __forceinline__ void load_column(T *S, int ldS, int hs, const Chunk<T
     const Tin *src = c.src + (int64_t)col * c.lda;
     T *dst = S + (size_t)col * ldS;
     if constexpr (Copy<T, Tin>::kAsync) {
-        for (int i = threadIdx.x; i < hs; i += blockDim.x) {
+        for (int i = threadIdx.x; i < hs; i += TSQR_FOLD_THREADS) {
             const bool ok = i < c.rows;
             if constexpr (sizeof(T) == 8)
                 cp_async8(dst + i, ok ? (const void *)(src + i) : (const void *)c.src, ok ? 8 : 0);
@@ -74,7 +86,7 @@ __device__ __forceinline__ void load_column(T *S, int ldS, int hs, const Chunk<T
         }
         cp_async_commit();
     } else {
-        for (int i = threadIdx.x; i < hs; i += blockDim.x)
+        for (int i = threadIdx.x; i < hs; i += TSQR_FOLD_THREADS)
             dst[i] = (i < c.rows) ? (T)widen(src[i]) : (T)0;
     }
 }
@@ -478,7 +490,7 @@ __device__ __forceinline__ void fold_leaf(T *__restrict__ S, const int ldS, cons
                                           const QChunk qc = QChunk{}) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int Wb = (blockDim.x >> 5) - 1;
+    const int Wb = (TSQR_FOLD_THREADS >> 5) - 1;
     const bool reducer = (warp == Wb);
     const int Hw = hs / Wb;
     const int r = Hw >> 5;
@@ -612,7 +624,7 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
                                            const bool worker_sums = true) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int Wp = (blockDim.x >> 5) - 1;  // worker warps 1..Wp
+    const int Wp = (TSQR_FOLD_THREADS >> 5) - 1;  // worker warps 1..Wp
     const int ss = seg_stride(n);
     double *seg = seg_all + (warp > 0 ? warp - 1 : 0) * ss;
 
@@ -749,7 +761,7 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
 // Packed upper triangle (smem) -> column-major n x n (global), zeros below the diagonal.
 __device__ __forceinline__ void store_packed(const double *__restrict__ Rp, int n,
                                              double *__restrict__ dst, int64_t ld) {
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         dst[row + (int64_t)col * ld] = (row <= col) ? Rp[rowoff(n, row) + col - row] : 0.0;
     }
@@ -758,7 +770,7 @@ __device__ __forceinline__ void store_packed(const double *__restrict__ Rp, int 
 // Column-major global (L2, bypassing L1) -> packed upper triangle in smem.
 __device__ __forceinline__ void load_packed_cg(const double *src, int64_t ld, int n,
                                                double *__restrict__ Rp) {
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         if (row <= col) Rp[rowoff(n, row) + col - row] = __ldcg(src + row + (int64_t)col * ld);
     }
@@ -767,7 +779,7 @@ __device__ __forceinline__ void load_packed_cg(const double *src, int64_t ld, in
 // Column-major global -> S (upper triangle kept, strict lower part stored as zero).
 __device__ __forceinline__ void load_tri_cg(const double *src, int64_t ld, int n,
                                             double *__restrict__ S, int ldS) {
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         S[row + col * ldS] = (row <= col) ? __ldcg(src + row + (int64_t)col * ld) : 0.0;
     }
@@ -778,7 +790,7 @@ __device__ __forceinline__ void store_normalized(const double *__restrict__ Rp, 
                                                  double *__restrict__ R, int64_t ldr,
                                                  int *status) {
     bool bad = false;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         double v = 0.0;
         if (row <= col) {
@@ -826,7 +838,7 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
     for (;;) {
         if (cnt == 1) {
             if constexpr (kStore) {
-                for (int k2 = threadIdx.x; k2 < n; k2 += blockDim.x)
+                for (int k2 = threadIdx.x; k2 < n; k2 += TSQR_FOLD_THREADS)
                     a.q.signs[k2] = (Rp[rowoff(n, k2)] < 0.0) ? -1.0 : 1.0;
             }
             store_normalized(Rp, n, a.R, a.ldr, a.status);
@@ -862,7 +874,7 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
             // the node's tails: rows 0..(nchild-1) n - 1 of S (zero below each diagonal)
             double *dst = a.q.node_V + id * (size_t)ldv * n;
             const int rows = (nchild - 1) * n;
-            for (int idx = threadIdx.x; idx < rows * n; idx += blockDim.x) {
+            for (int idx = threadIdx.x; idx < rows * n; idx += TSQR_FOLD_THREADS) {
                 const int col = idx / rows, row = idx - col * rows;
                 dst[row + (size_t)col * ldv] = Sd[row + (size_t)col * ldSd];
             }
@@ -891,7 +903,7 @@ __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, co
                                               const int worker_sum_nodes = kWorkerSumNodes) {
     extern __shared__ __align__(16) double smem[];
     const int n = a.n;
-    const SmemLayout L = smem_layout_s(n, s_doubles, blockDim.x >> 5);
+    const SmemLayout L = smem_layout_s(n, s_doubles, TSQR_FOLD_THREADS >> 5);
     T *S = reinterpret_cast<T *>(smem + L.S);
     double *Sd = smem + L.S;
     double *Rp = smem + L.Rp;
@@ -906,7 +918,7 @@ __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, co
     double *npart = smem + L.npart;
     unsigned int *flag = reinterpret_cast<unsigned int *>(smem + L.scal);
 
-    for (int i = threadIdx.x; i < n * (n + 1) / 2; i += blockDim.x) Rp[i] = 0.0;
+    for (int i = threadIdx.x; i < n * (n + 1) / 2; i += TSQR_FOLD_THREADS) Rp[i] = 0.0;
 
     // rows of this leaf, folded in chunks of h rows
     const int64_t u0 = ((int64_t)leaf * a.nunits) / a.nleaves;

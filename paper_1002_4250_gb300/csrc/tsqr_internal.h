@@ -34,6 +34,14 @@ cudaError_t f64_combine_launch(int n, const double *R1, int64_t ld1, const doubl
                                int ldS, int hs, size_t smem_bytes, int *status,
                                cudaStream_t stream);
 
+// Exact-Gram reduction (tsqr_gram.cu): rows a CTA slices at a time, shared memory, launch (one
+// cooperative launch of at most one CTA per SM).
+struct GramArgs;
+int gram_round_rows(int n);
+size_t gram_smem_bytes(int n);
+cudaError_t gram_prepare(int n, size_t smem_bytes);
+cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream);
+
 // Mixed path (tsqr_mixed.cu); `warps` counts bulk warps as for the FP64 path.
 int mixed_s_doubles(int n, int ldS);
 size_t mixed_smem_bytes(int n, int ldS, int warps);

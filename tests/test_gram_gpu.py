@@ -1,0 +1,143 @@
+"""GPU parity of the exact-Gram reduction (TSQR_LEAF_GRAM) against the CPU oracle, at the sizes
+where it can go wrong: the edges of its width classes, ragged row blocks, leading dimensions that
+take the narrow copies, columns whose exponents rise while they are summed, and the matrices it
+hands to the Householder reduction.  Bounds as in the FP64 parity tests: every entry within
+c(m) kappa u ||R_oracle||_F, c(m) = max(50, 2 sqrt(m)), Gram residual <= 1e-13."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def T():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1002_4250_gb300 as T
+    return T
+
+
+def _check(oracle, R, At):
+    A = oracle.from_torch_colmajor(At)
+    R = R.cpu().numpy()
+    Ro = oracle.householder_r(A, nthreads=16)
+    assert np.all(np.tril(R, -1) == 0) and np.all(np.diag(R) >= 0)
+    tol = max(50.0, 2.0 * np.sqrt(A.shape[0])) * oracle.kappa_from_r(Ro) * U * np.linalg.norm(Ro)
+    np.testing.assert_allclose(R, Ro, rtol=0, atol=tol)
+    assert oracle.gram_residual(A, R, nthreads=16) <= 1e-13
+
+
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 15, 16, 17, 23, 24, 25, 31, 32])
+@pytest.mark.parametrize("m,pad", [(1024, 0), (1087, 1), (70001, 0), (100003, 5)])
+def test_widths_and_ragged_rows(oracle, T, n, m, pad):
+    import torch
+    At = workloads.gaussian(m, n, seed=600 + n)
+    big = torch.full((n, m + pad), float("nan"), dtype=torch.float64)
+    big[:, :m] = At
+    R = T.tsqr_r(big.cuda().T[:m, :])
+    assert T.last_plan().leaf == T.LEAF_GRAM and T.tsqr_last_launch_count() == 1
+    _check(oracle, R, At)
+    assert T.tsqr_get_device_status() == T.SUCCESS
+
+
+@pytest.mark.parametrize("n", [5, 13, 30])
+@pytest.mark.parametrize("kind", ["grow", "outlier", "constant", "scales", "kappa"])
+def test_value_ranges(oracle, T, n, kind):
+    """Columns that grow by 2^40 on the way (exponents rise often), one entry 2^30 above the
+    rest in the middle, constant columns, columns of scales 2^-200 .. 2^200, kappa = 1e8."""
+    import torch
+    m = 150001
+    At = workloads.gaussian(m, n, seed=650 + n)
+    if kind == "grow":
+        At *= torch.exp2(torch.arange(m, dtype=torch.float64) * (40.0 / m))
+    elif kind == "outlier":
+        At[:, m // 2] *= 2.0 ** 30
+    elif kind == "constant":
+        At[0] = 0.1
+    elif kind == "scales":
+        At *= torch.exp2(torch.linspace(-200, 200, n, dtype=torch.float64).round())[:, None]
+    else:
+        At = workloads.conditioned(m, n, 1e8, seed=n)
+    R = T.tsqr_r(At.cuda().T)
+    if kind == "scales":  # column j of R scales with column j of A, exactly
+        s = torch.exp2(-torch.linspace(-200, 200, n, dtype=torch.float64).round())
+        R, At = R.cpu() * s[None, :], At * s[:, None]
+    _check(oracle, R, At)
+
+
+@pytest.mark.parametrize("n", [6, 16, 32])
+@pytest.mark.parametrize("kind", ["repeated", "zero", "zeros", "huge", "tiny", "nan", "inf"])
+def test_what_the_householder_reduction_takes_over(oracle, T, n, kind):
+    """Repeated and zero columns, entries whose squares leave FP64, NaN and Inf: the bytes and the
+    status are those of the one Householder reduction with the same leaves."""
+    import torch
+    m = 60013
+    At = workloads.gaussian(m, n, seed=700 + n)
+    if kind == "repeated":
+        At[n - 1] = At[1]
+    elif kind == "zero":
+        At[n // 2] = 0.0
+    elif kind == "zeros":
+        At.zero_()
+    elif kind == "huge":
+        At[2] *= 1e200
+    elif kind == "tiny":
+        At[2] *= 1e-200
+    else:
+        At[3, 12345] = float(kind)
+    Ad = At.cuda().T
+    T.tsqr_get_device_status()  # clears it
+    R = T.tsqr_r(Ad)
+    status = T.tsqr_get_device_status()
+    p = T.last_plan()
+    assert p.leaf == T.LEAF_GRAM
+    ref = T.tsqr_r_ex(Ad, plan=T.make_plan("hybrid", tile_rows=p.tile_rows, ctas=p.ctas,
+                                           warps=p.warps, arity=p.arity))
+    assert T.last_plan().leaf == 0
+    assert status == T.tsqr_get_device_status()
+    assert torch.equal(torch.nan_to_num(R), torch.nan_to_num(ref))
+    assert torch.equal(torch.isfinite(R), torch.isfinite(ref))
+    if kind in ("repeated", "zero", "zeros"):
+        A = oracle.from_torch_colmajor(At)
+        if kind != "zeros":
+            assert oracle.gram_residual(A, R.cpu().numpy(), nthreads=16) <= 1e-13
+        assert status == T.SUCCESS
+
+
+def test_capture_streams_and_plans(oracle, T):
+    """A captured call replays on new data; two streams run side by side; the plan a call reports
+    gives the same bytes; a plan that asks for the Gram where it does not serve is refused."""
+    import torch
+    m, n = 120000, 20
+    A1, A2 = (workloads.gaussian(m, n, seed=s).cuda() for s in (1, 2))
+    R1, R2 = T.tsqr_r(A1.T).clone(), T.tsqr_r(A2.T).clone()
+    assert torch.equal(T.tsqr_r_ex(A1.T, plan=T.last_plan()), R1)
+    buf, out = A1.clone(), T.empty_r(n, "cuda")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        T.tsqr_r(buf.T, R=out)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        T.tsqr_r(buf.T, R=out, stream=s)
+    buf.copy_(A2)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, R2)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = []
+    for k, st in enumerate(streams * 4):
+        with torch.cuda.stream(st):
+            outs.append((k, T.tsqr_r((A1 if k % 2 else A2).T)))
+    torch.cuda.synchronize()
+    for k, R in outs:
+        assert torch.equal(R, R1 if k % 2 else R2)
+    for bad in (T.make_plan("binary", tile_rows=256), T.make_plan("flat")):
+        bad.leaf = T.LEAF_GRAM
+        with pytest.raises(T.TsqrError) as e:
+            T.tsqr_r_ex(A1.T, plan=bad)
+        assert e.value.status == T.ERR_INVALID_ARG
