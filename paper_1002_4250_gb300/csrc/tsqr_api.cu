@@ -73,6 +73,11 @@ DeviceInfo device_info(int dev) {
     return d;
 }
 
+int current_sms() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess ? device_info(dev).sms : 0;
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
@@ -89,7 +94,8 @@ struct F64Plan {
     size_t smem = 0;
     TreeShape shape{};
     int64_t nodes = 0;
-    int gram_ctas = 0;             // TSQR_LEAF_GRAM: leaves of the Gram sum (0: no Gram)
+    int gram_ctas = 0;             // TSQR_LEAF_GRAM in one launch: leaves of the Gram sum (0: not)
+    bool gram_queue = false;       // TSQR_LEAF_GRAM by a queue, the Householder launch behind it
 };
 
 // Arguments of the Q^T apply for a factorization with storage `q` under plan p: B (m x ktot,
@@ -134,6 +140,7 @@ WyArgs wy_args(const F64Plan &p, const QStore &q, int64_t m, int n, int ldX, dou
     w.nchunks = (m + p.h - 1) / p.h;
     w.chunk_sc = q.chunk_sc;
     w.S = S;
+    w.skip = nullptr;
     return w;
 }
 
@@ -470,16 +477,18 @@ tsqr_status_t zero_r(double *R, int64_t n, int64_t ldr, cudaStream_t stream) {
     return TSQR_SUCCESS;
 }
 
-// The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to kGramMaxN columns.
+// The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to kGramRootMaxN columns.
 constexpr int64_t kGramMinRows = 1024;
 bool gram_fits(int64_t m, int64_t n) {
-    return n >= 1 && n <= kGramMaxN && m >= kGramMinRows && m >= 16 * n;
+    return n >= 1 && n <= kGramRootMaxN && m >= kGramMinRows && m >= 16 * n;
 }
+constexpr int kPanelsMinN = 56;
 
 // Plan of an FP64 R by one reduction: the exact-Gram reduction where it serves (AUTO, or a plan
 // that asks for TSQR_LEAF_GRAM), else the Householder leaves.  The Gram plan's other fields are
-// those of the Householder reduction the same launch falls back to: one CTA of 12 bulk warps
-// per SM, an even number of rows per lane (the kernel's inner block is two rows).
+// those of the Householder reduction it falls back to: up to kGramMaxN columns in the same
+// launch, one CTA of 12 bulk warps per SM with an even number of rows per lane (the kernel's
+// inner block is two rows); past that the AUTO plan's, in a launch of its own.
 tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
@@ -488,12 +497,19 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
         tuned.tree != TSQR_TREE_PANELS)
         over = &tuned;
     const bool asked = over && over->leaf == TSQR_LEAF_GRAM;
-    if (asked && (over->tree > TSQR_TREE_HYBRID || over->tree == TSQR_TREE_BINARY ||
-                  over->tree == TSQR_TREE_FLAT || !gram_fits(m, n)))
+    const bool serves = gram_fits(m, n) && n < kPanelsMinN;
+    if (asked && ((over->tree != TSQR_TREE_AUTO && over->tree != TSQR_TREE_HYBRID) || !serves))
         return TSQR_ERR_INVALID_ARG;
-    if (!asked && !(plan_is_auto(over) && gram_fits(m, n))) return plan_f64(m, n, over, p);
+    if (!asked && !(plan_is_auto(over) && serves)) return plan_f64(m, n, over, p);
     const DeviceInfo di = device_info(dev);
     if (di.sms <= 0) return TSQR_ERR_CUDA;
+    if (n > kGramMaxN) {
+        const tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, 0, 0, 0, 0};
+        const tsqr_status_t st = plan_f64(m, n, &fold, p);
+        p->leaf = TSQR_LEAF_GRAM;
+        p->gram_queue = true;
+        return st;
+    }
     p->tree = TSQR_TREE_HYBRID;
     p->leaf = TSQR_LEAF_GRAM;
     p->warps = kGramFoldWarps;
@@ -514,67 +530,120 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     return TSQR_SUCCESS;
 }
 
-// Inner nodes of the Gram sum's tree over `ctas` leaves.
-int64_t gram_inner_nodes(int64_t ctas) {
-    int64_t inner = 0;
-    for (int64_t c = ctas; c > 1;) {
-        c = (c + kGramArity - 1) / kGramArity;
-        inner += c;
-    }
-    return inner;
+// Workspace of a queued Gram sum of one matrix: the queue's counters (zeroed per call), then
+// tree slots.
+struct GramLayout {
+    int nb = 0, nset = 0, nslab = 0, inner = 0;
+    size_t words = 0, cnt_bytes = 0, bytes = 0;
+};
+// Slabs: about five items a CTA (the last wave stays short; an item's fixed cost, its pipeline's
+// start, the flush and the climb, is some 7 us), of at least 512 rows.
+GramLayout gram_layout(int64_t m, int64_t n, int sms) {
+    GramLayout w;
+    w.nb = (int)((n + 31) / 32);
+    w.nset = gram_sets(w.nb);
+    const int64_t nkb = (m + 63) / 64;
+    w.nslab = (int)std::max<int64_t>(1, std::min<int64_t>(5LL * sms / w.nset, nkb / 8));
+    w.inner = gram_inner_nodes(w.nslab);
+    w.words = 4 + (size_t)w.nset * w.inner;  // queue, failed, verdict, sets done, then the nodes
+    w.cnt_bytes = align_up(w.words * sizeof(unsigned int), 256);
+    w.bytes = w.cnt_bytes + (size_t)w.nset * (w.nslab + w.inner) * gram_slot_bytes(32);
+    return w;
+}
+// The Gram sum of [A | B] (B: columns na .. n-1, or none) and its factor R in the workspace at
+// base; *verdict: the device word that tells the launches behind it whether R is there.
+tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_t lda,
+                           const double *B, int64_t ldb, int64_t na, int64_t m, int64_t n,
+                           void *base, double *R, int64_t ldr, int *status,
+                           const unsigned int **verdict, cudaStream_t stream) {
+    if (cudaMemsetAsync(base, 0, w.words * sizeof(unsigned int), stream) != cudaSuccess)
+        return TSQR_ERR_CUDA;
+    unsigned int *head = (unsigned int *)base;
+    GramQueueArgs q;
+    std::memset(&q, 0, sizeof(q));
+    q.one.A = A;
+    q.one.B = B;
+    q.one.lda = lda;
+    q.one.ldb = ldb;
+    q.one.m = m;
+    q.one.n = (int)n;
+    q.one.na = (int)na;
+    q.one.nb = w.nb;
+    q.one.nslab = w.nslab;
+    q.one.nkb = (m + 63) / 64;
+    q.one.counters = head + 3;
+    q.one.slots = (unsigned char *)base + w.cnt_bytes;
+    q.one.verdict = head + 2;
+    q.one.R = R;
+    q.one.ldr = ldr;
+    q.nitems = w.nset * w.nslab;
+    q.queue = head;
+    q.failed = head + 1;
+    q.status = status;
+    *verdict = head + 2;
+    return gram_queue_launch(q, std::min(sms, q.nitems), stream) == cudaSuccess ? TSQR_SUCCESS
+                                                                               : TSQR_ERR_CUDA;
 }
 
-// Workspace of one reduction under plan p: counters (zeroed per call), then tree slots.
+// Workspace of one reduction under plan p: counters (zeroed per call), then tree slots, then the
+// Gram sum's.
 struct RLayout {
-    size_t cnt_words = 0, cnt_bytes = 0, bytes = 0;
+    size_t cnt_words = 0, cnt_bytes = 0, gram_off = 0, bytes = 0;
+    GramLayout g;
 };
-RLayout r_layout(const F64Plan &p, int64_t n) {
+RLayout r_layout(const F64Plan &p, int64_t m, int64_t n, int sms) {
     RLayout w;
     const size_t inner = p.gram_ctas ? (size_t)gram_inner_nodes(p.gram_ctas) : 0;
-    w.cnt_words = (size_t)p.nodes + (p.gram_ctas ? inner + 1 : 0);
+    w.cnt_words = (size_t)p.nodes + (p.gram_ctas ? inner + 2 : 0);
     w.cnt_bytes = align_up(w.cnt_words * sizeof(unsigned int), 256);
-    w.bytes = w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double);
-    if (p.gram_ctas)
-        w.bytes = align_up(w.bytes, 256) + (inner + p.gram_ctas) * gram_slot_bytes((int)n);
+    w.gram_off = align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
+    w.bytes = w.gram_off;
+    if (p.gram_ctas) w.bytes += (inner + p.gram_ctas) * gram_slot_bytes(gram_slot_block((int)n));
+    if (p.gram_queue) {
+        w.g = gram_layout(m, n, sms);
+        w.bytes += w.g.bytes;
+    }
     return w;
 }
 
-// One reduction of [A | B] (B: columns na .. n-1, or none) under plan p in the workspace at base
-// (r_layout(p, n).bytes), R to device memory.  Only the Gram plan takes a second matrix.
-tsqr_status_t enqueue_r(const F64Plan &p, const double *A, int64_t lda, const double *B,
-                        int64_t ldb, int64_t na, int64_t m, int64_t n, void *base, double *R,
-                        int64_t ldr, int *status, cudaStream_t stream) {
-    const RLayout w = r_layout(p, n);
+// One reduction of A under plan p in the workspace at base (r_layout's bytes), R to device
+// memory; the launches it takes are added to *launches.
+tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const double *A, int64_t lda,
+                        int64_t m, int64_t n, void *base, double *R, int64_t ldr, int *status,
+                        int *launches, cudaStream_t stream) {
     F64Args a = plan_args(p, A, m, n, lda);
     a.counters = (unsigned int *)base;
     a.slots = (double *)((char *)base + w.cnt_bytes);
     a.R = R;
     a.ldr = ldr;
     a.status = status;
+    if (p.gram_queue) {
+        const tsqr_status_t st = enqueue_gram(w.g, sms, A, lda, nullptr, 0, n, m, n,
+                                              (char *)base + w.gram_off, R, ldr, status, &a.skip, stream);
+        if (st != TSQR_SUCCESS) return st;
+        ++*launches;
+    }
     if ((p.gram_ctas ? gram_prepare((int)n, p.smem) : f64_prepare(p.smem)) != cudaSuccess)
         return TSQR_ERR_CUDA;
     if (cudaMemsetAsync(a.counters, 0, w.cnt_words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
+    ++*launches;
     if (!p.gram_ctas)
         return f64_launch(a, p.warps, p.smem, stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
     GramArgs g;
     std::memset(&g, 0, sizeof(g));
-    g.A = A;
-    g.B = B;
-    g.lda = lda;
-    g.ldb = ldb;
-    g.m = m;
-    g.n = (int)n;
-    g.na = (int)na;
-    g.ctas = p.gram_ctas;
-    g.nkb = (m + 63) / 64;
-    g.counters = a.counters + p.nodes;
-    g.verdict = g.counters + gram_inner_nodes(p.gram_ctas);
-    g.slots = (unsigned char *)base +
-              align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
-    g.slot_bytes = gram_slot_bytes((int)n);
-    g.R = R;
-    g.ldr = ldr;
+    g.p.A = A;
+    g.p.lda = lda;
+    g.p.m = m;
+    g.p.n = g.p.na = (int)n;
+    g.p.nb = 1;
+    g.p.nslab = p.gram_ctas;
+    g.p.nkb = (m + 63) / 64;
+    g.p.counters = a.counters + p.nodes;
+    g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas) + 1;
+    g.p.slots = (unsigned char *)base + w.gram_off;
+    g.p.R = R;
+    g.p.ldr = ldr;
     g.status = status;
     g.fold = a;
     cudaError_t e = gram_launch(g, p.smem, stream);
@@ -596,7 +665,6 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
 // leaves small and the updates blocked: 4,194,304 rows, n = 56 / 64 / 96 / 128: 775 / 828 /
 // 863 / 887 against 727 / 750 / 555 / 586 GFLOP/s (n = 48: 802 against 826, so one reduction
 // below 56).  Returns the panel width, or 0 for one reduction.
-constexpr int kPanelsMinN = 56;
 constexpr int kPanelsWidth = 16;
 
 int64_t panels_width(int64_t m, int64_t n, const tsqr_plan_t *over, int dev) {
@@ -636,12 +704,15 @@ tsqr_status_t run_f64(const double *A, int64_t m, int64_t n, int64_t lda, double
     tsqr_status_t st = plan_r(m, (int)n, over, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
+    const int sms = current_sms();
+    const RLayout w = r_layout(p, m, n, sms);
     Workspace *ws = nullptr;
-    st = get_workspace(stream, r_layout(p, n).bytes, &ws);
+    st = get_workspace(stream, w.bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
-    st = enqueue_r(p, A, lda, nullptr, 0, n, m, n, ws->base, R, ldr, ws->status, stream);
+    int launches = 0;
+    st = enqueue_r(p, w, sms, A, lda, m, n, ws->base, R, ldr, ws->status, &launches, stream);
     if (st != TSQR_SUCCESS) return st;
-    g_last_launches = 1;
+    g_last_launches = launches;
     return TSQR_SUCCESS;
 }
 
@@ -883,7 +954,9 @@ tsqr_status_t run_f64_host(const double *A, int64_t m, int64_t n, int64_t lda, d
     tsqr_status_t st = plan_r(m, (int)n, nullptr, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
-    const size_t r_off = align_up(r_layout(p, n).bytes, 256);
+    const int sms = current_sms();
+    const RLayout w = r_layout(p, m, n, sms);
+    const size_t r_off = align_up(w.bytes, 256);
     const size_t r_bytes = align_up((size_t)n * (size_t)n * sizeof(double), 256);
     const size_t a_bytes = Amapped ? 0 : (size_t)m * (size_t)n * sizeof(double);
     Workspace *ws = nullptr;
@@ -902,13 +975,14 @@ tsqr_status_t run_f64_host(const double *A, int64_t m, int64_t n, int64_t lda, d
         Ain = Ad;
         ld_in = m;
     }
-    st = enqueue_r(p, Ain, ld_in, nullptr, 0, n, m, n, base, Rd, n, ws->status, stream);
+    int launches = 0;
+    st = enqueue_r(p, w, sms, Ain, ld_in, m, n, base, Rd, n, ws->status, &launches, stream);
     if (st != TSQR_SUCCESS) return st;
     if (cudaMemcpy2DAsync(R, (size_t)ldr * sizeof(double), Rd, (size_t)n * sizeof(double),
                           (size_t)n * sizeof(double), (size_t)n, cudaMemcpyDeviceToHost,
                           stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    g_last_launches = 1;
+    g_last_launches = launches;
     return TSQR_SUCCESS;
 }
 
@@ -1245,19 +1319,23 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
     const DeviceInfo di = device_info(dev);
-    if (N <= nb && plan_is_auto(over) && gram_fits(m, N)) {  // one panel: tsqr_r's reduction
+    if (N <= nb && plan_is_auto(over) && gram_fits(m, N) && N < kPanelsMinN) {  // one panel: tsqr_r's reduction
         F64Plan p;
         tsqr_status_t st = plan_r(m, (int)N, over, &p);
         if (st != TSQR_SUCCESS) return st;
+        const RLayout w = r_layout(p, m, N, di.sms);
         Workspace *ws = nullptr;
-        st = get_workspace(stream, r_layout(p, N).bytes, &ws);
+        st = get_workspace(stream, w.bytes, &ws);
         if (st != TSQR_SUCCESS) return st;
-        st = enqueue_r(p, A, lda, nullptr, 0, N, m, N, ws->base, R, ldr, ws->status, stream);
+        int launches = 0;
+        st = enqueue_r(p, w, di.sms, A, lda, m, N, ws->base, R, ldr, ws->status, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
         g_last_plan = public_plan(p);
-        g_last_launches = 1;
+        g_last_launches = launches;
         return TSQR_SUCCESS;
     }
+    // by panels of the default width: the Gram sum first, the panels behind it
+    const bool gram = nb == 16 && plan_is_auto(over) && gram_fits(m, N);
     std::vector<CaqrPanel> panels;
     int64_t M = m;
     size_t max_fsmem = 0, max_qt = 0;
@@ -1371,10 +1449,20 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     constexpr int kBufs = sizeof(sizes) / sizeof(sizes[0]);
     size_t total = 0;
     for (size_t b : sizes) total += align_up(b, 256);
+    GramLayout gl;
+    if (gram) gl = gram_layout(m, N, di.sms);
     Workspace *ws = nullptr;
-    tsqr_status_t st = get_workspace(stream, total, &ws);
+    tsqr_status_t st = get_workspace(stream, total + gl.bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
     char *base = (char *)ws->base;
+    int launches = 0;
+    const unsigned int *skip = nullptr;
+    if (gram) {
+        st = enqueue_gram(gl, di.sms, A, lda, nullptr, 0, N, m, N, base + total, R, ldr, ws->status,
+                          &skip, stream);
+        if (st != TSQR_SUCCESS) return st;
+        ++launches;
+    }
     void *bufs[kBufs];
     size_t o = 0;
     for (int i = 0; i < kBufs; ++i) {
@@ -1386,11 +1474,13 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     double *nV = (double *)bufs[4], *nsc = (double *)bufs[5], *signs = (double *)bufs[6];
     unsigned int *qcounters = (unsigned int *)bufs[7];
     double *qslots = (double *)bufs[8], *C = (double *)bufs[9], *wyS = (double *)bufs[10];
-    // R's rows below each diagonal block stay zero; the kernels write the rest
-    if (cudaMemset2DAsync(R, (size_t)ldr * sizeof(double), 0, (size_t)N * sizeof(double),
-                          (size_t)N, stream) != cudaSuccess)
+    // R's rows below each diagonal block stay zero; the kernels write the rest (behind a Gram
+    // sum, whose R must stay, they are its root's zeros or a kernel's)
+    if (gram ? zero_lower_launch(R, ldr, (int)N, skip, stream) != cudaSuccess
+             : cudaMemset2DAsync(R, (size_t)ldr * sizeof(double), 0, (size_t)N * sizeof(double),
+                                 (size_t)N, stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    int launches = 0;
+    launches += gram ? 1 : 0;
     for (size_t pi = 0; pi < panels.size(); ++pi) {
         const CaqrPanel &c = panels[pi];
         // the panel's matrix: A itself for the first panel, then C (column j of the matrix is
@@ -1403,6 +1493,7 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
         a.R = R + c.j0 + c.j0 * ldr;
         a.ldr = ldr;
         a.status = ws->status;
+        a.skip = skip;
         a.q.V = V;
         a.q.ldv = c.M;
         a.q.chunk_sc = csc;
@@ -1417,6 +1508,7 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
         const int64_t trail = N - c.j0 - c.w;
         if (trail == 0) break;
         QtArgs t = qt_args(c.p, a.q, c.M, c.w, src + c.w * lds, lds, c.kc, (int)trail);
+        t.skip = skip;
         t.slots = qslots;
         t.counters = qcounters;
         t.C = R + c.j0 + (c.j0 + c.w) * ldr;
@@ -1429,7 +1521,8 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
                             stream) != cudaSuccess)
             return TSQR_ERR_CUDA;
         if (c.wy) {
-            const WyArgs wa = wy_args(c.p, a.q, c.M, c.w, c.ldX, wyS);
+            WyArgs wa = wy_args(c.p, a.q, c.M, c.w, c.ldX, wyS);
+            wa.skip = skip;
             t.wyS = wyS;
             const int grid = (int)std::min<int64_t>(wa.nchunks, 4LL * di.sms);
             if (wy_launch(wa, c.wy_smem, grid, stream) != cudaSuccess ||

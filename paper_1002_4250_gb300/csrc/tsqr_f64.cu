@@ -6,6 +6,7 @@ namespace tsqr {
 
 template <int B>
 __global__ void __launch_bounds__(416, 1) tsqr_f64_kernel(const F64Args a) {
+    if (skipped(a.skip)) return;
     // one row per lane (B = 1): the software-pipelined sweep hides the shared-memory latency
     // a single block per item exposes (measured +3% at n = 64); taller lanes keep the plain
     // loop, which measured faster there
@@ -44,6 +45,16 @@ __global__ void __launch_bounds__(288, 1) tsqr_f64_combine_kernel(int n, const d
         store_packed(Rp, n, R, ldr);
 }
 
+// The strict lower triangle of R (n x n) zeroed.
+__global__ void tsqr_zero_lower_kernel(double *R, int64_t ldr, int n, const unsigned int *skip) {
+    if (skipped(skip)) return;
+    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < (int64_t)n * n;
+         o += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t col = o / n, row = o - col * n;
+        if (row > col) R[row + col * ldr] = 0.0;
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // host-side launchers
 // ------------------------------------------------------------------------------------------
@@ -76,6 +87,13 @@ cudaError_t f64_launch(const F64Args &a, int warps, size_t smem_bytes, cudaStrea
         case 2: tsqr_f64_kernel<2><<<grid, block, smem_bytes, stream>>>(a); break;
         default: tsqr_f64_kernel<1><<<grid, block, smem_bytes, stream>>>(a); break;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t zero_lower_launch(double *R, int64_t ldr, int n, const unsigned int *skip,
+                              cudaStream_t stream) {
+    const int64_t blocks = ((int64_t)n * n + 1023) / 1024;
+    tsqr_zero_lower_kernel<<<(int)(blocks < 512 ? blocks : 512), 1024, 0, stream>>>(R, ldr, n, skip);
     return cudaGetLastError();
 }
 

@@ -66,7 +66,13 @@ struct F64Args {
     int64_t ldr;
     int *status;            // device status word (TSQR_STATUS_NONFINITE is or-ed in)
     QStore q;               // reflector storage (tsqr_qr's factorization only)
+    const unsigned int *skip;  // when *skip == 1 the launch has nothing to do (null: never)
 };
+
+// A launch that stands behind another way to the same result: *skip == 1 once that succeeded.
+#ifdef __CUDACC__
+__device__ __forceinline__ bool skipped(const unsigned int *skip) { return skip && *skip == 1u; }
+#endif
 
 // Mixed-precision kernel arguments: the FP64 arguments (base.A unused) plus A of another
 // type, and the FP64 view of the S region used by the tree operator.

@@ -10,8 +10,12 @@
 // rounding is that of the input's fixed-point form and of R's entries.
 //
 // The tree of Section 2 is the sum over the row blocks.  A matrix this form cannot serve (a
-// non-finite or extreme entry, a pivot below 2^-kGramPivotBits of its column's square) is found
-// by the root, and the same launch then runs the Householder reduction instead.
+// non-finite or extreme entry, a pivot below 2^-bits of its column's square) is found by the
+// root, and the Householder reduction then runs instead.
+//
+// Columns are taken in blocks of NB (32 for FP64, 64 for FP32 and BF16): a column set is a block
+// against itself or a block against a later one, and a work item is one set over one slab of
+// rows.
 #pragma once
 
 #include "tsqr_f64.cuh"
@@ -22,30 +26,59 @@ constexpr int kGramThreads = 512;
 constexpr int kGramWarps = kGramThreads / 32;
 constexpr int kGramFoldWarps = 12;  // bulk warps of the Householder reduction (and its reducer)
 constexpr int kGramArity = 16;      // children per node of the Gram sum's tree
-constexpr int kGramMaxN = 32;
+constexpr int kGramMaxN = 32;       // one column block: tsqr_r's single launch
+constexpr int kGramRootMaxN = 128;  // widest matrix one CTA factors
 
-struct GramArgs {
-    const void *A;         // m x na, leading dimension lda
-    const void *B;         // columns na .. n-1 (a second matrix beside A; null when na == n)
+// One matrix [A | B] (B: columns na .. n-1, or none) and where its sums go.
+struct GramProblem {
+    const void *A, *B;
     int64_t lda, ldb, m;
     int n, na;
-    int ctas;              // leaves: CTA c sums 64-row blocks [c nkb / ctas, (c+1) nkb / ctas)
+    int nb;                // column blocks; sets 0 .. nb-1 are a block against itself, then (0, 1),
+                           // (0, 2), (1, 2), (0, 3), ...
+    int nslab;             // slabs of rows: slab s holds 64-row blocks [s nkb / nslab, ...)
     int64_t nkb;           // ceil(m / 64)
-    unsigned int *counters;  // one per inner tree node, then the verdict word; zeroed per call
-    unsigned int *verdict;   // 0: not decided; 1: R is written; 2: run the Householder reduction
-    unsigned char *slots;    // one slot per tree node
-    size_t slot_bytes;
+    unsigned int *counters;  // per set: the tree's inner nodes; then one for the sets; zeroed
+    unsigned char *slots;    // per set: one slot per tree node
+    unsigned int *verdict;   // 0: not decided; 1: R is written; 2: the Householder reduction runs
     double *R;
     int64_t ldr;
+};
+
+struct GramArgs {          // tsqr_r's single launch: one problem of one column block
+    GramProblem p;
     int *status;
     F64Args fold;          // the Householder reduction (its A is FP64; nleaves <= grid)
 };
 
-// Slot of a node: 128 column exponents (the last int: non-zero for a leaf that cannot be
-// served), then the n (n + 1) / 2 sums (128-bit, (i, j) with i <= j at j (j + 1) / 2 + i).
+struct GramQueueArgs {     // a queue of work items
+    GramProblem one;       // the problem when probs is null
+    const GramProblem *probs;
+    const int2 *items;     // (problem, set + nsets slab) in the order they are taken; null: item
+                           // k of the one problem is set k % nsets of slab k / nsets
+    int nitems;
+    unsigned int *queue;   // next item, zeroed per call
+    unsigned int *failed;  // problems left to the Householder reduction, zeroed per call
+    int *status;
+};
+
+// Inner nodes and all nodes of the sum's tree over `leaves` leaves.
+__host__ __device__ inline int gram_inner_nodes(int leaves) {
+    int inner = 0;
+    for (int c = leaves; c > 1;) {
+        c = (c + kGramArity - 1) / kGramArity;
+        inner += c;
+    }
+    return inner;
+}
+__host__ __device__ inline int gram_sets(int nb) { return nb * (nb + 1) / 2; }
+
+// Slot of a node: 143 column exponents (block I's from 0, block J's from 64), a word that is
+// non-zero where a leaf cannot be served, then the sums (128-bit): (i, j) with i <= j at
+// j (j + 1) / 2 + i for a block against itself, i nj + j for two blocks.
 constexpr int kGramSlotHead = 576;
-inline size_t gram_slot_bytes(int n) {
-    return ((size_t)kGramSlotHead + (size_t)n * (n + 1) / 2 * 16 + 255) / 256 * 256;
+__host__ __device__ inline size_t gram_slot_bytes(int block) {  // block: columns of a block
+    return (size_t)kGramSlotHead + (size_t)block * block * 16;
 }
 
 }  // namespace tsqr

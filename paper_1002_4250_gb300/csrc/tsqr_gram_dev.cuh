@@ -1,0 +1,945 @@
+// Device code of the exact-Gram reduction (tsqr_gram.cuh has the method): digits of a slab of
+// rows into tensor-core operands, their exact sums, the tree over the slabs, and the
+// fixed-point Cholesky factor of the whole.
+#pragma once
+
+#include <cuda_bf16.h>
+#include <type_traits>
+
+#include "tsqr_fold.cuh"
+#include "tsqr_gram.cuh"
+#include "tsqr_tc.cuh"
+
+namespace tsqr {
+namespace gram {
+
+typedef unsigned long long u64;
+typedef __int128 i128;
+typedef unsigned __int128 u128;
+
+// Input types: S digits a column, the block of columns, the least pivot a column may keep
+// (relative to its square), the exponents its largest entry may have (biased; outside, squares
+// leave the range of the Householder leaves' arithmetic, which then decide what R is), and the
+// power of two of a whole number's unit for exponent word D (x = Q 2^(D + kUnit), Q in the
+// 64-bit form of eight digits).
+template <typename Tin>
+struct Type;
+template <>
+struct Type<double> {
+    static constexpr int kDigits = 8, kBlock = 32, kPivotBits = 64;
+    static constexpr int kExpLo = 1023 - 400, kExpHi = 1023 + 400, kUnit = -1086;
+};
+template <>
+struct Type<float> {
+    static constexpr int kDigits = 4, kBlock = 64, kPivotBits = 44;
+    static constexpr int kExpLo = 127 - 55, kExpHi = 127 + 55, kUnit = -190;
+};
+template <>
+struct Type<__nv_bfloat16> {
+    static constexpr int kDigits = 3, kBlock = 64, kPivotBits = 36;
+    static constexpr int kExpLo = 127 - 55, kExpHi = 127 + 55, kUnit = -190;
+};
+
+constexpr int cmin(int a, int b) { return a < b ? a : b; }
+constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int up16(int a) { return (a + 15) / 16 * 16; }
+
+// Shape of a column set: NI columns against themselves (NJ = 0), or against NJ others.
+// Operand rows: digit s of column i at s NI + i, then digit t of column j at S NI + t NJ + j.
+template <typename Tin, int NI, int NJ>
+struct Shape {
+    static constexpr int S = Type<Tin>::kDigits;
+    static constexpr bool kCross = NJ > 0;
+    static constexpr int MN = S * (NI + NJ);
+    // Row tiles of 128 accumulator lanes: TS digits of the NI columns each.  A block against
+    // itself needs a second tile only for its low digits against each other, (s, t) and (t, s)
+    // being mirrors: tile 1 takes digits TS .. S-1 against TS .. TE-1 (FP64: digits 4 to 7 against
+    // 4 and 5; what is left out, both digits 6 or 7, is below 2^-96 of the product).
+    static constexpr int TS = !kCross && S == 8 && NI > 16 ? 4 : cmin(S, 128 / NI);
+    static constexpr int kTiles = TS < S ? 2 : 1;
+    static constexpr int TE = kCross || kTiles == 1 ? S : S == 8 ? 6 : S;
+    static constexpr int NR = kCross ? NJ : NI;            // columns of a right-hand digit
+    static constexpr int N0 = up16(S * NR);
+    static constexpr int N1 = kTiles == 1 ? 0 : kCross ? N0 : up16((TE - TS) * NI);
+    static constexpr int kCols = N0 + N1;                  // tensor-memory columns
+    static constexpr int kSets = cmin(8, 512 / kCols);     // accumulator sets, 1,024 rows each
+    static_assert(kCols <= 512 && (kTiles == 1 || 2 * TS >= S), "accumulators fit");
+    // Slicing: a task is four columns of a 64-row block, a warp's round has kTasks of them.
+    static constexpr int kGroups = (NI + NJ) / 4;
+    static constexpr int kMaxTasks = sizeof(Tin) == 8 ? 1 : MN > 192 ? 1 : 2;
+    static constexpr int kRoundKb = cmin(16, kMaxTasks * kGramWarps / kGroups);
+    static constexpr int kSlots = kRoundKb * kGroups;      // tasks of a round
+    static constexpr int kTasks = (kSlots + kGramWarps - 1) / kGramWarps;
+    static_assert(kRoundKb >= 1 && kGroups <= kMaxTasks * kGramWarps, "a block a round");
+    static constexpr int kKbBytes = MN * 128;              // 64 FP16 per operand row
+    static constexpr int kStage = kRoundKb * kKbBytes;
+    // A task's raw bytes: a lane's eight entries; BF16 keeps 16 more a column (entries that
+    // are not 16-byte aligned straddle two pieces).
+    static constexpr int kTaskRaw = sizeof(Tin) == 2 ? 576 : 256 * (int)sizeof(Tin);
+    static constexpr int kRaw = kGramWarps * kTasks * kTaskRaw;
+    static constexpr int kRaws = cmin(8, 65536 / kRaw);    // rounds on their way
+    static_assert(kRaws >= 2, "a round is copied while another is sliced");
+    // Flush: partial sums (64-bit) of JP columns at a time over the stages, [part][row digit][j]
+    // [i]; parts: digits t < TA of tile 0 (or of the cross tiles), the others.
+    static constexpr int TA = kCross || kTiles == 1 ? cmin(4, S) : TS;
+    static constexpr bool kMirror = !kCross && kTiles == 2;
+    static constexpr int kParts = TA < S ? 2 : 1;
+    static constexpr int kRowDigits = kCross ? S : cmin(TS, S);
+    static constexpr int kLd = NI + 1;
+    static constexpr int per_j() {
+        return (kRowDigits * kParts + (kMirror ? S - TS : 0)) * kLd * 8;
+    }
+    static constexpr int kStages = 2 * kStage;
+    static constexpr int jp() {
+        int j = NR;
+        while (j * per_j() > kStages) j = (j / 2 + 7) / 8 * 8;
+        return j;
+    }
+    static constexpr int JP = jp();
+    static_assert(JP % 8 == 0 && NR % JP == 0 && JP * per_j() <= kStages, "flush buffers");
+    static constexpr int kU = NI * NR * 16;                // the 128-bit sums
+};
+
+struct alignas(16) Smem {   // beside the stages
+    uint64_t bar[2];
+    uint32_t tmem;
+    int flag, bad, item;
+    int D[128], E[128], Dnew[128];
+};
+
+// Shared memory: Smem, stages, raw rounds, U.  (Tile reads past the last operand row fall into
+// the raw rounds: rows and columns that no one reads back.)
+constexpr int kHead = 2048;
+static_assert(sizeof(Smem) <= kHead, "the stages start at a multiple of 1,024 bytes");
+template <typename Sh>
+constexpr size_t smem_bytes() {
+    return kHead + Sh::kStages + cmax(Sh::kRaws * Sh::kRaw, 16384) + Sh::kU;
+}
+
+// ------------------------------------------------------------------------------------------
+// Digits.  One entry in fixed point: |x| = Q units, d = D - exponent >= 2 (so Q fills at most
+// 62 of 64 bits, 30 of 32), plus 128 in every byte: byte k minus 128 is then the balanced digit
+// of weight 256^k.  (A shift by the word's size or more gives 0: zero and subnormal entries.)
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ u64 fix64(const double x, const int D, int &dmin) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const int d = D - ((hi >> 20) & 0x7ff);
+    dmin = min(dmin, d);
+    const u64 mant = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 43) | ((u64)(unsigned)lo << 11);
+    u64 q;
+    asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(mant), "r"((unsigned)d));
+    return q + 0x8080808080808080ull;
+}
+__device__ __forceinline__ uint32_t fix32(const uint32_t b, const int D, int &dmin) {
+    const int d = D - (int)((b >> 23) & 0xff);
+    dmin = min(dmin, d);
+    const uint32_t mant = ((b & 0x7fffff) | 0x800000) << 8;
+    uint32_t q;
+    asm("shr.u32 %0, %1, %2;" : "=r"(q) : "r"(mant), "r"((unsigned)d));
+    return q + 0x80808080u;
+}
+__device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// The four digits (FP16 pairs of two rows) of a 32-bit word of each row, most significant
+// first: a byte b under 0x64 is the FP16 1024 + b; sgn (1024 + b) - sgn 1152 is the signed digit.
+__device__ __forceinline__ void digits4(const uint32_t w0, const uint32_t w1, const uint32_t sgn,
+                                        const uint32_t off, uint32_t &s0, uint32_t &s1,
+                                        uint32_t &s2, uint32_t &s3) {
+    const uint32_t t = __byte_perm(w0, w1, 0x6273), b = __byte_perm(w0, w1, 0x4051);
+    s0 = hfma2_u(__byte_perm(t, 0x64646464u, 0x4140), sgn, off);
+    s1 = hfma2_u(__byte_perm(t, 0x64646464u, 0x4342), sgn, off);
+    s2 = hfma2_u(__byte_perm(b, 0x64646464u, 0x4140), sgn, off);
+    s3 = hfma2_u(__byte_perm(b, 0x64646464u, 0x4342), sgn, off);
+}
+
+// ------------------------------------------------------------------------------------------
+// Rows of a lane in a 64-row block: E = 16 / sizeof(Tin) consecutive rows at 8 E q + E c8 (eight
+// lanes read 128 consecutive bytes), the same for every column: the operand's rows are the
+// block's in another order, which the sums do not see.  A 16-byte piece q of the lane goes to
+// raw + 512 q (raw: the lane's), FP64 and FP32 in narrow copies where A is not 16-byte aligned.
+// BF16 copies aligned pieces always (144 bytes a column; the ninth piece by the last lane) and
+// reads its entries at the column's offset in them.  Rows past the end read as zeros.
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ void copy16(void *dst, const void *src, const int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(tc::smem_u32(dst)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
+template <typename Tin>
+__device__ __forceinline__ void copy_rows(unsigned char *raw, const Tin *p, const int64_t left,
+                                          const int c8, const bool vec, const void *any) {
+    if constexpr (sizeof(Tin) == 2) {
+        const uintptr_t first = (uintptr_t)p, base = first & ~(uintptr_t)15;
+        const uintptr_t end = left <= 0 ? 0 : first + 2 * (uintptr_t)(left < 64 ? left : 64);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q == 1 && (c8 != 7 || first == base)) break;
+            const uintptr_t at = base + 16 * (c8 + q);
+            const int bytes = at >= end ? 0 : end - at >= 16 ? 16 : (int)(end - at);
+            copy16(raw + 16 * q, bytes ? (const void *)at : any, bytes);
+        }
+    } else {
+        constexpr int E = 16 / (int)sizeof(Tin);
+        if (left >= 64 && vec) {
+#pragma unroll
+            for (int q = 0; q < 8 / E; ++q) copy16(raw + 512 * q, p + 8 * E * q + E * c8, 16);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int r = 8 * E * (e / E) + E * c8 + e % E;
+                unsigned char *to = raw + 512 * (e / E) + (int)sizeof(Tin) * (e % E);
+                if constexpr (sizeof(Tin) == 8)
+                    cp_async8(to, r < left ? p + r : any, r < left ? 8 : 0);
+                else
+                    cp_async4(to, r < left ? p + r : any, r < left ? 4 : 0);
+            }
+        }
+    }
+}
+// The lane's FP32 bit patterns (FP32 and BF16).  off: the column's byte offset in its 16-byte pieces.
+template <typename Tin>
+__device__ __forceinline__ void read_words(uint32_t (&w)[8], const unsigned char *raw, const int off) {
+    if constexpr (sizeof(Tin) == 4) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint4 t = *reinterpret_cast<const uint4 *>(raw + 512 * q);
+            w[4 * q] = t.x, w[4 * q + 1] = t.y, w[4 * q + 2] = t.z, w[4 * q + 3] = t.w;
+        }
+    } else if (off == 0) {
+        const uint4 t = *reinterpret_cast<const uint4 *>(raw);
+        const uint32_t v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[2 * q] = v[q] << 16, w[2 * q + 1] = v[q] & 0xffff0000u;
+    } else {
+        const unsigned short *h = reinterpret_cast<const unsigned short *>(raw + off);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = (uint32_t)h[e] << 16;
+    }
+}
+// Largest biased exponent of the lane's eight entries.
+template <typename Tin>
+__device__ __forceinline__ int max_exponent(const unsigned char *raw, const int off) {
+    int e = 0;
+    if constexpr (sizeof(Tin) == 8) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
+            e = max(e, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+        }
+    } else {
+        uint32_t w[8];
+        read_words<Tin>(w, raw, off);
+#pragma unroll
+        for (int p = 0; p < 8; ++p) e = max(e, (int)((w[p] >> 23) & 0xff));
+    }
+    return e;
+}
+// The lane's eight entries as digits: digit s to dst + s step.
+template <typename Tin>
+__device__ __forceinline__ void slice8(const unsigned char *raw, const int off, const int D,
+                                       int &dmin, unsigned char *dst, const int step) {
+    constexpr int S = Type<Tin>::kDigits;
+    uint32_t o[8][4];
+    if constexpr (sizeof(Tin) == 8) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
+            const u64 q0 = fix64(v.x, D, dmin), q1 = fix64(v.y, D, dmin);
+            const uint32_t sg =
+                __byte_perm(__double2hiint(v.x), __double2hiint(v.y), 0x7632) & 0x80008000u;
+            const uint32_t sgn = sg | 0x3c003c00u, of = sg ^ 0xe480e480u;
+            digits4((uint32_t)(q0 >> 32), (uint32_t)(q1 >> 32), sgn, of, o[0][p], o[1][p], o[2][p],
+                    o[3][p]);
+            digits4((uint32_t)q0, (uint32_t)q1, sgn, of, o[4][p], o[5][p], o[6][p], o[7][p]);
+        }
+    } else {
+        uint32_t w[8];
+        read_words<Tin>(w, raw, off);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t q0 = fix32(w[2 * p], D, dmin), q1 = fix32(w[2 * p + 1], D, dmin);
+            const uint32_t sg = __byte_perm(w[2 * p], w[2 * p + 1], 0x7632) & 0x80008000u;
+            const uint32_t sgn = sg | 0x3c003c00u, of = sg ^ 0xe480e480u;
+            digits4(q0, q1, sgn, of, o[0][p], o[1][p], o[2][p], o[3][p]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+        *reinterpret_cast<uint4 *>(dst + s * step) = make_uint4(o[s][0], o[s][1], o[s][2], o[s][3]);
+}
+
+// ------------------------------------------------------------------------------------------
+// 128-bit integers
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ i128 shr128(const i128 x, const int s) {
+    return s == 0 ? x : s >= 127 ? (x < 0 ? (i128)-1 : (i128)0) : x >> s;
+}
+__device__ __forceinline__ i128 shift128(const i128 x, const int s) {  // left for s > 0
+    return s >= 0 ? (i128)((u128)x << (s > 127 ? 127 : s)) : shr128(x, -s);
+}
+struct alignas(16) Q128 {
+    u64 lo, hi;
+};
+__device__ __forceinline__ i128 unpack(const Q128 q) { return (i128)(((u128)q.hi << 64) | q.lo); }
+__device__ __forceinline__ Q128 pack(const i128 x) {
+    Q128 q;
+    q.lo = (u64)x;
+    q.hi = (u64)((u128)x >> 64);
+    return q;
+}
+__device__ __forceinline__ i128 ldcg128(const void *p) {
+    const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2 *>(p));
+    return (i128)(((u128)t.y << 64) | t.x);
+}
+// (i, j), i <= j, of packed index o = j (j + 1) / 2 + i.
+__device__ __forceinline__ void unpack_index(const int o, int &i, int &j) {
+    j = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
+    while ((j + 1) * (j + 2) / 2 <= o) ++j;
+    while (j * (j + 1) / 2 > o) --j;
+    i = o - j * (j + 1) / 2;
+}
+
+// ------------------------------------------------------------------------------------------
+// One work item's view of the CTA: shared memory, tensor memory and the barriers' state.
+// ------------------------------------------------------------------------------------------
+struct Cta {
+    Smem *sm;
+    Q128 *U;           // the current item's sums
+    unsigned char *stages;
+    uint32_t tmem;
+    uint32_t par[2];   // parity of the next completion of each stage's barrier
+    bool ok;           // no wait has given up
+};
+template <typename Sh>
+__device__ __forceinline__ Q128 *sums_of(const Cta &c) {
+    return reinterpret_cast<Q128 *>(c.stages + Sh::kStages + cmax(Sh::kRaws * Sh::kRaw, 16384));
+}
+
+// Columns of an item: local column l < NI is column i0 + l of the matrix (l < ni), NI + l is j0 + l.
+struct Cols {
+    int i0, ni, j0, nj;
+};
+
+// The sums of one set over the 64-row blocks [kb0, kb1): in c.U (the lower half of a block
+// against itself holds what its mirror adds), exponents in sm.D, sm.bad where the rows cannot be
+// served.  Every thread of the CTA; all copies and tensor-core work have ended on return.
+template <typename Tin, int NI, int NJ>
+__device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, const int64_t kb0,
+                                         const int64_t kb1, Cta &c) {
+    using Sh = Shape<Tin, NI, NJ>;
+    using Ty = Type<Tin>;
+    constexpr int S = Sh::S;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    Smem &sm = *c.sm;
+    c.U = sums_of<Sh>(c);
+    if (tid == 0) sm.bad = 0;
+    if (tid < 128) sm.D[tid] = sm.E[tid] = 0;
+    for (int o = tid; o < NI * Sh::NR; o += kGramThreads) c.U[o] = Q128{0, 0};
+
+    const int rounds = (int)((kb1 - kb0 + Sh::kRoundKb - 1) / Sh::kRoundKb);
+    const Tin *A = (const Tin *)p.A, *B = (const Tin *)p.B;
+    constexpr int kAlign = 16 / (int)sizeof(Tin);
+    const bool vec = ((p.lda | (B ? p.ldb : 0)) & (kAlign - 1)) == 0 &&
+                     (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+    const int c8 = lane & 7;
+
+    // the lane's column, block and operand address in each of its tasks
+    struct Task {
+        const Tin *src;
+        int kbo, lc, dst, off;
+        bool mine;
+    };
+    Task tk[Sh::kTasks];
+#pragma unroll
+    for (int t = 0; t < Sh::kTasks; ++t) {
+        const int id = warp + t * kGramWarps;
+        tk[t].kbo = id / Sh::kGroups;
+        const int lc = 4 * (id % Sh::kGroups) + (lane >> 3);
+        const bool right = NJ > 0 && lc >= NI;
+        const int g = right ? cols.j0 + lc - NI : cols.i0 + lc;
+        tk[t].lc = lc;
+        tk[t].mine = id < Sh::kSlots && (right ? lc - NI < cols.nj : lc < cols.ni);
+        tk[t].src = (g < p.na ? A + (int64_t)g * p.lda : B + (int64_t)(g - p.na) * p.ldb) +
+                    (kb0 + tk[t].kbo) * 64;
+        tk[t].off = sizeof(Tin) == 2 ? (int)((uintptr_t)tk[t].src & 15) : 0;
+        const int row = right ? S * NI + lc - NI : lc;  // of digit 0; the others 8-row atoms away
+        tk[t].dst = tk[t].kbo * Sh::kKbBytes + (row >> 3) * 1024 + (row & 7) * 128 +
+                    ((c8 ^ (row & 7)) << 4);
+    }
+    unsigned char *const raw0 = c.stages + Sh::kStages + warp * Sh::kTasks * Sh::kTaskRaw +
+                                (sizeof(Tin) == 2 ? (lane >> 3) * 144 + c8 * 16 : lane * 16);
+    auto raw_of = [&](const int r, const int t) {
+        return raw0 + (r % Sh::kRaws) * Sh::kRaw + t * Sh::kTaskRaw;
+    };
+    // Round r of A on its way to shared memory (one cp.async group a round, empty at the end).
+    auto load_round = [&](const int r) {
+        if (r < rounds) {
+#pragma unroll
+            for (int t = 0; t < Sh::kTasks; ++t)
+                if (tk[t].mine) {
+                    const int64_t kb = kb0 + tk[t].kbo + (int64_t)r * Sh::kRoundKb;
+                    copy_rows<Tin>(raw_of(r, t), tk[t].src + (int64_t)r * (64 * Sh::kRoundKb),
+                                   kb < kb1 ? p.m - kb * 64 : 0, c8, vec, A);
+                }
+        }
+        cp_async_commit();
+    };
+    // The column exponents block kb of round r (64 rows) needs, to sm.Dnew: a column whose largest
+    // entry there is out of its range gets that entry's exponent and two bits to spare, the others
+    // keep theirs.  A column's exponents so follow from its slab alone, whatever set it is in: the
+    // sets of a matrix sum the digits of one and the same matrix.  True if any column changes.
+    auto scan_block = [&](const int r, const int kb) {
+#pragma unroll
+        for (int t = 0; t < Sh::kTasks; ++t) {
+            const bool here = tk[t].mine && tk[t].kbo == kb;
+            int e = here ? max_exponent<Tin>(raw_of(r, t), tk[t].off) : 0;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+            if (c8 == 0 && here) atomicMax(&sm.E[tk[t].lc], e);
+        }
+        __syncthreads();
+        bool up = false;
+        if (tid < NI + NJ) {
+            const int e = sm.E[tid];
+            if (e > Ty::kExpHi) sm.bad = 1;
+            up = e + 2 > sm.D[tid];
+            sm.Dnew[tid] = up ? max(e, Ty::kExpLo) + 4 : sm.D[tid];
+            sm.E[tid] = 0;
+        }
+        return __syncthreads_or(up) != 0;
+    };
+    auto zero_stages = [&]() {  // columns past the matrix's read as zeros
+        for (int i = tid; i < Sh::kStages / 16; i += kGramThreads)
+            reinterpret_cast<uint4 *>(c.stages)[i] = make_uint4(0, 0, 0, 0);
+        tc::fence_proxy_async();
+        __syncthreads();
+    };
+    const bool padded = cols.ni < NI || cols.nj < NJ;
+
+    constexpr uint32_t idesc0 = tc::instr_desc(0, 128, Sh::N0, false, false);
+    constexpr uint32_t idesc1 = Sh::kTiles == 2 ? tc::instr_desc(0, 128, Sh::N1, false, false) : 0;
+    const uint32_t sbase = tc::smem_u32(c.stages);
+    bool pend[2] = {false, false};
+    int sets = 0, in_set = 0;  // accumulator sets begun, 64-row blocks in the current one
+    auto wait_stage = [&](const int b) {
+        if (pend[b]) {
+            c.ok &= tc::mbar_wait(&sm.bar[b], c.par[b], 1LL << 24);
+            c.par[b] ^= 1;
+            pend[b] = false;
+        }
+    };
+
+    // Accumulators into U: every digit product's sum, weighted.  All tensor-core work is waited
+    // for; the stages are free on return.
+    auto flush = [&]() {
+        wait_stage(0);
+        wait_stage(1);
+        tc::fence_after_sync();
+        __syncthreads();
+        const int part = warp >> 2, lrow = 32 * (warp & 3) + lane, s = lrow / NI, i = lrow - s * NI;
+        const uint32_t lanes = c.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+        long long *buf = reinterpret_cast<long long *>(c.stages);
+        constexpr int kPart = Sh::kRowDigits * Sh::JP * Sh::kLd;     // words of a part
+        constexpr int kL1 = Sh::kParts * kPart;                      // then tile 1's, [s - TS][j][i]
+        // sum over the sets of K digits of columns at .. at + 7, weighted 256^(W - 1 - t)
+        auto digits = [&](auto K, auto W, long long (&x)[8], const uint32_t at) {
+            int v[K][8];
+#pragma unroll
+            for (int t = 0; t < K; ++t)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[t][e] = 0;
+            for (int set = 0; set < sets; ++set) {
+                float f[K][8];
+#pragma unroll
+                for (int t = 0; t < K; ++t) tc::tmem_ld8(at + set * Sh::kCols + t * Sh::NR, f[t]);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int t = 0; t < K; ++t)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[t][e] += __float2int_rn(f[t][e]);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                long long y = 0;
+#pragma unroll
+                for (int t = 0; t < W; ++t) y = y * 256 + (t < K ? v[t < K ? t : 0][e] : 0);
+                x[e] = y;
+            }
+        };
+        auto put = [&](const int at, const long long (&x)[8]) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) buf[at + e * Sh::kLd + i] = x[e];
+        };
+        for (int jb = 0; jb < Sh::NR; jb += Sh::JP) {
+            constexpr int kJ = Sh::JP / 8;
+            for (int task = part; task < Sh::kTiles * kJ; task += 4) {
+                const int tile = task / kJ, jl = 8 * (task - tile * kJ);
+                const uint32_t at = lanes + (tile ? Sh::N0 : 0) + jb + jl;
+                long long x[8];
+                if constexpr (Sh::kMirror) {
+                    if (tile == 1) {
+                        // digits TS .. TE-1, in the word whose last digit is 3 (S <= 4) or 7
+                        digits(std::integral_constant<int, Sh::TE - Sh::TS>(),
+                               std::integral_constant<int, (S > 4 ? 8 : 4) - Sh::TS>(), x, at);
+                        if (s < S - Sh::TS) put(kL1 + (s * Sh::JP + jl) * Sh::kLd, x);
+                        continue;
+                    }
+                }
+                {
+                    const int sr = s + tile * Sh::TS;  // the row's digit
+                    const bool keep = s < Sh::TS && sr < Sh::kRowDigits;
+                    digits(std::integral_constant<int, Sh::TA>(), std::integral_constant<int, 4>(), x, at);
+                    if (keep) put((sr * Sh::JP + jl) * Sh::kLd, x);
+                    if constexpr (Sh::kParts == 2) {
+                        digits(std::integral_constant<int, S - Sh::TA>(),
+                               std::integral_constant<int, (S > 4 ? 8 : 4) - Sh::TA>(), x,
+                               at + Sh::TA * Sh::NR);
+                        if (keep) put(kPart + (sr * Sh::JP + jl) * Sh::kLd, x);
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncthreads();
+            // weights: row digit s, word ending in digit e: 256^(7 - s) 256^(7 - e), in units of 2^24
+            auto add = [&](i128 &g, const long long x, const int sh) {
+                g += sh >= 0 ? (i128)x << (sh >= 0 ? sh : 0) : (i128)(x >> (sh < 0 ? -sh : 0));
+            };
+            for (int o = tid; o < NI * cmin(Sh::JP, Sh::NR); o += kGramThreads) {
+                const int ii = o % NI, jl = o / NI, j = jb + jl;
+                if (j >= Sh::NR) break;
+                i128 g = 0, mir = 0;
+#pragma unroll
+                for (int sr = 0; sr < Sh::kRowDigits; ++sr) {
+                    const int at = (sr * Sh::JP + jl) * Sh::kLd + ii;
+                    add(g, buf[at], 64 - 8 * sr);
+                    if (Sh::kParts == 2) add(mir, buf[kPart + at], (S > 4 ? 32 : 64) - 8 * sr);
+                }
+                if (Sh::kMirror) {
+#pragma unroll
+                    for (int sr = Sh::TS; sr < S; ++sr) {
+                        const long long x = buf[kL1 + ((sr - Sh::TS) * Sh::JP + jl) * Sh::kLd + ii];
+                        const int sh = (S > 4 ? 32 : 64) - 8 * sr;
+                        if (sr < Sh::TE)
+                            add(g, x, sh);
+                        else
+                            add(mir, x, sh);
+                    }
+                    g = (ii <= j ? g : 0) + (ii == j ? 2 * mir : mir);
+                } else {
+                    g = NJ > 0 || ii <= j ? g + mir : 0;
+                }
+                Q128 *u = c.U + ii * Sh::NR + j;
+                *u = pack(unpack(*u) + g);
+            }
+            __syncthreads();
+        }
+        sets = 0;
+        in_set = 0;
+    };
+
+    // Tensor-core work of blocks [k0, k1) of the round in stage b (one thread), into the current
+    // accumulator set (begun here when the last one is full or flushed).
+    auto multiply = [&](const int b, const int k0, const int k1) {
+        if (in_set == 0) ++sets;
+        if (tid == kGramThreads - 32) {
+            tc::fence_after_sync();
+            const uint32_t d0 = c.tmem + (uint32_t)(sets - 1) * Sh::kCols;
+#pragma unroll 1
+            for (int kb = k0; kb < k1; ++kb) {
+                const uint32_t base = sbase + b * Sh::kStage + kb * Sh::kKbBytes;
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const bool add = in_set > 0 || kb > k0 || ks > 0;
+                    const uint64_t ad = tc::smem_desc(base + 32 * ks, 16, 1024, tc::kSw128);
+                    const uint64_t bd =
+                        NJ > 0 ? tc::smem_desc(base + S * NI * 128 + 32 * ks, 16, 1024, tc::kSw128) : ad;
+                    tc::mma_f16(d0, ad, bd, idesc0, add);
+                    if (Sh::kTiles == 2) {
+                        const uint64_t a1 =
+                            tc::smem_desc(base + Sh::TS * NI * 128 + 32 * ks, 16, 1024, tc::kSw128);
+                        tc::mma_f16(d0 + Sh::N0, a1, NJ > 0 ? bd : a1, idesc1, add);
+                    }
+                }
+            }
+            tc::mma_commit(&sm.bar[b]);
+        }
+        pend[b] = true;
+        in_set += k1 - k0;
+    };
+    // Block kb (all: the whole round) of round r as digits in stage b; false where an entry is out
+    // of its column's range (the same for every thread).
+    auto slice = [&](const int r, const int b, const int kb, const bool all) {
+        int dmin = 2;
+#pragma unroll
+        for (int t = 0; t < Sh::kTasks; ++t)
+            if (tk[t].mine && (all || tk[t].kbo == kb))
+                slice8<Tin>(raw_of(r, t), tk[t].off, sm.D[tk[t].lc], dmin,
+                            c.stages + b * Sh::kStage + tk[t].dst,
+                            (NJ > 0 && tk[t].lc >= NI ? NJ : NI) * 128);
+        tc::fence_proxy_async();
+        return __syncthreads_or(dmin < 2) == 0;
+    };
+
+#pragma unroll 1
+    for (int r = 0; r < Sh::kRaws; ++r) load_round(r);
+    cp_async_wait<Sh::kRaws - 1>();
+    if (sizeof(Tin) == 2) __syncwarp();
+    __syncthreads();
+    scan_block(0, 0);
+    if (tid < NI + NJ) sm.D[tid] = sm.Dnew[tid];
+    if (padded)
+        zero_stages();
+    else
+        __syncthreads();
+    for (int r = 0; r < rounds && !sm.bad; ++r) {
+        const int b = r & 1;
+        cp_async_wait<Sh::kRaws - 1>();
+        if (sizeof(Tin) == 2) __syncwarp();
+        wait_stage(b);
+        if (slice(r, b, 0, true)) {
+            multiply(b, 0, Sh::kRoundKb);
+        } else {
+            // block by block: where an entry is above its column's range, what is accumulated goes
+            // to U, then the exponents rise and U's entries follow
+#pragma unroll 1
+            for (int kb = 0; kb < Sh::kRoundKb; ++kb) {
+                const bool up = scan_block(r, kb);
+                if (sm.bad) break;
+                if (up) {
+                    if (sets > 0) flush();
+                    for (int o = tid; o < NI * Sh::NR; o += kGramThreads) {
+                        const int i = o / Sh::NR, j = (NJ > 0 ? NI : 0) + o % Sh::NR;
+                        c.U[o] = pack(
+                            shr128(unpack(c.U[o]), sm.Dnew[i] - sm.D[i] + sm.Dnew[j] - sm.D[j]));
+                    }
+                    __syncthreads();
+                    if (tid < NI + NJ) sm.D[tid] = sm.Dnew[tid];
+                    if (padded)
+                        zero_stages();
+                    else
+                        __syncthreads();
+                }
+                slice(r, b, kb, false);
+                multiply(b, kb, kb + 1);
+                wait_stage(b);
+            }
+            if (sm.bad) break;
+        }
+        const bool full = in_set + Sh::kRoundKb > 16;
+        if (full) in_set = 0;
+        load_round(r + Sh::kRaws);
+        if (r + 1 == rounds || (full && sets == Sh::kSets)) {
+            flush();
+            if (r + 1 < rounds && padded) zero_stages();
+        }
+    }
+    cp_async_wait_all();
+    wait_stage(0);
+    wait_stage(1);
+    if (__syncthreads_or(!c.ok) && tid == 0) sm.bad = 1;
+    __syncthreads();
+}
+
+// ------------------------------------------------------------------------------------------
+// The tree over a set's slabs.  Publishes the leaf (exponents, sums); the last child of a node to
+// arrive adds its siblings, aligned to the largest exponents, and climbs on.  Returns true in the
+// CTA that has written the set's sum (the last slot of the set's tree).
+// ------------------------------------------------------------------------------------------
+template <int NI, int NJ, int NR>
+__device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const int set, const int slab,
+                      const size_t slot_bytes, Cta &c) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    Smem &sm = *c.sm;
+    const int inner = gram_inner_nodes(p.nslab);
+    unsigned int *counters = p.counters + (size_t)set * inner;
+    unsigned char *slots = p.slots + (size_t)set * (p.nslab + inner) * slot_bytes;
+    const int nout = NJ > 0 ? cols.ni * cols.nj : cols.ni * (cols.ni + 1) / 2;
+    auto decode = [&](const int o, int &i, int &j) {  // local columns of output o
+        if (NJ > 0) {
+            i = o / cols.nj;
+            j = o - i * cols.nj;
+        } else {
+            unpack_index(o, i, j);
+        }
+    };
+    {
+        unsigned char *mine = slots + (size_t)slab * slot_bytes;
+        int *head = reinterpret_cast<int *>(mine);
+        if (tid < 128) {
+            const int l = tid < 64 ? tid : NI + tid - 64;
+            head[tid] = (tid < 64 ? tid < cols.ni : tid - 64 < cols.nj) ? sm.D[l] : 0;
+        }
+        if (tid == 0) head[kGramSlotHead / 4 - 1] = sm.bad;
+        for (int o = tid; o < nout; o += kGramThreads) {
+            int i, j;
+            decode(o, i, j);
+            i128 g = unpack(c.U[i * NR + j]);
+            if (NJ == 0 && i < j) g += unpack(c.U[j * NR + i]);
+            reinterpret_cast<Q128 *>(mine + kGramSlotHead)[o] = pack(g);
+        }
+    }
+    int cnt = p.nslab, off = 0, t = slab, cidx = 0;
+    int *kd = reinterpret_cast<int *>(c.stages);  // children's exponents, 128 each; then the node's
+    while (cnt > 1) {
+        const int next_cnt = (cnt + kGramArity - 1) / kGramArity;
+        const int parent = t / kGramArity, first = parent * kGramArity;
+        const int nchild = min(kGramArity, cnt - first);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) sm.flag = atomicAdd(&counters[cidx + parent], 1u) + 1 == (unsigned)nchild;
+        __syncthreads();
+        if (!sm.flag) return false;
+        __threadfence();
+        const unsigned char *kids = slots + (size_t)(off + first) * slot_bytes;
+        unsigned char *node = slots + (size_t)(off + cnt + parent) * slot_bytes;
+        for (int e = tid; e < 128 * nchild; e += kGramThreads)
+            kd[e] = __ldcg(reinterpret_cast<const int *>(kids + (e >> 7) * slot_bytes) + (e & 127));
+        if (tid == 0) sm.bad = 0;
+        __syncthreads();
+        if (tid < 128) {
+            int d = 0;
+            for (int ch = 0; ch < nchild; ++ch) d = max(d, kd[128 * ch + tid]);
+            kd[128 * kGramArity + tid] = d;
+            reinterpret_cast<int *>(node)[tid] = d;
+        } else if (tid < 128 + nchild) {
+            if (__ldcg(reinterpret_cast<const int *>(kids + (tid - 128) * slot_bytes) +
+                       kGramSlotHead / 4 - 1))
+                sm.bad = 1;
+        }
+        __syncthreads();
+        if (tid == 0) reinterpret_cast<int *>(node)[kGramSlotHead / 4 - 1] = sm.bad;
+        for (int o = tid; o < nout; o += kGramThreads) {
+            int i, j;
+            decode(o, i, j);
+            const int jj = NJ > 0 ? 64 + j : j;
+            const int dij = kd[128 * kGramArity + i] + kd[128 * kGramArity + jj];
+            const unsigned char *e = kids + kGramSlotHead + (size_t)o * 16;
+            i128 g = 0;
+#pragma unroll 4
+            for (int ch = 0; ch < nchild; ++ch)
+                g += shr128(ldcg128(e + ch * slot_bytes), dij - kd[128 * ch + i] - kd[128 * ch + jj]);
+            reinterpret_cast<Q128 *>(node + kGramSlotHead)[o] = pack(g);
+        }
+        off += cnt;
+        cidx += next_cnt;
+        cnt = next_cnt;
+        t = parent;
+    }
+    __threadfence();
+    __syncthreads();
+    return true;
+}
+
+// ------------------------------------------------------------------------------------------
+// Root: the Cholesky factor of the summed Gram in fixed point.  Columns are scaled by powers of
+// two so that every diagonal lies in [1/4, 1); values are integers over 2^122.  Step k works on
+// row k scaled by 2^z (pivot in [1/4, 1) again): l = C(k, j) / pivot in [-2, 2], to about 2^-90
+// from a 46-bit reciprocal and one residual, then C(i, j) -= l_i C(k, j).  R(k, j) = l_j sqrt(pivot).
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ u128 mul122(const u128 a, const u128 b) {  // (a b) >> 122; a, b < 2^124
+    const u64 ah = (u64)(a >> 64), al = (u64)a, bh = (u64)(b >> 64), bl = (u64)b;
+    const u128 mid = (u128)ah * bl + (u128)al * bh + __umul64hi(al, bl);
+    return (((u128)ah * bh) << 6) + (mid >> 58);
+}
+__device__ __forceinline__ u128 mul60(const u128 a, const u64 r) {  // (a r) >> 60
+    return (((u128)(u64)(a >> 64) * r) << 4) + (((u128)(u64)a * r) >> 60);
+}
+// 2^60 (2^122 / d) to about 46 bits, d in [2^120, 2^122): the hardware's FP32 reciprocal and one
+// Newton step.
+__device__ __forceinline__ u64 recip60(const u128 d) {
+    const u64 x = (u64)(d >> 58);  // d / 2^122 = x / 2^64
+    const float f = __uint2float_rz((uint32_t)(x >> 32)) * 2.3283064365386963e-10f;
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(f));
+    const uint32_t yb = __float_as_uint(y);  // y in (1, 4]
+    const u64 r = (u64)((yb & 0x7fffff) | 0x800000) << (37 + (int)(yb >> 23) - 127);
+    const long long e = (1ll << 60) - (long long)__umul64hi(x, r);
+    return r + (u64)(__mul64hi((long long)r, e) << 4);
+}
+// x / 2^122 as a sum of two doubles (the second below the first's last place).
+struct D2 {
+    double hi, lo;
+};
+__device__ __forceinline__ D2 to_double(const i128 x) {
+    const long long top = (long long)(x >> 64);
+    const double h = (double)top;
+    const double r = (double)(top - (long long)h);
+    return D2{h * 0x1p-58, r * 0x1p-58 + (double)(u64)x * 0x1p-122};
+}
+__device__ __forceinline__ D2 sqrt2(const D2 x) {
+    const double s = sqrt(x.hi + x.lo);
+    return D2{s, (fma(-s, s, x.hi) + x.lo) / (2.0 * s)};
+}
+
+// C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it.  rowv: 3 n
+// entries of scratch.  g[j]: the power of two of R's column j.  Returns false if a pivot is too small.
+__device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int pivot_bits,
+                                         const int *g, double *R, const int64_t ldr) {
+    const int tid = threadIdx.x, nt = kGramThreads, warp = tid >> 5, lane = tid & 31;
+    Q128 *Lq = rowv, *Cp = rowv + n, *dv = rowv + 2 * n;
+    for (int k = 0; k < n; ++k) {
+        Q128 *Ck = C + rowoff(n, k) - k;
+        const i128 d0 = unpack(Ck[k]);
+        if (d0 < ((i128)1 << (122 - pivot_bits))) return false;  // the same for every thread
+        const u64 dh = (u64)((u128)d0 >> 64);
+        const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d0);
+        const int z = (122 - len) >> 1;
+        const int j = k + 1 + tid;
+        if (j < n || tid == 0) {
+            u128 d = (u128)d0;
+            if (z) d <<= 2 * z;
+            if (tid == 0) dv[k] = pack((i128)d);
+            if (j < n) {
+                const i128 c0 = unpack(Ck[j]);
+                const bool neg = c0 < 0;
+                u128 c = (u128)(neg ? -c0 : c0);
+                if (z) c <<= z;
+                const u64 r = recip60(d);
+                u128 q = mul60(c, r);
+                const i128 res = (i128)(c - mul122(q, d));
+                const u128 dq = mul60((u128)(res < 0 ? -res : res), r);
+                q = res < 0 ? q - dq : q + dq;
+                const Q128 l = pack(neg ? -(i128)q : (i128)q);
+                Lq[j] = l;
+                Ck[j] = l;
+                Cp[j] = pack(neg ? -(i128)c : (i128)c);
+            }
+        }
+        __syncthreads();
+        // trailing update, (i, j) with k < i <= j: a warp a row
+        for (int i = k + 1 + warp; i < n; i += nt >> 5) {
+            const i128 a = unpack(Lq[i]);
+            const u128 am = (u128)(a < 0 ? -a : a);
+            Q128 *Ci = C + rowoff(n, i) - i;
+            for (int jj = i + lane; jj < n; jj += 32) {
+                const i128 b = unpack(Cp[jj]);
+                const u128 q = mul122(am, (u128)(b < 0 ? -b : b));
+                const i128 x = unpack(Ci[jj]);
+                Ci[jj] = pack((a < 0) != (b < 0) ? x + (i128)q : x - (i128)q);
+            }
+        }
+        __syncthreads();
+    }
+    // R(k, k) = sqrt(C(k, k)) (still in place); R(k, j) = l sqrt(d): rounded once, near enough
+    D2 *sd = reinterpret_cast<D2 *>(Lq);
+    for (int k = tid; k < n; k += nt) sd[k] = sqrt2(to_double(unpack(dv[k])));
+    __syncthreads();
+    for (int o = tid; o < n * n; o += nt) {
+        const int col = o / n, row = o - col * n;
+        double v = 0.0;
+        if (row <= col) {
+            const D2 x = to_double(unpack(C[rowoff(n, row) - row + col]));
+            if (row == col) {
+                const D2 q = sqrt2(x);
+                v = q.hi + q.lo;
+            } else {
+                const D2 q = sd[row];
+                const double p = x.hi * q.hi;
+                v = p + (fma(x.hi, q.hi, -p) + (x.hi * q.lo + x.lo * q.hi));
+            }
+            v = scalbn(v, g[col]);
+        }
+        R[row + (int64_t)col * ldr] = v;
+    }
+    return true;
+}
+
+// Every set's sum (all written): gathered, scaled and factored; R written.  False: not served.
+template <typename Tin>
+__device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_bytes, Smem *smp,
+                                    unsigned char *base) {
+    constexpr int NB = Type<Tin>::kBlock;
+    const int tid = threadIdx.x, n = p.n;
+    Smem &sm = *smp;
+    Q128 *C = reinterpret_cast<Q128 *>(base);
+    Q128 *rowv = C + n * (n + 1) / 2;
+    const int per_set = p.nslab + gram_inner_nodes(p.nslab), nset = gram_sets(p.nb);
+    auto top = [&](const int set) {
+        return p.slots + ((size_t)(set + 1) * per_set - 1) * slot_bytes;
+    };
+    auto set_of = [&](const int I, const int J) {
+        return I == J ? I : p.nb + J * (J - 1) / 2 + I;
+    };
+    __syncthreads();
+    if (tid == 0) sm.bad = 0;
+    __syncthreads();
+    for (int s = tid; s < nset; s += kGramThreads)
+        if (__ldcg(reinterpret_cast<const int *>(top(s)) + kGramSlotHead / 4 - 1)) sm.bad = 1;
+    if (tid < n) {  // column exponents: the largest of the column's sets
+        const int b = tid / NB, l = tid - b * NB;
+        int d = 0;
+        for (int o = 0; o < p.nb; ++o) {
+            const int s = set_of(min(o, b), max(o, b));
+            d = max(d, __ldcg(reinterpret_cast<const int *>(top(s)) + (o < b ? 64 : 0) + l));
+        }
+        sm.D[tid] = d;
+    }
+    __syncthreads();
+    if (sm.bad) return false;
+    auto entry = [&](const int i, const int j) {  // the sum (i, j), i <= j, aligned to sm.D
+        const int I = i / NB, J = j / NB, li = i - I * NB, lj = j - J * NB;
+        const unsigned char *t = top(set_of(I, J));
+        const int *h = reinterpret_cast<const int *>(t);
+        const int nj = min(NB, n - J * NB);
+        const size_t o = I == J ? (size_t)(lj * (lj + 1) / 2 + li) : (size_t)(li * nj + lj);
+        const i128 x = ldcg128(t + kGramSlotHead + o * 16);
+        return shr128(x, sm.D[i] + sm.D[j] - __ldcg(h + li) - __ldcg(h + (I == J ? lj : 64 + lj)));
+    };
+    if (tid < n) {
+        const i128 d = entry(tid, tid);
+        const u64 dh = (u64)((u128)d >> 64);
+        const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d);
+        sm.E[tid] = d > 0 ? (122 - len) >> 1 : 0;  // shift of the column
+        if (!(d > 0)) sm.bad = 1;
+        sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + Type<Tin>::kUnit;
+    }
+    __syncthreads();
+    if (sm.bad) return false;
+    for (int o = tid; o < n * (n + 1) / 2; o += kGramThreads) {
+        int i, j;
+        unpack_index(o, i, j);
+        C[rowoff(n, i) - i + j] = pack(shift128(entry(i, j), sm.E[i] + sm.E[j]));
+    }
+    __syncthreads();
+    return factor_root(C, rowv, n, Type<Tin>::kPivotBits, sm.Dnew, p.R, p.ldr);
+}
+
+// One work item: its rows' sums and the climb.  True in the CTA that has written the set's sum.
+template <typename Tin, int NI, int NJ>
+__device__ __forceinline__ bool item_of(const GramProblem &p, const Cols cols, const int set,
+                                        const int slab, const size_t slot_bytes, Cta &c) {
+    const int64_t kb0 = (int64_t)slab * p.nkb / p.nslab, kb1 = (int64_t)(slab + 1) * p.nkb / p.nslab;
+    sum_rows<Tin, NI, NJ>(p, cols, kb0, kb1, c);
+    return climb<NI, NJ, Shape<Tin, NI, NJ>::NR>(p, cols, set, slab, slot_bytes, c);
+}
+
+// Tensor memory and barriers of the CTA; smem: its dynamic shared memory.
+__device__ __forceinline__ void cta_begin(Cta &c, unsigned char *smem) {
+    c.sm = reinterpret_cast<Smem *>(smem);
+    c.stages = smem + kHead;
+    if (threadIdx.x >> 5 == kGramWarps - 1) tc::tmem_alloc(&c.sm->tmem, 512);
+    if (threadIdx.x == 0) {
+        tc::mbar_init(&c.sm->bar[0], 1);
+        tc::mbar_init(&c.sm->bar[1], 1);
+        tc::fence_mbar_init();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    c.tmem = c.sm->tmem;
+    c.par[0] = c.par[1] = 0;
+    c.ok = true;
+}
+__device__ __forceinline__ void cta_end(const Cta &c) {
+    __syncthreads();
+    if (threadIdx.x >> 5 == kGramWarps - 1) {
+        tc::tmem_relinquish();
+        tc::tmem_dealloc(c.tmem, 512);
+    }
+}
+
+}  // namespace gram
+}  // namespace tsqr

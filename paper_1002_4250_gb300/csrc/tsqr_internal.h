@@ -29,6 +29,8 @@ size_t f64_smem_bytes(int n, int hs, int ldS, int warps);
 cudaError_t f64_prepare(size_t smem_bytes);
 int f64_blocks_per_sm(int warps, size_t smem_bytes);
 cudaError_t f64_launch(const F64Args &a, int warps, size_t smem_bytes, cudaStream_t stream);
+cudaError_t zero_lower_launch(double *R, int64_t ldr, int n, const unsigned int *skip,
+                              cudaStream_t stream);
 cudaError_t f64_combine_launch(int n, const double *R1, int64_t ld1, const double *R2,
                                int64_t ld2, double *R, int64_t ldr, int normalize, int warps,
                                int ldS, int hs, size_t smem_bytes, int *status,
@@ -38,9 +40,13 @@ cudaError_t f64_combine_launch(int n, const double *R1, int64_t ld1, const doubl
 // cooperative launch of at most one CTA per SM).
 struct GramArgs;
 int gram_round_rows(int n);
+int gram_slot_block(int n);
 size_t gram_smem_bytes(int n);
 cudaError_t gram_prepare(int n, size_t smem_bytes);
 cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream);
+// A queue of column sets and slabs on `grid` CTAs (at most one per SM).
+struct GramQueueArgs;
+cudaError_t gram_queue_launch(const GramQueueArgs &a, int grid, cudaStream_t stream);
 
 // Mixed path (tsqr_mixed.cu); `warps` counts bulk warps as for the FP64 path.
 int mixed_s_doubles(int n, int ldS);

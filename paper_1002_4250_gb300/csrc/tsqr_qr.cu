@@ -23,6 +23,7 @@ namespace tsqr {
 // ------------------------------------------------------------------------------------------
 template <int B>
 __global__ void __launch_bounds__(416, 1) tsqr_qr_factor_kernel(const F64Args a) {
+    if (skipped(a.skip)) return;
     leaf_tree_job<double, double, B, 1, B == 1, true>(a, a.A, a.ldS, a.ldS * a.n, blockIdx.x);
 }
 
@@ -450,6 +451,7 @@ __device__ __forceinline__ void qt_climb(const QtArgs &a, const int leaf, const 
 // ------------------------------------------------------------------------------------------
 template <int B>
 __global__ void __launch_bounds__(416, 1) tsqr_qt_kernel(const QtArgs a) {
+    if (skipped(a.skip)) return;
     extern __shared__ __align__(16) double smem[];
     const int n = a.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = blockIdx.y, kc = min(a.k, a.ktot - grp * a.k);
@@ -613,6 +615,7 @@ __device__ __forceinline__ void wy_s_from_g(const double *G, const double *sc, c
 }
 
 __global__ void __launch_bounds__(256) tsqr_wy_kernel(const WyArgs a) {
+    if (skipped(a.skip)) return;
     extern __shared__ __align__(16) double smem[];
     const int n = a.n, ldX = a.ldX;
     double *X = smem;               // ldX x n
@@ -752,6 +755,7 @@ __device__ __forceinline__ void wy_zupdate(double *Z, const double *X, const int
 // Y = S^T W, T -= Y and (where the whole product is wanted) Z -= X diag(c) Y, written to Cout.  Then the same climb.  Two passes over the chunk's rows
 // in place of n fused sweeps, and no per-reflector barriers.
 __global__ void __launch_bounds__(256, 1) tsqr_qt_wy_kernel(const QtArgs a) {
+    if (skipped(a.skip)) return;
     extern __shared__ __align__(16) double smem[];
     const int n = a.n;
     const int grp = blockIdx.y, kc = min(a.k, a.ktot - grp * a.k);

@@ -98,6 +98,7 @@ struct QtArgs {
     // The chunks' compact WY factors (per chunk id, n x n, from tsqr_wy_kernel), for the
     // blocked leaf part; unused by the reflector-by-reflector one.
     const double *wyS;
+    const unsigned int *skip; // as in F64Args
 };
 
 // Compact WY form of each chunk's reflectors.  Reflector J of a chunk is v_J = [e_J; c_J x_J]
@@ -112,6 +113,7 @@ struct WyArgs {
     int64_t nchunks;
     const double *chunk_sc;   // per chunk: tau_J, c_J
     double *S;                // out
+    const unsigned int *skip; // as in F64Args
 };
 
 // Blocked leaf part of the Q^T apply: the tails X diag(c) (ldS x n), B's chunk Z (ldS x kc),

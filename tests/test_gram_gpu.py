@@ -141,3 +141,51 @@ def test_capture_streams_and_plans(oracle, T):
         with pytest.raises(T.TsqrError) as e:
             T.tsqr_r_ex(A1.T, plan=bad)
         assert e.value.status == T.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("n", [33, 40, 41, 48, 49, 55, 56, 63, 64, 65, 72, 96, 97, 127, 128])
+@pytest.mark.parametrize("m,pad", [(2048, 0), (30011, 3)])
+def test_column_blocks(oracle, T, n, m, pad):
+    """Past 32 columns the sums go by blocks of 32 columns, a block against itself or another."""
+    import torch
+    At = workloads.gaussian(m, n, seed=800 + n)
+    At *= torch.exp2(torch.arange(m, dtype=torch.float64) * (6.0 / m))  # exponents rise
+    big = torch.full((n, m + pad), float("nan"), dtype=torch.float64)
+    big[:, :m] = At
+    Ad = big.cuda().T[:m, :]
+    R = T.tsqr_r(Ad)
+    p = T.last_plan()
+    assert (p.leaf, p.tree) == ((T.LEAF_GRAM, T.TREE_HYBRID) if n < 56 else (0, T.TREE_PANELS))
+    _check(oracle, R, At)
+    assert torch.equal(T.tsqr_r_ex(Ad, plan=p), R)
+
+
+@pytest.mark.parametrize("n", [40, 100])
+@pytest.mark.parametrize("kind", ["repeated", "zero", "nan", "kappa"])
+def test_column_blocks_handed_over(oracle, T, n, kind):
+    """What the Gram sum cannot serve runs the launches behind it: the Householder reduction's
+    bytes (its own plan, or panels of 16 as an explicit panel width that the Gram never takes)."""
+    import torch
+    m = 40009
+    At = workloads.gaussian(m, n, seed=850 + n)
+    if kind == "repeated":
+        At[n - 1] = At[1]
+    elif kind == "zero":
+        At[33] = 0.0
+    elif kind == "nan":
+        At[35, 12345] = float("nan")
+    else:
+        At = workloads.conditioned(m, n, 1e8, seed=n)  # served: no hand-over
+    Ad = At.cuda().T
+    T.tsqr_get_device_status()
+    R = T.tsqr_r(Ad)
+    status = T.tsqr_get_device_status()
+    assert status == (T.STATUS_NONFINITE if kind == "nan" else T.SUCCESS)
+    if kind == "kappa":
+        _check(oracle, R, At)
+    elif n < 56:
+        ref = T.tsqr_r_ex(Ad, plan=T.make_plan("hybrid"))
+        assert torch.equal(torch.nan_to_num(R), torch.nan_to_num(ref))
+    if kind in ("repeated", "zero"):
+        assert np.all(np.diag(R.cpu().numpy()) >= 0)
+        assert oracle.gram_residual(oracle.from_torch_colmajor(At), R.cpu().numpy(), nthreads=16) <= 1e-13
