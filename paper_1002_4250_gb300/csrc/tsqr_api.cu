@@ -538,16 +538,19 @@ struct GramLayout {
 };
 // Slabs: about five items a CTA (the last wave stays short; an item's fixed cost, its pipeline's
 // start, the flush and the climb, is some 7 us), of at least 512 rows.
+// One set: a slab a CTA.
 GramLayout gram_layout(int64_t m, int64_t n, int sms) {
     GramLayout w;
     w.nb = (int)((n + 31) / 32);
     w.nset = gram_sets(w.nb);
     const int64_t nkb = (m + 63) / 64;
-    w.nslab = (int)std::max<int64_t>(1, std::min<int64_t>(5LL * sms / w.nset, nkb / 8));
+    w.nslab = (int)std::max<int64_t>(
+        1, std::min<int64_t>(w.nset == 1 ? sms : 5LL * sms / w.nset, nkb / 8));
     w.inner = gram_inner_nodes(w.nslab);
     w.words = 4 + (size_t)w.nset * w.inner;  // queue, failed, verdict, sets done, then the nodes
     w.cnt_bytes = align_up(w.words * sizeof(unsigned int), 256);
-    w.bytes = w.cnt_bytes + (size_t)w.nset * (w.nslab + w.inner) * gram_slot_bytes(32);
+    w.bytes = w.cnt_bytes + (size_t)w.nset * (w.nslab + w.inner) *
+                                gram_slot_bytes(gram_block((int)n));
     return w;
 }
 // The Gram sum of [A | B] (B: columns na .. n-1, or none) and its factor R in the workspace at
@@ -598,7 +601,7 @@ RLayout r_layout(const F64Plan &p, int64_t m, int64_t n, int sms) {
     w.cnt_bytes = align_up(w.cnt_words * sizeof(unsigned int), 256);
     w.gram_off = align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
     w.bytes = w.gram_off;
-    if (p.gram_ctas) w.bytes += (inner + p.gram_ctas) * gram_slot_bytes(gram_slot_block((int)n));
+    if (p.gram_ctas) w.bytes += (inner + p.gram_ctas) * gram_slot_bytes(gram_block((int)n));
     if (p.gram_queue) {
         w.g = gram_layout(m, n, sms);
         w.bytes += w.g.bytes;
@@ -1004,22 +1007,33 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     const size_t cnt_bytes = align_up((size_t)p.nodes * sizeof(unsigned int), 256);
     const size_t slot_bytes = align_up((size_t)p.nodes * (size_t)na * na * sizeof(double), 256);
     const size_t aug_bytes = align_up((size_t)m * (size_t)na * sizeof(double), 256);
-    const size_t ra_bytes = (size_t)na * na * sizeof(double);
+    const size_t ra_bytes = align_up((size_t)na * na * sizeof(double), 256);
+    // the Gram sum of [A | B] where it serves (it reads A and B where they are); the copy and the
+    // Householder reduction stand behind it
+    const bool gram = plan_is_auto(over) && gram_fits(m, na);
+    const int sms = current_sms();
+    GramLayout gl;
+    if (gram) gl = gram_layout(m, na, sms);
     Workspace *ws = nullptr;
-    st = get_workspace(stream, cnt_bytes + slot_bytes + aug_bytes + ra_bytes, &ws);
+    st = get_workspace(stream, cnt_bytes + slot_bytes + aug_bytes + ra_bytes + gl.bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
     char *base = (char *)ws->base;
     double *aug = (double *)(base + cnt_bytes + slot_bytes);
     double *Ra = (double *)(base + cnt_bytes + slot_bytes + aug_bytes);
-    if (cudaMemcpy2DAsync(aug, (size_t)m * sizeof(double), A, (size_t)lda * sizeof(double),
-                          (size_t)m * sizeof(double), (size_t)n, cudaMemcpyDeviceToDevice,
-                          stream) != cudaSuccess ||
-        cudaMemcpy2DAsync(aug + n * m, (size_t)m * sizeof(double), B, (size_t)ldb * sizeof(double),
-                          (size_t)m * sizeof(double), (size_t)k, cudaMemcpyDeviceToDevice,
-                          stream) != cudaSuccess ||
+    F64Args a = plan_args(p, aug, m, na, m);
+    if (gram) {
+        st = enqueue_gram(gl, sms, A, lda, B, ldb, n, m, na, (char *)Ra + ra_bytes, Ra, na, ws->status,
+                          &a.skip, stream);
+        if (st != TSQR_SUCCESS) return st;
+        if (na < kPanelsMinN)
+            g_last_plan.leaf = TSQR_LEAF_GRAM;
+        else
+            g_last_plan = tsqr_plan_t{TSQR_TREE_PANELS, kPanelsWidth, 0, 0, 0, 0};
+    }
+    if (copy_cols_launch(A, lda, aug, m, m, (int)n, a.skip, stream) != cudaSuccess ||
+        copy_cols_launch(B, ldb, aug + n * m, m, m, (int)k, a.skip, stream) != cudaSuccess ||
         cudaMemsetAsync(base, 0, (size_t)p.nodes * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    F64Args a = plan_args(p, aug, m, na, m);
     a.counters = (unsigned int *)base;
     a.slots = (double *)(base + cnt_bytes);
     a.R = Ra;
@@ -1033,7 +1047,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     if (trsm_launch(Ra, na, Ra + n * na, na, X, ldx, (int)n, (int)k, ws->status, stream) !=
         cudaSuccess)
         return TSQR_ERR_CUDA;
-    g_last_launches = 2;
+    g_last_launches = gram ? 5 : 4;
     return TSQR_SUCCESS;
 }
 

@@ -55,6 +55,16 @@ __global__ void tsqr_zero_lower_kernel(double *R, int64_t ldr, int n, const unsi
     }
 }
 
+// Columns 0 .. n-1 of src (m rows) to dst.
+__global__ void tsqr_copy_cols_kernel(const double *src, int64_t lds, double *dst, int64_t ldd,
+                                      int64_t m, int n, const unsigned int *skip) {
+    if (skipped(skip)) return;
+    for (int col = blockIdx.y; col < n; col += gridDim.y)
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
+             i += (int64_t)gridDim.x * blockDim.x)
+            dst[i + col * ldd] = src[i + col * lds];
+}
+
 // ------------------------------------------------------------------------------------------
 // host-side launchers
 // ------------------------------------------------------------------------------------------
@@ -94,6 +104,14 @@ cudaError_t zero_lower_launch(double *R, int64_t ldr, int n, const unsigned int 
                               cudaStream_t stream) {
     const int64_t blocks = ((int64_t)n * n + 1023) / 1024;
     tsqr_zero_lower_kernel<<<(int)(blocks < 512 ? blocks : 512), 1024, 0, stream>>>(R, ldr, n, skip);
+    return cudaGetLastError();
+}
+
+cudaError_t copy_cols_launch(const double *src, int64_t lds, double *dst, int64_t ldd, int64_t m,
+                             int n, const unsigned int *skip, cudaStream_t stream) {
+    const int64_t blocks = (m + 1023) / 1024;
+    const dim3 grid((unsigned)(blocks < 128 ? blocks : 128), (unsigned)(n < 64 ? n : 64));
+    tsqr_copy_cols_kernel<<<grid, 1024, 0, stream>>>(src, lds, dst, ldd, m, n, skip);
     return cudaGetLastError();
 }
 

@@ -32,11 +32,11 @@ tsqr_gram_f64_kernel(const __grid_constant__ GramArgs a) {
     if (b < a.p.nslab) {
         Cta c;
         cta_begin(c, smem);
-        const bool root = item_of<double, NB, 0>(a.p, Cols{0, a.p.n, 0, 0}, 0, b, slot_bytes, c);
+        const bool root = item_of<NB, 0>(a.p, Cols{0, a.p.n, 0, 0}, 0, b, slot_bytes, c);
         if (!c.ok && tid == 0) atomicOr(a.status, kStatusTimeoutBit);
         cta_end(c);
         if (root) {
-            const bool good = finish<double>(a.p, slot_bytes, c.sm, c.stages);
+            const bool good = finish(a.p, slot_bytes, c.sm, c.stages);
             __syncthreads();
             if (tid == 0) {
                 __threadfence();
@@ -71,8 +71,7 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
     extern __shared__ __align__(1024) double smem_d[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(smem_d);
     const int tid = threadIdx.x;
-    constexpr int NB = Type<double>::kBlock;
-    const size_t slot_bytes = gram_slot_bytes(NB);
+    constexpr int NB = kBlock;
     Cta c;
     cta_begin(c, smem);
     for (;;) {
@@ -88,6 +87,7 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
             code = w.y;
         }
         const GramProblem &p = a.probs ? a.probs[which] : a.one;
+        const size_t slot_bytes = gram_slot_bytes(gram_block(p.n));
         const int nset = gram_sets(p.nb), slab = code / nset, set = code - slab * nset;
         Cols cols{0, 0, 0, 0};
         bool root;
@@ -95,26 +95,26 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
             cols.i0 = set * NB;
             cols.ni = min(NB, p.n - cols.i0);
             if (cols.ni <= 8)
-                root = item_of<double, 8, 0>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<8, 0>(p, cols, set, slab, slot_bytes, c);
             else if (cols.ni <= 16)
-                root = item_of<double, 16, 0>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<16, 0>(p, cols, set, slab, slot_bytes, c);
             else if (cols.ni <= 24)
-                root = item_of<double, 24, 0>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<24, 0>(p, cols, set, slab, slot_bytes, c);
             else
-                root = item_of<double, 32, 0>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<32, 0>(p, cols, set, slab, slot_bytes, c);
         } else {
             int I = 0, J = 1;
             for (int o = set - p.nb; o >= J; ++J) o -= J;
             I = set - p.nb - J * (J - 1) / 2;
             cols = Cols{I * NB, NB, J * NB, min(NB, p.n - J * NB)};
             if (cols.nj <= 8)
-                root = item_of<double, 32, 8>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<32, 8>(p, cols, set, slab, slot_bytes, c);
             else if (cols.nj <= 16)
-                root = item_of<double, 32, 16>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<32, 16>(p, cols, set, slab, slot_bytes, c);
             else if (cols.nj <= 24)
-                root = item_of<double, 32, 24>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<32, 24>(p, cols, set, slab, slot_bytes, c);
             else
-                root = item_of<double, 32, 32>(p, cols, set, slab, slot_bytes, c);
+                root = item_of<32, 32>(p, cols, set, slab, slot_bytes, c);
         }
         if (!root) continue;
         if (nset > 1) {
@@ -125,7 +125,7 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
             if (!c.sm->flag) continue;
             __threadfence();
         }
-        const bool good = finish<double>(p, slot_bytes, c.sm, c.stages);
+        const bool good = finish(p, slot_bytes, c.sm, c.stages);
         __syncthreads();
         if (tid == 0) {
             *p.verdict = good ? 1u : 2u;
@@ -144,18 +144,18 @@ struct Variant {
 };
 template <int NB>
 Variant variant() {
-    using Sh = Shape<double, NB, 0>;
+    using Sh = Shape<NB, 0>;
     return Variant{tsqr_gram_f64_kernel<NB>, smem_bytes<Sh>(), Sh::kRoundKb};
 }
 Variant variant_for(int n) {
     return n <= 8 ? variant<8>() : n <= 16 ? variant<16>() : n <= 24 ? variant<24>() : variant<32>();
 }
 constexpr size_t queue_smem() {
-    size_t b = smem_bytes<Shape<double, 8, 0>>();
-    for (size_t o : {smem_bytes<Shape<double, 16, 0>>(), smem_bytes<Shape<double, 24, 0>>(),
-                     smem_bytes<Shape<double, 32, 0>>(), smem_bytes<Shape<double, 32, 8>>(),
-                     smem_bytes<Shape<double, 32, 16>>(), smem_bytes<Shape<double, 32, 24>>(),
-                     smem_bytes<Shape<double, 32, 32>>()})
+    size_t b = smem_bytes<Shape<8, 0>>();
+    for (size_t o : {smem_bytes<Shape<16, 0>>(), smem_bytes<Shape<24, 0>>(),
+                     smem_bytes<Shape<32, 0>>(), smem_bytes<Shape<32, 8>>(),
+                     smem_bytes<Shape<32, 16>>(), smem_bytes<Shape<32, 24>>(),
+                     smem_bytes<Shape<32, 32>>()})
         b = o > b ? o : b;
     return b;
 }
@@ -166,7 +166,6 @@ static_assert(kHead + (kGramRootMaxN * (kGramRootMaxN + 1) / 2 + 3 * kGramRootMa
 }  // namespace
 
 int gram_round_rows(int n) { return 64 * variant_for(n).kb_round; }
-int gram_slot_block(int n) { return n <= 8 ? 8 : n <= 16 ? 16 : n <= 24 ? 24 : 32; }
 size_t gram_smem_bytes(int n) { return variant_for(n).smem; }
 
 cudaError_t gram_prepare(int n, size_t smem_bytes) {

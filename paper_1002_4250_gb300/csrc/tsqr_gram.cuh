@@ -13,9 +13,8 @@
 // non-finite or extreme entry, a pivot below 2^-bits of its column's square) is found by the
 // root, and the Householder reduction then runs instead.
 //
-// Columns are taken in blocks of NB (32 for FP64, 64 for FP32 and BF16): a column set is a block
-// against itself or a block against a later one, and a work item is one set over one slab of
-// rows.
+// Columns are taken in blocks of 32: a column set is a block against itself or a block against a
+// later one, and a work item is one set over one slab of rows.
 #pragma once
 
 #include "tsqr_f64.cuh"
@@ -31,7 +30,7 @@ constexpr int kGramRootMaxN = 128;  // widest matrix one CTA factors
 
 // One matrix [A | B] (B: columns na .. n-1, or none) and where its sums go.
 struct GramProblem {
-    const void *A, *B;
+    const double *A, *B;
     int64_t lda, ldb, m;
     int n, na;
     int nb;                // column blocks; sets 0 .. nb-1 are a block against itself, then (0, 1),
@@ -80,5 +79,8 @@ constexpr int kGramSlotHead = 576;
 __host__ __device__ inline size_t gram_slot_bytes(int block) {  // block: columns of a block
     return (size_t)kGramSlotHead + (size_t)block * block * 16;
 }
+
+// Columns of a matrix's blocks: a class of 8 for a matrix of one block, else 32.
+__host__ __device__ inline int gram_block(int n) { return n <= 24 ? (n + 7) / 8 * 8 : 32; }
 
 }  // namespace tsqr

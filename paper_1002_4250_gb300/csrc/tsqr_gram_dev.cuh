@@ -3,7 +3,6 @@
 // fixed-point Cholesky factor of the whole.
 #pragma once
 
-#include <cuda_bf16.h>
 #include <type_traits>
 
 #include "tsqr_fold.cuh"
@@ -17,77 +16,53 @@ typedef unsigned long long u64;
 typedef __int128 i128;
 typedef unsigned __int128 u128;
 
-// Input types: S digits a column, the block of columns, the least pivot a column may keep
-// (relative to its square), the exponents its largest entry may have (biased; outside, squares
-// leave the range of the Householder leaves' arithmetic, which then decide what R is), and the
-// power of two of a whole number's unit for exponent word D (x = Q 2^(D + kUnit), Q in the
-// 64-bit form of eight digits).
-template <typename Tin>
-struct Type;
-template <>
-struct Type<double> {
-    static constexpr int kDigits = 8, kBlock = 32, kPivotBits = 64;
-    static constexpr int kExpLo = 1023 - 400, kExpHi = 1023 + 400, kUnit = -1086;
-};
-template <>
-struct Type<float> {
-    static constexpr int kDigits = 4, kBlock = 64, kPivotBits = 44;
-    static constexpr int kExpLo = 127 - 55, kExpHi = 127 + 55, kUnit = -190;
-};
-template <>
-struct Type<__nv_bfloat16> {
-    static constexpr int kDigits = 3, kBlock = 64, kPivotBits = 36;
-    static constexpr int kExpLo = 127 - 55, kExpHi = 127 + 55, kUnit = -190;
-};
+constexpr int kDigits = 8;       // of a column
+constexpr int kBlock = 32;       // columns of a block
+// The least pivot a column may keep, relative to its square (2^-kPivotBits).
+constexpr int kPivotBits = 64;
+// Biased exponents a column's largest entry may have: outside, squares leave FP64's range (or
+// come near it) and the Householder reduction decides what R is.
+constexpr int kExpLo = 1023 - 400, kExpHi = 1023 + 400;
+constexpr int kUnit = -1086;     // |x| = Q 2^(D + kUnit) for a column's exponent word D
 
 constexpr int cmin(int a, int b) { return a < b ? a : b; }
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
-constexpr int up16(int a) { return (a + 15) / 16 * 16; }
 
 // Shape of a column set: NI columns against themselves (NJ = 0), or against NJ others.
 // Operand rows: digit s of column i at s NI + i, then digit t of column j at S NI + t NJ + j.
-template <typename Tin, int NI, int NJ>
+template <int NI, int NJ>
 struct Shape {
-    static constexpr int S = Type<Tin>::kDigits;
+    static constexpr int S = kDigits;
     static constexpr bool kCross = NJ > 0;
     static constexpr int MN = S * (NI + NJ);
     // Row tiles of 128 accumulator lanes: TS digits of the NI columns each.  A block against
     // itself needs a second tile only for its low digits against each other, (s, t) and (t, s)
     // being mirrors: tile 1 takes digits TS .. S-1 against TS .. TE-1 (FP64: digits 4 to 7 against
     // 4 and 5; what is left out, both digits 6 or 7, is below 2^-96 of the product).
-    static constexpr int TS = !kCross && S == 8 && NI > 16 ? 4 : cmin(S, 128 / NI);
+    static constexpr int TS = NI > 16 ? 4 : S;
     static constexpr int kTiles = TS < S ? 2 : 1;
-    static constexpr int TE = kCross || kTiles == 1 ? S : S == 8 ? 6 : S;
+    static constexpr int TE = kCross || kTiles == 1 ? S : 6;
     static constexpr int NR = kCross ? NJ : NI;            // columns of a right-hand digit
-    static constexpr int N0 = up16(S * NR);
-    static constexpr int N1 = kTiles == 1 ? 0 : kCross ? N0 : up16((TE - TS) * NI);
+    static constexpr int N0 = S * NR;
+    static constexpr int N1 = kTiles == 1 ? 0 : kCross ? N0 : (TE - TS) * NI;
     static constexpr int kCols = N0 + N1;                  // tensor-memory columns
     static constexpr int kSets = cmin(8, 512 / kCols);     // accumulator sets, 1,024 rows each
     static_assert(kCols <= 512 && (kTiles == 1 || 2 * TS >= S), "accumulators fit");
-    // Slicing: a task is four columns of a 64-row block, a warp's round has kTasks of them.
+    // Slicing: a task is four columns of a 64-row block, each warp has one a round.
     static constexpr int kGroups = (NI + NJ) / 4;
-    static constexpr int kMaxTasks = sizeof(Tin) == 8 ? 1 : MN > 192 ? 1 : 2;
-    static constexpr int kRoundKb = cmin(16, kMaxTasks * kGramWarps / kGroups);
-    static constexpr int kSlots = kRoundKb * kGroups;      // tasks of a round
-    static constexpr int kTasks = (kSlots + kGramWarps - 1) / kGramWarps;
-    static_assert(kRoundKb >= 1 && kGroups <= kMaxTasks * kGramWarps, "a block a round");
+    static constexpr int kRoundKb = kGramWarps / kGroups;
+    static_assert(kRoundKb >= 1, "a block a round");
     static constexpr int kKbBytes = MN * 128;              // 64 FP16 per operand row
     static constexpr int kStage = kRoundKb * kKbBytes;
-    // A task's raw bytes: a lane's eight entries; BF16 keeps 16 more a column (entries that
-    // are not 16-byte aligned straddle two pieces).
-    static constexpr int kTaskRaw = sizeof(Tin) == 2 ? 576 : 256 * (int)sizeof(Tin);
-    static constexpr int kRaw = kGramWarps * kTasks * kTaskRaw;
-    static constexpr int kRaws = cmin(8, 65536 / kRaw);    // rounds on their way
-    static_assert(kRaws >= 2, "a round is copied while another is sliced");
-    // Flush: partial sums (64-bit) of JP columns at a time over the stages, [part][row digit][j]
-    // [i]; parts: digits t < TA of tile 0 (or of the cross tiles), the others.
-    static constexpr int TA = kCross || kTiles == 1 ? cmin(4, S) : TS;
+    static constexpr int kRaw = kGramWarps * 2048;         // a round of A: 64 bytes a lane
+    static constexpr int kRaws = 2;                        // rounds on their way
+    // Flush: partial sums (64-bit) of JP columns at a time over the stages, [half][row digit]
+    // [j][i]; halves: digits 0-3 and 4-7 of the right-hand columns.
     static constexpr bool kMirror = !kCross && kTiles == 2;
-    static constexpr int kParts = TA < S ? 2 : 1;
-    static constexpr int kRowDigits = kCross ? S : cmin(TS, S);
+    static constexpr int kRowDigits = kCross ? S : TS;
     static constexpr int kLd = NI + 1;
     static constexpr int per_j() {
-        return (kRowDigits * kParts + (kMirror ? S - TS : 0)) * kLd * 8;
+        return (kRowDigits * 2 + (kMirror ? S - TS : 0)) * kLd * 8;
     }
     static constexpr int kStages = 2 * kStage;
     static constexpr int jp() {
@@ -113,12 +88,12 @@ constexpr int kHead = 2048;
 static_assert(sizeof(Smem) <= kHead, "the stages start at a multiple of 1,024 bytes");
 template <typename Sh>
 constexpr size_t smem_bytes() {
-    return kHead + Sh::kStages + cmax(Sh::kRaws * Sh::kRaw, 16384) + Sh::kU;
+    return kHead + Sh::kStages + Sh::kRaws * Sh::kRaw + Sh::kU;
 }
 
 // ------------------------------------------------------------------------------------------
 // Digits.  One entry in fixed point: |x| = Q units, d = D - exponent >= 2 (so Q fills at most
-// 62 of 64 bits, 30 of 32), plus 128 in every byte: byte k minus 128 is then the balanced digit
+// 62 of 64 bits), plus 128 in every byte: byte k minus 128 is then the balanced digit
 // of weight 256^k.  (A shift by the word's size or more gives 0: zero and subnormal entries.)
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ u64 fix64(const double x, const int D, int &dmin) {
@@ -129,14 +104,6 @@ __device__ __forceinline__ u64 fix64(const double x, const int D, int &dmin) {
     u64 q;
     asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(mant), "r"((unsigned)d));
     return q + 0x8080808080808080ull;
-}
-__device__ __forceinline__ uint32_t fix32(const uint32_t b, const int D, int &dmin) {
-    const int d = D - (int)((b >> 23) & 0xff);
-    dmin = min(dmin, d);
-    const uint32_t mant = ((b & 0x7fffff) | 0x800000) << 8;
-    uint32_t q;
-    asm("shr.u32 %0, %1, %2;" : "=r"(q) : "r"(mant), "r"((unsigned)d));
-    return q + 0x80808080u;
 }
 __device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t d;
@@ -156,118 +123,57 @@ __device__ __forceinline__ void digits4(const uint32_t w0, const uint32_t w1, co
 }
 
 // ------------------------------------------------------------------------------------------
-// Rows of a lane in a 64-row block: E = 16 / sizeof(Tin) consecutive rows at 8 E q + E c8 (eight
-// lanes read 128 consecutive bytes), the same for every column: the operand's rows are the
-// block's in another order, which the sums do not see.  A 16-byte piece q of the lane goes to
-// raw + 512 q (raw: the lane's), FP64 and FP32 in narrow copies where A is not 16-byte aligned.
-// BF16 copies aligned pieces always (144 bytes a column; the ninth piece by the last lane) and
-// reads its entries at the column's offset in them.  Rows past the end read as zeros.
+// Rows of a lane in a 64-row block: 16 q + 2 c8 + {0, 1}, q = 0..3 (eight lanes read 128
+// consecutive bytes), the same for every column: the operand's rows are the block's in another
+// order, which the sums do not see.  Piece q of the lane goes to raw + 512 q (the warp's q-th
+// pieces side by side) and only the lane itself reads it, so no barrier stands between; 8-byte
+// copies where A is not 16-byte aligned.  Rows past the end read as zeros (any: an address to name
+// where there is nothing to copy).
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ void copy16(void *dst, const void *src, const int bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(tc::smem_u32(dst)),
-                 "l"(src), "r"(bytes)
+__device__ __forceinline__ void copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tc::smem_u32(dst)), "l"(src)
                  : "memory");
 }
-template <typename Tin>
-__device__ __forceinline__ void copy_rows(unsigned char *raw, const Tin *p, const int64_t left,
-                                          const int c8, const bool vec, const void *any) {
-    if constexpr (sizeof(Tin) == 2) {
-        const uintptr_t first = (uintptr_t)p, base = first & ~(uintptr_t)15;
-        const uintptr_t end = left <= 0 ? 0 : first + 2 * (uintptr_t)(left < 64 ? left : 64);
+__device__ __forceinline__ void copy_rows(unsigned char *raw, const double *p, const int64_t left,
+                                          const int c8, const bool vec, const double *any) {
+    if (left >= 64 && vec) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (q == 1 && (c8 != 7 || first == base)) break;
-            const uintptr_t at = base + 16 * (c8 + q);
-            const int bytes = at >= end ? 0 : end - at >= 16 ? 16 : (int)(end - at);
-            copy16(raw + 16 * q, bytes ? (const void *)at : any, bytes);
-        }
+        for (int q = 0; q < 4; ++q) copy16(raw + 512 * q, p + 16 * q + 2 * c8);
     } else {
-        constexpr int E = 16 / (int)sizeof(Tin);
-        if (left >= 64 && vec) {
 #pragma unroll
-            for (int q = 0; q < 8 / E; ++q) copy16(raw + 512 * q, p + 8 * E * q + E * c8, 16);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int r = 8 * E * (e / E) + E * c8 + e % E;
-                unsigned char *to = raw + 512 * (e / E) + (int)sizeof(Tin) * (e % E);
-                if constexpr (sizeof(Tin) == 8)
-                    cp_async8(to, r < left ? p + r : any, r < left ? 8 : 0);
-                else
-                    cp_async4(to, r < left ? p + r : any, r < left ? 4 : 0);
-            }
+        for (int e = 0; e < 8; ++e) {
+            const int r = 16 * (e >> 1) + 2 * c8 + (e & 1);
+            cp_async8(raw + 512 * (e >> 1) + 8 * (e & 1), r < left ? p + r : any, r < left ? 8 : 0);
         }
-    }
-}
-// The lane's FP32 bit patterns (FP32 and BF16).  off: the column's byte offset in its 16-byte pieces.
-template <typename Tin>
-__device__ __forceinline__ void read_words(uint32_t (&w)[8], const unsigned char *raw, const int off) {
-    if constexpr (sizeof(Tin) == 4) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const uint4 t = *reinterpret_cast<const uint4 *>(raw + 512 * q);
-            w[4 * q] = t.x, w[4 * q + 1] = t.y, w[4 * q + 2] = t.z, w[4 * q + 3] = t.w;
-        }
-    } else if (off == 0) {
-        const uint4 t = *reinterpret_cast<const uint4 *>(raw);
-        const uint32_t v[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[2 * q] = v[q] << 16, w[2 * q + 1] = v[q] & 0xffff0000u;
-    } else {
-        const unsigned short *h = reinterpret_cast<const unsigned short *>(raw + off);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = (uint32_t)h[e] << 16;
     }
 }
 // Largest biased exponent of the lane's eight entries.
-template <typename Tin>
-__device__ __forceinline__ int max_exponent(const unsigned char *raw, const int off) {
+__device__ __forceinline__ int max_exponent(const unsigned char *raw) {
     int e = 0;
-    if constexpr (sizeof(Tin) == 8) {
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
-            e = max(e, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
-        }
-    } else {
-        uint32_t w[8];
-        read_words<Tin>(w, raw, off);
-#pragma unroll
-        for (int p = 0; p < 8; ++p) e = max(e, (int)((w[p] >> 23) & 0xff));
+    for (int p = 0; p < 4; ++p) {
+        const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
+        e = max(e, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
     }
     return e;
 }
 // The lane's eight entries as digits: digit s to dst + s step.
-template <typename Tin>
-__device__ __forceinline__ void slice8(const unsigned char *raw, const int off, const int D,
-                                       int &dmin, unsigned char *dst, const int step) {
-    constexpr int S = Type<Tin>::kDigits;
-    uint32_t o[8][4];
-    if constexpr (sizeof(Tin) == 8) {
+__device__ __forceinline__ void slice8(const unsigned char *raw, const int D, int &dmin,
+                                       unsigned char *dst, const int step) {
+    uint32_t o[kDigits][4];
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
-            const u64 q0 = fix64(v.x, D, dmin), q1 = fix64(v.y, D, dmin);
-            const uint32_t sg =
-                __byte_perm(__double2hiint(v.x), __double2hiint(v.y), 0x7632) & 0x80008000u;
-            const uint32_t sgn = sg | 0x3c003c00u, of = sg ^ 0xe480e480u;
-            digits4((uint32_t)(q0 >> 32), (uint32_t)(q1 >> 32), sgn, of, o[0][p], o[1][p], o[2][p],
-                    o[3][p]);
-            digits4((uint32_t)q0, (uint32_t)q1, sgn, of, o[4][p], o[5][p], o[6][p], o[7][p]);
-        }
-    } else {
-        uint32_t w[8];
-        read_words<Tin>(w, raw, off);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const uint32_t q0 = fix32(w[2 * p], D, dmin), q1 = fix32(w[2 * p + 1], D, dmin);
-            const uint32_t sg = __byte_perm(w[2 * p], w[2 * p + 1], 0x7632) & 0x80008000u;
-            const uint32_t sgn = sg | 0x3c003c00u, of = sg ^ 0xe480e480u;
-            digits4(q0, q1, sgn, of, o[0][p], o[1][p], o[2][p], o[3][p]);
-        }
+    for (int p = 0; p < 4; ++p) {
+        const double2 v = *reinterpret_cast<const double2 *>(raw + 512 * p);
+        const u64 q0 = fix64(v.x, D, dmin), q1 = fix64(v.y, D, dmin);
+        const uint32_t sg =
+            __byte_perm(__double2hiint(v.x), __double2hiint(v.y), 0x7632) & 0x80008000u;
+        const uint32_t sgn = sg | 0x3c003c00u, off = sg ^ 0xe480e480u;
+        digits4((uint32_t)(q0 >> 32), (uint32_t)(q1 >> 32), sgn, off, o[0][p], o[1][p], o[2][p],
+                o[3][p]);
+        digits4((uint32_t)q0, (uint32_t)q1, sgn, off, o[4][p], o[5][p], o[6][p], o[7][p]);
     }
 #pragma unroll
-    for (int s = 0; s < S; ++s)
+    for (int s = 0; s < kDigits; ++s)
         *reinterpret_cast<uint4 *>(dst + s * step) = make_uint4(o[s][0], o[s][1], o[s][2], o[s][3]);
 }
 
@@ -315,7 +221,7 @@ struct Cta {
 };
 template <typename Sh>
 __device__ __forceinline__ Q128 *sums_of(const Cta &c) {
-    return reinterpret_cast<Q128 *>(c.stages + Sh::kStages + cmax(Sh::kRaws * Sh::kRaw, 16384));
+    return reinterpret_cast<Q128 *>(c.stages + Sh::kStages + Sh::kRaws * Sh::kRaw);
 }
 
 // Columns of an item: local column l < NI is column i0 + l of the matrix (l < ni), NI + l is j0 + l.
@@ -326,11 +232,10 @@ struct Cols {
 // The sums of one set over the 64-row blocks [kb0, kb1): in c.U (the lower half of a block
 // against itself holds what its mirror adds), exponents in sm.D, sm.bad where the rows cannot be
 // served.  Every thread of the CTA; all copies and tensor-core work have ended on return.
-template <typename Tin, int NI, int NJ>
+template <int NI, int NJ>
 __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, const int64_t kb0,
                                          const int64_t kb1, Cta &c) {
-    using Sh = Shape<Tin, NI, NJ>;
-    using Ty = Type<Tin>;
+    using Sh = Shape<NI, NJ>;
     constexpr int S = Sh::S;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Smem &sm = *c.sm;
@@ -340,50 +245,30 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     for (int o = tid; o < NI * Sh::NR; o += kGramThreads) c.U[o] = Q128{0, 0};
 
     const int rounds = (int)((kb1 - kb0 + Sh::kRoundKb - 1) / Sh::kRoundKb);
-    const Tin *A = (const Tin *)p.A, *B = (const Tin *)p.B;
-    constexpr int kAlign = 16 / (int)sizeof(Tin);
-    const bool vec = ((p.lda | (B ? p.ldb : 0)) & (kAlign - 1)) == 0 &&
-                     (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+    const double *A = p.A, *B = p.B;
+    const bool vec = ((p.lda | (B ? p.ldb : 0)) & 1) == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
     const int c8 = lane & 7;
 
-    // the lane's column, block and operand address in each of its tasks
-    struct Task {
-        const Tin *src;
-        int kbo, lc, dst, off;
-        bool mine;
-    };
-    Task tk[Sh::kTasks];
-#pragma unroll
-    for (int t = 0; t < Sh::kTasks; ++t) {
-        const int id = warp + t * kGramWarps;
-        tk[t].kbo = id / Sh::kGroups;
-        const int lc = 4 * (id % Sh::kGroups) + (lane >> 3);
-        const bool right = NJ > 0 && lc >= NI;
-        const int g = right ? cols.j0 + lc - NI : cols.i0 + lc;
-        tk[t].lc = lc;
-        tk[t].mine = id < Sh::kSlots && (right ? lc - NI < cols.nj : lc < cols.ni);
-        tk[t].src = (g < p.na ? A + (int64_t)g * p.lda : B + (int64_t)(g - p.na) * p.ldb) +
-                    (kb0 + tk[t].kbo) * 64;
-        tk[t].off = sizeof(Tin) == 2 ? (int)((uintptr_t)tk[t].src & 15) : 0;
-        const int row = right ? S * NI + lc - NI : lc;  // of digit 0; the others 8-row atoms away
-        tk[t].dst = tk[t].kbo * Sh::kKbBytes + (row >> 3) * 1024 + (row & 7) * 128 +
-                    ((c8 ^ (row & 7)) << 4);
-    }
-    unsigned char *const raw0 = c.stages + Sh::kStages + warp * Sh::kTasks * Sh::kTaskRaw +
-                                (sizeof(Tin) == 2 ? (lane >> 3) * 144 + c8 * 16 : lane * 16);
-    auto raw_of = [&](const int r, const int t) {
-        return raw0 + (r % Sh::kRaws) * Sh::kRaw + t * Sh::kTaskRaw;
-    };
+    // the lane's column, block and operand address
+    const int kbo = warp / Sh::kGroups, lc = 4 * (warp % Sh::kGroups) + (lane >> 3);
+    const bool right = NJ > 0 && lc >= NI;
+    const bool mine = warp < Sh::kRoundKb * Sh::kGroups &&
+                      (right ? lc - NI < cols.nj : lc < cols.ni);
+    const int gcol = right ? cols.j0 + lc - NI : cols.i0 + lc;
+    const double *const src = (gcol < p.na ? A + (int64_t)gcol * p.lda
+                                           : B + (int64_t)(gcol - p.na) * p.ldb) + (kb0 + kbo) * 64;
+    const int row0 = right ? S * NI + lc - NI : lc;  // operand row of digit 0
+    unsigned char *const dst = c.stages + kbo * Sh::kKbBytes + (row0 >> 3) * 1024 +
+                               (row0 & 7) * 128 + ((c8 ^ (row0 & 7)) << 4);
+    const int step = (right ? NJ : NI) * 128;        // from digit to digit
+    unsigned char *const raw0 = c.stages + Sh::kStages + warp * 2048 + lane * 16;
+    auto raw_of = [&](const int r) { return raw0 + (r % Sh::kRaws) * Sh::kRaw; };
     // Round r of A on its way to shared memory (one cp.async group a round, empty at the end).
     auto load_round = [&](const int r) {
-        if (r < rounds) {
-#pragma unroll
-            for (int t = 0; t < Sh::kTasks; ++t)
-                if (tk[t].mine) {
-                    const int64_t kb = kb0 + tk[t].kbo + (int64_t)r * Sh::kRoundKb;
-                    copy_rows<Tin>(raw_of(r, t), tk[t].src + (int64_t)r * (64 * Sh::kRoundKb),
-                                   kb < kb1 ? p.m - kb * 64 : 0, c8, vec, A);
-                }
+        if (mine && r < rounds) {
+            const int64_t kb = kb0 + kbo + (int64_t)r * Sh::kRoundKb;
+            copy_rows(raw_of(r), src + (int64_t)r * (64 * Sh::kRoundKb),
+                      kb < kb1 ? p.m - kb * 64 : 0, c8, vec, A);
         }
         cp_async_commit();
     };
@@ -392,21 +277,18 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     // keep theirs.  A column's exponents so follow from its slab alone, whatever set it is in: the
     // sets of a matrix sum the digits of one and the same matrix.  True if any column changes.
     auto scan_block = [&](const int r, const int kb) {
+        const bool here = mine && kbo == kb;
+        int top = here ? max_exponent(raw_of(r)) : 0;
 #pragma unroll
-        for (int t = 0; t < Sh::kTasks; ++t) {
-            const bool here = tk[t].mine && tk[t].kbo == kb;
-            int e = here ? max_exponent<Tin>(raw_of(r, t), tk[t].off) : 0;
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-            if (c8 == 0 && here) atomicMax(&sm.E[tk[t].lc], e);
-        }
+        for (int o = 1; o < 8; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (c8 == 0 && here) atomicMax(&sm.E[lc], top);
         __syncthreads();
         bool up = false;
         if (tid < NI + NJ) {
             const int e = sm.E[tid];
-            if (e > Ty::kExpHi) sm.bad = 1;
+            if (e > kExpHi) sm.bad = 1;
             up = e + 2 > sm.D[tid];
-            sm.Dnew[tid] = up ? max(e, Ty::kExpLo) + 4 : sm.D[tid];
+            sm.Dnew[tid] = up ? max(e, kExpLo) + 4 : sm.D[tid];
             sm.E[tid] = 0;
         }
         return __syncthreads_or(up) != 0;
@@ -442,10 +324,10 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         const int part = warp >> 2, lrow = 32 * (warp & 3) + lane, s = lrow / NI, i = lrow - s * NI;
         const uint32_t lanes = c.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         long long *buf = reinterpret_cast<long long *>(c.stages);
-        constexpr int kPart = Sh::kRowDigits * Sh::JP * Sh::kLd;     // words of a part
-        constexpr int kL1 = Sh::kParts * kPart;                      // then tile 1's, [s - TS][j][i]
-        // sum over the sets of K digits of columns at .. at + 7, weighted 256^(W - 1 - t)
-        auto digits = [&](auto K, auto W, long long (&x)[8], const uint32_t at) {
+        constexpr int kHalf = Sh::kRowDigits * Sh::JP * Sh::kLd;     // words of a half
+        constexpr int kL1 = 2 * kHalf;                               // then tile 1's, [s - TS][j][i]
+        // sum over the sets of K <= 4 digits of columns at .. at + 7, weighted 256^(3 - t)
+        auto digits = [&](auto K, long long (&x)[8], const uint32_t at) {
             int v[K][8];
 #pragma unroll
             for (int t = 0; t < K; ++t)
@@ -465,8 +347,8 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             for (int e = 0; e < 8; ++e) {
                 long long y = 0;
 #pragma unroll
-                for (int t = 0; t < W; ++t) y = y * 256 + (t < K ? v[t < K ? t : 0][e] : 0);
-                x[e] = y;
+                for (int t = 0; t < K; ++t) y = y * 256 + v[t][e];
+                x[e] = y << (8 * (4 - K));
             }
         };
         auto put = [&](const int at, const long long (&x)[8]) {
@@ -479,26 +361,16 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
                 const int tile = task / kJ, jl = 8 * (task - tile * kJ);
                 const uint32_t at = lanes + (tile ? Sh::N0 : 0) + jb + jl;
                 long long x[8];
-                if constexpr (Sh::kMirror) {
-                    if (tile == 1) {
-                        // digits TS .. TE-1, in the word whose last digit is 3 (S <= 4) or 7
-                        digits(std::integral_constant<int, Sh::TE - Sh::TS>(),
-                               std::integral_constant<int, (S > 4 ? 8 : 4) - Sh::TS>(), x, at);
-                        if (s < S - Sh::TS) put(kL1 + (s * Sh::JP + jl) * Sh::kLd, x);
-                        continue;
-                    }
-                }
-                {
+                if (Sh::kMirror && tile == 1) {
+                    digits(std::integral_constant<int, Sh::kMirror ? Sh::TE - Sh::TS : 4>(), x, at);
+                    if (s < S - Sh::TS) put(kL1 + (s * Sh::JP + jl) * Sh::kLd, x);
+                } else {
                     const int sr = s + tile * Sh::TS;  // the row's digit
                     const bool keep = s < Sh::TS && sr < Sh::kRowDigits;
-                    digits(std::integral_constant<int, Sh::TA>(), std::integral_constant<int, 4>(), x, at);
+                    digits(std::integral_constant<int, 4>(), x, at);
                     if (keep) put((sr * Sh::JP + jl) * Sh::kLd, x);
-                    if constexpr (Sh::kParts == 2) {
-                        digits(std::integral_constant<int, S - Sh::TA>(),
-                               std::integral_constant<int, (S > 4 ? 8 : 4) - Sh::TA>(), x,
-                               at + Sh::TA * Sh::NR);
-                        if (keep) put(kPart + (sr * Sh::JP + jl) * Sh::kLd, x);
-                    }
+                    digits(std::integral_constant<int, 4>(), x, at + 4 * Sh::NR);
+                    if (keep) put(kHalf + (sr * Sh::JP + jl) * Sh::kLd, x);
                 }
             }
             tc::fence_before_sync();
@@ -507,21 +379,20 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             auto add = [&](i128 &g, const long long x, const int sh) {
                 g += sh >= 0 ? (i128)x << (sh >= 0 ? sh : 0) : (i128)(x >> (sh < 0 ? -sh : 0));
             };
-            for (int o = tid; o < NI * cmin(Sh::JP, Sh::NR); o += kGramThreads) {
+            for (int o = tid; o < NI * Sh::JP; o += kGramThreads) {
                 const int ii = o % NI, jl = o / NI, j = jb + jl;
-                if (j >= Sh::NR) break;
                 i128 g = 0, mir = 0;
 #pragma unroll
                 for (int sr = 0; sr < Sh::kRowDigits; ++sr) {
                     const int at = (sr * Sh::JP + jl) * Sh::kLd + ii;
                     add(g, buf[at], 64 - 8 * sr);
-                    if (Sh::kParts == 2) add(mir, buf[kPart + at], (S > 4 ? 32 : 64) - 8 * sr);
+                    add(mir, buf[kHalf + at], 32 - 8 * sr);
                 }
                 if (Sh::kMirror) {
 #pragma unroll
                     for (int sr = Sh::TS; sr < S; ++sr) {
                         const long long x = buf[kL1 + ((sr - Sh::TS) * Sh::JP + jl) * Sh::kLd + ii];
-                        const int sh = (S > 4 ? 32 : 64) - 8 * sr;
+                        const int sh = 32 - 8 * sr;
                         if (sr < Sh::TE)
                             add(g, x, sh);
                         else
@@ -573,12 +444,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     // of its column's range (the same for every thread).
     auto slice = [&](const int r, const int b, const int kb, const bool all) {
         int dmin = 2;
-#pragma unroll
-        for (int t = 0; t < Sh::kTasks; ++t)
-            if (tk[t].mine && (all || tk[t].kbo == kb))
-                slice8<Tin>(raw_of(r, t), tk[t].off, sm.D[tk[t].lc], dmin,
-                            c.stages + b * Sh::kStage + tk[t].dst,
-                            (NJ > 0 && tk[t].lc >= NI ? NJ : NI) * 128);
+        if (mine && (all || kbo == kb)) slice8(raw_of(r), sm.D[lc], dmin, dst + b * Sh::kStage, step);
         tc::fence_proxy_async();
         return __syncthreads_or(dmin < 2) == 0;
     };
@@ -586,7 +452,6 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
 #pragma unroll 1
     for (int r = 0; r < Sh::kRaws; ++r) load_round(r);
     cp_async_wait<Sh::kRaws - 1>();
-    if (sizeof(Tin) == 2) __syncwarp();
     __syncthreads();
     scan_block(0, 0);
     if (tid < NI + NJ) sm.D[tid] = sm.Dnew[tid];
@@ -597,8 +462,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     for (int r = 0; r < rounds && !sm.bad; ++r) {
         const int b = r & 1;
         cp_async_wait<Sh::kRaws - 1>();
-        if (sizeof(Tin) == 2) __syncwarp();
-        wait_stage(b);
+            wait_stage(b);
         if (slice(r, b, 0, true)) {
             multiply(b, 0, Sh::kRoundKb);
         } else {
@@ -776,14 +640,13 @@ __device__ __forceinline__ D2 sqrt2(const D2 x) {
 
 // C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it.  rowv: 3 n
 // entries of scratch.  g[j]: the power of two of R's column j.  Returns false if a pivot is too small.
-__device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int pivot_bits,
-                                         const int *g, double *R, const int64_t ldr) {
+static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g, double *R, const int64_t ldr) {
     const int tid = threadIdx.x, nt = kGramThreads, warp = tid >> 5, lane = tid & 31;
     Q128 *Lq = rowv, *Cp = rowv + n, *dv = rowv + 2 * n;
     for (int k = 0; k < n; ++k) {
         Q128 *Ck = C + rowoff(n, k) - k;
         const i128 d0 = unpack(Ck[k]);
-        if (d0 < ((i128)1 << (122 - pivot_bits))) return false;  // the same for every thread
+        if (d0 < ((i128)1 << (122 - kPivotBits))) return false;  // the same for every thread
         const u64 dh = (u64)((u128)d0 >> 64);
         const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d0);
         const int z = (122 - len) >> 1;
@@ -848,10 +711,9 @@ __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const
 }
 
 // Every set's sum (all written): gathered, scaled and factored; R written.  False: not served.
-template <typename Tin>
-__device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_bytes, Smem *smp,
+static __device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_bytes, Smem *smp,
                                     unsigned char *base) {
-    constexpr int NB = Type<Tin>::kBlock;
+    constexpr int NB = kBlock;
     const int tid = threadIdx.x, n = p.n;
     Smem &sm = *smp;
     Q128 *C = reinterpret_cast<Q128 *>(base);
@@ -894,7 +756,7 @@ __device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_byte
         const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d);
         sm.E[tid] = d > 0 ? (122 - len) >> 1 : 0;  // shift of the column
         if (!(d > 0)) sm.bad = 1;
-        sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + Type<Tin>::kUnit;
+        sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + kUnit;
     }
     __syncthreads();
     if (sm.bad) return false;
@@ -904,16 +766,16 @@ __device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_byte
         C[rowoff(n, i) - i + j] = pack(shift128(entry(i, j), sm.E[i] + sm.E[j]));
     }
     __syncthreads();
-    return factor_root(C, rowv, n, Type<Tin>::kPivotBits, sm.Dnew, p.R, p.ldr);
+    return factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr);
 }
 
 // One work item: its rows' sums and the climb.  True in the CTA that has written the set's sum.
-template <typename Tin, int NI, int NJ>
+template <int NI, int NJ>
 __device__ __forceinline__ bool item_of(const GramProblem &p, const Cols cols, const int set,
                                         const int slab, const size_t slot_bytes, Cta &c) {
     const int64_t kb0 = (int64_t)slab * p.nkb / p.nslab, kb1 = (int64_t)(slab + 1) * p.nkb / p.nslab;
-    sum_rows<Tin, NI, NJ>(p, cols, kb0, kb1, c);
-    return climb<NI, NJ, Shape<Tin, NI, NJ>::NR>(p, cols, set, slab, slot_bytes, c);
+    sum_rows<NI, NJ>(p, cols, kb0, kb1, c);
+    return climb<NI, NJ, Shape<NI, NJ>::NR>(p, cols, set, slab, slot_bytes, c);
 }
 
 // Tensor memory and barriers of the CTA; smem: its dynamic shared memory.

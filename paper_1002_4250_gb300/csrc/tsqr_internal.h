@@ -31,6 +31,8 @@ int f64_blocks_per_sm(int warps, size_t smem_bytes);
 cudaError_t f64_launch(const F64Args &a, int warps, size_t smem_bytes, cudaStream_t stream);
 cudaError_t zero_lower_launch(double *R, int64_t ldr, int n, const unsigned int *skip,
                               cudaStream_t stream);
+cudaError_t copy_cols_launch(const double *src, int64_t lds, double *dst, int64_t ldd, int64_t m,
+                             int n, const unsigned int *skip, cudaStream_t stream);
 cudaError_t f64_combine_launch(int n, const double *R1, int64_t ld1, const double *R2,
                                int64_t ld2, double *R, int64_t ldr, int normalize, int warps,
                                int ldS, int hs, size_t smem_bytes, int *status,
@@ -40,7 +42,6 @@ cudaError_t f64_combine_launch(int n, const double *R1, int64_t ld1, const doubl
 // cooperative launch of at most one CTA per SM).
 struct GramArgs;
 int gram_round_rows(int n);
-int gram_slot_block(int n);
 size_t gram_smem_bytes(int n);
 cudaError_t gram_prepare(int n, size_t smem_bytes);
 cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream);

@@ -928,6 +928,73 @@ __global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs 
 // R X = C for R upper triangular (n x n), C (n x k, leading dimension ldc): one warp per column,
 // rows last to first, each row's sum over the solved rows split across the lanes (a fixed
 // butterfly).  A zero or non-finite result is noted in the status word.
+// R X = C for n <= 32 T: one warp a column, row i of the running right-hand side in lane i % 32.
+// From the last row up, x_i goes to every lane by shuffles and is taken out of the rows above, the
+// next columns of R already on their way (their loads do not wait for x).  The quotient is a
+// product with the row's reciprocal (a division, some 375 cycles, would be most of a row's chain)
+// and its residual: x_i and the right-hand side are kept as a double and what its rounding left
+// out, so X carries the rounding of its last addition.  n = 32, one column: row sums with
+// divisions took 20 us.
+template <int T>
+__global__ void __launch_bounds__(256) tsqr_trsm_small_kernel(const double *R, int64_t ldr,
+                                                              const double *C, int64_t ldc, double *X,
+                                                              int64_t ldx, int n, int k, int *status) {
+    constexpr int kAhead = 4;
+    const int lane = threadIdx.x & 31;
+    const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (q >= k) return;
+    double s[T], lo[T], inv[T], dia[T], col[kAhead][T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        const int i = lane + 32 * t;
+        s[t] = i < n ? C[i + (int64_t)q * ldc] : 0.0;
+        lo[t] = 0.0;
+        dia[t] = i < n ? R[i + (int64_t)i * ldr] : 1.0;
+        inv[t] = 1.0 / dia[t];
+    }
+    auto fetch = [&](const int i, double (&v)[T]) {
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const int r = lane + 32 * t;
+            v[t] = r < i ? R[r + (int64_t)i * ldr] : 0.0;
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) fetch(n - 1 - u, col[u]);
+    bool bad = false;
+    for (int i0 = n - 1; i0 >= 0; i0 -= kAhead) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int i = i0 - u;
+            if (i < 0) continue;
+            double x = 0.0, y = 0.0;
+#pragma unroll
+            for (int t = 0; t < T; ++t)
+                if (t == i >> 5) {
+                    x = s[t] * inv[t];
+                    y = (fma(-x, dia[t], s[t]) + lo[t]) * inv[t];
+                    if (lane == (i & 31)) s[t] = x + y;
+                }
+            x = __shfl_sync(0xffffffffu, x, i & 31);
+            y = __shfl_sync(0xffffffffu, y, i & 31);
+            bad |= !isfinite(x);
+#pragma unroll
+            for (int t = 0; t < T; ++t)
+                if (lane + 32 * t < i) {
+                    const double p = col[u][t] * x, e = fma(col[u][t], x, -p);
+                    const double d = s[t] - p, v = d - s[t];
+                    lo[t] += ((s[t] - (d - v)) - (p + v)) - fma(col[u][t], y, e);
+                    s[t] = d;
+                }
+            fetch(i - kAhead, col[u]);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+        if (lane + 32 * t < n) X[lane + 32 * t + (int64_t)q * ldx] = s[t];
+    if (bad && lane == 0 && status) atomicOr(status, kStatusNonfiniteBit);
+}
+
 __global__ void __launch_bounds__(1024) tsqr_trsm_kernel(const double *R, int64_t ldr,
                                                          const double *C, int64_t ldc, double *X,
                                                          int64_t ldx, int n, int k, int *status) {
@@ -1034,6 +1101,16 @@ cudaError_t qt_wy_launch(const QtArgs &a, size_t smem_bytes, cudaStream_t stream
 cudaError_t trsm_launch(const double *R, int64_t ldr, const double *C, int64_t ldc, double *X,
                         int64_t ldx, int n, int k, int *status, cudaStream_t stream) {
     const int warps = 8;
+    if (n <= 128) {
+        const dim3 grid((k + 7) / 8), block(k < 8 ? 32 * k : 256);
+        if (n <= 32)
+            tsqr_trsm_small_kernel<1><<<grid, block, 0, stream>>>(R, ldr, C, ldc, X, ldx, n, k, status);
+        else if (n <= 64)
+            tsqr_trsm_small_kernel<2><<<grid, block, 0, stream>>>(R, ldr, C, ldc, X, ldx, n, k, status);
+        else
+            tsqr_trsm_small_kernel<4><<<grid, block, 0, stream>>>(R, ldr, C, ldc, X, ldx, n, k, status);
+        return cudaGetLastError();
+    }
     tsqr_trsm_kernel<<<(k + warps - 1) / warps, warps * 32, 0, stream>>>(R, ldr, C, ldc, X, ldx,
                                                                         n, k, status);
     return cudaGetLastError();

@@ -189,3 +189,28 @@ def test_column_blocks_handed_over(oracle, T, n, kind):
     if kind in ("repeated", "zero"):
         assert np.all(np.diag(R.cpu().numpy()) >= 0)
         assert oracle.gram_residual(oracle.from_torch_colmajor(At), R.cpu().numpy(), nthreads=16) <= 1e-13
+
+
+@pytest.mark.parametrize("m,n,k,pad", [(2048, 31, 1, 0), (30011, 32, 1, 1), (20000, 8, 2, 0),
+                                       (50001, 96, 24, 3), (40000, 55, 1, 0)])
+def test_least_squares_of_two_matrices(oracle, T, m, n, k, pad):
+    """[A | B] summed where A and B are; X against the oracle's least squares."""
+    import torch
+    At = workloads.gaussian(m, n, seed=n)
+    Bt = workloads.gaussian(m, k, seed=k + 1)
+    big = torch.full((n, m + pad), float("nan"), dtype=torch.float64)
+    big[:, :m] = At
+    X, R = T.tsqr_lstsq(big.cuda().T[:m, :], Bt.cuda().T)
+    _check(oracle, R, At)
+    A, B = oracle.from_torch_colmajor(At), oracle.from_torch_colmajor(Bt)
+    Xo = oracle.lstsq(A, B, nthreads=16)
+    kap = oracle.kappa_from_r(oracle.householder_r(A, nthreads=16))
+    res = np.linalg.norm(B - A @ Xo)
+    tol = max(50.0, 2.0 * np.sqrt(m)) * (kap + kap ** 2 * res /
+                                         (np.linalg.norm(A, 2) * np.linalg.norm(Xo))) * U
+    assert np.linalg.norm(X.cpu().numpy() - Xo) <= tol * np.linalg.norm(Xo)
+    At[n // 2] = At[0]  # dependent: the copy and the Householder reduction behind the sum
+    T.tsqr_get_device_status()
+    X, R = T.tsqr_lstsq(At.cuda().T, Bt.cuda().T)
+    T.tsqr_get_device_status()
+    assert oracle.gram_residual(oracle.from_torch_colmajor(At), R.cpu().numpy(), nthreads=16) <= 1e-13
