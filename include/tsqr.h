@@ -73,7 +73,7 @@ typedef enum { TSQR_PREC_F64 = 0, TSQR_PREC_MIXED = 1 } tsqr_prec_t;
  *         columns (0 = 16), each panel's R by its own TSQR reduction (AUTO plan, reflectors
  *         kept) and its Q^T applied to the columns right of it, as tsqr_caqr_r does (Section
  *         5's panel and update).  R equals one reduction's up to rounding.  With 16 columns (or
- *         0), up to TSQR_MAX_N columns and m >= max(1024, 16 n), the exact sum of TSQR_LEAF_GRAM is
+ *         0), up to TSQR_MAX_N columns and m >= max(256, 4 n), the exact sum of TSQR_LEAF_GRAM is
  *         tried first and the panels run only where it cannot serve.
  * AUTO picks HYBRID, or PANELS for FP64 R with n >= 56 and m >= 8 n, where it measured faster
  * (4,194,304 rows, n = 56 / 64 / 96 / 128: 775 / 828 / 863 / 887 against 727 / 750 / 555 / 586
@@ -101,7 +101,7 @@ typedef enum {
  *         (62 bits, in eight 8-bit digits), the digits' products are summed on the tensor cores
  *         (exact: whole numbers below 2^24 in FP32 accumulators), put together in 128-bit
  *         integers, added over the row blocks, and the sum is factored in 122-bit fixed point.
- *         m >= 1024, m >= 16 n; n < 56 here, wider through the PANELS tree.  A matrix it cannot
+ *         m >= 256, m >= 4 n; n < 56 here, wider through the PANELS tree.  A matrix it cannot
  *         serve (a NaN or Inf, entries outside 2^-400 .. 2^400, a pivot below 2^-64 of its
  *         column's square: zero or dependent columns) is found on the device, and the
  *         Householder leaves and tree that the plan's other fields describe run instead: up to 32

@@ -478,9 +478,9 @@ tsqr_status_t zero_r(double *R, int64_t n, int64_t ldr, cudaStream_t stream) {
 }
 
 // The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to kGramRootMaxN columns.
-constexpr int64_t kGramMinRows = 1024;
+constexpr int64_t kGramMinRows = 256;
 bool gram_fits(int64_t m, int64_t n) {
-    return n >= 1 && n <= kGramRootMaxN && m >= kGramMinRows && m >= 16 * n;
+    return n >= 1 && n <= kGramRootMaxN && m >= kGramMinRows && m >= 4 * n;
 }
 constexpr int kPanelsMinN = 56;
 
@@ -1799,6 +1799,66 @@ bool batch_plan_is_auto(const tsqr_batch_plan_t *p) {
                   p->leaf == 0);
 }
 
+// Gram problems (one per matrix of the batch; addresses of the workspace as offsets, in words and
+// bytes) and work items, the costliest first, of the matrices the sum serves.
+void plan_gram_batch(const void *const *ptrs, const int64_t *ms, const int32_t *ns,
+                     const int64_t *offsets, int32_t count, double *R_packed, int sms,
+                     std::vector<GramProblem> *probs, std::vector<int2> *items, size_t *words,
+                     size_t *slot_bytes, int32_t *served) {
+    // an item's cost: its rows times its columns (slicing), a block of 64 rows counting the fixed
+    // cost of an item as some kFixed more
+    constexpr double kFixed = 12.0;
+    double work = 0.0;
+    for (int32_t i = 0; i < count; ++i)
+        if (gram_fits(ms[i], ns[i])) {
+            const int nb = (ns[i] + 31) / 32;
+            work += (double)((ms[i] + 63) / 64) * ns[i] * nb;  // every column is sliced nb times
+        }
+    const double target = std::max(work / (4.0 * sms), 16.0 * 32);  // about four items a CTA
+    probs->assign(count, GramProblem{});
+    std::vector<std::pair<double, int2>> list;
+    for (int32_t i = 0; i < count; ++i) {
+        if (!gram_fits(ms[i], ns[i])) continue;
+        GramProblem &g = (*probs)[i];
+        g.A = (const double *)ptrs[i];
+        g.lda = g.m = ms[i];
+        g.n = g.na = ns[i];
+        g.nb = (ns[i] + 31) / 32;
+        g.nkb = (ms[i] + 63) / 64;
+        const int nset = gram_sets(g.nb);
+        const double all = (double)g.nkb * ns[i] * g.nb;
+        g.nslab = (int)std::max<double>(
+            1.0, std::min<double>(std::ceil(all / (nset * target)), (double)g.nkb / 8));
+        const int inner = gram_inner_nodes(g.nslab);
+        g.counters = (unsigned int *)*words;
+        *words += (size_t)nset * inner + 1;
+        g.slots = (unsigned char *)*slot_bytes;
+        *slot_bytes += (size_t)nset * (g.nslab + inner) * gram_slot_bytes(gram_block(ns[i]));
+        g.R = R_packed + offsets[i];
+        g.ldr = ns[i];
+        ++*served;
+        for (int set = 0; set < nset; ++set) {
+            int cols;
+            if (set < g.nb) {
+                cols = std::min(32, ns[i] - 32 * set);
+            } else {
+                int J = 1, o = set - g.nb;
+                while (o >= J) o -= J++;
+                cols = 32 + std::min(32, ns[i] - 32 * J);
+            }
+            for (int sl = 0; sl < g.nslab; ++sl)
+                list.push_back({((double)g.nkb / g.nslab + kFixed) * cols, make_int2(i, set + nset * sl)});
+        }
+    }
+    *slot_bytes = align_up(*slot_bytes, 256);
+    std::stable_sort(list.begin(), list.end(),
+                     [](const std::pair<double, int2> &a, const std::pair<double, int2> &b) {
+                         return a.first > b.first;
+                     });
+    items->reserve(list.size());
+    for (const auto &e : list) items->push_back(e.second);
+}
+
 tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int32_t *ns,
                           const int64_t *offsets, int32_t count, double *R_packed, int dt,
                           const tsqr_batch_plan_t *bp_in, cudaStream_t stream) {
@@ -1823,9 +1883,10 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
         return TSQR_ERR_INVALID_ARG;
     for (int b = 0; b < 4; ++b)
         if (bp.arity[b] != 0 && (bp.arity[b] < 2 || bp.arity[b] > 8)) return TSQR_ERR_INVALID_ARG;
-    if (bp.leaf != 0 && bp.leaf != TSQR_LEAF_FOLD && bp.leaf != TSQR_LEAF_PANELS)
-        return TSQR_ERR_INVALID_ARG;
     const bool mixed = dt != 0;
+    if (bp.leaf != 0 && bp.leaf != TSQR_LEAF_FOLD && bp.leaf != TSQR_LEAF_PANELS &&
+        (mixed || bp.leaf != TSQR_LEAF_GRAM))
+        return TSQR_ERR_INVALID_ARG;
     int nmax = 1;
     for (int32_t i = 0; i < count; ++i) nmax = std::max(nmax, (int)ns[i]);
     if (bp.leaf == TSQR_LEAF_PANELS && (!mixed || nmax > kMixedWyMaxN)) return TSQR_ERR_UNSUPPORTED;
@@ -1948,19 +2009,43 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
                          return a.first > b.first;
                      });
     if (items.size() > (size_t)0x7fffffff) return TSQR_ERR_UNSUPPORTED;
+    // FP64 (AUTO, or a plan that asks for it): the Gram sum of every problem it serves first, the
+    // fold behind it for the others and for those it finds it cannot serve
+    const bool gram = !mixed && (batch_plan_is_auto(&bp) || bp.leaf == TSQR_LEAF_GRAM);
+    std::vector<GramProblem> gprobs;
+    std::vector<int2> gitems;
+    size_t gwords = 0, gslots = 0;  // counters past the queue's two words, slot bytes
+    int32_t served = 0;
+    if (gram) plan_gram_batch(ptrs, ms, ns, offsets, count, R_packed, di.sms, &gprobs, &gitems,
+                              &gwords, &gslots, &served);
     // table: problems then items, copied once and reused while the batch is unchanged
-    std::vector<char> table(sizeof(BatchProblem) * probs.size() + sizeof(int2) * items.size());
+    const size_t tp = align_up(sizeof(BatchProblem) * probs.size(), 16);
+    const size_t ti = align_up(sizeof(int2) * items.size(), 16);
+    const size_t tg = served ? align_up(sizeof(GramProblem) * gprobs.size(), 16) : 0;
+    std::vector<char> table(tp + ti + tg + sizeof(int2) * gitems.size());
     std::memcpy(table.data(), probs.data(), sizeof(BatchProblem) * probs.size());
-    int2 *it_host = reinterpret_cast<int2 *>(table.data() + sizeof(BatchProblem) * probs.size());
+    int2 *it_host = reinterpret_cast<int2 *>(table.data() + tp);
     for (size_t k = 0; k < items.size(); ++k) it_host[k] = items[k].second;
 
-    const size_t head_bytes = align_up((size_t)(1 + nodes_total) * sizeof(unsigned int), 256);
+    const size_t words = 1 + (size_t)nodes_total + (served ? 2 + (size_t)count + gwords : 0);
+    const size_t head_bytes = align_up(words * sizeof(unsigned int), 256);
     const size_t slots_bytes = align_up((size_t)slot_doubles * sizeof(double), 256);
     Workspace *ws = nullptr;
-    tsqr_status_t st = get_workspace(stream, head_bytes + slots_bytes + table.size(), &ws);
+    tsqr_status_t st = get_workspace(stream, head_bytes + slots_bytes + gslots + table.size(), &ws);
     if (st != TSQR_SUCCESS) return st;
-    const size_t table_off = head_bytes + slots_bytes;
+    const size_t table_off = head_bytes + slots_bytes + gslots;
     char *base = (char *)ws->base;
+    unsigned int *gq = reinterpret_cast<unsigned int *>(base) + 1 + nodes_total;  // queue, failed
+    if (served) {
+        for (int32_t i = 0; i < count; ++i) {  // offsets become addresses
+            GramProblem &g = gprobs[i];
+            g.counters = gq + 2 + count + (size_t)g.counters;
+            g.slots = (unsigned char *)base + head_bytes + slots_bytes + (size_t)g.slots;
+            g.verdict = gq + 2 + i;
+        }
+        std::memcpy(table.data() + tp + ti, gprobs.data(), sizeof(GramProblem) * gprobs.size());
+        std::memcpy(table.data() + tp + ti + tg, gitems.data(), sizeof(int2) * gitems.size());
+    }
     if (ws->table != table || ws->table_off != table_off) {
         if (cudaMemcpyAsync(base + table_off, table.data(), table.size(), cudaMemcpyHostToDevice,
                             stream) != cudaSuccess)
@@ -1970,26 +2055,39 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
     }
     BatchArgs b;
     b.probs = reinterpret_cast<const BatchProblem *>(base + table_off);
-    b.items = reinterpret_cast<const int2 *>(base + table_off + sizeof(BatchProblem) * probs.size());
+    b.items = reinterpret_cast<const int2 *>(base + table_off + tp);
     b.nitems = (int)items.size();
     b.queue = reinterpret_cast<unsigned int *>(base);
     b.counters = b.queue + 1;
     b.slots = reinterpret_cast<double *>(base + head_bytes);
     b.status = ws->status;
-    if (cudaMemsetAsync(base, 0, (size_t)(1 + nodes_total) * sizeof(unsigned int), stream) !=
-        cudaSuccess)
+    b.verdicts = served ? gq + 2 : nullptr;
+    b.failed = served == count ? gq + 1 : nullptr;
+    if (cudaMemsetAsync(base, 0, words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
+    if (served) {
+        GramQueueArgs q;
+        std::memset(&q, 0, sizeof(q));
+        q.probs = reinterpret_cast<const GramProblem *>(base + table_off + tp + ti);
+        q.items = reinterpret_cast<const int2 *>(base + table_off + tp + ti + tg);
+        q.nitems = (int)gitems.size();
+        q.queue = gq;
+        q.failed = gq + 1;
+        q.status = ws->status;
+        if (gram_queue_launch(q, std::min(di.sms, q.nitems), stream) != cudaSuccess)
+            return TSQR_ERR_CUDA;
+    }
     const int grid = (int)std::min<int64_t>(ctas, (int64_t)items.size());
     if ((wy ? batched_wy_launch(b, grid, dt == 2, wy_h, wy_tcols, smem, stream)
             : batched_launch(kdt, b, grid, W, smem, stream)) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    g_last_launches = 1;
+    g_last_launches = served ? 2 : 1;
     tsqr_batch_plan_t used{};
     used.warps = W;
     used.ctas_per_sm = wy ? 1 : budget == one_per_sm ? 1 : 2;
     used.leaves_per_cta = lpc;
     for (int b2 = 0; b2 < 4; ++b2) used.arity[b2] = bp.arity[b2];
-    used.leaf = mixed ? (wy ? TSQR_LEAF_PANELS : TSQR_LEAF_FOLD) : 0;
+    used.leaf = mixed ? (wy ? TSQR_LEAF_PANELS : TSQR_LEAF_FOLD) : gram ? TSQR_LEAF_GRAM : 0;
     g_last_batch_plan = used;
     return TSQR_SUCCESS;
 }

@@ -10,6 +10,7 @@ namespace tsqr {
 template <typename T, typename Tin>
 __device__ __forceinline__ void batched_body(const BatchArgs &b) {
     __shared__ int s_item;
+    if (b.failed && *b.failed == 0) return;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = (int)atomicAdd(b.queue, 1u);
@@ -17,8 +18,10 @@ __device__ __forceinline__ void batched_body(const BatchArgs &b) {
         const int it = s_item;
         if (it >= b.nitems) return;
         const int2 w = b.items[it];
+        if (b.verdicts && skipped(b.verdicts + w.x)) continue;
         const BatchProblem P = b.probs[w.x];
         F64Args a;
+        a.skip = nullptr;
         a.A = static_cast<const double *>(P.A);
         a.m = P.m;
         a.lda = P.lda;

@@ -103,6 +103,9 @@ struct BatchArgs {
     double *slots;
     unsigned int *counters;  // zeroed per call
     int *status;
+    // Behind a Gram sum (else null): per problem, 1 where its R is there already; and, where
+    // every problem had its sum, the number of those it could not serve.
+    const unsigned int *verdicts, *failed;
 };
 
 // Leading dimension of the tree operator's FP64 view of the S region: odd, and room for

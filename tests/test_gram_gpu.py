@@ -214,3 +214,50 @@ def test_least_squares_of_two_matrices(oracle, T, m, n, k, pad):
     X, R = T.tsqr_lstsq(At.cuda().T, Bt.cuda().T)
     T.tsqr_get_device_status()
     assert oracle.gram_residual(oracle.from_torch_colmajor(At), R.cpu().numpy(), nthreads=16) <= 1e-13
+
+
+def test_batch_served_and_handed_over(oracle, T):
+    """A batch of matrices the sum serves (one and several column blocks, ragged), matrices it is
+    not tried on (too few rows), and matrices it hands over (a zero column, a repeated one, NaN)."""
+    import torch
+    g = torch.Generator().manual_seed(31)
+    ms = [300, 4097, 70001, 20000, 513, 255, 100, 0, 9000, 8192, 5000, 40000, 260, 3000]
+    ns = [5, 16, 33, 64, 128, 8, 64, 4, 24, 40, 7, 100, 65, 1]
+    bad = {8: "zero", 9: "repeated", 10: "nan"}
+    offs = [0]
+    for m, n in zip(ms, ns):
+        offs.append(offs[-1] + m * n)
+    buf = torch.randn(offs[-1], generator=g, dtype=torch.float64)
+    for i, kind in bad.items():
+        A = buf[offs[i]:offs[i + 1]].view(ns[i], ms[i])
+        if kind == "zero":
+            A[3] = 0.0
+        elif kind == "repeated":
+            A[ns[i] - 1] = A[0]
+        else:
+            A[2, 77] = float("nan")
+    bd = buf.cuda()
+    roff = [0]
+    for n in ns:
+        roff.append(roff[-1] + n * n)
+    ptrs = [bd.data_ptr() + 8 * o for o in offs[:-1]]
+    T.tsqr_get_device_status()
+    R = torch.full((roff[-1],), float("nan"), dtype=torch.float64, device="cuda")
+    T.tsqr_r_batched(ptrs, ms, ns, roff, R)
+    assert T.last_batch_plan().leaf == T.LEAF_GRAM
+    assert T.tsqr_get_device_status() == T.STATUS_NONFINITE
+    again = torch.zeros_like(R)
+    T.tsqr_r_batched(ptrs, ms, ns, roff, again, plan=T.last_batch_plan())
+    assert torch.equal(torch.nan_to_num(again), torch.nan_to_num(R))
+    T.tsqr_get_device_status()  # clears it
+    for i, (m, n) in enumerate(zip(ms, ns)):
+        Ri = R[roff[i]:roff[i + 1]].view(n, n).T
+        At = buf[offs[i]:offs[i + 1]].view(n, m)
+        if bad.get(i) == "nan":
+            assert not torch.isfinite(Ri).all()
+        elif m == 0:
+            assert torch.all(Ri == 0)
+        elif i in bad or m < 4 * n:
+            assert oracle.gram_residual(oracle.from_torch_colmajor(At), Ri.cpu().numpy()) <= 1e-13
+        else:
+            _check(oracle, Ri, At)
