@@ -477,10 +477,11 @@ tsqr_status_t zero_r(double *R, int64_t n, int64_t ldr, cudaStream_t stream) {
     return TSQR_SUCCESS;
 }
 
-// The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to kGramRootMaxN columns.
-constexpr int64_t kGramMinRows = 256;
+// The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to 2,048 columns (the fixed-
+// point matrix is then 64 MB).
+constexpr int64_t kGramMinRows = 256, kGramMaxCols = 2048;
 bool gram_fits(int64_t m, int64_t n) {
-    return n >= 1 && n <= kGramRootMaxN && m >= kGramMinRows && m >= 4 * n;
+    return n >= 1 && n <= kGramMaxCols && m >= kGramMinRows && m >= 4 * n;
 }
 constexpr int kPanelsMinN = 56;
 
@@ -534,7 +535,7 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
 // tree slots.
 struct GramLayout {
     int nb = 0, nset = 0, nslab = 0, inner = 0;
-    size_t words = 0, cnt_bytes = 0, bytes = 0;
+    size_t words = 0, cnt_bytes = 0, wide_off = 0, bytes = 0;
 };
 // Slabs: about five items a CTA (the last wave stays short; an item's fixed cost, its pipeline's
 // start, the flush and the climb, is some 7 us), of at least 512 rows.
@@ -547,10 +548,14 @@ GramLayout gram_layout(int64_t m, int64_t n, int sms) {
     w.nslab = (int)std::max<int64_t>(
         1, std::min<int64_t>(w.nset == 1 ? sms : 5LL * sms / w.nset, nkb / 8));
     w.inner = gram_inner_nodes(w.nslab);
-    w.words = 4 + (size_t)w.nset * w.inner;  // queue, failed, verdict, sets done, then the nodes
+    w.words = 5 + (size_t)w.nset * w.inner;  // queue, failed, verdict, bad, then the nodes, sets done
     w.cnt_bytes = align_up(w.words * sizeof(unsigned int), 256);
     w.bytes = w.cnt_bytes + (size_t)w.nset * (w.nslab + w.inner) *
                                 gram_slot_bytes(gram_block((int)n));
+    if (n > kGramRootMaxN) {  // the fixed-point matrix, a block row, pivots, per-column words
+        w.wide_off = align_up(w.bytes, 256);
+        w.bytes = w.wide_off + (size_t)n * n * 16 + (size_t)n * (32 * 16 + 16 + 4 * sizeof(int));
+    }
     return w;
 }
 // The Gram sum of [A | B] (B: columns na .. n-1, or none) and its factor R in the workspace at
@@ -558,7 +563,7 @@ GramLayout gram_layout(int64_t m, int64_t n, int sms) {
 tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_t lda,
                            const double *B, int64_t ldb, int64_t na, int64_t m, int64_t n,
                            void *base, double *R, int64_t ldr, int *status,
-                           const unsigned int **verdict, cudaStream_t stream) {
+                           const unsigned int **verdict, int *launches, cudaStream_t stream) {
     if (cudaMemsetAsync(base, 0, w.words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
     unsigned int *head = (unsigned int *)base;
@@ -574,7 +579,7 @@ tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_
     q.one.nb = w.nb;
     q.one.nslab = w.nslab;
     q.one.nkb = (m + 63) / 64;
-    q.one.counters = head + 3;
+    q.one.counters = head + 4;
     q.one.slots = (unsigned char *)base + w.cnt_bytes;
     q.one.verdict = head + 2;
     q.one.R = R;
@@ -584,8 +589,28 @@ tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_
     q.failed = head + 1;
     q.status = status;
     *verdict = head + 2;
-    return gram_queue_launch(q, std::min(sms, q.nitems), stream) == cudaSuccess ? TSQR_SUCCESS
-                                                                               : TSQR_ERR_CUDA;
+    if (gram_queue_launch(q, std::min(sms, q.nitems), stream) != cudaSuccess) return TSQR_ERR_CUDA;
+    ++*launches;
+    if (n <= kGramRootMaxN) return TSQR_SUCCESS;
+    GramWideArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.p = q.one;
+    char *at = (char *)base + w.wide_off;
+    g.C = at;
+    at += (size_t)n * n * 16;
+    g.P = at;
+    at += (size_t)n * 32 * 16;
+    g.d = at;
+    at += (size_t)n * 16;
+    g.D = (int *)at;
+    g.E = g.D + n;
+    g.g = g.E + n;
+    g.z = g.g + n;
+    g.bad = head + 3;
+    const int k = gram_wide_launch(g, stream);
+    if (k < 0) return TSQR_ERR_CUDA;
+    *launches += k;
+    return TSQR_SUCCESS;
 }
 
 // Workspace of one reduction under plan p: counters (zeroed per call), then tree slots, then the
@@ -622,9 +647,9 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
     a.status = status;
     if (p.gram_queue) {
         const tsqr_status_t st = enqueue_gram(w.g, sms, A, lda, nullptr, 0, n, m, n,
-                                              (char *)base + w.gram_off, R, ldr, status, &a.skip, stream);
+                                              (char *)base + w.gram_off, R, ldr, status, &a.skip, launches,
+                                              stream);
         if (st != TSQR_SUCCESS) return st;
-        ++*launches;
     }
     if ((p.gram_ctas ? gram_prepare((int)n, p.smem) : f64_prepare(p.smem)) != cudaSuccess)
         return TSQR_ERR_CUDA;
@@ -1011,6 +1036,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     // the Gram sum of [A | B] where it serves (it reads A and B where they are); the copy and the
     // Householder reduction stand behind it
     const bool gram = plan_is_auto(over) && gram_fits(m, na);
+    int launches = 0;
     const int sms = current_sms();
     GramLayout gl;
     if (gram) gl = gram_layout(m, na, sms);
@@ -1023,7 +1049,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     F64Args a = plan_args(p, aug, m, na, m);
     if (gram) {
         st = enqueue_gram(gl, sms, A, lda, B, ldb, n, m, na, (char *)Ra + ra_bytes, Ra, na, ws->status,
-                          &a.skip, stream);
+                          &a.skip, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
         if (na < kPanelsMinN)
             g_last_plan.leaf = TSQR_LEAF_GRAM;
@@ -1047,7 +1073,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     if (trsm_launch(Ra, na, Ra + n * na, na, X, ldx, (int)n, (int)k, ws->status, stream) !=
         cudaSuccess)
         return TSQR_ERR_CUDA;
-    g_last_launches = gram ? 5 : 4;
+    g_last_launches = launches + 4;
     return TSQR_SUCCESS;
 }
 
@@ -1473,9 +1499,8 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     const unsigned int *skip = nullptr;
     if (gram) {
         st = enqueue_gram(gl, di.sms, A, lda, nullptr, 0, N, m, N, base + total, R, ldr, ws->status,
-                          &skip, stream);
+                          &skip, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
-        ++launches;
     }
     void *bufs[kBufs];
     size_t o = 0;

@@ -116,7 +116,7 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
             else
                 root = item_of<32, 32>(p, cols, set, slab, slot_bytes, c);
         }
-        if (!root) continue;
+        if (!root || p.n > kGramRootMaxN) continue;  // (a wider matrix is factored by its own launches)
         if (nset > 1) {
             if (tid == 0)
                 c.sm->flag = atomicAdd(p.counters + (size_t)nset * gram_inner_nodes(p.nslab), 1u) + 1 ==

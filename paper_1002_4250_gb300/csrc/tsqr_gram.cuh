@@ -61,6 +61,15 @@ struct GramQueueArgs {     // a queue of work items
     int *status;
 };
 
+struct GramWideArgs {      // more columns than one CTA factors
+    GramProblem p;
+    void *C;               // n x n fixed-point values, row-major (upper part)
+    void *P;               // 32 x n: the current block row before its division by the pivots
+    void *d;               // n scaled pivots
+    int *D, *E, *g, *z;    // per column: exponent word, shift, R's power of two; per row: pivot shift
+    unsigned int *bad;     // non-zero: the sum cannot serve (zeroed per call)
+};
+
 // Inner nodes and all nodes of the sum's tree over `leaves` leaves.
 __host__ __device__ inline int gram_inner_nodes(int leaves) {
     int inner = 0;

@@ -48,6 +48,10 @@ cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t strea
 // A queue of column sets and slabs on `grid` CTAs (at most one per SM).
 struct GramQueueArgs;
 cudaError_t gram_queue_launch(const GramQueueArgs &a, int grid, cudaStream_t stream);
+// The factor of the set sums of more than kGramRootMaxN columns (tsqr_gram_wide.cu); the launches
+// it took, or -1.
+struct GramWideArgs;
+int gram_wide_launch(const GramWideArgs &a, cudaStream_t stream);
 
 // Mixed path (tsqr_mixed.cu); `warps` counts bulk warps as for the FP64 path.
 int mixed_s_doubles(int n, int ldS);

@@ -261,3 +261,33 @@ def test_batch_served_and_handed_over(oracle, T):
             assert oracle.gram_residual(oracle.from_torch_colmajor(At), Ri.cpu().numpy()) <= 1e-13
         else:
             _check(oracle, Ri, At)
+
+
+@pytest.mark.parametrize("m,n", [(520, 129), (1100, 160), (20000, 200), (9001, 290), (5000, 512)])
+def test_wide_factor(oracle, T, m, n):
+    """Past 128 columns the summed Gram is factored by block rows; bounds of the panels' tests."""
+    At = workloads.gaussian(m, n, seed=n)
+    A = oracle.from_torch_colmajor(At)
+    R = T.tsqr_caqr_r(At.cuda().T).cpu().numpy()
+    Ro = oracle.householder_r(A, nthreads=16)
+    assert np.all(np.tril(R, -1) == 0) and np.all(np.diag(R) >= 0)
+    c = max(50.0, 2.0 * np.sqrt(m * n / 32.0))
+    np.testing.assert_allclose(R, Ro, rtol=0, atol=c * oracle.kappa_from_r(Ro) * U * np.linalg.norm(Ro))
+    assert oracle.gram_residual(A, R, nthreads=16) <= 1e-13
+
+
+@pytest.mark.parametrize("kind", ["repeated", "nan", "kappa"])
+def test_wide_handed_over(oracle, T, kind):
+    m, n = 12001, 180
+    At = workloads.gaussian(m, n, seed=77)
+    if kind == "repeated":
+        At[170] = At[3]
+    elif kind == "nan":
+        At[100, 5000] = float("nan")
+    else:
+        At = workloads.conditioned(m, n, 1e8, seed=7)
+    T.tsqr_get_device_status()
+    R = T.tsqr_caqr_r(At.cuda().T).cpu().numpy()
+    assert T.tsqr_get_device_status() == (T.STATUS_NONFINITE if kind == "nan" else T.SUCCESS)
+    if kind != "nan":
+        assert oracle.gram_residual(oracle.from_torch_colmajor(At), R, nthreads=16) <= 1e-13
