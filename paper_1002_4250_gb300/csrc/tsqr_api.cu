@@ -45,6 +45,20 @@ struct Workspace {
     // batched calls: the problem table and work items last copied to base + table_off
     std::vector<char> table;
     size_t table_off = 0;
+    // Page-locked copies of the last tables on their way to the device: the copy runs on the stream,
+    // after the call has returned, and on a host whose pageable memory the device reads in place
+    // (Grace) nothing stages it before.  A slot is reused once its copy is done.
+    struct Staged {
+        void *host = nullptr;
+        size_t bytes = 0;
+        cudaEvent_t done = nullptr;
+        bool used = false;
+    };
+    Staged staged[4];
+    int next_staged = 0;
+    // Tables of captured calls: a graph reads them at every replay, and a replay puts its table in
+    // the workspace unseen, so calls after a capture always copy theirs.
+    std::vector<std::vector<char>> captured;
 };
 
 std::mutex g_mu;
@@ -467,6 +481,38 @@ tsqr_status_t get_workspace(cudaStream_t stream, size_t bytes, Workspace **out) 
         w.bytes = nb;
     }
     *out = &w;
+    return TSQR_SUCCESS;
+}
+
+// `table` to device memory at dst, on the stream.
+tsqr_status_t upload_table(Workspace *w, const std::vector<char> &table, void *dst,
+                           cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) return TSQR_ERR_CUDA;
+    if (cap != cudaStreamCaptureStatusNone) {
+        w->captured.push_back(table);
+        return cudaMemcpyAsync(dst, w->captured.back().data(), table.size(), cudaMemcpyHostToDevice,
+                               stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
+    }
+    Workspace::Staged &s = w->staged[w->next_staged];
+    w->next_staged = (w->next_staged + 1) % 4;
+    if (s.used && cudaEventSynchronize(s.done) != cudaSuccess) return TSQR_ERR_CUDA;
+    s.used = false;
+    if (!s.done && cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess)
+        return TSQR_ERR_CUDA;
+    if (s.bytes < table.size()) {
+        if (s.host) cudaFreeHost(s.host);
+        s.host = nullptr;
+        s.bytes = 0;
+        const size_t nb = align_up(table.size(), 1 << 16);
+        if (cudaMallocHost(&s.host, nb) != cudaSuccess) return TSQR_ERR_ALLOC;
+        s.bytes = nb;
+    }
+    std::memcpy(s.host, table.data(), table.size());
+    if (cudaMemcpyAsync(dst, s.host, table.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        cudaEventRecord(s.done, stream) != cudaSuccess)
+        return TSQR_ERR_CUDA;
+    s.used = true;
     return TSQR_SUCCESS;
 }
 
@@ -2072,10 +2118,9 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
         std::memcpy(table.data() + tp + ti + tg, gitems.data(), sizeof(int2) * gitems.size());
     }
     if (ws->table != table || ws->table_off != table_off) {
-        if (cudaMemcpyAsync(base + table_off, table.data(), table.size(), cudaMemcpyHostToDevice,
-                            stream) != cudaSuccess)
-            return TSQR_ERR_CUDA;
-        ws->table = table;
+        st = upload_table(ws, table, base + table_off, stream);
+        if (st != TSQR_SUCCESS) return st;
+        ws->table = ws->captured.empty() ? std::move(table) : std::vector<char>();
         ws->table_off = table_off;
     }
     BatchArgs b;
@@ -2469,6 +2514,10 @@ void tsqr_release_workspace(void) {
         cudaDeviceSynchronize();
         if (kv.second.base) cudaFree(kv.second.base);
         if (kv.second.status) cudaFree(kv.second.status);
+        for (Workspace::Staged &s : kv.second.staged) {
+            if (s.host) cudaFreeHost(s.host);
+            if (s.done) cudaEventDestroy(s.done);
+        }
     }
     g_ws.clear();
     cudaSetDevice(cur);

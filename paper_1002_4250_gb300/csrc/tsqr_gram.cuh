@@ -21,8 +21,8 @@
 
 namespace tsqr {
 
-constexpr int kGramThreads = 512;
-constexpr int kGramWarps = kGramThreads / 32;
+constexpr int kGramSlicers = 16;    // warps that cut entries into digits; one more multiplies
+constexpr int kGramThreads = 32 * (kGramSlicers + 1);
 constexpr int kGramFoldWarps = 12;  // bulk warps of the Householder reduction (and its reducer)
 constexpr int kGramArity = 16;      // children per node of the Gram sum's tree
 constexpr int kGramMaxN = 32;       // one column block: tsqr_r's single launch

@@ -45,16 +45,21 @@ struct Shape {
     static constexpr int NR = kCross ? NJ : NI;            // columns of a right-hand digit
     static constexpr int N0 = S * NR;
     static constexpr int N1 = kTiles == 1 ? 0 : kCross ? N0 : (TE - TS) * NI;
-    static constexpr int kCols = N0 + N1;                  // tensor-memory columns
+    // Narrow sets put two 64-row blocks into one product: block k+1's operand rows follow block
+    // k's, so a 128-row tile against twice the columns holds both blocks' sums on its diagonal
+    // (a product takes some 95 cycles however few its columns).
+    static constexpr int kPair = !kCross && MN <= 64 ? 2 : 1;
+    static constexpr int kCols = kPair * N0 + N1;          // tensor-memory columns
     static constexpr int kSets = cmin(8, 512 / kCols);     // accumulator sets, 1,024 rows each
+    static_assert((kSets & (kSets - 1)) == 0, "a power of two");
     static_assert(kCols <= 512 && (kTiles == 1 || 2 * TS >= S), "accumulators fit");
     // Slicing: a task is four columns of a 64-row block, each warp has one a round.
     static constexpr int kGroups = (NI + NJ) / 4;
-    static constexpr int kRoundKb = kGramWarps / kGroups;
+    static constexpr int kRoundKb = kGramSlicers / kGroups;
     static_assert(kRoundKb >= 1, "a block a round");
     static constexpr int kKbBytes = MN * 128;              // 64 FP16 per operand row
     static constexpr int kStage = kRoundKb * kKbBytes;
-    static constexpr int kRaw = kGramWarps * 2048;         // a round of A: 64 bytes a lane
+    static constexpr int kRaw = kGramSlicers * 2048;         // a round of A: 64 bytes a lane
     static constexpr int kRaws = 2;                        // rounds on their way
     // Flush: partial sums (64-bit) of JP columns at a time over the stages, [half][row digit]
     // [j][i]; halves: digits 0-3 and 4-7 of the right-hand columns.
@@ -62,7 +67,7 @@ struct Shape {
     static constexpr int kRowDigits = kCross ? S : TS;
     static constexpr int kLd = NI + 1;
     static constexpr int per_j() {
-        return (kRowDigits * 2 + (kMirror ? S - TS : 0)) * kLd * 8;
+        return (kPair * kRowDigits * 2 + (kMirror ? S - TS : 0)) * kLd * 8;
     }
     static constexpr int kStages = 2 * kStage;
     static constexpr int jp() {
@@ -76,9 +81,13 @@ struct Shape {
 };
 
 struct alignas(16) Smem {   // beside the stages
-    uint64_t bar[2];
+    uint64_t full[2];       // a stage is sliced: one arrival a warp
+    uint64_t free[2];       // a stage is multiplied: the tensor cores' commit
+    uint64_t drain;         // all tensor-core work so far is done
     uint32_t tmem;
     int flag, bad, item;
+    int above;              // an entry was above its column's range
+    int stop;               // the round that was not multiplied for it; -1: none
     int D[128], E[128], Dnew[128];
 };
 
@@ -216,7 +225,6 @@ struct Cta {
     Q128 *U;           // the current item's sums
     unsigned char *stages;
     uint32_t tmem;
-    uint32_t par[2];   // parity of the next completion of each stage's barrier
     bool ok;           // no wait has given up
 };
 template <typename Sh>
@@ -301,31 +309,73 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     };
     const bool padded = cols.ni < NI || cols.nj < NJ;
 
-    constexpr uint32_t idesc0 = tc::instr_desc(0, 128, Sh::N0, false, false);
+    constexpr uint32_t idesc0 = tc::instr_desc(0, 128, Sh::kPair * Sh::N0, false, false);
     constexpr uint32_t idesc1 = Sh::kTiles == 2 ? tc::instr_desc(0, 128, Sh::N1, false, false) : 0;
-    const uint32_t sbase = tc::smem_u32(c.stages);
-    bool pend[2] = {false, false};
-    int sets = 0, in_set = 0;  // accumulator sets begun, 64-row blocks in the current one
-    auto wait_stage = [&](const int b) {
-        if (pend[b]) {
-            c.ok &= tc::mbar_wait(&sm.bar[b], c.par[b], 1LL << 24);
-            c.par[b] ^= 1;
-            pend[b] = false;
+    const uint64_t desc0 = tc::smem_desc(tc::smem_u32(c.stages), 16, 1024, tc::kSw128);
+    const bool issuer = tid == kGramThreads - 32;  // the thread that issues the tensor-core work
+    constexpr long long kPolls = 1LL << 22;
+    volatile int *const above = &sm.above, *const stop = &sm.stop;
+    int blocks = 0;                 // 64-row blocks in the accumulators
+    int used[2] = {0, 0};           // rounds given to each stage since the barriers' last start
+    uint32_t drained = 0;           // completions of sm.drain since then
+    auto restart_barriers = [&]() {  // between two CTA barriers; nothing is in flight
+        if (tid == 0) {
+            for (int b = 0; b < 2; ++b) {
+                tc::mbar_inval(&sm.full[b]);
+                tc::mbar_init(&sm.full[b], kGramSlicers);
+                tc::mbar_inval(&sm.free[b]);
+                tc::mbar_init(&sm.free[b], 1);
+            }
+            tc::mbar_inval(&sm.drain);
+            tc::mbar_init(&sm.drain, 1);
+            tc::fence_mbar_init();
+            *above = 0;
+            *stop = -1;
         }
+        used[0] = used[1] = 0;
+        drained = 0;
+    };
+    // Waits for a barrier's phase, or for the stop: true where the phase is complete (the same for
+    // the warp's lanes).
+    auto wait_or_stop = [&](uint64_t *bar, const uint32_t parity) {
+        bool done = !c.ok;  // a wait that gave up: no further one holds the CTA up
+        for (long long it = 0; !done; ++it) {
+            done = tc::mbar_test(bar, parity);
+            if (!done && *stop >= 0) break;
+            if (it >= kPolls) {
+                c.ok = false;
+                done = true;
+            }
+        }
+        return __any_sync(0xffffffffu, done) != 0;
+    };
+    // The last commits to the stages' barriers (the multiplying warp, which has counted the rounds it
+    // issued): a commit that arrives after its barrier is gone would write to memory that is another's.
+    auto settle = [&]() {
+        if (warp == kGramSlicers)
+            for (int b = 0; b < 2; ++b)
+                if (used[b] > 0 && c.ok) c.ok = tc::mbar_wait(&sm.free[b], (used[b] - 1) & 1, kPolls);
+    };
+    auto drain = [&]() {  // every thread; the issuer's work so far
+        if (issuer) tc::mma_commit(&sm.drain);
+        if (c.ok) c.ok = tc::mbar_wait(&sm.drain, drained & 1, kPolls);
+        ++drained;
     };
 
-    // Accumulators into U: every digit product's sum, weighted.  All tensor-core work is waited
-    // for; the stages are free on return.
+    // Accumulators into U: every digit product's sum, weighted.  The tensor cores are drained
+    // before, and the stages are free on return.
     auto flush = [&]() {
-        wait_stage(0);
-        wait_stage(1);
         tc::fence_after_sync();
         __syncthreads();
-        const int part = warp >> 2, lrow = 32 * (warp & 3) + lane, s = lrow / NI, i = lrow - s * NI;
-        const uint32_t lanes = c.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+        const int part = warp >> 2, lrow = (32 * (warp & 3) + lane) % (128 / Sh::kPair);
+        const int s = lrow / NI, i = lrow - s * NI;
+        // (a pair's second block: the second half of the lanes and of the columns)
+        const int second = Sh::kPair == 2 ? (warp & 3) >> 1 : 0;
+        const uint32_t lanes = c.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + second * Sh::N0;
         long long *buf = reinterpret_cast<long long *>(c.stages);
         constexpr int kHalf = Sh::kRowDigits * Sh::JP * Sh::kLd;     // words of a half
         constexpr int kL1 = 2 * kHalf;                               // then tile 1's, [s - TS][j][i]
+        constexpr int kSecond = 2 * kHalf;                           // (or a pair's second block)
         // sum over the sets of K <= 4 digits of columns at .. at + 7, weighted 256^(3 - t)
         auto digits = [&](auto K, long long (&x)[8], const uint32_t at) {
             int v[K][8];
@@ -333,7 +383,8 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             for (int t = 0; t < K; ++t)
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[t][e] = 0;
-            for (int set = 0; set < sets; ++set) {
+#pragma unroll 1
+            for (int set = 0; set < cmin(Sh::kSets, 4 * blocks / Sh::kPair); ++set) {
                 float f[K][8];
 #pragma unroll
                 for (int t = 0; t < K; ++t) tc::tmem_ld8(at + set * Sh::kCols + t * Sh::NR, f[t]);
@@ -357,7 +408,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         };
         for (int jb = 0; jb < Sh::NR; jb += Sh::JP) {
             constexpr int kJ = Sh::JP / 8;
-            for (int task = part; task < Sh::kTiles * kJ; task += 4) {
+            for (int task = part; task < Sh::kTiles * kJ && part < 4; task += 4) {
                 const int tile = task / kJ, jl = 8 * (task - tile * kJ);
                 const uint32_t at = lanes + (tile ? Sh::N0 : 0) + jb + jl;
                 long long x[8];
@@ -368,9 +419,9 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
                     const int sr = s + tile * Sh::TS;  // the row's digit
                     const bool keep = s < Sh::TS && sr < Sh::kRowDigits;
                     digits(std::integral_constant<int, 4>(), x, at);
-                    if (keep) put((sr * Sh::JP + jl) * Sh::kLd, x);
+                    if (keep) put(second * kSecond + (sr * Sh::JP + jl) * Sh::kLd, x);
                     digits(std::integral_constant<int, 4>(), x, at + 4 * Sh::NR);
-                    if (keep) put(kHalf + (sr * Sh::JP + jl) * Sh::kLd, x);
+                    if (keep) put(second * kSecond + kHalf + (sr * Sh::JP + jl) * Sh::kLd, x);
                 }
             }
             tc::fence_before_sync();
@@ -385,8 +436,9 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
 #pragma unroll
                 for (int sr = 0; sr < Sh::kRowDigits; ++sr) {
                     const int at = (sr * Sh::JP + jl) * Sh::kLd + ii;
-                    add(g, buf[at], 64 - 8 * sr);
-                    add(mir, buf[kHalf + at], 32 - 8 * sr);
+                    add(g, buf[at] + (Sh::kPair == 2 ? buf[kSecond + at] : 0), 64 - 8 * sr);
+                    add(mir, buf[kHalf + at] + (Sh::kPair == 2 ? buf[kSecond + kHalf + at] : 0),
+                        32 - 8 * sr);
                 }
                 if (Sh::kMirror) {
 #pragma unroll
@@ -407,48 +459,37 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             }
             __syncthreads();
         }
-        sets = 0;
-        in_set = 0;
+        blocks = 0;
     };
 
-    // Tensor-core work of blocks [k0, k1) of the round in stage b (one thread), into the current
-    // accumulator set (begun here when the last one is full or flushed).
+    // Tensor-core work of blocks [k0, k1) of the round in stage b (the issuer).  The 16-row steps go
+    // round the accumulator sets.  (Descriptors by addition: their low bits hold the address over
+    // 16; built from addresses they cost more than the products.)
     auto multiply = [&](const int b, const int k0, const int k1) {
-        if (in_set == 0) ++sets;
-        if (tid == kGramThreads - 32) {
-            tc::fence_after_sync();
-            const uint32_t d0 = c.tmem + (uint32_t)(sets - 1) * Sh::kCols;
+        tc::fence_after_sync();
+        uint64_t ad = desc0 + (uint32_t)((b * Sh::kStage + k0 * Sh::kKbBytes) >> 4);
 #pragma unroll 1
-            for (int kb = k0; kb < k1; ++kb) {
-                const uint32_t base = sbase + b * Sh::kStage + kb * Sh::kKbBytes;
+        for (int kb = k0; kb < k1; kb += Sh::kPair, ad += Sh::kPair * Sh::kKbBytes >> 4) {
+            const int step0 = 4 * (blocks + kb - k0) / Sh::kPair;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    const bool add = in_set > 0 || kb > k0 || ks > 0;
-                    const uint64_t ad = tc::smem_desc(base + 32 * ks, 16, 1024, tc::kSw128);
-                    const uint64_t bd =
-                        NJ > 0 ? tc::smem_desc(base + S * NI * 128 + 32 * ks, 16, 1024, tc::kSw128) : ad;
-                    tc::mma_f16(d0, ad, bd, idesc0, add);
-                    if (Sh::kTiles == 2) {
-                        const uint64_t a1 =
-                            tc::smem_desc(base + Sh::TS * NI * 128 + 32 * ks, 16, 1024, tc::kSw128);
-                        tc::mma_f16(d0 + Sh::N0, a1, NJ > 0 ? bd : a1, idesc1, add);
-                    }
-                }
+            for (int ks = 0; ks < 4; ++ks) {
+                const uint32_t d0 = c.tmem + (uint32_t)((step0 + ks) % Sh::kSets) * Sh::kCols;
+                const bool add = step0 + ks >= Sh::kSets;
+                const uint64_t bd = ad + 2 * ks + (NJ > 0 ? S * NI * 8 : 0);
+                tc::mma_f16(d0, ad + 2 * ks, bd, idesc0, add);
+                if (Sh::kTiles == 2)
+                    tc::mma_f16(d0 + Sh::N0, ad + 2 * ks + Sh::TS * NI * 8,
+                                NJ > 0 ? bd : ad + 2 * ks + Sh::TS * NI * 8, idesc1, add);
             }
-            tc::mma_commit(&sm.bar[b]);
         }
-        pend[b] = true;
-        in_set += k1 - k0;
-    };
-    // Block kb (all: the whole round) of round r as digits in stage b; false where an entry is out
-    // of its column's range (the same for every thread).
-    auto slice = [&](const int r, const int b, const int kb, const bool all) {
-        int dmin = 2;
-        if (mine && (all || kbo == kb)) slice8(raw_of(r), sm.D[lc], dmin, dst + b * Sh::kStage, step);
-        tc::fence_proxy_async();
-        return __syncthreads_or(dmin < 2) == 0;
     };
 
+    // Rounds run without a CTA barrier: a warp slices its task of a round into the round's stage as
+    // soon as the tensor cores are done with the round before the last (free), and the last warp,
+    // which slices nothing, issues a round's products once all have arrived (full).  A warp that meets an entry
+    // above its column's range says so before it arrives; the last warp then issues nothing and
+    // sets the stop, which every wait watches, and the whole CTA takes that round block by block.
+    restart_barriers();
 #pragma unroll 1
     for (int r = 0; r < Sh::kRaws; ++r) load_round(r);
     cp_async_wait<Sh::kRaws - 1>();
@@ -459,50 +500,115 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         zero_stages();
     else
         __syncthreads();
-    for (int r = 0; r < rounds && !sm.bad; ++r) {
+    int r = 0;
+    int r_at = 0, blocks_at = 0;  // blocks in the accumulators before round r_at
+    while (r < rounds && !sm.bad) {
         const int b = r & 1;
-        cp_async_wait<Sh::kRaws - 1>();
-            wait_stage(b);
-        if (slice(r, b, 0, true)) {
-            multiply(b, 0, Sh::kRoundKb);
-        } else {
-            // block by block: where an entry is above its column's range, what is accumulated goes
-            // to U, then the exponents rise and U's entries follow
-#pragma unroll 1
-            for (int kb = 0; kb < Sh::kRoundKb; ++kb) {
-                const bool up = scan_block(r, kb);
-                if (sm.bad) break;
-                if (up) {
-                    if (sets > 0) flush();
-                    for (int o = tid; o < NI * Sh::NR; o += kGramThreads) {
-                        const int i = o / Sh::NR, j = (NJ > 0 ? NI : 0) + o % Sh::NR;
-                        c.U[o] = pack(
-                            shr128(unpack(c.U[o]), sm.Dnew[i] - sm.D[i] + sm.Dnew[j] - sm.D[j]));
-                    }
-                    __syncthreads();
-                    if (tid < NI + NJ) sm.D[tid] = sm.Dnew[tid];
-                    if (padded)
-                        zero_stages();
-                    else
-                        __syncthreads();
-                }
-                slice(r, b, kb, false);
-                multiply(b, kb, kb + 1);
-                wait_stage(b);
+        bool go;
+        if (warp < kGramSlicers) {
+            cp_async_wait<Sh::kRaws - 1>();
+            go = used[b] == 0 || wait_or_stop(&sm.free[b], (used[b] - 1) & 1);
+            if (go) {
+                int dmin = 2;
+                if (mine) slice8(raw_of(r), sm.D[lc], dmin, dst + b * Sh::kStage, step);
+                if (__any_sync(0xffffffffu, dmin < 2) && lane == 0) *above = 1;
+                tc::fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&sm.full[b]);
             }
+        } else {
+            if (c.ok) c.ok = tc::mbar_wait(&sm.full[b], used[b] & 1, kPolls);
+            __syncwarp();
+            // (one lane reads it for all: another warp may be saying so of the next round)
+            go = __shfl_sync(0xffffffffu, lane == 0 ? *above : 0, 0) == 0;
+            if (issuer) {
+                if (go) {
+                    multiply(b, 0, Sh::kRoundKb);
+                    tc::mma_commit(&sm.free[b]);
+                } else {
+                    *stop = r;
+                }
+            }
+            __syncwarp();
+        }
+        if (go) {
+            ++used[b];
+            blocks += Sh::kRoundKb;
+            load_round(r + Sh::kRaws);
+            if (r + 1 == rounds || blocks + Sh::kRoundKb > 16 * Sh::kSets * Sh::kPair) {
+                if (issuer) tc::mma_commit(&sm.drain);
+                __syncwarp();
+                go = wait_or_stop(&sm.drain, drained & 1);
+                if (go) {
+                    ++drained;
+                    flush();
+                    if (r + 1 < rounds && padded) zero_stages();
+                    r_at = r + 1;
+                    blocks_at = 0;
+                }
+            }
+        }
+        if (go) {
+            ++r;
+            continue;
+        }
+        // ---- round *stop block by block: where an entry is above its column's range, what is
+        //      accumulated goes to U, then the exponents rise and U's entries follow
+        __syncthreads();
+        r = *stop;
+        blocks = blocks_at + (r - r_at) * Sh::kRoundKb;
+        settle();
+        drain();
+        cp_async_wait_all();
+        __syncthreads();
+        restart_barriers();
+#pragma unroll 1
+        for (int q = 0; q < Sh::kRaws; ++q) load_round(r + q);
+        cp_async_wait<Sh::kRaws - 1>();
+        if (Sh::kPair == 2) zero_stages();
+        __syncthreads();
+#pragma unroll 1
+        for (int kb = 0; kb < Sh::kRoundKb; ++kb) {
+            const bool up = scan_block(r, kb);
             if (sm.bad) break;
+            if (up) {
+                if (blocks > 0) flush();
+                for (int o = tid; o < NI * Sh::NR; o += kGramThreads) {
+                    const int i = o / Sh::NR, j = (NJ > 0 ? NI : 0) + o % Sh::NR;
+                    c.U[o] =
+                        pack(shr128(unpack(c.U[o]), sm.Dnew[i] - sm.D[i] + sm.Dnew[j] - sm.D[j]));
+                }
+                __syncthreads();
+                if (tid < NI + NJ) sm.D[tid] = sm.Dnew[tid];
+                if (padded || Sh::kPair == 2)
+                    zero_stages();
+                else
+                    __syncthreads();
+            }
+            int dmin = 2;
+            // (in block 0 of stage 0; a pair's second block reads as zeros)
+            if (mine && kbo == kb)
+                slice8(raw_of(r), sm.D[lc], dmin, dst - kbo * Sh::kKbBytes, step);
+            tc::fence_proxy_async();
+            __syncthreads();
+            if (issuer) multiply(0, 0, 1);
+            blocks += Sh::kPair;
+            drain();
+            if (blocks + Sh::kRoundKb > 16 * Sh::kSets * Sh::kPair) {
+                flush();
+                if (padded || Sh::kPair == 2) zero_stages();
+            }
         }
-        const bool full = in_set + Sh::kRoundKb > 16;
-        if (full) in_set = 0;
+        if (sm.bad) break;
         load_round(r + Sh::kRaws);
-        if (r + 1 == rounds || (full && sets == Sh::kSets)) {
-            flush();
-            if (r + 1 < rounds && padded) zero_stages();
-        }
+        ++r;
+        if (r == rounds) flush();
+        r_at = r;
+        blocks_at = blocks;
+        __syncthreads();
     }
     cp_async_wait_all();
-    wait_stage(0);
-    wait_stage(1);
+    settle();
     if (__syncthreads_or(!c.ok) && tid == 0) sm.bad = 1;
     __syncthreads();
 }
@@ -782,22 +888,24 @@ __device__ __forceinline__ bool item_of(const GramProblem &p, const Cols cols, c
 __device__ __forceinline__ void cta_begin(Cta &c, unsigned char *smem) {
     c.sm = reinterpret_cast<Smem *>(smem);
     c.stages = smem + kHead;
-    if (threadIdx.x >> 5 == kGramWarps - 1) tc::tmem_alloc(&c.sm->tmem, 512);
+    if (threadIdx.x >> 5 == kGramSlicers) tc::tmem_alloc(&c.sm->tmem, 512);
     if (threadIdx.x == 0) {
-        tc::mbar_init(&c.sm->bar[0], 1);
-        tc::mbar_init(&c.sm->bar[1], 1);
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_init(&c.sm->full[b], kGramSlicers);
+            tc::mbar_init(&c.sm->free[b], 1);
+        }
+        tc::mbar_init(&c.sm->drain, 1);
         tc::fence_mbar_init();
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     c.tmem = c.sm->tmem;
-    c.par[0] = c.par[1] = 0;
     c.ok = true;
 }
 __device__ __forceinline__ void cta_end(const Cta &c) {
     __syncthreads();
-    if (threadIdx.x >> 5 == kGramWarps - 1) {
+    if (threadIdx.x >> 5 == kGramSlicers) {
         tc::tmem_relinquish();
         tc::tmem_dealloc(c.tmem, 512);
     }

@@ -291,3 +291,28 @@ def test_wide_handed_over(oracle, T, kind):
     assert T.tsqr_get_device_status() == (T.STATUS_NONFINITE if kind == "nan" else T.SUCCESS)
     if kind != "nan":
         assert oracle.gram_residual(oracle.from_torch_colmajor(At), R, nthreads=16) <= 1e-13
+
+
+def test_batches_in_flight_keep_their_tables(T):
+    """Two batches in turn on one stream with nothing waited for: each call's table of problems (some
+    100 KB here) has to last until the device has read it, also after the call has returned."""
+    import torch
+    calls = []
+    for seed in (1, 2):
+        buf, ms, ns, offs = workloads.varlen_batch(700, 300, 3000, seed=seed, device="cuda")
+        roff = [0]
+        for n in ns:
+            roff.append(roff[-1] + n * n)
+        ptrs = [buf.data_ptr() + 8 * o for o in offs[:-1]]
+        ref = torch.zeros(roff[-1], dtype=torch.float64, device="cuda")
+        T.tsqr_r_batched(ptrs, ms, ns, roff, ref)
+        torch.cuda.synchronize()
+        calls.append((buf, ptrs, ms, ns, roff, ref))
+    outs = []
+    for k in range(12):
+        buf, ptrs, ms, ns, roff, ref = calls[k % 2]
+        outs.append(torch.zeros_like(ref))
+        T.tsqr_r_batched(ptrs, ms, ns, roff, outs[-1])
+    torch.cuda.synchronize()
+    for k, out in enumerate(outs):
+        assert torch.equal(out, calls[k % 2][5])
