@@ -106,10 +106,16 @@ typedef enum {
  *         column's square: zero or dependent columns) is found on the device, and the
  *         Householder leaves and tree that the plan's other fields describe run instead: up to 32
  *         columns in the same launch, past that in the launches behind it.
+ *   GRAM_Q tsqr_qr's form of GRAM, up to 32 columns: the root also inverts R (in 110-bit fixed
+ *         point) and Q = A R^-1 is formed on the tensor cores from A's and the inverse's digits,
+ *         where its error bound is below 2^-47 (conditions up to some 100 to 1,000); past that
+ *         the Householder reduction and its reflectors give R and Q.  In tsqr_r_ex: the R that
+ *         tsqr_qr gives.
  * AUTO picks, FP64: GRAM where it serves; MIXED: PANELS for n <= 112 (FP32 from n = 9, BF16 from
  * n = 3), where it measured faster, else FOLD. */
 typedef enum {
-    TSQR_LEAF_AUTO = 0, TSQR_LEAF_FOLD = 1, TSQR_LEAF_PANELS = 2, TSQR_LEAF_GRAM = 3
+    TSQR_LEAF_AUTO = 0, TSQR_LEAF_FOLD = 1, TSQR_LEAF_PANELS = 2, TSQR_LEAF_GRAM = 3,
+    TSQR_LEAF_GRAM_Q = 4
 } tsqr_leaf_t;
 
 /* Optional plan override.  Zero fields mean "choose".  The chosen plan fixes the arithmetic

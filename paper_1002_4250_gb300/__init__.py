@@ -26,7 +26,7 @@ SUCCESS, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_CUDA, ERR_ALLOC, ERR_TIMEOUT, STA
 F64, F32, BF16 = 0, 1, 2
 PREC_F64, PREC_MIXED = 0, 1
 TREE_AUTO, TREE_BINARY, TREE_FLAT, TREE_HYBRID, TREE_PANELS = 0, 1, 2, 3, 4
-LEAF_AUTO, LEAF_FOLD, LEAF_PANELS, LEAF_GRAM = 0, 1, 2, 3
+LEAF_AUTO, LEAF_FOLD, LEAF_PANELS, LEAF_GRAM, LEAF_GRAM_Q = 0, 1, 2, 3, 4
 MAX_N = 128
 _TREES = {"auto": TREE_AUTO, "binary": TREE_BINARY, "flat": TREE_FLAT, "hybrid": TREE_HYBRID,
           "panels": TREE_PANELS}

@@ -24,6 +24,8 @@ size_t wy_smem_bytes(int n, int ldX);
 cudaError_t wy_launch(const WyArgs &a, size_t smem_bytes, int grid, cudaStream_t stream);
 size_t qt_wy_smem_bytes(int n, int kc, int ldS, bool fused = false);
 size_t q_leaf_wy_smem_bytes(int n, int qn, int ldS, bool fused);
+cudaError_t q_gram_launch(const GramQArgs &g, const QLeafArgs &a, int sms, size_t leaf_smem,
+                          cudaStream_t stream);
 cudaError_t q_leaf_wy_launch(const QLeafArgs &a, size_t smem_bytes, cudaStream_t stream);
 cudaError_t qt_wy_launch(const QtArgs &a, size_t smem_bytes, cudaStream_t stream);
 cudaError_t trsm_launch(const double *R, int64_t ldr, const double *C, int64_t ldc, double *X,
@@ -543,9 +545,10 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     if (plan_is_auto(over) && tuned_plan(dev, m, n, false, &tuned) &&
         tuned.tree != TSQR_TREE_PANELS)
         over = &tuned;
-    const bool asked = over && over->leaf == TSQR_LEAF_GRAM;
+    const bool with_q = over && over->leaf == TSQR_LEAF_GRAM_Q;
+    const bool asked = over && (over->leaf == TSQR_LEAF_GRAM || with_q);
     const bool serves = gram_fits(m, n) && n < kPanelsMinN;
-    if (asked && ((over->tree != TSQR_TREE_AUTO && over->tree != TSQR_TREE_HYBRID) || !serves))
+    if (asked && ((over->tree != TSQR_TREE_AUTO && over->tree != TSQR_TREE_HYBRID) || !serves || (with_q && n > kGramMaxN)))
         return TSQR_ERR_INVALID_ARG;
     if (!asked && !(plan_is_auto(over) && serves)) return plan_f64(m, n, over, p);
     const DeviceInfo di = device_info(dev);
@@ -558,11 +561,18 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
         return st;
     }
     p->tree = TSQR_TREE_HYBRID;
-    p->leaf = TSQR_LEAF_GRAM;
+    p->leaf = with_q ? TSQR_LEAF_GRAM_Q : TSQR_LEAF_GRAM;
     p->warps = kGramFoldWarps;
     const size_t budget = std::min(di.smem_block_optin, di.smem_sm - 1024);
     int r = max_rows_per_lane_p(n, p->warps, budget, false);
-    while (r > 0 && (r % 2 || good_r(r) != r)) --r;
+    auto q_fits = [&](const int rows) {  // Q's blocked leaf pass in one column group
+        const int hs = 32 * p->warps * rows;
+        int blk = 1, vec = 1;
+        block_for(rows, false, &blk, &vec);
+        return q_leaf_wy_smem_bytes(n, n, ld_for(hs, vec), true) <= di.smem_block_optin &&
+               wy_smem_bytes(n, hs | 1) <= di.smem_block_optin;
+    };
+    while (r > 0 && (r % 2 || good_r(r) != r || (with_q && !q_fits(r)))) --r;
     tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, di.sms, p->warps, 0, 0};
     const tsqr_status_t st = plan_with_r(m, n, &fold, false, r, di, p);
     if (st != TSQR_SUCCESS) return st;
@@ -662,7 +672,7 @@ tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_
 // Workspace of one reduction under plan p: counters (zeroed per call), then tree slots, then the
 // Gram sum's.
 struct RLayout {
-    size_t cnt_words = 0, cnt_bytes = 0, gram_off = 0, bytes = 0;
+    size_t cnt_words = 0, cnt_bytes = 0, gram_off = 0, form_off = 0, bytes = 0;
     GramLayout g;
 };
 RLayout r_layout(const F64Plan &p, int64_t m, int64_t n, int sms) {
@@ -672,12 +682,38 @@ RLayout r_layout(const F64Plan &p, int64_t m, int64_t n, int sms) {
     w.cnt_bytes = align_up(w.cnt_words * sizeof(unsigned int), 256);
     w.gram_off = align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
     w.bytes = w.gram_off;
-    if (p.gram_ctas) w.bytes += (inner + p.gram_ctas) * gram_slot_bytes(gram_block((int)n));
+    if (p.gram_ctas) {
+        w.bytes += align_up((inner + p.gram_ctas) * gram_slot_bytes(gram_block((int)n)), 256);
+        w.form_off = w.bytes;
+        if (p.leaf == TSQR_LEAF_GRAM_Q) w.bytes += align_up(sizeof(GramQForm), 256);
+    }
     if (p.gram_queue) {
         w.g = gram_layout(m, n, sms);
         w.bytes += w.g.bytes;
     }
     return w;
+}
+
+// The single launch's Gram arguments behind the Householder reduction's (r_layout's workspace).
+GramArgs gram_args(const F64Plan &p, const RLayout &w, const F64Args &a, void *base) {
+    GramArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.p.A = a.A;
+    g.p.lda = a.lda;
+    g.p.m = a.m;
+    g.p.n = g.p.na = a.n;
+    g.p.nb = 1;
+    g.p.nslab = p.gram_ctas;
+    g.p.nkb = (a.m + 63) / 64;
+    g.p.counters = a.counters + p.nodes;
+    g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas) + 1;
+    g.p.slots = (unsigned char *)base + w.gram_off;
+    g.p.R = a.R;
+    g.p.ldr = a.ldr;
+    if (p.leaf == TSQR_LEAF_GRAM_Q) g.p.Q = (GramQForm *)((char *)base + w.form_off);
+    g.status = a.status;
+    g.fold = a;
+    return g;
 }
 
 // One reduction of A under plan p in the workspace at base (r_layout's bytes), R to device
@@ -704,22 +740,7 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
     ++*launches;
     if (!p.gram_ctas)
         return f64_launch(a, p.warps, p.smem, stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
-    GramArgs g;
-    std::memset(&g, 0, sizeof(g));
-    g.p.A = A;
-    g.p.lda = lda;
-    g.p.m = m;
-    g.p.n = g.p.na = (int)n;
-    g.p.nb = 1;
-    g.p.nslab = p.gram_ctas;
-    g.p.nkb = (m + 63) / 64;
-    g.p.counters = a.counters + p.nodes;
-    g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas) + 1;
-    g.p.slots = (unsigned char *)base + w.gram_off;
-    g.p.R = R;
-    g.p.ldr = ldr;
-    g.status = status;
-    g.fold = a;
+    const GramArgs g = gram_args(p, w, a, base);
     cudaError_t e = gram_launch(g, p.smem, stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         // a context that owns only part of the device: the plan's Householder reduction
@@ -732,6 +753,28 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
 
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
                        int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream);
+
+// tsqr_qr's plan: the Gram factor and Q = A R^-1 where AUTO can take them (one column block; the
+// plan's other fields are those of the reflectors that stand behind it), else plan_store's.
+// ms, against plan_store's: 4,194,304 x 32 1.14 / 24.4, 16,777,216 x 8 1.04 / 7.76, 100,003 x 32
+// 0.144 / 1.66, 10,000 x 16 0.069 / 0.38, 3,000 x 5 0.046 / 0.22.  A matrix left to the reflectors
+// pays for the sum: 4,194,304 x 32 24.65 / 24.36, and up to 16 columns for the 12-warp chunks the
+// single launch folds in (1,000,000 x 16 2.25 / 1.88).
+tsqr_status_t plan_qr(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
+    tsqr_plan_t tuned;
+    const bool any = plan_is_auto(over) ? !tuned_plan(dev, m, n, false, &tuned) ||
+                                              tuned.leaf == TSQR_LEAF_GRAM
+                                        : over->leaf == TSQR_LEAF_GRAM || over->leaf == TSQR_LEAF_GRAM_Q;
+    if (any && n <= kGramMaxN && gram_fits(m, n)) {
+        const tsqr_plan_t ask{TSQR_TREE_HYBRID, 0, 0, 0, 0, TSQR_LEAF_GRAM_Q};
+        if (plan_r(m, n, &ask, p) == TSQR_SUCCESS && p->gram_ctas && p->unit % p->h == 0)
+            return TSQR_SUCCESS;
+        *p = F64Plan();
+    }
+    return plan_store(m, n, over, p);
+}
 
 // Panels (TSQR_TREE_PANELS): the AUTO plan of a tall FP64 matrix from n = 56 on, where the one
 // reduction's leaves hold one CTA per SM and n reflectors per chunk, while panels of 16 columns
@@ -798,7 +841,7 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
     g_last_launches = 0;
     g_last_plan = tsqr_plan_t{};
     F64Plan p;
-    tsqr_status_t st = plan_store(m, (int)n, over, &p);
+    tsqr_status_t st = plan_qr(m, (int)n, over, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
     if (p.unit % p.h != 0) return TSQR_ERR_UNSUPPORTED;  // chunk ids = first row / h
@@ -853,8 +896,7 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
     const size_t nn = (size_t)n * (size_t)n;
     const size_t wys_bytes =
         (wyq && !fuse) ? align_up((size_t)nchunks * nn * sizeof(double), 256) : 0;
-    const size_t cnt_bytes = align_up((size_t)p.nodes * sizeof(unsigned int), 256);
-    const size_t slot_bytes = align_up((size_t)p.nodes * nn * sizeof(double), 256);
+    const RLayout rl = r_layout(p, m, n, di.sms);
     const size_t csc_bytes = align_up((size_t)nchunks * 2 * n * sizeof(double), 256);
     const size_t nv_bytes = align_up((size_t)p.nodes * (p.arity - 1) * nn * sizeof(double), 256);
     const size_t nsc_bytes = align_up((size_t)p.nodes * 2 * n * sizeof(double), 256);
@@ -862,17 +904,18 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
     const size_t sgn_bytes = align_up((size_t)n * sizeof(double), 256);
     const size_t v_bytes = grouped ? align_up((size_t)m * (size_t)n * sizeof(double), 256) : 0;
     Workspace *ws = nullptr;
-    st = get_workspace(stream, cnt_bytes + slot_bytes + csc_bytes + nv_bytes + nsc_bytes +
-                                   blk_bytes + sgn_bytes + v_bytes + wys_bytes, &ws);
+    const size_t r_bytes = align_up(rl.bytes, 256);
+    st = get_workspace(stream, r_bytes + csc_bytes + nv_bytes + nsc_bytes + blk_bytes + sgn_bytes +
+                                   v_bytes + wys_bytes, &ws);
     if (st != TSQR_SUCCESS) return st;
     char *base = (char *)ws->base;
     F64Args a = plan_args(p, A, m, n, lda);
     a.counters = (unsigned int *)base;
-    a.slots = (double *)(base + cnt_bytes);
+    a.slots = (double *)(base + rl.cnt_bytes);
     a.R = R;
     a.ldr = ldr;
     a.status = ws->status;
-    size_t o = cnt_bytes + slot_bytes;
+    size_t o = r_bytes;
     a.q.V = Q;
     a.q.ldv = ldq;
     a.q.chunk_sc = (double *)(base + o);
@@ -891,10 +934,31 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
     }
     o += v_bytes;
     double *wyS = (double *)(base + o);
-    if (cudaMemsetAsync(a.counters, 0, (size_t)p.nodes * sizeof(unsigned int), stream) !=
-        cudaSuccess)
+    if (cudaMemsetAsync(a.counters, 0, rl.cnt_words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    if (qr_factor_launch(a, p.warps, p.smem, stream) != cudaSuccess) return TSQR_ERR_CUDA;
+    GramQArgs gq;
+    std::memset(&gq, 0, sizeof(gq));
+    cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+    if (p.gram_ctas) {
+        const GramArgs g = gram_args(p, rl, a, base);
+        gq.A = A;
+        gq.Q = Q;
+        gq.lda = lda;
+        gq.ldq = ldq;
+        gq.m = m;
+        gq.n = (int)n;
+        gq.ntiles = (m + gram_q_rows((int)n) - 1) / gram_q_rows((int)n);
+        gq.form = g.p.Q;
+        gq.verdict = g.p.verdict;
+        gq.status = ws->status;
+        if (gram_prepare((int)n, p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
+        e = gram_launch(g, p.smem, stream);
+    }
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // (also a context that owns part of the device)
+        cudaGetLastError();
+        e = qr_factor_launch(a, p.warps, p.smem, stream);
+    }
+    if (e != cudaSuccess) return TSQR_ERR_CUDA;
     int launches = 1;
     if (wyq && !fuse) {
         const WyArgs wa = wy_args(p, a.q, m, (int)n, ldX, wyS);
@@ -917,6 +981,7 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
         t.signs = a.q.signs;
         t.B = blocks;
         t.qg = qg;
+        t.skip = gq.verdict;
         if (q_tree_launch(t, sh.count[L], tree_smem, stream) != cudaSuccess) return TSQR_ERR_CUDA;
         ++launches;
     }
@@ -941,7 +1006,8 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
     for (int q0 = 0; q0 < n; q0 += qn) {
         l.q0 = q0;
         l.qn = (int)std::min<int64_t>(qn, n - q0);
-        if ((wyq ? q_leaf_wy_launch(l, leaf_smem, stream)
+        if ((p.gram_ctas ? q_gram_launch(gq, l, di.sms, leaf_smem, stream)
+             : wyq       ? q_leaf_wy_launch(l, leaf_smem, stream)
                  : q_leaf_launch(l, qblk, qwarps, leaf_smem, stream)) != cudaSuccess)
             return TSQR_ERR_CUDA;
         ++launches;
@@ -1143,7 +1209,7 @@ bool plan_wy(int w, const F64Plan &p, const DeviceInfo &di, int *ldX, size_t *wy
 // reports which.
 tsqr_status_t plan_store(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     // the exact-Gram reduction keeps no reflectors: those calls' own plan
-    if (over && over->leaf == TSQR_LEAF_GRAM) over = nullptr;
+    if (over && (over->leaf == TSQR_LEAF_GRAM || over->leaf == TSQR_LEAF_GRAM_Q)) over = nullptr;
     // the passes that keep and apply the reflectors run 4, 8 or 12 bulk warps
     if (over && over->warps % 4 != 0) return TSQR_ERR_INVALID_ARG;
     tsqr_status_t st = plan_f64(m, n, over, p);

@@ -19,6 +19,11 @@ __device__ __noinline__ void fold_job(const F64Args &f, const int leaf) {
     leaf_tree_job<double, double, 2, 1, false>(f, f.A, f.ldS, f.ldS * f.n, leaf);
 }
 
+// The same keeping its reflectors (tsqr_qr).
+__device__ __noinline__ void fold_store_job(const F64Args &f, const int leaf) {
+    leaf_tree_job<double, double, 2, 1, false, true>(f, f.A, f.ldS, f.ldS * f.n, leaf);
+}
+
 // One FP64 matrix of at most 32 columns in one launch: CTA c sums slab c, the root factors, every
 // CTA waits for its verdict and runs its leaf of the Householder reduction where the Gram cannot
 // serve.  One CTA per SM, launched cooperatively.
@@ -61,7 +66,10 @@ tsqr_gram_f64_kernel(const __grid_constant__ GramArgs a) {
     const int v = sm.flag;
     __syncthreads();
     if (v != 2 || b >= a.fold.nleaves || tid >= TSQR_FOLD_THREADS) return;
-    fold_job(a.fold, b);
+    if (a.fold.q.V)
+        fold_store_job(a.fold, b);
+    else
+        fold_job(a.fold, b);
 }
 
 // A queue of work items (sets of columns over slabs of rows) of one matrix or many: the CTA that

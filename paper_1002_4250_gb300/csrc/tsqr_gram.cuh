@@ -42,12 +42,34 @@ struct GramProblem {
     unsigned int *verdict;   // 0: not decided; 1: R is written; 2: the Householder reduction runs
     double *R;
     int64_t ldr;
+    struct GramQForm *Q;     // where the root leaves R's inverse (at most kGramMaxN columns), or null
+};
+
+// What Q = A R^-1 needs (tsqr_gram_q.cuh): A's columns' exponent words, and the columns of the
+// scaled inverse in fixed point, 2^62 units to 2^F.
+struct GramQForm {
+    int D[kGramMaxN], F[kGramMaxN];
+    long long w[kGramMaxN * kGramMaxN];  // (i, j) at 32 j + i
 };
 
 struct GramArgs {          // tsqr_r's single launch: one problem of one column block
     GramProblem p;
     int *status;
     F64Args fold;          // the Householder reduction (its A is FP64; nleaves <= grid)
+};
+
+// Q = A R^-1 (tsqr_gram_q.cuh).  Rows of a tile: up to 16 columns, two or four 128-row blocks of A
+// stand side by side in it.
+__host__ __device__ inline int gram_q_rows(const int n) { return n <= 8 ? 512 : n <= 16 ? 256 : 128; }
+struct GramQArgs {
+    const double *A;
+    double *Q;
+    int64_t lda, ldq, m;
+    int n;
+    int64_t ntiles;               // tiles of gram_q_rows rows
+    const GramQForm *form;
+    const unsigned int *verdict;  // 1: the Gram factor is there
+    int *status;
 };
 
 struct GramQueueArgs {     // a queue of work items

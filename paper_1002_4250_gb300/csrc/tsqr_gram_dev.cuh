@@ -816,6 +816,75 @@ static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n
     return true;
 }
 
+__device__ __forceinline__ int bits128(const u128 x) {
+    const u64 h = (u64)(x >> 64);
+    return h ? 128 - __clzll((long long)h) : 64 - __clzll((long long)(u64)x);
+}
+// The inverse of the factor just formed, for Q = A R^-1 (p.Q): R = diag(rho) M 2^g by columns, with
+// M(k, k) = 2^-z_k and M(k, j) = l, so column j of the inverse is M^-1 e_j / rho_j: a warp a
+// column, its entries one a lane, 110 bits after the point through the substitution (which a
+// growth past 2^11 ends), then 62 bits against the column's largest entry.  Q's columns come
+// out with an error of about sqrt(m n) 2^(F - 73): sm.bad where that is above 2^-47 (a
+// bound; what Q^T Q - I shows is 2^-50, as with reflectors), an A whose Q the reflectors give.
+static __device__ __noinline__ void invert_root(const GramProblem &p, const Q128 *C, const Q128 *dv,
+                                                Smem &sm) {
+    const int n = p.n, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned all = 0xffffffffu;
+    const int limit = 52 - (64 - __clzll((long long)(p.m * n - 1)));  // of 2 F
+    for (int j = warp; j < kGramMaxN; j += kGramThreads >> 5) {
+        if (j >= n) {  // a column of zeros
+            p.Q->w[kGramMaxN * j + lane] = 0;
+            if (lane == 0) {
+                p.Q->D[j] = 2047 + 64;
+                p.Q->F[j] = 0;
+            }
+            continue;
+        }
+        const int z = lane < n ? (bits128((u128)unpack(dv[lane])) -
+                                  bits128((u128)unpack(C[rowoff(n, lane)]))) >> 1 : 0;
+        i128 x = lane == j ? (i128)1 << 110 : (i128)0;
+        bool bad = false;
+        for (int k = j; k >= 0; --k) {
+            if (lane == k) {
+                if (bits128((u128)(x < 0 ? -x : x)) + z > 121) {
+                    bad = true;
+                    x = 0;
+                }
+                x = (i128)((u128)x << z);
+            }
+            const u64 hi = __shfl_sync(all, (u64)((u128)x >> 64), k), lo = __shfl_sync(all, (u64)x, k);
+            if (lane < k) {
+                const i128 xk = (i128)(((u128)hi << 64) | lo);
+                const i128 l = unpack(C[rowoff(n, lane) - lane + k]);
+                const u128 q = mul122((u128)(l < 0 ? -l : l), (u128)(xk < 0 ? -xk : xk));
+                x = (l < 0) != (xk < 0) ? (i128)((u128)x + q) : (i128)((u128)x - q);
+            }
+        }
+        // 1 / rho, in (1, 2], times 2^62
+        const D2 rho = sqrt2(to_double(unpack(dv[j])));
+        const double y = 1.0 / rho.hi, dy = y * (fma(-y, rho.hi, 1.0) - y * rho.lo);
+        const u64 inv = __double2ull_rn(y * 0x1p62) + (u64)__double2ll_rn(dy * 0x1p62);
+        const u128 ax = (u128)(x < 0 ? -x : x);
+        const u128 v = (((u128)(u64)(ax >> 64) * inv) << 2) + (((u128)(u64)ax * inv) >> 62);
+        const int e = lane <= j ? sm.E[lane] : 0;
+        int F = v ? bits128(v) - 110 + e : -1000;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) F = max(F, __shfl_xor_sync(all, F, o));
+        const int s = e - 48 - F;  // v 2^(e - 110) in units of 2^(F - 62)
+        long long w;
+        if (s >= 0)
+            w = (long long)(v << min(s, 64));
+        else
+            w = s < -126 ? 0 : (long long)((v + ((u128)1 << (-s - 1))) >> -s);
+        p.Q->w[kGramMaxN * j + lane] = x < 0 ? -w : w;
+        if (lane == 0) {
+            p.Q->D[j] = sm.D[j];
+            p.Q->F[j] = F;
+        }
+        if (__any_sync(all, bad || 2 * F > limit) && lane == 0) sm.bad = 1;
+    }
+}
+
 // Every set's sum (all written): gathered, scaled and factored; R written.  False: not served.
 static __device__ __noinline__ bool finish(const GramProblem &p, const size_t slot_bytes, Smem *smp,
                                     unsigned char *base) {
@@ -872,7 +941,12 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
         C[rowoff(n, i) - i + j] = pack(shift128(entry(i, j), sm.E[i] + sm.E[j]));
     }
     __syncthreads();
-    return factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr);
+    if (!factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr)) return false;
+    if (p.Q) {
+        invert_root(p, C, rowv + 2 * n, sm);
+        __syncthreads();
+    }
+    return !sm.bad;
 }
 
 // One work item: its rows' sums and the climb.  True in the CTA that has written the set's sum.

@@ -13,10 +13,13 @@
 #include <cuda_runtime.h>
 
 #include "tsqr_fold.cuh"
+#include "tsqr_gram_q.cuh"
 #include "tsqr_internal.h"
 #include "tsqr_qr.cuh"
 
 namespace tsqr {
+
+constexpr int kWyThreads = 256;  // of the blocked (compact WY) passes
 
 // ------------------------------------------------------------------------------------------
 // Factorization with storage: tsqr_r's leaf + tree kernel keeping its reflectors in a.q.
@@ -47,6 +50,7 @@ const void *qr_factor_fn(int blk) {
 __global__ void __launch_bounds__(256) tsqr_q_tree_kernel(const QTreeArgs a) {
     extern __shared__ __align__(16) double smem[];
     const int n = a.n, k = a.arity, t = blockIdx.x;
+    if (skipped(a.skip)) return;
     const int first = t * k;
     const int nchild = min(k, a.child_cnt - first);
     const size_t id = (size_t)a.level_off + t;
@@ -574,7 +578,7 @@ __global__ void __launch_bounds__(416, 1) tsqr_qt_kernel(const QtArgs a) {
 __device__ __forceinline__ void wy_gram(const double *X, const int ldX, const int rows,
                                         const int n, double *G) {
     const int npairs = n * (n - 1) / 2;
-    for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
+    for (int p = threadIdx.x; p < npairs; p += kWyThreads) {
         // pair p -> (i, J), i < J, column by column: J = the largest with J(J-1)/2 <= p
         int J = (int)((1.0 + sqrt(1.0 + 8.0 * p)) * 0.5);
         while (J * (J - 1) / 2 > p) --J;
@@ -597,13 +601,13 @@ __device__ __forceinline__ void wy_gram(const double *X, const int ldX, const in
 // be complete (a barrier before); S is complete after the call's last barrier.
 __device__ __forceinline__ void wy_s_from_g(const double *G, const double *sc, const int n,
                                             double *S) {
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n; idx += kWyThreads) {
         for (int i = 0; i < n; ++i) S[i + idx * n] = (i == idx) ? sc[2 * idx] : 0.0;
     }
     for (int J = 1; J < n; ++J) {
         __syncthreads();  // columns 0 .. J-1 are complete
         int tpr = 1;
-        while (tpr < 32 && 2 * tpr * J <= (int)blockDim.x) tpr *= 2;
+        while (tpr < 32 && 2 * tpr * J <= kWyThreads) tpr *= 2;
         const int team = threadIdx.x / tpr, sub = threadIdx.x - team * tpr;
         const int i = team < J ? team : J - 1;  // spare teams shadow the last row
         double v = 0.0;
@@ -839,7 +843,7 @@ __global__ void __launch_bounds__(256, 1) tsqr_qt_wy_kernel(const QtArgs a) {
 // Per chunk, last to first: Y = S T, T -= Y, and the chunk's rows of Q, -X diag(c) Y, are
 // written straight from registers.  Only half the flops of the sweep (no dot products with
 // the chunk's rows, which are zero before the chunk's reflectors reach them).
-__global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs a) {
+__device__ __forceinline__ void q_leaf_wy_job(const QLeafArgs &a, const int leaf) {
     extern __shared__ __align__(16) double smem[];
     const int n = a.n, qn = a.qn, q0 = a.q0;
     const QLeafWyLayout L = q_leaf_wy_layout(n, qn, a.ldS, a.wyS == nullptr);
@@ -848,8 +852,7 @@ __global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs 
     double *S = smem + L.S;
     double *Y = smem + L.Y;
     double *cs = smem + L.cs;
-    const int leaf = blockIdx.x;
-    for (int idx = threadIdx.x; idx < n * qn; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * qn; idx += kWyThreads) {
         const int col = idx / n, row = idx - col * n;
         top[idx] = a.single ? ((row == q0 + col) ? a.signs[row] : 0.0)
                             : a.B[(size_t)leaf * n * n + row + (size_t)(q0 + col) * n];
@@ -865,20 +868,20 @@ __global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs 
         const int64_t cid = row0 / a.h;
         const double *csc = a.chunk_sc + cid * 2 * n;
         __syncthreads();  // the previous chunk's X, S and Y are no longer read
-        for (int idx = threadIdx.x; idx < rows * n; idx += blockDim.x) {
+        for (int idx = threadIdx.x; idx < rows * n; idx += kWyThreads) {
             const int col = idx / rows, i = idx - col * rows;
             cp_async8(X + i + (size_t)col * a.ldS, a.V + row0 + i + (int64_t)col * a.ldv, 8);
         }
         if (a.wyS) {
             const double *Sg = a.wyS + cid * (int64_t)n * n;
-            for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x)
+            for (int idx = threadIdx.x; idx < n * n; idx += kWyThreads)
                 cp_async8(S + idx, Sg + idx, 8);
         }
         cp_async_commit();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) cs[j] = csc[2 * j + 1];
+        for (int j = threadIdx.x; j < n; j += kWyThreads) cs[j] = csc[2 * j + 1];
         cp_async_wait_all();
         __syncthreads();
-        for (int idx = threadIdx.x; idx < rows * n; idx += blockDim.x) {  // X diag(c)
+        for (int idx = threadIdx.x; idx < rows * n; idx += kWyThreads) {  // X diag(c)
             const int col = idx / rows, i = idx - col * rows;
             X[i + (size_t)col * a.ldS] *= cs[col];
         }
@@ -888,17 +891,17 @@ __global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs 
             __syncthreads();
             wy_s_from_g(smem + L.G, csc, n, S);
         }
-        for (int o = threadIdx.x; o < n * qn; o += blockDim.x) {  // Y = S T (S upper)
+        for (int o = threadIdx.x; o < n * qn; o += kWyThreads) {  // Y = S T (S upper)
             const int i = o % n, q = o / n;
             double v = 0.0;
             for (int j = i; j < n; ++j) v = fma(S[i + j * n], top[j + q * n], v);
             Y[o] = v;
         }
         __syncthreads();
-        for (int o = threadIdx.x; o < n * qn; o += blockDim.x) top[o] -= Y[o];
+        for (int o = threadIdx.x; o < n * qn; o += kWyThreads) top[o] -= Y[o];
         // Q rows: thread tiles of 4 rows (tr apart) by 2 columns, -sum_j X(r, j) Y(j, q)
         const int tr = (rows + 3) >> 2, tq = (qn + 1) >> 1;
-        for (int u = threadIdx.x; u < tr * tq; u += blockDim.x) {
+        for (int u = threadIdx.x; u < tr * tq; u += kWyThreads) {
             const int rr = u % tr, qa = 2 * (u / tr), qb = min(qa + 1, qn - 1);
             int rw[4];
 #pragma unroll
@@ -923,6 +926,21 @@ __global__ void __launch_bounds__(256, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs 
             }
         }
     }
+}
+__global__ void __launch_bounds__(kWyThreads, 1) tsqr_q_leaf_wy_kernel(const QLeafArgs a) {
+    q_leaf_wy_job(a, blockIdx.x);
+}
+__device__ __noinline__ void q_leaf_wy_call(const QLeafArgs &a, const int leaf) { q_leaf_wy_job(a, leaf); }
+
+// Q's rows where the root has decided: from the Gram factor's inverse, or (the first kWyThreads
+// threads) from the reflectors.
+__global__ void __launch_bounds__(kGramThreads, 1)
+tsqr_q_gram_kernel(const __grid_constant__ GramQArgs g, const __grid_constant__ QLeafArgs a) {
+    extern __shared__ __align__(1024) double smem_d[];
+    if (*g.verdict == 1u)
+        gram::q_rows(g, reinterpret_cast<unsigned char *>(smem_d));
+    else if (threadIdx.x < kWyThreads && blockIdx.x < a.nleaves)
+        q_leaf_wy_call(a, blockIdx.x);
 }
 
 // R X = C for R upper triangular (n x n), C (n x k, leading dimension ldc): one warp per column,
@@ -1073,6 +1091,16 @@ cudaError_t q_leaf_wy_launch(const QLeafArgs &a, size_t smem_bytes, cudaStream_t
     return cudaGetLastError();
 }
 
+cudaError_t q_gram_launch(const GramQArgs &g, const QLeafArgs &a, int sms, size_t leaf_smem,
+                          cudaStream_t stream) {
+    const size_t smem = leaf_smem > gram::kQSmem ? leaf_smem : gram::kQSmem;
+    const cudaError_t e = set_smem_attrs(tsqr_q_gram_kernel, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = g.ntiles < sms ? g.ntiles : sms;
+    tsqr_q_gram_kernel<<<(int)(grid > a.nleaves ? grid : a.nleaves), kGramThreads, smem, stream>>>(g, a);
+    return cudaGetLastError();
+}
+
 size_t wy_smem_bytes(int n, int ldX) {
     return sizeof(double) * ((size_t)ldX * n + 2 * (size_t)n * n);
 }
@@ -1083,8 +1111,6 @@ cudaError_t wy_launch(const WyArgs &a, size_t smem_bytes, int grid, cudaStream_t
     tsqr_wy_kernel<<<grid, 256, smem_bytes, stream>>>(a);
     return cudaGetLastError();
 }
-
-constexpr int kWyThreads = 256;
 
 size_t qt_wy_smem_bytes(int n, int kc, int ldS, bool fused) {
     return sizeof(double) * (size_t)wy_layout(n, kc, ldS, kWyThreads, fused).total;

@@ -21,6 +21,7 @@ struct QTreeArgs {
     double *B;                // per node id: n x n block, leading dimension n (in and out)
     int qg;                   // columns per group: the blocks' columns are independent, and
                               // the kernel takes them qg at a time to bound shared memory
+    const unsigned int *skip; // device word, or null: 1 where Q comes from the Gram factor
 };
 
 // The leaf pass: the leaf partition of the factorization (m, unit, nunits, nleaves, h) and

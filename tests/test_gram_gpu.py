@@ -316,3 +316,58 @@ def test_batches_in_flight_keep_their_tables(T):
     torch.cuda.synchronize()
     for k, out in enumerate(outs):
         assert torch.equal(out, calls[k % 2][5])
+
+
+@pytest.mark.parametrize("m,n", [(256, 1), (512, 8), (513, 7), (1025, 8), (256, 9), (257, 16),
+                                 (20479, 15), (257, 17), (12800, 24), (39041, 25), (19457, 32)])
+def test_qr_from_the_gram_factor(oracle, T, m, n):
+    """Q = A R^-1 at the edges of its tiles (512, 256 and 128 rows a tile for up to 8, 16 and 32
+    columns, 152 tiles a wave) and width classes, leading dimensions padded; R is tsqr_r_ex's under
+    the plan reported, and what the oracle gives."""
+    import torch
+    At = workloads.gaussian(m, n, seed=700 + n)
+    big = torch.full((n, m + 3), float("nan"), dtype=torch.float64)
+    big[:, :m] = At
+    Ad = big.cuda().T[:m, :]
+    Qbig = torch.full((n, m + 5), float("nan"), dtype=torch.float64, device="cuda")
+    Q, R = T.tsqr_qr(Ad, Q=Qbig.T[:m, :])
+    p = T.last_plan()
+    assert p.leaf == T.LEAF_GRAM_Q
+    assert torch.equal(T.tsqr_r_ex(Ad, plan=p), R)
+    _check(oracle, R, At)
+    Qo, Ro = oracle.householder_qr(oracle.from_torch_colmajor(At), nthreads=16)
+    tol = max(50.0, 2.0 * np.sqrt(m)) * oracle.kappa_from_r(Ro) * U * np.linalg.norm(Qo)
+    np.testing.assert_allclose(Q.cpu().numpy(), Qo, rtol=0, atol=tol)
+    Qd = Q.cpu().numpy()
+    assert np.abs(Qd.T @ Qd - np.eye(n)).max() <= 50 * U
+    assert torch.isnan(Qbig[:, m:]).all()
+    assert T.tsqr_get_device_status() == T.SUCCESS
+
+
+@pytest.mark.parametrize("kind", ["kappa10", "kappa100", "kappa1e4", "outlier", "zeros", "integers"])
+@pytest.mark.parametrize("n", [8, 13, 32])
+def test_qr_value_ranges(oracle, T, n, kind):
+    """On both sides of the line to the reflectors: conditions 10, 100 and 1e4, an entry 2^30 above
+    the rest (a column its peak dominates), rows of zeros, small whole numbers.  Orthonormal to
+    50 u and A = Q R to c(m) u either way."""
+    import torch
+    m = 50001
+    if kind.startswith("kappa"):
+        At = workloads.conditioned(m, n, float(kind[5:]), seed=n)
+    else:
+        At = workloads.gaussian(m, n, seed=720 + n)
+    if kind == "outlier":
+        At[:, m // 2] *= 2.0 ** 30
+        At[1, m // 2] = 1.0
+    elif kind == "zeros":
+        At[:, 1000:40000] = 0.0
+    elif kind == "integers":
+        At = torch.round(At * 4.0)
+    Ad = At.cuda().T
+    Q, R = T.tsqr_qr(Ad)
+    assert torch.equal(T.tsqr_r_ex(Ad, plan=T.last_plan()), R)
+    A, Qh, Rh = oracle.from_torch_colmajor(At), Q.cpu().numpy(), R.cpu().numpy()
+    assert np.abs(Qh.T @ Qh - np.eye(n)).max() <= 50 * U
+    assert np.linalg.norm(A - Qh @ Rh) <= 2.0 * np.sqrt(m) * U * np.linalg.norm(A)
+    if kind == "zeros":
+        assert np.all(Qh[1000:40000] == 0)
