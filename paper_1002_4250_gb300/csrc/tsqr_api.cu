@@ -44,9 +44,8 @@ struct Workspace {
     void *base = nullptr;   // counters + slots (grown on demand)
     size_t bytes = 0;
     int *status = nullptr;  // device status word (lives as long as the workspace entry)
-    // batched calls: the problem table and work items last copied to base + table_off
-    std::vector<char> table;
-    size_t table_off = 0;
+    // Batched calls copy their problem table into the workspace on every call: what else runs on the
+    // stream, graph replays included, uses the same workspace and leaves nothing of it.
     // Page-locked copies of the last tables on their way to the device: the copy runs on the stream,
     // after the call has returned, and on a host whose pageable memory the device reads in place
     // (Grace) nothing stages it before.  A slot is reused once its copy is done.
@@ -58,8 +57,7 @@ struct Workspace {
     };
     Staged staged[4];
     int next_staged = 0;
-    // Tables of captured calls: a graph reads them at every replay, and a replay puts its table in
-    // the workspace unseen, so calls after a capture always copy theirs.
+    // Tables of captured calls: a graph reads them at every replay.
     std::vector<std::vector<char>> captured;
 };
 
@@ -477,7 +475,6 @@ tsqr_status_t get_workspace(cudaStream_t stream, size_t bytes, Workspace **out) 
         if (w.base) cudaFreeAsync(w.base, stream);
         w.base = nullptr;
         w.bytes = 0;
-        w.table.clear();
         const size_t nb = align_up(bytes, 1 << 20);
         if (cudaMallocAsync(&w.base, nb, stream) != cudaSuccess) return TSQR_ERR_ALLOC;
         w.bytes = nb;
@@ -2155,7 +2152,7 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
     int32_t served = 0;
     if (gram) plan_gram_batch(ptrs, ms, ns, offsets, count, R_packed, di.sms, &gprobs, &gitems,
                               &gwords, &gslots, &served);
-    // table: problems then items, copied once and reused while the batch is unchanged
+    // table: problems then items
     const size_t tp = align_up(sizeof(BatchProblem) * probs.size(), 16);
     const size_t ti = align_up(sizeof(int2) * items.size(), 16);
     const size_t tg = served ? align_up(sizeof(GramProblem) * gprobs.size(), 16) : 0;
@@ -2183,12 +2180,8 @@ tsqr_status_t run_batched(const void *const *ptrs, const int64_t *ms, const int3
         std::memcpy(table.data() + tp + ti, gprobs.data(), sizeof(GramProblem) * gprobs.size());
         std::memcpy(table.data() + tp + ti + tg, gitems.data(), sizeof(int2) * gitems.size());
     }
-    if (ws->table != table || ws->table_off != table_off) {
-        st = upload_table(ws, table, base + table_off, stream);
-        if (st != TSQR_SUCCESS) return st;
-        ws->table = ws->captured.empty() ? std::move(table) : std::vector<char>();
-        ws->table_off = table_off;
-    }
+    st = upload_table(ws, table, base + table_off, stream);
+    if (st != TSQR_SUCCESS) return st;
     BatchArgs b;
     b.probs = reinterpret_cast<const BatchProblem *>(base + table_off);
     b.items = reinterpret_cast<const int2 *>(base + table_off + tp);

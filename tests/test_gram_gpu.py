@@ -371,3 +371,44 @@ def test_qr_value_ranges(oracle, T, n, kind):
     assert np.linalg.norm(A - Qh @ Rh) <= 2.0 * np.sqrt(m) * U * np.linalg.norm(A)
     if kind == "zeros":
         assert np.all(Qh[1000:40000] == 0)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_batch_repeated_after_another_call(T, dtype):
+    """The same batch (same buffers) before and after a call that takes the same workspace, and
+    after the replay of a graph that does: its problem table is its own each time."""
+    import torch
+    dt = torch.float64 if dtype == "f64" else torch.float32
+    ms, ns = [600 + 37 * i for i in range(24)], [(8, 16, 32, 64)[i % 4] for i in range(24)]
+    offs, roff = [0], [0]
+    for m, n in zip(ms, ns):
+        offs.append(offs[-1] + m * n)
+        roff.append(roff[-1] + n * n)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    buf = torch.randn(offs[-1], generator=g, dtype=dt, device="cuda")
+    wide = torch.randn(128, 60000, generator=g, dtype=torch.float64, device="cuda").T
+    code = (T.F64, T.PREC_F64) if dtype == "f64" else (T.F32, T.PREC_MIXED)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+
+    def batch():
+        R = torch.empty(roff[-1], dtype=torch.float64, device="cuda")
+        T.tsqr_r_batched([buf.data_ptr() + buf.element_size() * o for o in offs[:-1]], ms, ns, roff,
+                         R, dtype=code[0], prec=code[1])
+        return R
+
+    with torch.cuda.stream(s):
+        Rw = T.tsqr_r(wide)  # the workspace at its full size before the first table
+        first = batch()
+        T.tsqr_r(wide, R=Rw)
+        second = batch()
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            T.tsqr_r(wide, R=Rw)
+        third = batch()
+        graph.replay()
+        fourth = batch()
+    s.synchronize()
+    for R in (second, third, fourth):
+        assert torch.equal(first, R)
