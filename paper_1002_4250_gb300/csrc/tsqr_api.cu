@@ -600,7 +600,7 @@ GramLayout gram_layout(int64_t m, int64_t n, int sms) {
     const int64_t nkb = (m + 63) / 64;
     w.nslab = (int)std::max<int64_t>(
         1, std::min<int64_t>(w.nset == 1 ? sms : 5LL * sms / w.nset, nkb / 8));
-    w.inner = gram_inner_nodes(w.nslab);
+    w.inner = gram_inner_nodes(w.nslab, (int)n);
     w.words = 5 + (size_t)w.nset * w.inner;  // queue, failed, verdict, bad, then the nodes, sets done
     w.cnt_bytes = align_up(w.words * sizeof(unsigned int), 256);
     w.bytes = w.cnt_bytes + (size_t)w.nset * (w.nslab + w.inner) *
@@ -674,7 +674,7 @@ struct RLayout {
 };
 RLayout r_layout(const F64Plan &p, int64_t m, int64_t n, int sms) {
     RLayout w;
-    const size_t inner = p.gram_ctas ? (size_t)gram_inner_nodes(p.gram_ctas) : 0;
+    const size_t inner = p.gram_ctas ? (size_t)gram_inner_nodes(p.gram_ctas, (int)n) : 0;
     w.cnt_words = (size_t)p.nodes + (p.gram_ctas ? inner + 2 : 0);
     w.cnt_bytes = align_up(w.cnt_words * sizeof(unsigned int), 256);
     w.gram_off = align_up(w.cnt_bytes + (size_t)p.nodes * (size_t)n * (size_t)n * sizeof(double), 256);
@@ -703,7 +703,7 @@ GramArgs gram_args(const F64Plan &p, const RLayout &w, const F64Args &a, void *b
     g.p.nslab = p.gram_ctas;
     g.p.nkb = (a.m + 63) / 64;
     g.p.counters = a.counters + p.nodes;
-    g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas) + 1;
+    g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas, a.n) + 1;
     g.p.slots = (unsigned char *)base + w.gram_off;
     g.p.R = a.R;
     g.p.ldr = a.ldr;
@@ -1963,7 +1963,7 @@ void plan_gram_batch(const void *const *ptrs, const int64_t *ms, const int32_t *
         const double all = (double)g.nkb * ns[i] * g.nb;
         g.nslab = (int)std::max<double>(
             1.0, std::min<double>(std::ceil(all / (nset * target)), (double)g.nkb / 8));
-        const int inner = gram_inner_nodes(g.nslab);
+        const int inner = gram_inner_nodes(g.nslab, g.n);
         g.counters = (unsigned int *)*words;
         *words += (size_t)nset * inner + 1;
         g.slots = (unsigned char *)*slot_bytes;

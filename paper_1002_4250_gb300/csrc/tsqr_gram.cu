@@ -127,7 +127,7 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
         if (!root || p.n > kGramRootMaxN) continue;  // (a wider matrix is factored by its own launches)
         if (nset > 1) {
             if (tid == 0)
-                c.sm->flag = atomicAdd(p.counters + (size_t)nset * gram_inner_nodes(p.nslab), 1u) + 1 ==
+                c.sm->flag = atomicAdd(p.counters + (size_t)nset * gram_inner_nodes(p.nslab, p.n), 1u) + 1 ==
                              (unsigned)nset;
             __syncthreads();
             if (!c.sm->flag) continue;

@@ -24,7 +24,6 @@ namespace tsqr {
 constexpr int kGramSlicers = 16;    // warps that cut entries into digits; one more multiplies
 constexpr int kGramThreads = 32 * (kGramSlicers + 1);
 constexpr int kGramFoldWarps = 12;  // bulk warps of the Householder reduction (and its reducer)
-constexpr int kGramArity = 16;      // children per node of the Gram sum's tree
 constexpr int kGramMaxN = 32;       // one column block: tsqr_r's single launch
 constexpr int kGramRootMaxN = 128;  // widest matrix one CTA factors
 
@@ -92,11 +91,17 @@ struct GramWideArgs {      // more columns than one CTA factors
     unsigned int *bad;     // non-zero: the sum cannot serve (zeroed per call)
 };
 
-// Inner nodes and all nodes of the sum's tree over `leaves` leaves.
-__host__ __device__ inline int gram_inner_nodes(int leaves) {
+// Children per node of the Gram sum's tree: a level costs some 8,000 cycles (a fence, a counter, the
+// children's exponents, their sums), so up to 24 columns, whose sums are small, one level takes
+// all the slabs (10,000 x 16, 40 of them: 20,000 cycles in two levels of 16, 9,000 in one); wider,
+// one CTA reading them all takes as long as the second level.
+__host__ __device__ inline int gram_arity(int n) { return n <= 24 ? 160 : 16; }
+// Inner nodes of the tree over `leaves` leaves.
+__host__ __device__ inline int gram_inner_nodes(int leaves, int n) {
     int inner = 0;
+    const int arity = gram_arity(n);
     for (int c = leaves; c > 1;) {
-        c = (c + kGramArity - 1) / kGramArity;
+        c = (c + arity - 1) / arity;
         inner += c;
     }
     return inner;

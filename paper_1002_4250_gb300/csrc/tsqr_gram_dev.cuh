@@ -408,20 +408,21 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         };
         for (int jb = 0; jb < Sh::NR; jb += Sh::JP) {
             constexpr int kJ = Sh::JP / 8;
-            for (int task = part; task < Sh::kTiles * kJ && part < 4; task += 4) {
-                const int tile = task / kJ, jl = 8 * (task - tile * kJ);
-                const uint32_t at = lanes + (tile ? Sh::N0 : 0) + jb + jl;
+            // a task: four right-hand digits of eight columns; tile 0's halves, then tile 1's
+            constexpr int kTasks = Sh::kMirror ? 3 * kJ : 2 * Sh::kTiles * kJ;
+            for (int task = part; task < kTasks && part < 4; task += 4) {
+                const int which = task / kJ, jl = 8 * (task - which * kJ);
+                const int tile = which >> 1, half = which & 1;
+                const uint32_t at = lanes + (tile ? Sh::N0 : 0) + jb + jl + half * (4 * Sh::NR);
                 long long x[8];
                 if (Sh::kMirror && tile == 1) {
                     digits(std::integral_constant<int, Sh::kMirror ? Sh::TE - Sh::TS : 4>(), x, at);
                     if (s < S - Sh::TS) put(kL1 + (s * Sh::JP + jl) * Sh::kLd, x);
                 } else {
                     const int sr = s + tile * Sh::TS;  // the row's digit
-                    const bool keep = s < Sh::TS && sr < Sh::kRowDigits;
                     digits(std::integral_constant<int, 4>(), x, at);
-                    if (keep) put(second * kSecond + (sr * Sh::JP + jl) * Sh::kLd, x);
-                    digits(std::integral_constant<int, 4>(), x, at + 4 * Sh::NR);
-                    if (keep) put(second * kSecond + kHalf + (sr * Sh::JP + jl) * Sh::kLd, x);
+                    if (s < Sh::TS && sr < Sh::kRowDigits)
+                        put(second * kSecond + half * kHalf + (sr * Sh::JP + jl) * Sh::kLd, x);
                 }
             }
             tc::fence_before_sync();
@@ -623,7 +624,7 @@ __device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const 
                       const size_t slot_bytes, Cta &c) {
     const int tid = threadIdx.x, lane = tid & 31;
     Smem &sm = *c.sm;
-    const int inner = gram_inner_nodes(p.nslab);
+    const int inner = gram_inner_nodes(p.nslab, p.n);
     unsigned int *counters = p.counters + (size_t)set * inner;
     unsigned char *slots = p.slots + (size_t)set * (p.nslab + inner) * slot_bytes;
     const int nout = NJ > 0 ? cols.ni * cols.nj : cols.ni * (cols.ni + 1) / 2;
@@ -652,11 +653,13 @@ __device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const 
         }
     }
     int cnt = p.nslab, off = 0, t = slab, cidx = 0;
-    int *kd = reinterpret_cast<int *>(c.stages);  // children's exponents, 128 each; then the node's
+    constexpr int kHeads = NJ > 0 ? 64 : 32;  // exponents of a child: block I's, then block J's
+    const int arity = gram_arity(p.n);
+    int *kd = reinterpret_cast<int *>(c.stages);  // the node's exponents, then its children's
     while (cnt > 1) {
-        const int next_cnt = (cnt + kGramArity - 1) / kGramArity;
-        const int parent = t / kGramArity, first = parent * kGramArity;
-        const int nchild = min(kGramArity, cnt - first);
+        const int next_cnt = (cnt + arity - 1) / arity;
+        const int parent = t / arity, first = parent * arity;
+        const int nchild = min(arity, cnt - first);
         __threadfence();
         __syncthreads();
         if (tid == 0) sm.flag = atomicAdd(&counters[cidx + parent], 1u) + 1 == (unsigned)nchild;
@@ -665,33 +668,49 @@ __device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const 
         __threadfence();
         const unsigned char *kids = slots + (size_t)(off + first) * slot_bytes;
         unsigned char *node = slots + (size_t)(off + cnt + parent) * slot_bytes;
-        for (int e = tid; e < 128 * nchild; e += kGramThreads)
-            kd[e] = __ldcg(reinterpret_cast<const int *>(kids + (e >> 7) * slot_bytes) + (e & 127));
         if (tid == 0) sm.bad = 0;
+        for (int e = tid; e < kHeads * nchild; e += kGramThreads) {
+            const int l = e % kHeads;
+            kd[kHeads + e] = __ldcg(reinterpret_cast<const int *>(kids + e / kHeads * slot_bytes) +
+                                    (l < 32 ? l : 32 + l));
+        }
+        int bad = 0;
+        if (tid < nchild)
+            bad = __ldcg(reinterpret_cast<const int *>(kids + tid * slot_bytes) + kGramSlotHead / 4 - 1);
         __syncthreads();
-        if (tid < 128) {
+        if (bad) sm.bad = 1;
+        if (tid < kHeads) {
             int d = 0;
-            for (int ch = 0; ch < nchild; ++ch) d = max(d, kd[128 * ch + tid]);
-            kd[128 * kGramArity + tid] = d;
-            reinterpret_cast<int *>(node)[tid] = d;
-        } else if (tid < 128 + nchild) {
-            if (__ldcg(reinterpret_cast<const int *>(kids + (tid - 128) * slot_bytes) +
-                       kGramSlotHead / 4 - 1))
-                sm.bad = 1;
+            for (int ch = 1; ch <= nchild; ++ch) d = max(d, kd[kHeads * ch + tid]);
+            kd[tid] = d;
+            reinterpret_cast<int *>(node)[tid < 32 ? tid : 32 + tid] = d;
         }
         __syncthreads();
         if (tid == 0) reinterpret_cast<int *>(node)[kGramSlotHead / 4 - 1] = sm.bad;
-        for (int o = tid; o < nout; o += kGramThreads) {
+        // an output's children go to as many threads as there are for it
+        const int parts = max(1, min(nchild, kGramThreads / nout));
+        Q128 *part = reinterpret_cast<Q128 *>(c.stages + (((arity + 1) * kHeads * 4 + 15) & ~15));
+        for (int u = tid; u < nout * parts; u += kGramThreads) {
+            const int o = u % nout;
             int i, j;
             decode(o, i, j);
-            const int jj = NJ > 0 ? 64 + j : j;
-            const int dij = kd[128 * kGramArity + i] + kd[128 * kGramArity + jj];
+            const int jj = NJ > 0 ? 32 + j : j;
+            const int dij = kd[i] + kd[jj];
             const unsigned char *e = kids + kGramSlotHead + (size_t)o * 16;
             i128 g = 0;
-#pragma unroll 4
-            for (int ch = 0; ch < nchild; ++ch)
-                g += shr128(ldcg128(e + ch * slot_bytes), dij - kd[128 * ch + i] - kd[128 * ch + jj]);
-            reinterpret_cast<Q128 *>(node + kGramSlotHead)[o] = pack(g);
+#pragma unroll 8
+            for (int ch = u / nout; ch < nchild; ch += parts)
+                g += shr128(ldcg128(e + ch * slot_bytes),
+                            dij - kd[kHeads * (ch + 1) + i] - kd[kHeads * (ch + 1) + jj]);
+            (parts > 1 ? part[u] : reinterpret_cast<Q128 *>(node + kGramSlotHead)[o]) = pack(g);
+        }
+        if (parts > 1) {
+            __syncthreads();
+            for (int o = tid; o < nout; o += kGramThreads) {
+                i128 g = 0;
+                for (int q = 0; q < parts; ++q) g += unpack(part[q * nout + o]);
+                reinterpret_cast<Q128 *>(node + kGramSlotHead)[o] = pack(g);
+            }
         }
         off += cnt;
         cidx += next_cnt;
@@ -709,13 +728,11 @@ __device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const 
 // row k scaled by 2^z (pivot in [1/4, 1) again): l = C(k, j) / pivot in [-2, 2], to about 2^-90
 // from a 46-bit reciprocal and one residual, then C(i, j) -= l_i C(k, j).  R(k, j) = l_j sqrt(pivot).
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ u128 mul122(const u128 a, const u128 b) {  // (a b) >> 122; a, b < 2^124
+// (a b) >> 122 to 2^8 (2^-114: far below the columns' own rounding), a, b < 2^124: one full product
+// of words and the high halves of two.
+__device__ __forceinline__ u128 mul122(const u128 a, const u128 b) {
     const u64 ah = (u64)(a >> 64), al = (u64)a, bh = (u64)(b >> 64), bl = (u64)b;
-    const u128 mid = (u128)ah * bl + (u128)al * bh + __umul64hi(al, bl);
-    return (((u128)ah * bh) << 6) + (mid >> 58);
-}
-__device__ __forceinline__ u128 mul60(const u128 a, const u64 r) {  // (a r) >> 60
-    return (((u128)(u64)(a >> 64) * r) << 4) + (((u128)(u64)a * r) >> 60);
+    return ((u128)ah * bh + __umul64hi(ah, bl) + __umul64hi(al, bh)) << 6;
 }
 // 2^60 (2^122 / d) to about 46 bits, d in [2^120, 2^122): the hardware's FP32 reciprocal and one
 // Newton step.
@@ -728,6 +745,13 @@ __device__ __forceinline__ u64 recip60(const u128 d) {
     const u64 r = (u64)((yb & 0x7fffff) | 0x800000) << (37 + (int)(yb >> 23) - 127);
     const long long e = (1ll << 60) - (long long)__umul64hi(x, r);
     return r + (u64)(__mul64hi((long long)r, e) << 4);
+}
+// 2^122 c / d to about 2^-90 from r = recip60(d): 46 bits, then the residual's quotient; c <= 2 d.
+__device__ __forceinline__ u128 quotient(const u128 c, const u128 d, const u64 r) {
+    const u64 q = __umul64hi((u64)(c >> 60), r);  // of weight 2^64
+    const u128 qd = (((u128)q * (u64)(d >> 64)) << 6) + (((u128)q * (u64)d) >> 58);
+    const long long res = (long long)((i128)(c - qd) >> 16);  // below 2^62
+    return ((u128)q << 64) + (u128)((i128)__mul64hi(res, (long long)r) << 20);
 }
 // x / 2^122 as a sum of two doubles (the second below the first's last place).
 struct D2 {
@@ -744,42 +768,118 @@ __device__ __forceinline__ D2 sqrt2(const D2 x) {
     return D2{s, (fma(-s, s, x.hi) + x.lo) / (2.0 * s)};
 }
 
+__device__ __forceinline__ int bits128(const u128 x) {
+    const u64 h = (u64)(x >> 64);
+    return h ? 128 - __clzll((long long)h) : 64 - __clzll((long long)(u64)x);
+}
+// 2^64 sqrt(d / 2^122) to about 2^-62 of it, d in [2^120, 2^122): the hardware's FP32 reciprocal
+// square root, two Newton steps, and the residual's share.
+__device__ __forceinline__ u64 sqrt64(const u128 d) {
+    const u64 x = (u64)(d >> 58);
+    const float f = __uint2float_rz((uint32_t)(x >> 32)) * 2.3283064365386963e-10f;
+    float yf;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(yf) : "f"(f));
+    const uint32_t yb = __float_as_uint(yf);  // in [1, 2]
+    u64 y = (u64)((yb & 0x7fffff) | 0x800000) << (39 + (int)(yb >> 23) - 127);
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+        const long long e = (1ll << 62) - (long long)__umul64hi(x, __umul64hi(y, y) << 2);
+        y += (u64)(__mul64hi((long long)y, e) << 1);
+    }
+    const u64 q = __umul64hi(x, y);  // of 2^62
+    const long long res = (long long)((i128)((d << 2) - (u128)q * q) >> 8);
+    const u64 v = (q << 2) + (u64)(__mul64hi(res, (long long)y) >> 51);
+    return v >> 62 ? v : ~0ull;
+}
+// p 2^e, p in [2^62, 2^64), rounded to FP64 (in range).
+__device__ __forceinline__ double round64(u64 p, int e, const bool neg) {
+    if (!(p >> 63)) {
+        p <<= 1;
+        --e;
+    }
+    const u64 m = (p >> 11) + ((p >> 10) & 1);
+    return __longlong_as_double((long long)((((u64)(1023 + 52 + 11 - 1 + e) << 52) + m) |
+                                            ((u64)neg << 63)));
+}
+
 // C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it.  rowv: 3 n
-// entries of scratch.  g[j]: the power of two of R's column j.  Returns false if a pivot is too small.
-static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g, double *R, const int64_t ldr) {
+// entries of scratch (the scaled pivots stay in the last n).  g[j]: the power of two of R's column j.
+// Returns false if a pivot is too small (*low: zero on entry, then non-zero).
+//
+// A chain of n steps, each a reciprocal, a quotient and a multiplication deep.  The first n threads
+// hold column j = tid: row k's l are theirs, and while the others take row k off the rows below they
+// find the next pivot (from the diagonal as it was and l's own share) and its reciprocal.  In
+// integers to the last: R's entries too, the chip's FP64 units being two lanes an SM.  Up to 32
+// columns the trailing matrix stays in registers.  n = 32: 71 us of a 1,000-row call before, with
+// full products, the reciprocal in the chain and R in double-double.
+static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g,
+                                                double *R, const int64_t ldr, int *low) {
     const int tid = threadIdx.x, nt = kGramThreads, warp = tid >> 5, lane = tid & 31;
+    constexpr i128 kLeast = (i128)1 << (122 - kPivotBits);
     Q128 *Lq = rowv, *Cp = rowv + n, *dv = rowv + 2 * n;
+    // Up to 32 columns a thread keeps its entry (ti, tj) of C in registers until its row's turn.
+    const bool owns = n <= kGramMaxN;
+    int ti = -1, tj = 0;
+    i128 own = 0;
+    if (owns && tid < n * (n + 1) / 2) {
+        int a, b;
+        unpack_index(n * (n + 1) / 2 - 1 - tid, a, b);
+        ti = n - 1 - b;
+        tj = n - 1 - a;
+        own = unpack(C[tid]);
+    }
+    i128 diag = tid < n ? unpack(C[rowoff(n, tid)]) : (i128)0;
+    u128 d = 0, mine = 0;  // the pivot scaled to [1/4, 1), and the thread's own once it has been
+    u64 r = 0;
+    int z = 0, myz = 0;
+    auto pivot = [&](const i128 d0) {
+        z = (122 - bits128((u128)d0)) >> 1;
+        d = (u128)d0 << (2 * z);
+        r = recip60(d);
+    };
+    {
+        const i128 d0 = unpack(C[0]);
+        if (d0 < kLeast) return false;  // the same for every thread
+        if (tid < n) pivot(d0);
+    }
     for (int k = 0; k < n; ++k) {
         Q128 *Ck = C + rowoff(n, k) - k;
-        const i128 d0 = unpack(Ck[k]);
-        if (d0 < ((i128)1 << (122 - kPivotBits))) return false;  // the same for every thread
-        const u64 dh = (u64)((u128)d0 >> 64);
-        const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d0);
-        const int z = (122 - len) >> 1;
-        const int j = k + 1 + tid;
-        if (j < n || tid == 0) {
-            u128 d = (u128)d0;
-            if (z) d <<= 2 * z;
-            if (tid == 0) dv[k] = pack((i128)d);
-            if (j < n) {
-                const i128 c0 = unpack(Ck[j]);
+        u128 lm = 0, cm = 0;  // |l| and |c| of the thread's column
+        if (tid < n) {
+            if (tid == k) {
+                dv[k] = pack((i128)d);
+                mine = d;
+                myz = z;
+            } else if (tid > k) {
+                const i128 c0 = unpack(Ck[tid]);
                 const bool neg = c0 < 0;
-                u128 c = (u128)(neg ? -c0 : c0);
-                if (z) c <<= z;
-                const u64 r = recip60(d);
-                u128 q = mul60(c, r);
-                const i128 res = (i128)(c - mul122(q, d));
-                const u128 dq = mul60((u128)(res < 0 ? -res : res), r);
-                q = res < 0 ? q - dq : q + dq;
-                const Q128 l = pack(neg ? -(i128)q : (i128)q);
-                Lq[j] = l;
-                Ck[j] = l;
-                Cp[j] = pack(neg ? -(i128)c : (i128)c);
+                cm = (u128)(neg ? -c0 : c0) << z;
+                lm = quotient(cm, d, r);
+                const Q128 l = pack(neg ? -(i128)lm : (i128)lm);
+                Lq[tid] = l;
+                Ck[tid] = l;
+                Cp[tid] = pack(neg ? -(i128)cm : (i128)cm);
+                if (tid == k + 1) Lq[k] = pack(diag);
             }
         }
+        if (k + 1 == n) break;
         __syncthreads();
-        // trailing update, (i, j) with k < i <= j: a warp a row
-        for (int i = k + 1 + warp; i < n; i += nt >> 5) {
+        if (tid < n) {
+            const i128 a = unpack(Lq[k + 1]), b = unpack(Cp[k + 1]);
+            const i128 d0 = unpack(Lq[k]) -
+                            (i128)mul122((u128)(a < 0 ? -a : a), (u128)(b < 0 ? -b : b));
+            if (d0 < kLeast) *low = 1;
+            diag -= (i128)mul122(lm, cm);
+            pivot(d0 < kLeast ? kLeast : d0);
+        }
+        // trailing update, (i, j) with k < i <= j: a thread an entry, or a warp a row
+        if (ti > k) {
+            const i128 a = unpack(Lq[ti]), b = unpack(Cp[tj]);
+            const u128 q = mul122((u128)(a < 0 ? -a : a), (u128)(b < 0 ? -b : b));
+            own = (a < 0) != (b < 0) ? own + (i128)q : own - (i128)q;
+            if (ti == k + 1) C[tid] = pack(own);
+        }
+        for (int i = k + 1 + (nt >> 5) - 1 - warp; i < n && !owns; i += nt >> 5) {
             const i128 a = unpack(Lq[i]);
             const u128 am = (u128)(a < 0 ? -a : a);
             Q128 *Ci = C + rowoff(n, i) - i;
@@ -791,35 +891,29 @@ static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n
             }
         }
         __syncthreads();
+        if (*low) return false;
     }
-    // R(k, k) = sqrt(C(k, k)) (still in place); R(k, j) = l sqrt(d): rounded once, near enough
-    D2 *sd = reinterpret_cast<D2 *>(Lq);
-    for (int k = tid; k < n; k += nt) sd[k] = sqrt2(to_double(unpack(dv[k])));
+    // R(k, k) = sqrt(d_k) 2^-z_k, R(k, j) = l sqrt(d_k)
+    __syncthreads();
+    if (tid < n) Lq[tid] = Q128{sqrt64(mine), (u64)myz};
     __syncthreads();
     for (int o = tid; o < n * n; o += nt) {
         const int col = o / n, row = o - col * n;
         double v = 0.0;
-        if (row <= col) {
-            const D2 x = to_double(unpack(C[rowoff(n, row) - row + col]));
-            if (row == col) {
-                const D2 q = sqrt2(x);
-                v = q.hi + q.lo;
-            } else {
-                const D2 q = sd[row];
-                const double p = x.hi * q.hi;
-                v = p + (fma(x.hi, q.hi, -p) + (x.hi * q.lo + x.lo * q.hi));
-            }
-            v = scalbn(v, g[col]);
+        if (row < col) {
+            const i128 l = unpack(C[rowoff(n, row) - row + col]);
+            const u128 a = (u128)(l < 0 ? -l : l);
+            const int b = bits128(a);
+            const u64 top = b > 64 ? (u64)(a >> (b - 64)) : (u64)a << ((64 - b) & 63);
+            if (b) v = round64(__umul64hi(top, Lq[row].lo), b - 186 + g[col], l < 0);
+        } else if (row == col) {
+            v = round64(Lq[row].lo, g[col] - 64 - (int)Lq[row].hi, false);
         }
         R[row + (int64_t)col * ldr] = v;
     }
     return true;
 }
 
-__device__ __forceinline__ int bits128(const u128 x) {
-    const u64 h = (u64)(x >> 64);
-    return h ? 128 - __clzll((long long)h) : 64 - __clzll((long long)(u64)x);
-}
 // The inverse of the factor just formed, for Q = A R^-1 (p.Q): R = diag(rho) M 2^g by columns, with
 // M(k, k) = 2^-z_k and M(k, j) = l, so column j of the inverse is M^-1 e_j / rho_j: a warp a
 // column, its entries one a lane, 110 bits after the point through the substitution (which a
@@ -893,7 +987,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
     Smem &sm = *smp;
     Q128 *C = reinterpret_cast<Q128 *>(base);
     Q128 *rowv = C + n * (n + 1) / 2;
-    const int per_set = p.nslab + gram_inner_nodes(p.nslab), nset = gram_sets(p.nb);
+    const int per_set = p.nslab + gram_inner_nodes(p.nslab, p.n), nset = gram_sets(p.nb);
     auto top = [&](const int set) {
         return p.slots + ((size_t)(set + 1) * per_set - 1) * slot_bytes;
     };
@@ -941,7 +1035,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
         C[rowoff(n, i) - i + j] = pack(shift128(entry(i, j), sm.E[i] + sm.E[j]));
     }
     __syncthreads();
-    if (!factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr)) return false;
+    if (!factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr, &sm.bad)) return false;
     if (p.Q) {
         invert_root(p, C, rowv + 2 * n, sm);
         __syncthreads();

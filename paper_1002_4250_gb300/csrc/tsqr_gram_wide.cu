@@ -14,7 +14,7 @@ using namespace gram;
 constexpr int kBw = 32;  // rows of a block
 
 __device__ __forceinline__ const unsigned char *set_top(const GramProblem &p, const int I, const int J) {
-    const int per_set = p.nslab + gram_inner_nodes(p.nslab);
+    const int per_set = p.nslab + gram_inner_nodes(p.nslab, p.n);
     const int set = I == J ? I : p.nb + J * (J - 1) / 2 + I;
     return p.slots + ((size_t)(set + 1) * per_set - 1) * gram_slot_bytes(kBlock);
 }
@@ -72,15 +72,10 @@ __device__ __forceinline__ i128 smul122(const i128 a, const i128 b) {
     const u128 q = mul122((u128)(a < 0 ? -a : a), (u128)(b < 0 ? -b : b));
     return (a < 0) != (b < 0) ? -(i128)q : (i128)q;
 }
-// c / d for a pivot d in [1/4, 1) with reciprocal r (factor_root's quotient).
-__device__ __forceinline__ i128 quotient(const i128 c0, const u128 d, const u64 r) {
-    const bool neg = c0 < 0;
-    const u128 c = (u128)(neg ? -c0 : c0);
-    u128 q = mul60(c, r);
-    const i128 res = (i128)(c - mul122(q, d));
-    const u128 dq = mul60((u128)(res < 0 ? -res : res), r);
-    q = res < 0 ? q - dq : q + dq;
-    return neg ? -(i128)q : (i128)q;
+// c / d for a pivot d in [1/4, 1) with reciprocal r.
+__device__ __forceinline__ i128 squotient(const i128 c, const u128 d, const u64 r) {
+    const i128 q = (i128)quotient((u128)(c < 0 ? -c : c), d, r);
+    return c < 0 ? -q : q;
 }
 __device__ __forceinline__ i128 shfl128(const i128 x, const int src) {
     const u64 lo = __shfl_sync(0xffffffffu, (u64)x, src);
@@ -123,7 +118,7 @@ __global__ void __launch_bounds__(256) tsqr_gram_panel_kernel(const GramWideArgs
             } else {
                 i128 c = unpack(L[k][tid]);
                 if (z) c = (i128)((u128)c << z);
-                const Q128 l = pack(quotient(c, d, r));
+                const Q128 l = pack(squotient(c, d, r));
                 row[tid] = l;
                 rowp[tid] = pack(c);
                 L[k][tid] = l;
@@ -157,7 +152,7 @@ __global__ void __launch_bounds__(256) tsqr_gram_panel_kernel(const GramWideArgs
         const int z = zs[lane];
         if (z) c = (i128)((u128)c << z);
         P[(int64_t)lane * n + j] = pack(c);
-        C[(int64_t)(k0 + lane) * n + j] = pack(quotient(c, (u128)unpack(piv[lane]), rec[lane]));
+        C[(int64_t)(k0 + lane) * n + j] = pack(squotient(c, (u128)unpack(piv[lane]), rec[lane]));
     }
 }
 
