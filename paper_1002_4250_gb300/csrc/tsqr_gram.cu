@@ -96,7 +96,13 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
         }
         const GramProblem &p = a.probs ? a.probs[which] : a.one;
         const size_t slot_bytes = gram_slot_bytes(gram_block(p.n));
-        const int nset = gram_sets(p.nb), slab = code / nset, set = code - slab * nset;
+        const int nset = gram_sets(p.nb);
+        int slab = code / nset, set = code - slab * nset;
+        if (!a.probs && code >= a.cut) {  // the last slabs set by set
+            const int tail = p.nslab - a.cut / nset, q = code - a.cut, o = q / tail;
+            slab = p.nslab - tail + q - o * tail;
+            set = o < nset - p.nb ? p.nb + o : o - (nset - p.nb);
+        }
         Cols cols{0, 0, 0, 0};
         bool root;
         if (set < p.nb) {

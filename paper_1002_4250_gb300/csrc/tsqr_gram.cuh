@@ -75,8 +75,10 @@ struct GramQueueArgs {     // a queue of work items
     GramProblem one;       // the problem when probs is null
     const GramProblem *probs;
     const int2 *items;     // (problem, set + nsets slab) in the order they are taken; null: item
-                           // k of the one problem is set k % nsets of slab k / nsets
-    int nitems;
+                           // k of the one problem is set k % nsets of slab k / nsets, so that a
+                           // slab's sets find its rows in L2; from item cut on, the two-block
+                           // sets (twice the work) of all slabs left, then the others
+    int nitems, cut;
     unsigned int *queue;   // next item, zeroed per call
     unsigned int *failed;  // problems left to the Householder reduction, zeroed per call
     int *status;
