@@ -802,18 +802,25 @@ __device__ __forceinline__ double round64(u64 p, int e, const bool neg) {
                                             ((u64)neg << 63)));
 }
 
+// l sqrt(d) 2^g from s = sqrt64(d).
+__device__ __forceinline__ double r_entry(const i128 l, const u64 s, const int g) {
+    const u128 a = (u128)(l < 0 ? -l : l);
+    const int b = bits128(a);
+    const u64 top = b > 64 ? (u64)(a >> (b - 64)) : (u64)a << ((64 - b) & 63);
+    return b ? round64(__umul64hi(top, s), b - 186 + g, l < 0) : 0.0;
+}
+
 // C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it.  rowv: 3 n
-// entries of scratch (the scaled pivots stay in the last n).  g[j]: the power of two of R's column j.
-// Returns false if a pivot is too small (*low: zero on entry, then non-zero).
+// entries of scratch (the scaled pivots stay in the last n).  Thread k < n returns pivot k, scaled,
+// and its shift.  Returns false if a pivot is too small (*low: zero on entry, then non-zero).
 //
 // A chain of n steps, each a reciprocal, a quotient and a multiplication deep.  The first n threads
 // hold column j = tid: row k's l are theirs, and while the others take row k off the rows below they
-// find the next pivot (from the diagonal as it was and l's own share) and its reciprocal.  In
-// integers to the last: R's entries too, the chip's FP64 units being two lanes an SM.  Up to 32
-// columns the trailing matrix stays in registers.  n = 32: 71 us of a 1,000-row call before, with
-// full products, the reciprocal in the chain and R in double-double.
-static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g,
-                                                double *R, const int64_t ldr, int *low) {
+// find the next pivot (from the diagonal as it was and l's own share) and its reciprocal.  Up to 32
+// columns the trailing matrix stays in registers.  (1,000 x 32, with what follows here: 53 us a call,
+// 72 with full products, the reciprocal in the chain and R in double-double.)
+static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int n, int *low,
+                                                 u128 &mine, int &myz) {
     const int tid = threadIdx.x, nt = kGramThreads, warp = tid >> 5, lane = tid & 31;
     constexpr i128 kLeast = (i128)1 << (122 - kPivotBits);
     Q128 *Lq = rowv, *Cp = rowv + n, *dv = rowv + 2 * n;
@@ -829,9 +836,11 @@ static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n
         own = unpack(C[tid]);
     }
     i128 diag = tid < n ? unpack(C[rowoff(n, tid)]) : (i128)0;
-    u128 d = 0, mine = 0;  // the pivot scaled to [1/4, 1), and the thread's own once it has been
+    u128 d = 0;  // the pivot scaled to [1/4, 1)
     u64 r = 0;
-    int z = 0, myz = 0;
+    int z = 0;
+    mine = 0;
+    myz = 0;
     auto pivot = [&](const i128 d0) {
         z = (122 - bits128((u128)d0)) >> 1;
         d = (u128)d0 << (2 * z);
@@ -893,7 +902,18 @@ static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n
         __syncthreads();
         if (*low) return false;
     }
-    // R(k, k) = sqrt(d_k) 2^-z_k, R(k, j) = l sqrt(d_k)
+    return true;
+}
+
+// R from the chain's l and pivots: R(k, k) = sqrt(d_k) 2^-z_k, R(k, j) = l sqrt(d_k), g[j] the power
+// of two of column j; in integers to the last (the chip has two FP64 lanes an SM).
+static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g,
+                                                double *R, const int64_t ldr, int *low) {
+    const int tid = threadIdx.x, nt = kGramThreads;
+    Q128 *Lq = rowv;
+    u128 mine;
+    int myz;
+    if (!factor_chain(C, rowv, n, low, mine, myz)) return false;
     __syncthreads();
     if (tid < n) Lq[tid] = Q128{sqrt64(mine), (u64)myz};
     __syncthreads();
@@ -901,11 +921,7 @@ static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n
         const int col = o / n, row = o - col * n;
         double v = 0.0;
         if (row < col) {
-            const i128 l = unpack(C[rowoff(n, row) - row + col]);
-            const u128 a = (u128)(l < 0 ? -l : l);
-            const int b = bits128(a);
-            const u64 top = b > 64 ? (u64)(a >> (b - 64)) : (u64)a << ((64 - b) & 63);
-            if (b) v = round64(__umul64hi(top, Lq[row].lo), b - 186 + g[col], l < 0);
+            v = r_entry(unpack(C[rowoff(n, row) - row + col]), Lq[row].lo, g[col]);
         } else if (row == col) {
             v = round64(Lq[row].lo, g[col] - 64 - (int)Lq[row].hi, false);
         }

@@ -83,71 +83,54 @@ __device__ __forceinline__ i128 shfl128(const i128 x, const int src) {
     return (i128)(((u128)hi << 64) | lo);
 }
 
-// Block row kb: its diagonal block factored, then the columns right of it, one warp a column:
-// lane i holds row i; step k takes row k's multiple off the rows below.
-__global__ void __launch_bounds__(256) tsqr_gram_panel_kernel(const GramWideArgs a, const int kb) {
-    __shared__ Q128 L[kBw][kBw + 1], row[kBw], rowp[kBw], piv[kBw];
+// Block row kb: its diagonal block factored (by every CTA for itself: the root's chain), then the
+// columns right of it, one warp a column: lane i holds row i; step k takes row k's multiple off the
+// rows below.  Bound by the chain of 32 pivots, 1.7k cycles each of some 45 us.
+__global__ void __launch_bounds__(kGramThreads) tsqr_gram_panel_kernel(const GramWideArgs a, const int kb) {
+    __shared__ Q128 L[kBw * (kBw + 1) / 2], rowv[3 * kBw];
     __shared__ u64 rec[kBw];
-    __shared__ int zs[kBw];
+    __shared__ int zs[kBw], low;
     if (*a.bad) return;
     const int n = a.p.n, k0 = kb * kBw, w = min(kBw, n - k0);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int kWarps = kGramThreads / 32;
     Q128 *C = reinterpret_cast<Q128 *>(a.C), *P = reinterpret_cast<Q128 *>(a.P);
-    for (int o = tid; o < kBw * kBw; o += 256) {
-        const int i = o / kBw, j = o % kBw;
-        L[i][j] = i <= j && j < w ? C[(int64_t)(k0 + i) * n + k0 + j] : Q128{0, 0};
+    for (int o = tid; o < w * w; o += kGramThreads) {
+        const int i = o / w, j = o % w;
+        if (i <= j) L[rowoff(w, i) - i + j] = C[(int64_t)(k0 + i) * n + k0 + j];
+    }
+    if (tid == 0) low = 0;
+    __syncthreads();
+    u128 mine;
+    int myz;
+    if (!factor_chain(L, rowv, w, &low, mine, myz)) {  // (the same for every thread of every CTA)
+        if (tid == 0) *a.bad = 1;
+        return;
+    }
+    const Q128 *piv = rowv + 2 * w;
+    if (tid < w) {
+        rec[tid] = recip60(mine);
+        zs[tid] = myz;
     }
     __syncthreads();
-    for (int k = 0; k < w; ++k) {
-        const i128 d0 = unpack(L[k][k]);
-        if (d0 < ((i128)1 << (122 - kPivotBits))) {  // the same for every thread of every CTA
-            if (tid == 0) *a.bad = 1;
-            return;
-        }
-        const u64 dh = (u64)((u128)d0 >> 64);
-        const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d0);
-        const int z = (122 - len) >> 1;
-        if (tid < kBw && tid >= k) {
-            u128 d = (u128)d0;
-            if (z) d <<= 2 * z;
-            const u64 r = recip60(d);
-            if (tid == k) {
-                piv[k] = pack((i128)d);
-                rec[k] = r;
-                zs[k] = z;
-            } else {
-                i128 c = unpack(L[k][tid]);
-                if (z) c = (i128)((u128)c << z);
-                const Q128 l = pack(squotient(c, d, r));
-                row[tid] = l;
-                rowp[tid] = pack(c);
-                L[k][tid] = l;
-            }
-        }
-        __syncthreads();
-        for (int i = k + 1 + warp; i < w; i += 8)
-            if (lane >= i)
-                L[i][lane] = pack(unpack(L[i][lane]) - smul122(unpack(row[i]), unpack(rowp[lane])));
-        __syncthreads();
-    }
     if (blockIdx.x == 0) {
-        for (int o = tid; o < w * w; o += 256) {
+        for (int o = tid; o < w * w; o += kGramThreads) {
             const int i = o / w, j = o % w;
             // (mirrored: other CTAs may still be reading the block itself)
-            if (i < j) C[(int64_t)(k0 + j) * n + k0 + i] = L[i][j];
+            if (i < j) C[(int64_t)(k0 + j) * n + k0 + i] = L[rowoff(w, i) - i + j];
         }
         if (tid < w) {
             reinterpret_cast<Q128 *>(a.d)[k0 + tid] = piv[tid];
             a.z[k0 + tid] = zs[tid];
         }
     }
-    for (int j = k0 + kBw + blockIdx.x * 8 + warp; j < n; j += gridDim.x * 8) {  // (w == kBw here)
+    for (int j = k0 + kBw + blockIdx.x * kWarps + warp; j < n; j += gridDim.x * kWarps) {  // (w == kBw here)
         i128 c = unpack(C[(int64_t)(k0 + lane) * n + j]);
         for (int k = 0; k < kBw - 1; ++k) {
             i128 ck = shfl128(c, k);
             const int z = zs[k];
             if (z) ck = (i128)((u128)ck << z);
-            if (lane > k) c -= smul122(unpack(L[k][lane]), ck);
+            if (lane > k) c -= smul122(unpack(L[rowoff(kBw, k) - k + lane]), ck);
         }
         const int z = zs[lane];
         if (z) c = (i128)((u128)c << z);
@@ -158,8 +141,9 @@ __global__ void __launch_bounds__(256) tsqr_gram_panel_kernel(const GramWideArgs
 
 // C(I, J) -= sum over block row kb of l(k, i) c(k, j), 32 x 32 a CTA.  Values as x = h 2^62 + l with
 // signed h and 0 <= l < 2^62: of a product over 2^122 the high product and the upper words of the
-// mixed ones are summed (2^-118 a term is left out).
-__global__ void __launch_bounds__(256) tsqr_gram_update_kernel(const GramWideArgs a, const int kb) {
+// mixed ones are summed (2^-118 a term is left out).  A thread an output: few tiles, so latency
+// counts (17 us a launch at 512 columns, 21 with four outputs a thread).
+__global__ void __launch_bounds__(1024) tsqr_gram_update_kernel(const GramWideArgs a, const int kb) {
     __shared__ long long lh[kBw][kBw], ll[kBw][kBw], ch[kBw][kBw], cl[kBw][kBw];
     if (*a.bad) return;
     const int n = a.p.n, k0 = kb * kBw, first = k0 + kBw;
@@ -171,8 +155,8 @@ __global__ void __launch_bounds__(256) tsqr_gram_update_kernel(const GramWideArg
     Q128 *C = reinterpret_cast<Q128 *>(a.C);
     const Q128 *P = reinterpret_cast<const Q128 *>(a.P);
     constexpr long long kMask = (1ll << 62) - 1;
-    for (int e = tid; e < kBw * kBw; e += 256) {
-        const int k = e / kBw, x = e % kBw;
+    {
+        const int k = tid / kBw, x = tid % kBw;
         const i128 l = i0 + x < n ? unpack(C[(int64_t)(k0 + k) * n + i0 + x]) : (i128)0;
         const i128 c = j0 + x < n ? unpack(P[(int64_t)k * n + j0 + x]) : (i128)0;
         lh[k][x] = (long long)(l >> 62);
@@ -182,25 +166,18 @@ __global__ void __launch_bounds__(256) tsqr_gram_update_kernel(const GramWideArg
     }
     __syncthreads();
     const int jx = tid & 31, iy = tid >> 5;
-    i128 hh[4] = {0, 0, 0, 0};
-    long long mm[4] = {0, 0, 0, 0};
-#pragma unroll 2
+    i128 hh = 0;
+    long long mm = 0;
+#pragma unroll 4
     for (int k = 0; k < kBw; ++k) {
-        const long long bh = ch[k][jx], bl = cl[k][jx];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const long long ah = lh[k][iy + 8 * u], al = ll[k][iy + 8 * u];
-            hh[u] += (i128)ah * bh;
-            mm[u] += __mul64hi(ah, bl) + __mul64hi(al, bh);
-        }
+        const long long ah = lh[k][iy], al = ll[k][iy], bh = ch[k][jx], bl = cl[k][jx];
+        hh += (i128)ah * bh;
+        mm += __mul64hi(ah, bl) + __mul64hi(al, bh);
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int i = i0 + iy + 8 * u, j = j0 + jx;
-        if (i <= j && j < n) {
-            Q128 *e = C + (int64_t)i * n + j;
-            *e = pack(unpack(*e) - (hh[u] * 4 + (i128)mm[u] * 16));
-        }
+    const int i = i0 + iy, j = j0 + jx;
+    if (i <= j && j < n) {
+        Q128 *e = C + (int64_t)i * n + j;
+        *e = pack(unpack(*e) - (hh * 4 + (i128)mm * 16));
     }
 }
 
@@ -213,23 +190,21 @@ __global__ void tsqr_gram_write_kernel(const GramWideArgs a) {
     const Q128 *C = reinterpret_cast<const Q128 *>(a.C), *d = reinterpret_cast<const Q128 *>(a.d);
     // a CTA writes tiles of 32 x 32 (rows of C in, columns of R out)
     __shared__ double t[kBw][kBw + 1];
+    __shared__ u64 sq[kBw];
     const int nb = (n + kBw - 1) / kBw;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int tile = blockIdx.x; tile < nb * nb; tile += gridDim.x) {
         const int i0 = tile / nb * kBw, j0 = tile % nb * kBw;
+        if (ty == 0) sq[tx] = i0 <= j0 && i0 + tx < n ? sqrt64((u128)unpack(d[i0 + tx])) : 0;
+        __syncthreads();
         for (int u = ty; u < kBw; u += 8) {
             const int i = i0 + u, j = j0 + tx;
             double v = 0.0;
             if (i <= j && j < n) {
-                const D2 s = sqrt2(to_double(unpack(d[i])));
-                if (i == j) {
-                    v = scalbn(s.hi + s.lo, a.g[j] - a.z[i]);
-                } else {
-                    // (a diagonal block's l are mirrored, see the panel kernel)
-                    const D2 x = to_double(unpack(i0 == j0 ? C[(int64_t)j * n + i] : C[(int64_t)i * n + j]));
-                    const double p = x.hi * s.hi;
-                    v = scalbn(p + (fma(x.hi, s.hi, -p) + (x.hi * s.lo + x.lo * s.hi)), a.g[j]);
-                }
+                // (a diagonal block's l are mirrored, see the panel kernel)
+                v = i == j ? round64(sq[u], a.g[j] - 64 - a.z[i], false)
+                           : r_entry(unpack(i0 == j0 ? C[(int64_t)j * n + i] : C[(int64_t)i * n + j]),
+                                     sq[u], a.g[j]);
             }
             t[u][tx] = v;
         }
@@ -253,12 +228,12 @@ int gram_wide_launch(const GramWideArgs &a, cudaStream_t stream) {
     launches += 2;
     for (int kb = 0; kb < nb; ++kb) {
         const int right = n - (kb + 1) * kBw;
-        const int ctas = right > 0 ? (right + 7) / 8 : 1;
-        tsqr_gram_panel_kernel<<<ctas < 1024 ? ctas : 1024, 256, 0, stream>>>(a, kb);
+        const int ctas = right > 0 ? (right + kGramThreads / 32 - 1) / (kGramThreads / 32) : 1;
+        tsqr_gram_panel_kernel<<<ctas < 1024 ? ctas : 1024, kGramThreads, 0, stream>>>(a, kb);
         ++launches;
         if (right <= 0) break;
         const int t = (right + kBw - 1) / kBw;
-        tsqr_gram_update_kernel<<<t * (t + 1) / 2, 256, 0, stream>>>(a, kb);
+        tsqr_gram_update_kernel<<<t * (t + 1) / 2, 1024, 0, stream>>>(a, kb);
         ++launches;
     }
     tsqr_gram_write_kernel<<<nb * nb < 1024 ? nb * nb : 1024, 256, 0, stream>>>(a);
