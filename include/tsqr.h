@@ -11,6 +11,11 @@
  * through tsqr_caqr_r, any width) run by panels of columns, each a reduction of its own
  * followed by an update of the columns right of it (Section 5).
  *
+ * FP64 calls on tall matrices take another form of the same reduction where it serves
+ * (TSQR_LEAF_GRAM): the row blocks' exact Gram matrices are summed along the tree, in whole
+ * numbers on the tensor cores, and the root factors the sum; the Householder leaves and tree
+ * stand behind it for the matrices it cannot serve, which is decided on the device.
+ *
  * Conventions shared by every entry point:
  *   - Matrices are column-major: element (i, j) of A is A[i + j*lda].
  *   - R is n x n, written in full: the upper triangle with diag(R) >= 0 (Section 2: R is unique
@@ -75,9 +80,9 @@ typedef enum { TSQR_PREC_F64 = 0, TSQR_PREC_MIXED = 1 } tsqr_prec_t;
  *         5's panel and update).  R equals one reduction's up to rounding.  With 16 columns (or
  *         0), up to TSQR_MAX_N columns and m >= max(256, 4 n), the exact sum of TSQR_LEAF_GRAM is
  *         tried first and the panels run only where it cannot serve.
- * AUTO picks HYBRID, or PANELS for FP64 R with n >= 56 and m >= 8 n, where it measured faster
- * (4,194,304 rows, n = 56 / 64 / 96 / 128: 775 / 828 / 863 / 887 against 727 / 750 / 555 / 586
- * GFLOP/s; at n = 48 one reduction is faster, 826 against 802).                           */
+ * AUTO picks HYBRID, or PANELS for FP64 R with n >= 56 and m >= 8 n, where its Householder form
+ * measured faster (4,194,304 rows, n = 56 / 64 / 96 / 128: 775 / 828 / 863 / 887 against 727 / 750 /
+ * 555 / 586 GFLOP/s; at n = 48 one reduction is faster, 826 against 802).                  */
 typedef enum {
     TSQR_TREE_AUTO = 0, TSQR_TREE_BINARY = 1, TSQR_TREE_FLAT = 2, TSQR_TREE_HYBRID = 3,
     TSQR_TREE_PANELS = 4
@@ -105,8 +110,9 @@ typedef enum {
  *         serve (a NaN or Inf, entries outside 2^-400 .. 2^400, a pivot below 2^-64 of its
  *         column's square: zero or dependent columns) is found on the device, and the
  *         Householder leaves and tree that the plan's other fields describe run instead: up to 32
- *         columns in the same launch, past that in the launches behind it.
- *   GRAM_Q tsqr_qr's form of GRAM, up to 32 columns: the root also inverts R (in 110-bit fixed
+ *         columns in the same launch, past that in the launches behind it.  R's entries are
+ *         within about half a last place, relative to their column, of the exact factor's.
+ * GRAM_Q: tsqr_qr's form of GRAM, up to 32 columns: the root also inverts R (in 110-bit fixed
  *         point) and Q = A R^-1 is formed on the tensor cores from A's and the inverse's digits,
  *         where its error bound is below 2^-47 (conditions up to some 100 to 1,000); past that
  *         the Householder reduction and its reflectors give R and Q.  In tsqr_r_ex: the R that
@@ -130,8 +136,8 @@ typedef struct {
                            in one sweep (the R factor of [R_1; ...; R_c], equal to a sequence of
                            binary operators by associativity, Section 2).  0 = as many as the
                            kernel's shared memory holds.                                     */
-    int32_t leaf;       /* tsqr_leaf_t (FP64: 0 or GRAM, whose plan is AUTO's whatever the other
-                           fields say).  With PANELS,
+    int32_t leaf;       /* tsqr_leaf_t (FP64: 0, GRAM or GRAM_Q, whose plans are AUTO's
+                           whatever the other fields say).  With PANELS,
                            tile_rows is the chunk height (256, 384, 512, 640, 768 or 1024) of a HYBRID
                            plan, warps is 8 (or 0).                                          */
 } tsqr_plan_t;
@@ -190,13 +196,16 @@ tsqr_status_t tsqr_qr_uppers(int64_t n, const double *R1, int64_t ld1, const dou
 /* Thin QR: Q (m x n, orthonormal columns) and R (n x n, diag(R) >= 0) with A = Q R, FP64.
  * Section 3 notes that the Q factor is obtained by applying the Householder transformations
  * of the reduction to the identity, which requires keeping every node's Householder vectors
- * and the shape of the tree.  This call does that: the factorization is tsqr_r's (same plan,
- * same kernels, the same R bit for bit; with the AUTO plan, except at widths where tsqr_r's
- * plan runs a number of bulk warps other than 4, 8 or 12, or chunks too tall for the Q passes'
- * buffers, which take the four-warp plan instead: tsqr_last_plan reports the plan used) with
- * the reflectors of every leaf chunk and tree node
- * kept, then Q = H [I_n; 0] (with the sign convention applied to Q's columns) is formed top-down
- * through the tree and backwards through each leaf's chunks.  Q is unique for A of full rank
+ * and the shape of the tree.  With an explicit plan, past 32 columns, or where the matrix asks for
+ * it, this call does that: the factorization is tsqr_r's Householder form (same plan, kernels and
+ * R bit for bit; widths whose plan runs a number of bulk warps other than 4, 8 or 12, or chunks
+ * too tall for the Q passes' buffers, take the four-warp plan) with the reflectors of every leaf
+ * chunk and tree node kept, then Q = H [I_n; 0] (with the sign convention applied to Q's columns)
+ * is formed top-down through the tree and backwards through each leaf's chunks.  Up to 32 columns
+ * (AUTO, m >= max(256, 4 n)) R comes from the exact Gram sum and Q = A R^-1 from digit products on
+ * the tensor cores, in the same launches, where that leaves Q orthonormal to working accuracy
+ * (TSQR_LEAF_GRAM_Q: conditions up to some 100 to 1,000).  tsqr_last_plan reports the plan used;
+ * tsqr_r_ex with it gives the same R bit for bit.  Q is unique for A of full rank
  * (as R is); with Householder reflectors it is then orthonormal to working accuracy however
  * ill-conditioned A is.  For rank-deficient A (a zero on R's diagonal) A = Q R still holds,
  * but the columns of Q beyond the rank are not guaranteed orthonormal: each leaf's first chunk
@@ -215,7 +224,7 @@ tsqr_status_t tsqr_qr_uppers(int64_t n, const double *R1, int64_t ld1, const dou
  * columns in groups and the tails go to workspace instead of Q.  Workspace: about (2 + arity)
  * n^2 doubles per tree node plus 2n per chunk, plus m x n when grouped, from the per-stream
  * pool.  Launches: the factorization, one per tree level below the root, and one leaf pass per
- * column group. */
+ * column group (up to 32 columns the same ones, which return at once where Q = A R^-1 serves). */
 tsqr_status_t tsqr_qr(const double *A, int64_t m, int64_t n, int64_t lda, double *Q,
                       int64_t ldq, double *R, int64_t ldr, const tsqr_plan_t *plan,
                       tsqr_stream_t stream);
@@ -232,10 +241,12 @@ tsqr_status_t tsqr_qr(const double *A, int64_t m, int64_t n, int64_t lda, double
  *   R : device n x n (ldr >= n) receiving R, or NULL.
  *   plan as for tsqr_qr (NULL = AUTO).
  * With few right-hand sides (k <= max(1, n / 4) and n + k <= TSQR_MAX_N) the augmented matrix
- * [A | B] is factorized instead (its R holds R and (Q^T B)(0:n, :) side by side) and one
- * triangular solve follows; R then equals tsqr_r's up to rounding.  Otherwise the columns of B
+ * [A | B] is factorized instead (its R holds R and (Q^T B)(0:n, :) side by side; with the AUTO
+ * plan by the exact Gram sum of [A | B], read where they are, and by the Householder reduction
+ * of a copy where that cannot serve) and one triangular solve follows; R then equals tsqr_r's
+ * up to rounding.  Otherwise the columns of B
  * go k_g = min(k, n) at a time (two launches per group after the factorization) and R is
- * tsqr_qr's bit for bit (tsqr_r's under the plan tsqr_last_plan reports).
+ * tsqr_r_ex's bit for bit under the plan tsqr_last_plan reports (a Householder one).
  * Above TSQR_MAX_N columns (AUTO plan only) [A | B] is copied to a buffer allocated for the
  * call (stream-ordered, m (n + k) doubles, plus (n + k)^2 for its R) and factorized by panels
  * as tsqr_caqr_r does; its R holds R and (Q^T B)(0:n, :) side by side, then one triangular
@@ -262,7 +273,9 @@ tsqr_status_t tsqr_lstsq(const double *A, int64_t m, int64_t n, int64_t lda, con
  * matrix (the rows' order does not change R).  Workspace: the matrix right of the first panel
  * with those rows added (about 8 (m + (n / panel) (L - 1) panel) n bytes), the panel's stored
  * reflectors (8 m panel bytes) and small tree buffers, from the per-stream pool.  Launches:
- * three per panel (the factorization, its chunks' compact WY factors and the update; two where
+ * (the exact Gram sum, AUTO plan and panel width, up to 2,048 columns and m >= max(256, 4 n): the
+ * sum, and past 128 columns two per 32 columns and three more for its factor, after which the
+ * panels' launches return at once unless it could not serve;) three per panel (the factorization, its chunks' compact WY factors and the update; two where
  * the blocked update does not fit) except the last (the factorization alone).  Returns
  * TSQR_ERR_INVALID_ARG for bad sizes, TSQR_ERR_UNSUPPORTED for a panel above TSQR_MAX_N or a
  * plan tsqr_qr would refuse, TSQR_ERR_ALLOC when the workspace cannot be had. */
@@ -271,7 +284,7 @@ tsqr_status_t tsqr_caqr_r(const double *A, int64_t m, int64_t n, int64_t lda, do
                           tsqr_stream_t stream);
 
 /* Varlen batch of independent problems: R_i = R factor of A_i for i < count, each the TSQR of
- * Section 2 (steps 1 and 2) with its own leaves and tree, all in one persistent launch.
+ * Section 2 (steps 1 and 2) with its own leaves and tree, all from one queue.
  *   ptrs    : host array of `count` device pointers; A_i is column-major m_i x n_i with
  *             lda_i = m_i (e.g. all pointing into one packed buffer).
  *   ms, ns  : host arrays of count rows (>= 0) and columns (1..TSQR_MAX_N).
@@ -279,8 +292,10 @@ tsqr_status_t tsqr_caqr_r(const double *A, int64_t m, int64_t n, int64_t lda, do
  *             offsets[i+1] - offsets[i] >= n_i^2; R_i is written column-major with ld n_i at
  *             R_packed + offsets[i].
  *   R_packed: device FP64 buffer of at least offsets[count] elements.
- *   dtype, prec as for tsqr_r_ex.  All problems are factorized by one launch: FP64 and wider
- *   mixed batches by the fold leaf, mixed batches up to 112 columns by the blocked
+ *   dtype, prec as for tsqr_r_ex.  All problems are factorized by one persistent launch.  With the
+ *   AUTO knobs an FP64 batch runs two: the exact Gram sums of the problems they serve
+ *   (TSQR_LEAF_GRAM: m_i >= max(256, 4 n_i)), then the fold leaf for the others and for those
+ *   found not to be served.  FP64 batches with explicit knobs and wider mixed batches run the fold leaf, mixed batches up to 112 columns by the blocked
  *   tensor-core leaf of TSQR_LEAF_PANELS (see tsqr_batch_plan_t's leaf).                    */
 tsqr_status_t tsqr_r_batched(const void *const *ptrs, const int64_t *ms, const int32_t *ns,
                              const int64_t *offsets, int32_t count, double *R_packed,
@@ -298,7 +313,8 @@ tsqr_status_t tsqr_r_batched(const void *const *ptrs, const int64_t *ms, const i
  *   arity[b]       : tree arity of the problems in width bucket b (n <= 8, <= 16, <= 32,
  *                    > 32), 2 .. 8, lowered to what the width's shared memory holds (0: the
  *                    largest that fits).
- *   leaf           : mixed precision only, a tsqr_leaf_t: FOLD, or PANELS (the blocked
+ *   leaf           : FP64: 0, or GRAM (the two launches of AUTO, the other knobs being the fold
+ *                    leaf's).  Mixed precision: FOLD, or PANELS (the blocked
  *                    tensor-core leaf of tsqr_r_ex, for batches up to 112 columns; chunks as
  *                    tall as the widest problem allows, 8 warps, one CTA per SM, so warps and
  *                    ctas_per_sm do not apply).  0: PANELS up to 112 columns, else FOLD.
@@ -351,11 +367,10 @@ tsqr_status_t tsqr_last_batch_plan(tsqr_batch_plan_t *out);
  * loop that must not allocate after start-up, or a process whose framework has already
  * reserved the device's memory for its own caching allocator.  The paper has no counterpart;
  * this is a deployment variant of tsqr_r.
- *   Same arguments as tsqr_r (FP64).  It always runs ONE reduction with the AUTO plan's
- *   one-reduction partition (tsqr_resolve_plan's plan, or the tuned plan of the bucket): where
- *   tsqr_r's AUTO plan runs by panels (n >= 56, m >= 8 n), this call does not, and its R equals
- *   tsqr_r's within the parity tolerance, not bit for bit; elsewhere the plan, kernel and R are
- *   tsqr_r's.  Instead of the per-stream workspace it uses one static device array of
+ *   Same arguments as tsqr_r (FP64).  It always runs ONE Householder reduction (the HYBRID plan
+ *   that tsqr_last_plan reports, or the tuned plan of the bucket), never the exact Gram sum or the
+ *   panels: its R equals tsqr_r's within the parity tolerance, not bit for bit.  Instead of the
+ *   per-stream workspace it uses one static device array of
  *   TSQR_NOALLOC_SCRATCH_BYTES that every GPU loading the library holds until the process
  *   exits.  It calls no cudaMalloc, cudaFree or other allocating routine.
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress)
@@ -382,7 +397,7 @@ tsqr_status_t tsqr_r_noalloc(const double *A, int64_t m, int64_t n, int64_t lda,
  * MPI library (Section 1).
  *   A, m, n, lda, dtype, prec, R, ldr as for tsqr_r_ex; R is overwritten (the last candidate's
  *   result).  best: optional, receives the chosen plan.
- *   Candidates: HYBRID slabs as tall as fit 1, 2 or 3 CTAs per SM, and half as tall, with that
+ *   Candidates: for FP64 the GRAM leaf; HYBRID slabs as tall as fit 1, 2 or 3 CTAs per SM, and half as tall, with that
  *   many CTAs per SM on every SM; 4, 5, 6, 8 or 12 bulk warps; for FP64 from n = 48 (m >= 8 n) the
  *   PANELS tree with 16- and 32-column panels; for the mixed path up to n = 112 the blocked
  *   leaf with every chunk height (256 to 1024 rows) the width's shared and tensor memory hold,

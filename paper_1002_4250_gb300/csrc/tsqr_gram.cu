@@ -24,6 +24,13 @@ __device__ __noinline__ void fold_store_job(const F64Args &f, const int leaf) {
     leaf_tree_job<double, double, 2, 1, false, true>(f, f.A, f.ldS, f.ldS * f.n, leaf);
 }
 
+// What bounds it: shared memory.  A 128-row round at 32 columns moves some 275 KB through it (A in
+// and out 64, its digits 64, the products' operands 147), 2.15k of the 3.2k cycles a round takes;
+// cutting alone is 1.2k, the products 0.8k.  Then the flush of every 1,024 rows' sums (7k cycles).
+// The Householder leaves it stands before are bound by FP64 arithmetic.  us: 4,194,304 x 32 10,103
+// before, 486 now (HBM's share 161); 16,777,216 x 8 2,697 / 399 (161); 10,000 x 16 198 / 38.9,
+// latency: the sums 14k cycles, the tree 9k, the root 25k.
+//
 // One FP64 matrix of at most 32 columns in one launch: CTA c sums slab c, the root factors, every
 // CTA waits for its verdict and runs its leaf of the Householder reduction where the Gram cannot
 // serve.  One CTA per SM, launched cooperatively.
@@ -73,7 +80,11 @@ tsqr_gram_f64_kernel(const __grid_constant__ GramArgs a) {
 }
 
 // A queue of work items (sets of columns over slabs of rows) of one matrix or many: the CTA that
-// completes a matrix's last set factors it.
+// completes a matrix's last set factors it.  Bound by the two-block sets, 3.9k cycles a 64-row round:
+// the digits of 64 columns 1.4k, 64 KB of operands read for each of eight products, the flush 0.9k
+// a round (one accumulator set, so every 1,024 rows).  us, Householder / here: 4,194,304 x 128 154,700 /
+// 7,210; 1,000,000 x 50 with an odd leading dimension (8-byte copies) 6,650 / 660; 512 problems 27,300
+// / 1,470.
 __global__ void __launch_bounds__(kGramThreads, 1)
 tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
     extern __shared__ __align__(1024) double smem_d[];
