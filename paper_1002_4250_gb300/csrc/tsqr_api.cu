@@ -756,8 +756,8 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
 
 // tsqr_qr's plan: the Gram factor and Q = A R^-1 where AUTO can take them (one column block; the
 // plan's other fields are those of the reflectors that stand behind it), else plan_store's.
-// ms, against plan_store's: 4,194,304 x 32 1.14 / 24.4, 16,777,216 x 8 1.04 / 7.76, 100,003 x 32
-// 0.144 / 1.66, 10,000 x 16 0.069 / 0.38, 3,000 x 5 0.046 / 0.22.  A matrix left to the reflectors
+// ms, against plan_store's: 4,194,304 x 32 1.02 / 24.4, 16,777,216 x 8 0.92 / 7.76, 100,003 x 32
+// 0.123 / 1.66, 10,000 x 16 0.064 / 0.38, 3,000 x 5 0.046 / 0.22.  A matrix left to the reflectors
 // pays for the sum: 4,194,304 x 32 24.65 / 24.36, and up to 16 columns for the 12-warp chunks the
 // single launch folds in (1,000,000 x 16 2.25 / 1.88).
 tsqr_status_t plan_qr(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {

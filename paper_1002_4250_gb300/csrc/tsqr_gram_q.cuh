@@ -8,11 +8,13 @@
 // 14, is below 2^-62 of the largest product.
 //
 // A tile is 32 KB in and 32 KB out (320 us of copy rate at 4,194,304 x 32) against some 25
-// instructions an entry to cut it and 45 to put its eight sums together and round them to FP64,
-// in integers: the chip's FP64 units would take longer than the tile's memory traffic.  Measured
-// 630 us there (with the sums in 64-bit multiply-adds and a 64-bit leading-zero count, 840 us);
-// the reflectors' passes, bound by FP64, took 14 ms.  One 128-row tile whatever the width took
-// 2.4 ms at 16,777,216 x 8, four side by side take 0.6 ms.
+// instructions an entry to cut it and 40 to put its eight sums together and round them to FP64,
+// in integers: the chip's FP64 units would take longer than the tile's memory traffic.  The shift
+// and logic unit bounds it (63% busy when the pass took 630 us), so sums and shifts that a
+// multiply-add can do go there, and whole tiles go without bounds checks: 530 us (840 with the
+// sums in 64-bit multiply-adds and a 64-bit leading-zero count).  The reflectors' passes, bound by
+// FP64, took 14 ms.  One 128-row tile whatever the width took 2.4 ms at 16,777,216 x 8, four side
+// by side take 0.5 ms.
 #pragma once
 
 #include "tsqr_gram_dev.cuh"
@@ -28,27 +30,40 @@ constexpr size_t kQSmem = kQHead + kQInverse + 2 * kQStage;
 
 struct alignas(16) QSmem {
     uint64_t full[2], done[2];
-    uint32_t tmem;
+    uint32_t tmem, p8;
     int D[kGramMaxN], F[kGramMaxN];
 };
 static_assert(sizeof(QSmem) <= kQHead, "the operands start at a multiple of 1,024 bytes");
 
-// Four accumulators of weights 256^3 .. 1 as a 64-bit number times 2^16.  (f + 1.5 2^23: f, a
-// whole number below 2^22, in the low bits; two of them fit 32.)
-__device__ __forceinline__ long long word4(const float f0, const float f1, const float f2,
-                                           const float f3) {
-    constexpr float kMagic = 12582912.0f;
-    constexpr uint32_t kBits = 0x4B400000u, kBias = (kBits << 8) + kBits;
-    const uint32_t a = (__float_as_uint(f0 + kMagic) << 8) + __float_as_uint(f1 + kMagic) - kBias;
-    const uint32_t b = (__float_as_uint(f2 + kMagic) << 8) + __float_as_uint(f3 + kMagic) - kBias;
-    const long long lo = (long long)(int)b * 65536;
-    return (long long)(((u64)(a + (uint32_t)((u64)lo >> 32)) << 32) | (uint32_t)lo);
+// Multipliers the compiler must not see as shifts: the unit that shifts and adds is the busy one
+// (63% against the multiplier's 20), and a multiply-add does both.
+struct Powers {
+    uint32_t p8, p16, m20;  // 2^8, 2^16, -2^20
+};
+__device__ __forceinline__ uint32_t mad_u32(const uint32_t a, const uint32_t b, const uint32_t c) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
 }
-// (H 2^32 + L) 2^(e - 16), rounded to FP64 (H, L: word4's).  Integers throughout: the 96-bit sum
+// Four accumulators of weights 256^3 .. 1 as a 64-bit number times 2^16.  (f + 1.5 2^23: f, a
+// whole number below 2^22, in the low bits; two of them fit 32, with their offsets 32 unsigned.)
+__device__ __forceinline__ long long word4(const float f0, const float f1, const float f2,
+                                           const float f3, const Powers &c) {
+    constexpr float kMagic = 12582912.0f;
+    constexpr u64 kBits = 0x4B400000u, kBias = (kBits * 256 + kBits) & 0xffffffffu;
+    constexpr u64 kOff = 0 - (kBias << 32) - (kBias << 16);
+    const uint32_t a = mad_u32(__float_as_uint(f0 + kMagic), c.p8, __float_as_uint(f1 + kMagic));
+    const uint32_t b = mad_u32(__float_as_uint(f2 + kMagic), c.p8, __float_as_uint(f3 + kMagic));
+    const u64 hi = ((u64)(a + (uint32_t)(kOff >> 32)) << 32) | (uint32_t)kOff;
+    u64 r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(b), "r"(c.p16), "l"(hi));
+    return (long long)r;
+}
+// (H 2^32 + L) 2^(e - 16), rounded to FP64 (H, L: word4's; e20: e's place in the exponent field).  Integers throughout: the 96-bit sum
 // is shifted until its sign bit is the top one, cut to 64 bits and rounded to 53.  small: a sum
 // below 2^48, whose leading bits need another word.
-__device__ __forceinline__ double round_sum(const long long H, const long long L, const int e,
-                                            bool &small) {
+__device__ __forceinline__ double round_sum(const long long H, const long long L,
+                                            const uint32_t e20, const Powers &c, bool &small) {
     const long long hi = H + (L >> 32);  // 2^32 of it
     const uint32_t w2 = (uint32_t)((u64)hi >> 32), w1 = (uint32_t)hi, w0 = (uint32_t)L;
     const uint32_t s = (uint32_t)((int)w2 >> 31), x = w2 ^ s;
@@ -56,10 +71,12 @@ __device__ __forceinline__ double round_sum(const long long H, const long long L
     const int sh = __clz((int)x) - 1;
     const uint32_t t1 = __funnelshift_l(w1, w2, sh) ^ s, t0 = __funnelshift_l(w0, w1, sh) ^ s;
     const u64 m = ((((u64)t1 << 32) | t0) + 512) >> 10;  // 2^52 .. 2^53
-    const uint32_t top = (uint32_t)(m >> 32) + ((uint32_t)(e - sh) << 20);
+    const uint32_t top = mad_u32((uint32_t)sh, c.m20, (uint32_t)(m >> 32) + e20);
     return __hiloint2double((int)(top | (s & 0x80000000u)), (int)(uint32_t)m);
 }
-__device__ __noinline__ double round_small(const long long H, const long long L, const int e) {
+__device__ __noinline__ double round_small(const long long H, const long long L,
+                                            const uint32_t e20) {
+    const int e = (int)(e20 >> 20);
     // 64 bits and the sign hold the sum (in units of 2^-16)
     const u64 v = ((u64)H << 32) + (u64)L;
     const bool neg = H + (L >> 32) < 0;
@@ -88,6 +105,7 @@ __device__ __forceinline__ void q_rows(const GramQArgs &a, unsigned char *smem) 
             tc::mbar_init(&sm.done[b], 1);
         }
         tc::fence_mbar_init();
+        *(volatile uint32_t *)&sm.p8 = 256;
     }
     if (tid < kGramMaxN) {
         sm.D[tid] = a.form->D[tid];
@@ -151,17 +169,28 @@ __device__ __forceinline__ void q_rows(const GramQArgs &a, unsigned char *smem) 
         // the thread's row of 8 columns; lane of the operand and place of the columns in it
         const int lr = 32 * (warp & 3) + lane, place = warp >> 2;
         const int r = 128 * (place / groups) + lr, c0 = 8 * (place % groups);
-        int D[8], F[8];
+        Powers pw;
+        pw.p8 = *(volatile uint32_t *)&sm.p8;
+        pw.p16 = pw.p8 * pw.p8;
+        pw.m20 = 0u - pw.p16 * 16;
+        int D[8];
+        uint32_t F[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             D[e] = sm.D[c0 + e];
-            F[e] = 1023 + 52 - 1 + 42 - 16 - 79 + sm.F[c0 + e];
+            F[e] = (uint32_t)(1023 + 52 - 1 + 42 - 16 - 79 + sm.F[c0 + e]) << 20;
         }
+        const bool whole = c0 + 8 <= a.n;  // no column of the thread is missing
         double v[8];
         auto load = [&](const int64_t t) {
             const int64_t row = t * rows + r;
             const bool in = t < a.ntiles && row < a.m;
             const double *p = a.A + row + c0 * a.lda;
+            if (whole && (t + 1) * rows <= a.m) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = p[e * a.lda];
+                return;
+            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = in && c0 + e < a.n ? p[e * a.lda] : 0.0;
         };
@@ -182,16 +211,33 @@ __device__ __forceinline__ void q_rows(const GramQArgs &a, unsigned char *smem) 
                     for (int d = 0; d < 4; ++d) tc::tmem_ld8(at + 32 * (4 * g + d), f[d]);
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) half[g][e] = word4(f[0][e], f[1][e], f[2][e], f[3][e]);
+                    for (int e = 0; e < 8; ++e) half[g][e] = word4(f[0][e], f[1][e], f[2][e], f[3][e], pw);
                 }
                 const int64_t row = t * rows + r;
                 double *q = a.Q + row + c0 * a.ldq;
+                double x[8];
+                bool any = false;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     bool small;
-                    double x = round_sum(half[0][e], half[1][e], F[e], small);
-                    if (small) x = round_small(half[0][e], half[1][e], F[e]);
-                    if (row < a.m && c0 + e < a.n) q[e * a.ldq] = x;
+                    x[e] = round_sum(half[0][e], half[1][e], F[e], pw, small);
+                    any |= small;
+                }
+                if (any) {  // (seldom; which of them, again)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        bool small;
+                        round_sum(half[0][e], half[1][e], F[e], pw, small);
+                        if (small) x[e] = round_small(half[0][e], half[1][e], F[e]);
+                    }
+                }
+                if (whole && (t + 1) * rows <= a.m) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) q[e * a.ldq] = x[e];
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (row < a.m && c0 + e < a.n) q[e * a.ldq] = x[e];
                 }
             }
             tc::fence_before_sync();
