@@ -310,7 +310,7 @@ def bench_ours(args, world, rank, local):
                      "peak_note": "measured copy bandwidth; A is read once (the kernel's own bound "
                                   "is shared memory)",
                      "peak_measured": pk["hbm_gbs"], "frac_of_measured": roof["a_read_frac_of_hbm"]})
-    traffic_path = os.path.join(ROOT, "profiles", "tsqr_f64_kernel_traffic.json")
+    traffic_path = os.path.join(ROOT, "profiles", "tsqr_gram_f64_kernel_traffic.json")
     if os.path.exists(traffic_path):
         with open(traffic_path) as f:
             tr = json.load(f)
@@ -694,9 +694,12 @@ def bench_batched(dev, threads):
 
 # The sources the FP64 leaf + tree kernel's code comes from: its translation unit and the
 # device headers (the C-ABI header it also includes holds declarations only).
-KERNEL_SOURCES = ("paper_1002_4250_gb300/csrc/tsqr_f64.cu",
-                  "paper_1002_4250_gb300/csrc/tsqr_f64.cuh",
+KERNEL_SOURCES = ("paper_1002_4250_gb300/csrc/tsqr_gram.cu",
+                  "paper_1002_4250_gb300/csrc/tsqr_gram.cuh",
+                  "paper_1002_4250_gb300/csrc/tsqr_gram_dev.cuh",
+                  "paper_1002_4250_gb300/csrc/tsqr_tc.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_fold.cuh",
+                  "paper_1002_4250_gb300/csrc/tsqr_f64.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_internal.h")
 
 
