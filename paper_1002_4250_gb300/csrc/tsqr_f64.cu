@@ -110,7 +110,9 @@ cudaError_t zero_lower_launch(double *R, int64_t ldr, int n, const unsigned int 
 cudaError_t copy_cols_launch(const double *src, int64_t lds, double *dst, int64_t ldd, int64_t m,
                              int n, const unsigned int *skip, cudaStream_t stream) {
     const int64_t blocks = (m + 1023) / 1024;
-    const dim3 grid((unsigned)(blocks < 128 ? blocks : 128), (unsigned)(n < 64 ? n : 64));
+    // two waves of CTAs, not a CTA for every column: mostly there is nothing to copy, and 4,096 CTAs
+    // take 7 us to find that out
+    const dim3 grid((unsigned)(blocks < 152 ? blocks : 152), (unsigned)(n < 4 ? n : 4));
     tsqr_copy_cols_kernel<<<grid, 1024, 0, stream>>>(src, lds, dst, ldd, m, n, skip);
     return cudaGetLastError();
 }
