@@ -1092,8 +1092,17 @@ __device__ __forceinline__ void cta_begin(Cta &c, unsigned char *smem) {
     c.tmem = c.sm->tmem;
     c.ok = true;
 }
+// (The barriers' lives end too: what follows in the same launch, the Householder reduction, takes the
+// memory they stand in.  A CTA barrier stands between this and that.)
 __device__ __forceinline__ void cta_end(const Cta &c) {
     __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_inval(&c.sm->full[b]);
+            tc::mbar_inval(&c.sm->free[b]);
+        }
+        tc::mbar_inval(&c.sm->drain);
+    }
     if (threadIdx.x >> 5 == kGramSlicers) {
         tc::tmem_relinquish();
         tc::tmem_dealloc(c.tmem, 512);

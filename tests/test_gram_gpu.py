@@ -412,3 +412,32 @@ def test_batch_repeated_after_another_call(T, dtype):
     s.synchronize()
     for R in (second, third, fourth):
         assert torch.equal(first, R)
+
+
+@pytest.mark.parametrize("n", [7, 32, 40, 64])
+def test_hand_over_under_capture(T, n):
+    """A captured call whose replays are served and handed over in turn (the Householder reduction
+    takes the shared memory that the sum's barriers stood in): each replay gives the direct call's
+    bytes."""
+    import torch
+    m = 30011
+    good = workloads.gaussian(m, n, seed=860 + n).cuda()
+    zero, repeated = good.clone(), good.clone()
+    zero[n // 2] = 0.0
+    repeated[n - 1] = repeated[0]
+    ref = [T.tsqr_r(A.T).clone() for A in (good, zero, repeated)]
+    buf, out = good.clone(), T.empty_r(n, "cuda")
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        T.tsqr_r(buf.T, R=out)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        T.tsqr_r(buf.T, R=out, stream=s)
+    for k in (0, 1, 0, 2, 1, 2, 0):
+        buf.copy_((good, zero, repeated)[k])
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref[k]), k
+    assert T.tsqr_get_device_status() == T.SUCCESS
