@@ -90,9 +90,11 @@ __global__ void __launch_bounds__(kGramThreads) tsqr_gram_panel_kernel(const Gra
     __shared__ Q128 L[kBw * (kBw + 1) / 2], rowv[3 * kBw];
     __shared__ u64 rec[kBw];
     __shared__ int zs[kBw], low;
-    if (*a.bad) return;
     const int n = a.p.n, k0 = kb * kBw, w = min(kBw, n - k0);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // one thread's read decides for the CTA: another CTA of this launch may be setting the word, and
+    // threads that saw it would be missing from the barriers of those that did not
+    if (__syncthreads_or(tid == 0 && __ldcg(a.bad) != 0)) return;
     constexpr int kWarps = kGramThreads / 32;
     Q128 *C = reinterpret_cast<Q128 *>(a.C), *P = reinterpret_cast<Q128 *>(a.P);
     for (int o = tid; o < w * w; o += kGramThreads) {

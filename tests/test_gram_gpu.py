@@ -441,3 +441,25 @@ def test_hand_over_under_capture(T, n):
         torch.cuda.synchronize()
         assert torch.equal(out, ref[k]), k
     assert T.tsqr_get_device_status() == T.SUCCESS
+
+
+def test_wide_handed_over_on_streams(oracle, T):
+    """A dependent column in the first block row of the wide factor, found by every CTA of that
+    launch, with other calls of the kind on two more streams (CTAs start late): the same bytes each
+    time, and A's Gram."""
+    import torch
+    m, n = 3000, 700
+    At = workloads.gaussian(m, n, seed=78)
+    At[9] = At[4]
+    Ad = At.cuda().T
+    ref = T.tsqr_caqr_r(Ad).clone()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = []
+    for st in streams * 3:
+        st.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(st):
+            outs.append(T.tsqr_caqr_r(Ad))
+    torch.cuda.synchronize()
+    for R in outs:
+        assert torch.equal(R, ref)
+    assert oracle.gram_residual(oracle.from_torch_colmajor(At), ref.cpu().numpy(), nthreads=16) <= 1e-13
