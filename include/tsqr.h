@@ -107,8 +107,9 @@ typedef enum {
  *         (exact: whole numbers below 2^24 in FP32 accumulators), put together in 128-bit
  *         integers, added over the row blocks, and the sum is factored in 122-bit fixed point.
  *         m >= 256, m >= 4 n; n < 56 here, wider through the PANELS tree.  A matrix it cannot
- *         serve (a NaN or Inf, entries outside 2^-400 .. 2^400, a pivot below 2^-64 of its
- *         column's square: zero or dependent columns) is found on the device, and the
+ *         serve (a NaN or Inf, a column whose largest entry is outside some 2^-400 .. 2^400, a
+ *         pivot below 2^-64 of its column's square: zero or dependent columns) is found on the
+ *         device, and the
  *         Householder leaves and tree that the plan's other fields describe run instead: up to 32
  *         columns in the same launch, past that in the launches behind it.  R's entries are
  *         within about half a last place, relative to their column, of the exact factor's.

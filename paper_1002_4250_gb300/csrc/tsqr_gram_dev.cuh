@@ -21,8 +21,11 @@ constexpr int kBlock = 32;       // columns of a block
 // The least pivot a column may keep, relative to its square (2^-kPivotBits).
 constexpr int kPivotBits = 64;
 // Biased exponents a column's largest entry may have: outside, squares leave FP64's range (or
-// come near it) and the Householder reduction decides what R is.
+// come near it) and the Householder reduction decides what R is.  A slab's exponent word goes no
+// lower than kLeastD, whatever its entries; a column that is there in every slab has lost digits
+// (2^-430: half of them), or is zero, and is not served.
 constexpr int kExpLo = 1023 - 400, kExpHi = 1023 + 400;
+constexpr int kLeastD = kExpLo + 4;
 constexpr int kUnit = -1086;     // |x| = Q 2^(D + kUnit) for a column's exponent word D
 
 constexpr int cmin(int a, int b) { return a < b ? a : b; }
@@ -301,7 +304,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             const int e = sm.E[tid];
             if (e > kExpHi) sm.bad = 1;
             up = e + 2 > sm.D[tid];
-            sm.Dnew[tid] = up ? max(e, kExpLo) + 4 : sm.D[tid];
+            sm.Dnew[tid] = up ? max(e + 4, kLeastD) : sm.D[tid];
             sm.E[tid] = 0;
         }
         return __syncthreads_or(up) != 0;
@@ -1028,6 +1031,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
             d = max(d, __ldcg(reinterpret_cast<const int *>(top(s)) + (o < b ? 64 : 0) + l));
         }
         sm.D[tid] = d;
+        if (d <= kLeastD) sm.bad = 1;
     }
     __syncthreads();
     if (sm.bad) return false;

@@ -53,7 +53,7 @@ __global__ void tsqr_gram_scale_kernel(const GramWideArgs a) {
     const int e = g > 0 ? (122 - len) >> 1 : 0;
     a.E[j] = e;
     a.g[j] = 73 - e + d + kUnit;
-    if (bad || !(g > 0)) *a.bad = 1;
+    if (bad || d <= kLeastD || !(g > 0)) *a.bad = 1;
 }
 
 __global__ void tsqr_gram_fill_kernel(const GramWideArgs a) {

@@ -463,3 +463,54 @@ def test_wide_handed_over_on_streams(oracle, T):
     for R in outs:
         assert torch.equal(R, ref)
     assert oracle.gram_residual(oracle.from_torch_colmajor(At), ref.cpu().numpy(), nthreads=16) <= 1e-13
+
+
+@pytest.mark.parametrize("p", [-396, -405, -430, -460])
+@pytest.mark.parametrize("which", ["one", "all"])
+@pytest.mark.parametrize("call,m,n", [("r", 4096, 4), ("r", 20011, 32), ("r", 20011, 40),
+                                      ("r", 20011, 100), ("host", 9001, 12), ("qr", 20011, 16),
+                                      ("caqr", 6007, 180), ("lstsq", 20011, 20), ("batch", 4096, 33)])
+def test_columns_of_small_scale(oracle, T, call, m, n, which, p):
+    """Columns whose largest entry is at 2^p, about the least the fixed point serves (2^-400) and
+    below: column j of R scales with column j of A exactly, so R scaled back meets the unscaled
+    matrix's bounds, whichever reduction gave it."""
+    import torch
+    At = workloads.gaussian(m, n, seed=900 + n)
+    e = torch.zeros(n, dtype=torch.float64)
+    if which == "one":
+        e[n // 2] = p
+    else:
+        e[:] = p
+    S = torch.exp2(e)
+    As = (At * S[:, None]).contiguous()
+    T.tsqr_get_device_status()
+    if call == "r":
+        R = T.tsqr_r(As.cuda().T)
+    elif call == "host":
+        R = T.tsqr_r_host(As.pin_memory().T)
+        torch.cuda.synchronize()
+    elif call == "caqr":
+        R = T.tsqr_caqr_r(As.cuda().T)
+    elif call == "qr":
+        Q, R = T.tsqr_qr(As.cuda().T)
+        Qh = Q.cpu().numpy()
+        assert np.abs(Qh.T @ Qh - np.eye(n)).max() <= 50 * U
+    elif call == "lstsq":
+        Bt = workloads.gaussian(m, 2, seed=5)  # the second right-hand side of the columns' scale
+        X, R = T.tsqr_lstsq(As.cuda().T, (Bt * torch.exp2(
+            torch.tensor([0.0, p], dtype=torch.float64))[:, None]).cuda().T)
+        A, B = oracle.from_torch_colmajor(At), oracle.from_torch_colmajor(Bt)
+        Xo = oracle.lstsq(A, B, nthreads=16)
+        Xh = X.cpu().numpy() * S.numpy()[:, None] * np.exp2([0.0, -p])
+        kap = oracle.kappa_from_r(oracle.householder_r(A, nthreads=16))
+        tol = 2.0 * np.sqrt(m) * (kap + kap ** 2 * np.linalg.norm(B - A @ Xo) /
+                                  (np.linalg.norm(A, 2) * np.linalg.norm(Xo))) * U
+        assert np.linalg.norm(Xh - Xo) <= tol * np.linalg.norm(Xo)
+    else:
+        buf = torch.cat([workloads.gaussian(m, n, seed=1).reshape(-1), As.reshape(-1)]).cuda()
+        out = torch.empty(2 * n * n, dtype=torch.float64, device="cuda")
+        T.tsqr_r_batched([buf.data_ptr(), buf.data_ptr() + 8 * m * n], [m, m], [n, n],
+                         [0, n * n, 2 * n * n], out)
+        R = out[n * n:].view(n, n).T
+    assert T.tsqr_get_device_status() == T.SUCCESS
+    _check(oracle, R.cpu() * torch.exp2(-e)[None, :], At)
