@@ -522,11 +522,18 @@ tsqr_status_t zero_r(double *R, int64_t n, int64_t ldr, cudaStream_t stream) {
     return TSQR_SUCCESS;
 }
 
+// Slabs of the Gram sum at most: about five items a CTA (the last wave stays short; an item's fixed
+// cost, its pipeline's start, the flush and the climb, is some 7 us).  One set: a slab a CTA.
+int64_t gram_max_slabs(int64_t n, int sms) {
+    const int nset = gram_sets((int)((n + 31) / 32));
+    return std::max<int64_t>(1, nset == 1 ? sms : 5LL * sms / nset);
+}
 // The exact-Gram reduction (tsqr_gram.cuh) serves tall matrices up to 2,048 columns (the fixed-
-// point matrix is then 64 MB).
+// point matrix is then 64 MB), whose slabs are no longer than its sums hold.
 constexpr int64_t kGramMinRows = 256, kGramMaxCols = 2048;
 bool gram_fits(int64_t m, int64_t n) {
-    return n >= 1 && n <= kGramMaxCols && m >= kGramMinRows && m >= 4 * n;
+    if (n < 1 || n > kGramMaxCols || m < kGramMinRows || m < 4 * n) return false;
+    return m <= kGramSlabRows || m / gram_max_slabs(n, current_sms()) + 64 <= kGramSlabRows;
 }
 constexpr int kPanelsMinN = 56;
 
@@ -590,16 +597,13 @@ struct GramLayout {
     int nb = 0, nset = 0, nslab = 0, inner = 0;
     size_t words = 0, cnt_bytes = 0, wide_off = 0, bytes = 0;
 };
-// Slabs: about five items a CTA (the last wave stays short; an item's fixed cost, its pipeline's
-// start, the flush and the climb, is some 7 us), of at least 512 rows.
-// One set: a slab a CTA.
+// Slabs of at least 512 rows.
 GramLayout gram_layout(int64_t m, int64_t n, int sms) {
     GramLayout w;
     w.nb = (int)((n + 31) / 32);
     w.nset = gram_sets(w.nb);
     const int64_t nkb = (m + 63) / 64;
-    w.nslab = (int)std::max<int64_t>(
-        1, std::min<int64_t>(w.nset == 1 ? sms : 5LL * sms / w.nset, nkb / 8));
+    w.nslab = (int)std::max<int64_t>(1, std::min<int64_t>(gram_max_slabs(n, sms), nkb / 8));
     w.inner = gram_inner_nodes(w.nslab, (int)n);
     w.words = 5 + (size_t)w.nset * w.inner;  // queue, failed, verdict, bad, then the nodes, sets done
     w.cnt_bytes = align_up(w.words * sizeof(unsigned int), 256);
@@ -632,6 +636,7 @@ tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_
     q.one.nb = w.nb;
     q.one.nslab = w.nslab;
     q.one.nkb = (m + 63) / 64;
+    q.one.guard = gram_guard(m);
     q.one.counters = head + 4;
     q.one.slots = (unsigned char *)base + w.cnt_bytes;
     q.one.verdict = head + 2;
@@ -705,6 +710,7 @@ GramArgs gram_args(const F64Plan &p, const RLayout &w, const F64Args &a, void *b
     g.p.nb = 1;
     g.p.nslab = p.gram_ctas;
     g.p.nkb = (a.m + 63) / 64;
+    g.p.guard = gram_guard(a.m);
     g.p.counters = a.counters + p.nodes;
     g.p.verdict = g.p.counters + gram_inner_nodes(p.gram_ctas, a.n) + 1;
     g.p.slots = (unsigned char *)base + w.gram_off;
@@ -1962,10 +1968,13 @@ void plan_gram_batch(const void *const *ptrs, const int64_t *ms, const int32_t *
         g.n = g.na = ns[i];
         g.nb = (ns[i] + 31) / 32;
         g.nkb = (ms[i] + 63) / 64;
+        g.guard = gram_guard(ms[i]);
         const int nset = gram_sets(g.nb);
         const double all = (double)g.nkb * ns[i] * g.nb;
         g.nslab = (int)std::max<double>(
-            1.0, std::min<double>(std::ceil(all / (nset * target)), (double)g.nkb / 8));
+            1.0, std::min<double>(std::max(std::ceil(all / (nset * target)),
+                                           std::ceil(g.nkb / (kGramSlabRows / 64.0 - 1.0))),
+                                  (double)g.nkb / 8));
         const int inner = gram_inner_nodes(g.nslab, g.n);
         g.counters = (unsigned int *)*words;
         *words += (size_t)nset * inner + 1;

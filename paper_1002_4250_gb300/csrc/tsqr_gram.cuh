@@ -36,6 +36,7 @@ struct GramProblem {
                            // (0, 2), (1, 2), (0, 3), ...
     int nslab;             // slabs of rows: slab s holds 64-row blocks [s nkb / nslab, ...)
     int64_t nkb;           // ceil(m / 64)
+    int guard;             // bits (an even number) by which a slab's sums are shifted down: gram_guard(m)
     unsigned int *counters;  // per set: the tree's inner nodes; then one for the sets; zeroed
     unsigned char *slots;    // per set: one slot per tree node
     unsigned int *verdict;   // 0: not decided; 1: R is written; 2: the Householder reduction runs
@@ -50,6 +51,16 @@ struct GramQForm {
     int D[kGramMaxN], F[kGramMaxN];
     long long w[kGramMaxN * kGramMaxN];  // (i, j) at 32 j + i
 };
+
+// A row adds less than 2^100 to a sum (entries below 2^62 units, products in units of 2^24), so a
+// slab of up to 2^26 rows stays within 127 bits.  More rows than that in all: the slabs' sums are
+// shifted down before they are added (far below the columns' own rounding: the sum is long).
+constexpr int64_t kGramSlabRows = (int64_t)1 << 26;
+__host__ __device__ inline int gram_guard(int64_t m) {
+    int g = 0;
+    while ((m >> g) > kGramSlabRows) g += 2;
+    return g;
+}
 
 struct GramArgs {          // tsqr_r's single launch: one problem of one column block
     GramProblem p;

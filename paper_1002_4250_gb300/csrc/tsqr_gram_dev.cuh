@@ -657,7 +657,7 @@ __device__ __noinline__ bool climb(const GramProblem &p, const Cols cols, const 
             decode(o, i, j);
             i128 g = unpack(c.U[i * NR + j]);
             if (NJ == 0 && i < j) g += unpack(c.U[j * NR + i]);
-            reinterpret_cast<Q128 *>(mine + kGramSlotHead)[o] = pack(g);
+            reinterpret_cast<Q128 *>(mine + kGramSlotHead)[o] = pack(g >> p.guard);
         }
     }
     int cnt = p.nslab, off = 0, t = slab, cidx = 0;
@@ -984,7 +984,7 @@ static __device__ __noinline__ void invert_root(const GramProblem &p, const Q128
         const u64 inv = __double2ull_rn(y * 0x1p62) + (u64)__double2ll_rn(dy * 0x1p62);
         const u128 ax = (u128)(x < 0 ? -x : x);
         const u128 v = (((u128)(u64)(ax >> 64) * inv) << 2) + (((u128)(u64)ax * inv) >> 62);
-        const int e = lane <= j ? sm.E[lane] : 0;
+        const int e = lane <= j ? sm.E[lane] - p.guard / 2 : 0;
         int F = v ? bits128(v) - 110 + e : -1000;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) F = max(F, __shfl_xor_sync(all, F, o));
@@ -1050,7 +1050,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
         const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d);
         sm.E[tid] = d > 0 ? (122 - len) >> 1 : 0;  // shift of the column
         if (!(d > 0)) sm.bad = 1;
-        sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + kUnit;
+        sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + kUnit + p.guard / 2;
     }
     __syncthreads();
     if (sm.bad) return false;

@@ -52,7 +52,7 @@ __global__ void tsqr_gram_scale_kernel(const GramWideArgs a) {
     const int len = gh ? 128 - __clzll((long long)gh) : 64 - __clzll((long long)(u64)g);
     const int e = g > 0 ? (122 - len) >> 1 : 0;
     a.E[j] = e;
-    a.g[j] = 73 - e + d + kUnit;
+    a.g[j] = 73 - e + d + kUnit + p.guard / 2;
     if (bad || d <= kLeastD || !(g > 0)) *a.bad = 1;
 }
 

@@ -514,3 +514,38 @@ def test_columns_of_small_scale(oracle, T, call, m, n, which, p):
         R = out[n * n:].view(n, n).T
     assert T.tsqr_get_device_status() == T.SUCCESS
     _check(oracle, R.cpu() * torch.exp2(-e)[None, :], At)
+
+
+@pytest.mark.parametrize("call", ["r", "qr", "lstsq", "batch"])
+def test_rows_past_what_128_bits_hold(T, call):
+    """402,653,184 rows of 1.75, every slab's first block (which sets the exponent) four times
+    smaller: the squares' sum is 1.15 2^128 in the units of a slab.  Two columns, the second with
+    signs in turn: orthogonal, so R is the norm times I, within c(m) u."""
+    import torch
+    m = 3 << 27
+    slabs = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    At = torch.full((2, m), 1.75, dtype=torch.float64, device="cuda")
+    first = torch.arange(slabs, device="cuda") * (m // 64) // slabs
+    At.view(2, m // 64, 64)[:, first] = 0.4375
+    At[1, 1::2] *= -1.0
+    norm = np.sqrt((m - 64 * slabs) * 1.75 ** 2 + 64 * slabs * 0.4375 ** 2)
+    tol = 2.0 * np.sqrt(m) * U
+    T.tsqr_get_device_status()
+    if call == "r":
+        R = T.tsqr_r(At.T)
+    elif call == "qr":
+        Q, R = T.tsqr_qr(At.T)
+        At *= 1.0 / norm
+        assert (Q.T - At).abs().max().item() <= tol / np.sqrt(m)
+    elif call == "lstsq":
+        B = At[1:].clone()
+        B[:, :m // 8] = At[0, :m // 8]  # an eighth of the first column's square, the rest orthogonal
+        X, R = T.tsqr_lstsq(At[:1].T, B.T)
+        assert abs(X.item() - 0.125) <= 4.0 * tol and abs(R.item() - norm) <= tol * norm
+        return
+    else:
+        R = torch.empty(4, dtype=torch.float64, device="cuda")
+        T.tsqr_r_batched([At.data_ptr()], [m], [2], [0, 4], R)
+        R = R.view(2, 2).T
+    assert T.tsqr_get_device_status() == T.SUCCESS
+    assert (R.cpu() - norm * torch.eye(2, dtype=torch.float64)).abs().max().item() <= tol * norm
