@@ -3,6 +3,7 @@
 // fixed-point Cholesky factor of the whole.
 #pragma once
 
+#include <climits>
 #include <type_traits>
 
 #include "tsqr_fold.cuh"
@@ -89,7 +90,7 @@ struct alignas(16) Smem {   // beside the stages
     uint64_t drain;         // all tensor-core work so far is done
     uint32_t tmem;
     int flag, bad, item;
-    int above;              // an entry was above its column's range
+    int above;              // the first round with an entry above its column's range
     int stop;               // the round that was not multiplied for it; -1: none
     int D[128], E[128], Dnew[128];
 };
@@ -337,7 +338,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             tc::mbar_inval(&sm.drain);
             tc::mbar_init(&sm.drain, 1);
             tc::fence_mbar_init();
-            *above = 0;
+            *above = INT_MAX;
             *stop = -1;
         }
         used[0] = used[1] = 0;
@@ -496,8 +497,9 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     // Rounds run without a CTA barrier: a warp slices its task of a round into the round's stage as
     // soon as the tensor cores are done with the round before the last (free), and the last warp,
     // which slices nothing, issues a round's products once all have arrived (full).  A warp that meets an entry
-    // above its column's range says so before it arrives; the last warp then issues nothing and
-    // sets the stop, which every wait watches, and the whole CTA takes that round block by block.
+    // above its column's range leaves the round's number before it arrives (the least one stays); the
+    // last warp then issues nothing for that round and sets the stop, which every wait watches, and
+    // the whole CTA takes that round block by block.
     restart_barriers();
 #pragma unroll 1
     for (int r = 0; r < Sh::kRaws; ++r) load_round(r);
@@ -520,7 +522,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             if (go) {
                 int dmin = 2;
                 if (mine) slice8(raw_of(r), sm.D[lc], dmin, dst + b * Sh::kStage, step);
-                if (__any_sync(0xffffffffu, dmin < 2) && lane == 0) *above = 1;
+                if (__any_sync(0xffffffffu, dmin < 2) && lane == 0) atomicMin(&sm.above, r);
                 tc::fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&sm.full[b]);
@@ -528,8 +530,10 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         } else {
             if (c.ok) c.ok = tc::mbar_wait(&sm.full[b], used[b] & 1, kPolls);
             __syncwarp();
-            // (one lane reads it for all: another warp may be saying so of the next round)
-            go = __shfl_sync(0xffffffffu, lane == 0 ? *above : 0, 0) == 0;
+            // (one lane reads it for all: another warp may be saying so of the next round, which
+            // is not this one's to stop for: where the rounds break off decides where the sums are
+            // cut, and has to follow from the data alone)
+            go = __shfl_sync(0xffffffffu, lane == 0 ? *above : 0, 0) > r;
             if (issuer) {
                 if (go) {
                     multiply(b, 0, Sh::kRoundKb);

@@ -549,3 +549,35 @@ def test_rows_past_what_128_bits_hold(T, call):
         R = R.view(2, 2).T
     assert T.tsqr_get_device_status() == T.SUCCESS
     assert (R.cpu() - norm * torch.eye(2, dtype=torch.float64)).abs().max().item() <= tol * norm
+
+
+@pytest.mark.parametrize("n", [8, 16, 24, 32, 40])
+def test_same_bytes_where_exponents_rise(T, n):
+    """One column whose peaks (2^6, 2^10, ...: its exponent rises twelve times in a slab, at other
+    places in each) break the rounds off, beside columns of condition 1e9, whose last pivots magnify
+    a difference in how their sums are cut: the same bytes on every run, alone and beside other
+    work."""
+    import torch
+    blocks = 300 if n > 8 else 700
+    m = 152 * 64 * blocks
+    g = torch.Generator(device="cuda").manual_seed(n)
+    V = torch.linalg.qr(torch.randn(n - 1, n - 1, dtype=torch.float64, device="cuda", generator=g))[0]
+    s = torch.logspace(0, -9, n - 1, dtype=torch.float64, device="cuda")
+    At = torch.randn(n, m, dtype=torch.float64, device="cuda", generator=g)
+    At[:-1] = (V * s) @ At[:-1]
+    gc = torch.Generator().manual_seed(n)
+    for slab in range(152):
+        peaks = torch.randperm(blocks - 20, generator=gc)[:12].sort().values + 10
+        At[-1, ((slab * blocks + peaks) * 64 + 11).cuda()] = torch.exp2(
+            6 + 4 * torch.arange(12, dtype=torch.float64)).cuda()
+    ref = T.tsqr_r(At.T).clone()
+    side, noise = torch.cuda.Stream(), torch.randn(2048, 2048, device="cuda")
+    outs = []
+    for k in range(60):
+        if k % 3 == 0:
+            with torch.cuda.stream(side):
+                noise = noise @ noise * 1e-3
+        outs.append(T.tsqr_r(At.T))
+    torch.cuda.synchronize()
+    assert sum(not torch.equal(R, ref) for R in outs) == 0
+    assert T.tsqr_get_device_status() == T.SUCCESS
