@@ -240,7 +240,7 @@ tsqr_status_t tsqr_qr(const double *A, int64_t m, int64_t n, int64_t lda, double
  *   B : device, column-major m x k, ldb >= m, k >= 0; read only.
  *   X : device, column-major n x k, ldx >= n.
  *   R : device n x n (ldr >= n) receiving R, or NULL.
- *   plan as for tsqr_qr (NULL = AUTO).
+ *   plan as for tsqr_qr (NULL = AUTO; a GRAM plan, as tsqr_r and this call report, is AUTO).
  * With few right-hand sides (k <= max(1, n / 4) and n + k <= TSQR_MAX_N) the augmented matrix
  * [A | B] is factorized instead (its R holds R and (Q^T B)(0:n, :) side by side; with the AUTO
  * plan by the exact Gram sum of [A | B], read where they are, and by the Householder reduction
@@ -268,7 +268,8 @@ tsqr_status_t tsqr_lstsq(const double *A, int64_t m, int64_t n, int64_t lda, con
  *   R     : device, column-major n x n, ldr >= n; the upper triangle with diag(R) >= 0, the
  *           strict lower triangle written as 0.  Must not overlap A.
  *   panel : panel width, 1 .. TSQR_MAX_N; 0 = 16 (or n if smaller).
- *   plan  : NULL = AUTO, else the plan used for every panel's factorization (as for tsqr_qr).
+ *   plan  : NULL = AUTO, else the plan used for every panel's factorization (as for tsqr_qr; a
+ *           GRAM plan, as reported for a matrix of one panel, is AUTO).
  * Each panel's update keeps every row of the panel's matrix and adds the n-row blocks its tree
  * nodes leave behind: a panel factorized on L leaves adds (L - 1) panel rows to the next
  * matrix (the rows' order does not change R).  Workspace: the matrix right of the first panel

@@ -294,6 +294,13 @@ bool plan_is_auto(const tsqr_plan_t *p) {
                   p->arity == 0 && p->leaf == 0);
 }
 
+// A plan that asks for the exact-Gram reduction: AUTO's, whatever its other fields (those of the
+// Householder reduction behind the sum) say.
+bool asks_gram(const tsqr_plan_t *p) {
+    return p && (p->leaf == TSQR_LEAF_GRAM || p->leaf == TSQR_LEAF_GRAM_Q) &&
+           (p->tree == TSQR_TREE_AUTO || p->tree == TSQR_TREE_HYBRID);
+}
+
 bool tuned_plan(int dev, int64_t m, int n, bool mixed, tsqr_plan_t *out) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(TuneKey{dev, n, mixed ? 1 : 0, floor_log2(std::max<int64_t>(m, 1))});
@@ -1143,6 +1150,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
                                   cudaStream_t stream) {
     const int64_t na = n + k;
     F64Plan p;
+    if (asks_gram(over) && gram_fits(m, na)) over = nullptr;
     tsqr_status_t st = plan_f64(m, (int)na, over, &p);
     if (st != TSQR_SUCCESS) return st;
     g_last_plan = public_plan(p);
@@ -1169,10 +1177,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
         st = enqueue_gram(gl, sms, A, lda, B, ldb, n, m, na, (char *)Ra + ra_bytes, Ra, na, ws->status,
                           &a.skip, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
-        if (na < kPanelsMinN)
-            g_last_plan.leaf = TSQR_LEAF_GRAM;
-        else
-            g_last_plan = tsqr_plan_t{TSQR_TREE_PANELS, kPanelsWidth, 0, 0, 0, 0};
+        g_last_plan.leaf = TSQR_LEAF_GRAM;
     }
     if (copy_cols_launch(A, lda, aug, m, m, (int)n, a.skip, stream) != cudaSuccess ||
         copy_cols_launch(B, ldb, aug + n * m, m, m, (int)k, a.skip, stream) != cudaSuccess ||
@@ -1477,6 +1482,7 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
     const DeviceInfo di = device_info(dev);
+    if (asks_gram(over)) over = nullptr;
     if (N <= nb && plan_is_auto(over) && gram_fits(m, N) && N < kPanelsMinN) {  // one panel: tsqr_r's reduction
         F64Plan p;
         tsqr_status_t st = plan_r(m, (int)N, over, &p);
@@ -2315,7 +2321,8 @@ tsqr_status_t tsqr_lstsq(const double *A, int64_t m, int64_t n, int64_t lda, con
         ldb < std::max<int64_t>(1, m) || ldx < n || (R && ldr < n))
         return TSQR_ERR_INVALID_ARG;
     if (!A || (k > 0 && (!B || !X))) return TSQR_ERR_INVALID_ARG;
-    if (plan && plan->warps % 4 != 0) return TSQR_ERR_INVALID_ARG;  // as for tsqr_qr
+    if (plan && !asks_gram(plan) && plan->warps % 4 != 0)
+        return TSQR_ERR_INVALID_ARG;  // as for tsqr_qr
     if (n > TSQR_MAX_N) {
         if (!plan_is_auto(plan) || n + k > 0x7fffffffLL) return TSQR_ERR_UNSUPPORTED;
         return run_lstsq_panels(A, m, n, lda, B, ldb, k, X, ldx, R, ldr, (cudaStream_t)stream);
@@ -2331,7 +2338,8 @@ tsqr_status_t tsqr_caqr_r(const double *A, int64_t m, int64_t n, int64_t lda, do
     if (bad_dims(m, n, lda, ldr) || n < 1 || m < n || panel < 0 || !A || !R)
         return TSQR_ERR_INVALID_ARG;
     if (panel > TSQR_MAX_N || n > 0x7fffffffLL) return TSQR_ERR_UNSUPPORTED;
-    if (plan && plan->warps % 4 != 0) return TSQR_ERR_INVALID_ARG;  // as for tsqr_qr
+    if (plan && !asks_gram(plan) && plan->warps % 4 != 0)
+        return TSQR_ERR_INVALID_ARG;  // as for tsqr_qr
     const int64_t nb = panel > 0 ? panel : std::min<int64_t>(n, kCaqrPanel);
     return run_caqr(A, m, n, lda, R, ldr, nb, plan, (cudaStream_t)stream);
 }

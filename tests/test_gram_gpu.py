@@ -581,3 +581,45 @@ def test_same_bytes_where_exponents_rise(T, n):
     torch.cuda.synchronize()
     assert sum(not torch.equal(R, ref) for R in outs) == 0
     assert T.tsqr_get_device_status() == T.SUCCESS
+
+
+@pytest.mark.parametrize("m,n,k", [(20011, 20, 1), (9001, 40, 2), (9001, 60, 3), (20011, 96, 24)])
+@pytest.mark.parametrize("kind", ["served", "handed over"])
+def test_least_squares_plans_go_back(T, m, n, k, kind):
+    """The plan least squares reports gives the same bytes when it is passed back (on both sides of 56
+    columns of [A | B]), served or handed over; so does tsqr_r's, where that is the sum's."""
+    import torch
+    At = workloads.gaussian(m, n, seed=n)
+    if kind == "handed over":
+        At[n - 1] = At[0]
+    A, B = At.cuda().T, workloads.gaussian(m, k, seed=k).cuda().T
+    T.tsqr_r(A)
+    pr = T.last_plan()
+    X, R = T.tsqr_lstsq(A, B)
+    p = T.last_plan()
+    assert (p.tree, p.leaf) == (T.TREE_HYBRID, T.LEAF_GRAM) and p.tile_rows > 0
+    for plan in [p] + ([pr] if pr.leaf == T.LEAF_GRAM else []):
+        X1, R1 = T.tsqr_lstsq(A, B, plan=plan)
+        assert torch.equal(R1, R) and torch.equal(torch.nan_to_num(X1), torch.nan_to_num(X))
+    bad = T.make_plan("binary", tile_rows=256)
+    bad.leaf = T.LEAF_GRAM
+    for A1, B1, plan in [(A, B, bad), (A[:200], B[:200], p)]:  # no tree of the sum's, too few rows
+        with pytest.raises(T.TsqrError) as e:
+            T.tsqr_lstsq(A1, B1, plan=plan)
+        assert e.value.status == T.ERR_INVALID_ARG
+    T.tsqr_get_device_status()  # clears it
+
+
+@pytest.mark.parametrize("m,n,panel", [(9001, 12, 0), (9001, 12, 16), (20011, 40, 64)])
+@pytest.mark.parametrize("kind", ["served", "handed over"])
+def test_one_panel_plans_go_back(T, m, n, panel, kind):
+    """The plan tsqr_caqr_r reports for one panel gives the same bytes when it is passed back."""
+    import torch
+    At = workloads.gaussian(m, n, seed=n)
+    if kind == "handed over":
+        At[n - 1] = At[0]
+    A = At.cuda().T
+    R = T.tsqr_caqr_r(A, panel=panel)
+    p = T.last_plan()
+    assert p.leaf == T.LEAF_GRAM
+    assert torch.equal(T.tsqr_caqr_r(A, panel=panel, plan=p), R)
