@@ -78,8 +78,8 @@ typedef enum { TSQR_PREC_F64 = 0, TSQR_PREC_MIXED = 1 } tsqr_prec_t;
  *         columns (0 = 16), each panel's R by its own TSQR reduction (AUTO plan, reflectors
  *         kept) and its Q^T applied to the columns right of it, as tsqr_caqr_r does (Section
  *         5's panel and update).  R equals one reduction's up to rounding.  With 16 columns (or
- *         0), up to TSQR_MAX_N columns and m >= max(256, 4 n), the exact sum of TSQR_LEAF_GRAM is
- *         tried first and the panels run only where it cannot serve.
+ *         0), up to 2,048 columns and m >= max(256, 4 n), the exact sum of TSQR_LEAF_GRAM is tried
+ *         first and the panels run only where it cannot serve; with leaf FOLD they run alone.
  * AUTO picks HYBRID, or PANELS for FP64 R with n >= 56 and m >= 8 n, where its Householder form
  * measured faster (4,194,304 rows, n = 56 / 64 / 96 / 128: 775 / 828 / 863 / 887 against 727 / 750 /
  * 555 / 586 GFLOP/s; at n = 48 one reduction is faster, 826 against 802).                  */
@@ -137,8 +137,9 @@ typedef struct {
                            in one sweep (the R factor of [R_1; ...; R_c], equal to a sequence of
                            binary operators by associativity, Section 2).  0 = as many as the
                            kernel's shared memory holds.                                     */
-    int32_t leaf;       /* tsqr_leaf_t (FP64: 0, GRAM or GRAM_Q, whose plans are AUTO's
-                           whatever the other fields say).  With PANELS,
+    int32_t leaf;       /* tsqr_leaf_t (FP64: 0; GRAM or GRAM_Q, whose plans are AUTO's
+                           whatever the other fields say; FOLD with the PANELS tree: the
+                           panels without the sum).  MIXED, with leaf PANELS,
                            tile_rows is the chunk height (256, 384, 512, 640, 768 or 1024) of a HYBRID
                            plan, warps is 8 (or 0).                                          */
 } tsqr_plan_t;

@@ -765,7 +765,8 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
 }
 
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
-                       int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream);
+                       int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream,
+                       bool sums = true);
 
 // tsqr_qr's plan: the Gram factor and Q = A R^-1 where AUTO can take them (one column block; the
 // plan's other fields are those of the reflectors that stand behind it), else plan_store's.
@@ -807,6 +808,12 @@ int64_t panels_width(int64_t m, int64_t n, const tsqr_plan_t *over, int dev) {
     return 0;
 }
 
+// A PANELS plan that names a Householder leaf: the panels alone, no Gram sum before them.
+bool panels_alone(const tsqr_plan_t *p) {
+    return p && p->tree == TSQR_TREE_PANELS && p->leaf != TSQR_LEAF_AUTO &&
+           p->leaf != TSQR_LEAF_GRAM && p->leaf != TSQR_LEAF_GRAM_Q;
+}
+
 tsqr_status_t run_f64(const double *A, int64_t m, int64_t n, int64_t lda, double *R, int64_t ldr,
                       const tsqr_plan_t *over, cudaStream_t stream) {
     g_last_launches = 0;
@@ -820,11 +827,13 @@ tsqr_status_t run_f64(const double *A, int64_t m, int64_t n, int64_t lda, double
         if (nb > 0) {
             if (nb > TSQR_MAX_N) return TSQR_ERR_INVALID_ARG;
             if (m < n) return n > TSQR_MAX_N ? TSQR_ERR_UNSUPPORTED : TSQR_ERR_INVALID_ARG;
-            const tsqr_status_t st = run_caqr(A, m, n, lda, R, ldr, nb, nullptr, stream);
+            const bool alone = panels_alone(over);
+            const tsqr_status_t st = run_caqr(A, m, n, lda, R, ldr, nb, nullptr, stream, !alone);
             g_last_plan = tsqr_plan_t{};
             if (st == TSQR_SUCCESS) {
                 g_last_plan.tree = TSQR_TREE_PANELS;
                 g_last_plan.tile_rows = (int32_t)nb;
+                if (alone) g_last_plan.leaf = TSQR_LEAF_FOLD;
             }
             return st;
         }
@@ -1476,14 +1485,15 @@ struct CaqrPanel {
 
 
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
-                       int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream) {
+                       int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream,
+                       const bool sums) {
     g_last_launches = 0;
     g_last_plan = tsqr_plan_t{};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
     const DeviceInfo di = device_info(dev);
     if (asks_gram(over)) over = nullptr;
-    if (N <= nb && plan_is_auto(over) && gram_fits(m, N) && N < kPanelsMinN) {  // one panel: tsqr_r's reduction
+    if (sums && N <= nb && plan_is_auto(over) && gram_fits(m, N) && N < kPanelsMinN) {  // one panel: tsqr_r's reduction
         F64Plan p;
         tsqr_status_t st = plan_r(m, (int)N, over, &p);
         if (st != TSQR_SUCCESS) return st;
@@ -1499,7 +1509,7 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
         return TSQR_SUCCESS;
     }
     // by panels of the default width: the Gram sum first, the panels behind it
-    const bool gram = nb == 16 && plan_is_auto(over) && gram_fits(m, N);
+    const bool gram = sums && nb == 16 && plan_is_auto(over) && gram_fits(m, N);
     std::vector<CaqrPanel> panels;
     int64_t M = m;
     size_t max_fsmem = 0, max_qt = 0;
@@ -2623,6 +2633,7 @@ tsqr_status_t tsqr_resolve_plan(int64_t m, int64_t n, int32_t dtype, int32_t pre
             *out = tsqr_plan_t{};
             out->tree = TSQR_TREE_PANELS;
             out->tile_rows = (int32_t)nb;
+            if (panels_alone(plan)) out->leaf = TSQR_LEAF_FOLD;
             return TSQR_SUCCESS;
         }
     }

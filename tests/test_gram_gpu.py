@@ -623,3 +623,37 @@ def test_one_panel_plans_go_back(T, m, n, panel, kind):
     p = T.last_plan()
     assert p.leaf == T.LEAF_GRAM
     assert torch.equal(T.tsqr_caqr_r(A, panel=panel, plan=p), R)
+
+
+@pytest.mark.parametrize("m,n", [(40009, 56), (40000, 64), (30011, 80), (100003, 96), (65537, 128),
+                                 (12001, 180)])
+def test_householder_panels_on_request(oracle, T, m, n):
+    """Panels of the default width without the sum before them (leaf FOLD): within parity of the
+    oracle on a matrix the sum serves; and the bytes of AUTO's call on matrices it hands over."""
+    import torch
+    plan = T.make_plan("panels", tile_rows=16, leaf="fold")
+    At = workloads.gaussian(m, n, seed=n + 1)
+    R = T.tsqr_r_ex(At.cuda().T, plan=plan)
+    p = T.last_plan()
+    assert (p.tree, p.tile_rows, p.leaf) == (T.TREE_PANELS, 16, T.LEAF_FOLD)
+    if n <= 128:
+        r = T.tsqr_resolve_plan(m, n, plan=plan)
+        assert (r.tree, r.tile_rows, r.leaf) == (T.TREE_PANELS, 16, T.LEAF_FOLD)
+        _check(oracle, R, At)
+    served = T.tsqr_r(At.cuda().T)
+    assert T.last_plan().leaf == 0 and not torch.equal(R, served)
+    for kind in ("repeated", "zero", "nan"):
+        B = At.clone()
+        if kind == "repeated":
+            B[n - 2] = B[1]
+        elif kind == "zero":
+            B[n // 2] = 0.0
+        else:
+            B[n - 3, m // 2] = float("nan")
+        T.tsqr_get_device_status()
+        Ra = T.tsqr_r(B.cuda().T)
+        sa = T.tsqr_get_device_status()
+        Rb = T.tsqr_r_ex(B.cuda().T, plan=plan)
+        assert sa == T.tsqr_get_device_status()
+        assert torch.equal(torch.nan_to_num(Ra), torch.nan_to_num(Rb)), kind
+        assert torch.equal(torch.isfinite(Ra), torch.isfinite(Rb)), kind
