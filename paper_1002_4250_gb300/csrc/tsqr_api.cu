@@ -490,6 +490,14 @@ tsqr_status_t get_workspace(cudaStream_t stream, size_t bytes, Workspace **out) 
     return TSQR_SUCCESS;
 }
 
+// While it lives, this thread's host allocations and event waits neither fail for a capture that
+// another thread has in hand nor break it off.
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // `table` to device memory at dst, on the stream.
 tsqr_status_t upload_table(Workspace *w, const std::vector<char> &table, void *dst,
                            cudaStream_t stream) {
@@ -500,6 +508,7 @@ tsqr_status_t upload_table(Workspace *w, const std::vector<char> &table, void *d
         return cudaMemcpyAsync(dst, w->captured.back().data(), table.size(), cudaMemcpyHostToDevice,
                                stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
     }
+    const BesideCaptures beside;
     Workspace::Staged &s = w->staged[w->next_staged];
     w->next_staged = (w->next_staged + 1) % 4;
     if (s.used && cudaEventSynchronize(s.done) != cudaSuccess) return TSQR_ERR_CUDA;

@@ -657,3 +657,60 @@ def test_householder_panels_on_request(oracle, T, m, n):
         assert sa == T.tsqr_get_device_status()
         assert torch.equal(torch.nan_to_num(Ra), torch.nan_to_num(Rb)), kind
         assert torch.equal(torch.isfinite(Ra), torch.isfinite(Rb)), kind
+
+
+def _batch_call(T, count=24, m0=600):
+    """A small FP64 batch: (call(stream) -> R, R's reference)."""
+    import torch
+    ms, ns = [m0 + 37 * i for i in range(count)], [(8, 16, 32, 40)[i % 4] for i in range(count)]
+    offs, roff = [0], [0]
+    for m, n in zip(ms, ns):
+        offs.append(offs[-1] + m * n)
+        roff.append(roff[-1] + n * n)
+    g = torch.Generator(device="cuda").manual_seed(count)
+    buf = torch.randn(offs[-1], generator=g, dtype=torch.float64, device="cuda")
+    ptrs = [buf.data_ptr() + 8 * o for o in offs[:-1]]
+
+    def call(R, stream):
+        T.tsqr_r_batched(ptrs, ms, ns, roff, R, stream=stream)
+
+    ref = torch.empty(roff[-1], dtype=torch.float64, device="cuda")
+    call(ref, None)
+    torch.cuda.synchronize()
+    return call, ref, buf
+
+
+def test_batch_beside_a_capture_of_another_thread(T):
+    """One thread captures a graph in the strictest mode while another runs batches on a stream of its
+    own (whose workspace is there; their tables are new): both succeed."""
+    import threading
+
+    import torch
+    call, ref, _keep = _batch_call(T)
+    x = torch.ones(1000, device="cuda")
+    outs = [torch.zeros_like(ref) for _ in range(8)]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    errors = []
+    call(outs[0], s2)
+
+    def work():
+        try:
+            for R in outs:
+                call(R, s2)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s1, capture_error_mode="global"):
+        x += 1.0
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        x += 1.0
+    g.replay()
+    torch.cuda.synchronize()
+    assert not errors
+    assert (x == 3.0).all()
+    for R in outs:
+        assert torch.equal(R, ref)
