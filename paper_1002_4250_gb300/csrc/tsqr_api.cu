@@ -48,15 +48,17 @@ struct Workspace {
     // stream, graph replays included, uses the same workspace and leaves nothing of it.
     // Page-locked copies of the last tables on their way to the device: the copy runs on the stream,
     // after the call has returned, and on a host whose pageable memory the device reads in place
-    // (Grace) nothing stages it before.  A slot is reused once its copy is done.
+    // (Grace) nothing stages it before.  A ring, the oldest at next_staged, whose slots are reused
+    // once their copies are done and which grows to kMaxStaged while they are not: with that many
+    // tables on their way the host waits for the oldest (with four it waited from the fifth call on).
     struct Staged {
         void *host = nullptr;
         size_t bytes = 0;
-        cudaEvent_t done = nullptr;
-        bool used = false;
+        cudaEvent_t done = nullptr;  // after the last copy from it
     };
-    Staged staged[4];
-    int next_staged = 0;
+    static constexpr size_t kMaxStaged = 32;
+    std::vector<Staged> staged;
+    size_t next_staged = 0;
     // Tables of captured calls: a graph reads them at every replay.
     std::vector<std::vector<char>> captured;
 };
@@ -509,25 +511,40 @@ tsqr_status_t upload_table(Workspace *w, const std::vector<char> &table, void *d
                                stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
     }
     const BesideCaptures beside;
-    Workspace::Staged &s = w->staged[w->next_staged];
-    w->next_staged = (w->next_staged + 1) % 4;
-    if (s.used && cudaEventSynchronize(s.done) != cudaSuccess) return TSQR_ERR_CUDA;
-    s.used = false;
-    if (!s.done && cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess)
-        return TSQR_ERR_CUDA;
+    std::vector<Workspace::Staged> &ring = w->staged;
+    bool idle = false, roomy = false;
+    if (w->next_staged < ring.size()) {
+        const Workspace::Staged &o = ring[w->next_staged];
+        const cudaError_t e = cudaEventQuery(o.done);
+        if (e == cudaErrorNotReady)
+            cudaGetLastError();  // (it would be the next launch's error)
+        else if (e != cudaSuccess)
+            return TSQR_ERR_CUDA;
+        idle = e == cudaSuccess;
+        roomy = o.bytes >= table.size();
+    }
+    if ((!idle || !roomy) && ring.size() < Workspace::kMaxStaged) {
+        Workspace::Staged fresh;
+        if (cudaEventCreateWithFlags(&fresh.done, cudaEventDisableTiming) != cudaSuccess)
+            return TSQR_ERR_CUDA;
+        ring.insert(ring.begin() + w->next_staged, fresh);
+    }
+    Workspace::Staged &s = ring[w->next_staged];
+    if (cudaEventSynchronize(s.done) != cudaSuccess) return TSQR_ERR_CUDA;  // (at once, mostly)
     if (s.bytes < table.size()) {
         if (s.host) cudaFreeHost(s.host);
         s.host = nullptr;
         s.bytes = 0;
-        const size_t nb = align_up(table.size(), 1 << 16);
+        size_t nb = 1 << 16;
+        while (nb < table.size()) nb *= 2;
         if (cudaMallocHost(&s.host, nb) != cudaSuccess) return TSQR_ERR_ALLOC;
         s.bytes = nb;
     }
+    w->next_staged = (w->next_staged + 1) % ring.size();
     std::memcpy(s.host, table.data(), table.size());
     if (cudaMemcpyAsync(dst, s.host, table.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess ||
         cudaEventRecord(s.done, stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
-    s.used = true;
     return TSQR_SUCCESS;
 }
 

@@ -714,3 +714,28 @@ def test_batch_beside_a_capture_of_another_thread(T):
     assert (x == 3.0).all()
     for R in outs:
         assert torch.equal(R, ref)
+
+
+def test_batch_calls_do_not_wait_for_the_stream(T):
+    """Thirty batch calls, small and larger tables in turn, on a stream that is busy for some 0.2 s:
+    the calls return while it is; and a second thirty with the slots at hand."""
+    import time
+
+    import torch
+    small, large = _batch_call(T), _batch_call(T, count=900, m0=260)
+    outs = [torch.zeros_like(b[1]) for b in (small, large)]
+    s = torch.cuda.Stream()
+    for (call, _, _), out in zip((small, large), outs):  # the workspace at its full size
+        call(out, s)
+    for _ in range(2):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(400_000_000)
+        t0 = time.perf_counter()
+        for k in range(30):
+            (small, large)[k % 2][0](outs[k % 2], s)
+        took = time.perf_counter() - t0
+        assert not s.query() and took < 0.15, took
+    torch.cuda.synchronize()
+    for (_, ref, _), out in zip((small, large), outs):
+        assert torch.equal(out, ref)
