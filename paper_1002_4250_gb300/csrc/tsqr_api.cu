@@ -59,8 +59,6 @@ struct Workspace {
     static constexpr size_t kMaxStaged = 32;
     std::vector<Staged> staged;
     size_t next_staged = 0;
-    // Tables of captured calls: a graph reads them at every replay.
-    std::vector<std::vector<char>> captured;
 };
 
 std::mutex g_mu;
@@ -504,11 +502,24 @@ struct BesideCaptures {
 tsqr_status_t upload_table(Workspace *w, const std::vector<char> &table, void *dst,
                            cudaStream_t stream) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) return TSQR_ERR_CUDA;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamGetCaptureInfo(stream, &cap, nullptr, &graph) != cudaSuccess) return TSQR_ERR_CUDA;
     if (cap != cudaStreamCaptureStatusNone) {
-        w->captured.push_back(table);
-        return cudaMemcpyAsync(dst, w->captured.back().data(), table.size(), cudaMemcpyHostToDevice,
-                               stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
+        // a graph reads its table at every replay: it owns a copy, as its executable forms do
+        auto *own = new std::vector<char>(table);
+        cudaUserObject_t obj;
+        if (cudaUserObjectCreate(&obj, own,
+                                 [](void *p) { delete static_cast<std::vector<char> *>(p); }, 1,
+                                 cudaUserObjectNoDestructorSync) != cudaSuccess) {
+            delete own;
+            return TSQR_ERR_CUDA;
+        }
+        if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+            cudaUserObjectRelease(obj, 1);
+            return TSQR_ERR_CUDA;
+        }
+        return cudaMemcpyAsync(dst, own->data(), own->size(), cudaMemcpyHostToDevice, stream) ==
+                       cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
     }
     const BesideCaptures beside;
     std::vector<Workspace::Staged> &ring = w->staged;
