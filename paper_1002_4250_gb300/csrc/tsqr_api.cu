@@ -621,14 +621,19 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
                wy_smem_bytes(n, hs | 1) <= di.smem_block_optin;
     };
     while (r > 0 && (r % 2 || good_r(r) != r || (with_q && !q_fits(r)))) --r;
+    // the shortest chunk that leaves every CTA one, where the matrix is short enough
+    const int64_t lanes = 32LL * p->warps;
+    for (int s = 2; s < r; s += 2)
+        if (good_r(s) == s && m <= s * lanes * di.sms && (!with_q || q_fits(s))) r = s;
     tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, di.sms, p->warps, 0, 0};
     const tsqr_status_t st = plan_with_r(m, n, &fold, false, r, di, p);
     if (st != TSQR_SUCCESS) return st;
-    if (p->blk % 2) {  // a matrix of few rows: two rows per lane all the same
+    if (p->hs / (32 * p->warps) % 2) {  // a matrix of few rows: two rows per lane all the same
         fold.tile_rows = 64 * p->warps;
         const tsqr_status_t st2 = plan_with_r(m, n, &fold, false, r, di, p);
         if (st2 != TSQR_SUCCESS) return st2;
     }
+    p->blk = 2;  // the launch's block, whatever else would divide the rows per lane
     const int64_t kb = gram_round_rows(n) / 64, nkb = (m + 63) / 64;
     p->gram_ctas = (int)std::min<int64_t>(di.sms, (nkb + kb - 1) / kb);
     p->smem = std::max(p->smem, gram_smem_bytes(n));

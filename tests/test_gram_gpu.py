@@ -777,3 +777,19 @@ def test_captured_batches_give_their_tables_back(T):
         if k == 4:
             before = resident()
     assert resident() - before < 20 << 20
+
+
+@pytest.mark.parametrize("n", range(1, 33))
+def test_chunks_behind_the_sum(T, n):
+    """The Householder leaves behind the single launch fold chunks that fill shared memory where there
+    are rows for it (four tenths of an SM's, a number of rows that blocks well), and where there are
+    not, as many leaves as chunks of the least height (two rows a lane) give."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    p = T.tsqr_resolve_plan(1 << 24, n)
+    assert p.leaf == T.LEAF_GRAM
+    per_sm = -(-p.ctas // sms)
+    assert p.ctas == per_sm * sms and per_sm * p.tile_rows * n * 8 >= 0.4 * 227 * 1024
+    for m in (10000, 100003):
+        p = T.tsqr_resolve_plan(m, n)
+        assert p.ctas >= min(0.8 * sms, m // (64 * p.warps))
