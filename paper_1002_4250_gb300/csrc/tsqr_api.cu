@@ -584,8 +584,8 @@ constexpr int kPanelsMinN = 56;
 // Plan of an FP64 R by one reduction: the exact-Gram reduction where it serves (AUTO, or a plan
 // that asks for TSQR_LEAF_GRAM), else the Householder leaves.  The Gram plan's other fields are
 // those of the Householder reduction it falls back to: up to kGramMaxN columns in the same
-// launch, one CTA of 12 bulk warps per SM with an even number of rows per lane (the kernel's
-// inner block is two rows); past that the AUTO plan's, in a launch of its own.
+// launch (several leaves a CTA, or one for tsqr_qr, which keeps their reflectors); past that the
+// AUTO plan's, in a launch of its own.
 tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
@@ -610,33 +610,45 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     }
     p->tree = TSQR_TREE_HYBRID;
     p->leaf = with_q ? TSQR_LEAF_GRAM_Q : TSQR_LEAF_GRAM;
-    p->warps = kGramFoldWarps;
-    const size_t budget = std::min(di.smem_block_optin, di.smem_sm - 1024);
+    const GramFold shape = with_q ? kGramFoldQ : kGramFoldR;
+    p->warps = shape.warps;
+    const size_t budget = std::min(di.smem_block_optin, di.smem_sm - 1024) / shape.groups / 16 * 16;
     int r = max_rows_per_lane_p(n, p->warps, budget, false);
-    auto q_fits = [&](const int rows) {  // Q's blocked leaf pass in one column group
+    auto usable = [&](const int rows) {
+        // from three rows on a multiple of three: a lane's run of rows times an odd number of columns
+        // then starts in another shared-memory bank than its neighbours' (us, 8 rows a lane / 6:
+        // 16,777,216 x 8 with a zero column 4,277 / 3,225, thin QR 1,000,000 x 8 at kappa 1e6
+        // 1,163 / 874)
+        if (!with_q) return rows < 3 || (rows % 3 == 0 && good_r(rows) == rows);
+        // the form that keeps its reflectors blocks by two rows, and Q's blocked leaf pass takes a
+        // chunk in one column group
         const int hs = 32 * p->warps * rows;
-        int blk = 1, vec = 1;
-        block_for(rows, false, &blk, &vec);
-        return q_leaf_wy_smem_bytes(n, n, ld_for(hs, vec), true) <= di.smem_block_optin &&
+        return rows % (rows < 6 ? 2 : 6) == 0 &&
+               q_leaf_wy_smem_bytes(n, n, ld_for(hs, 1), true) <= di.smem_block_optin &&
                wy_smem_bytes(n, hs | 1) <= di.smem_block_optin;
     };
-    while (r > 0 && (r % 2 || good_r(r) != r || (with_q && !q_fits(r)))) --r;
-    // the shortest chunk that leaves every CTA one, where the matrix is short enough
-    const int64_t lanes = 32LL * p->warps;
-    for (int s = 2; s < r; s += 2)
-        if (good_r(s) == s && m <= s * lanes * di.sms && (!with_q || q_fits(s))) r = s;
-    tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, di.sms, p->warps, 0, 0};
+    while (r > 0 && !usable(r)) --r;
+    // the shortest chunk that leaves every group one, where the matrix is short enough
+    const int64_t groups = (int64_t)di.sms * shape.groups;
+    for (int s = 2; s < r; ++s)
+        if (usable(s) && m <= 32 * s * p->warps * groups) r = s;
+    tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, (int32_t)groups, p->warps, 0, 0};
     const tsqr_status_t st = plan_with_r(m, n, &fold, false, r, di, p);
     if (st != TSQR_SUCCESS) return st;
-    if (p->hs / (32 * p->warps) % 2) {  // a matrix of few rows: two rows per lane all the same
-        fold.tile_rows = 64 * p->warps;
-        const tsqr_status_t st2 = plan_with_r(m, n, &fold, false, r, di, p);
-        if (st2 != TSQR_SUCCESS) return st2;
+    if (!with_q) {
+        const int rows = p->hs / (32 * p->warps);
+        p->blk = rows % 3 == 0 ? 3 : rows % 2 == 0 ? 2 : 1;  // (what the launch has)
+    } else {
+        if (p->hs / (32 * p->warps) % 2) {  // a matrix of few rows: two rows per lane all the same
+            fold.tile_rows = 64 * p->warps;
+            const tsqr_status_t st2 = plan_with_r(m, n, &fold, false, r, di, p);
+            if (st2 != TSQR_SUCCESS) return st2;
+        }
+        p->blk = 2;
     }
-    p->blk = 2;  // the launch's block, whatever else would divide the rows per lane
     const int64_t kb = gram_round_rows(n) / 64, nkb = (m + 63) / 64;
     p->gram_ctas = (int)std::min<int64_t>(di.sms, (nkb + kb - 1) / kb);
-    p->smem = std::max(p->smem, gram_smem_bytes(n));
+    p->smem = std::max(shape.groups * align_up(p->smem, 16), gram_smem_bytes(n));
     return TSQR_SUCCESS;
 }
 
@@ -767,6 +779,7 @@ GramArgs gram_args(const F64Plan &p, const RLayout &w, const F64Args &a, void *b
     g.p.ldr = a.ldr;
     if (p.leaf == TSQR_LEAF_GRAM_Q) g.p.Q = (GramQForm *)((char *)base + w.form_off);
     g.status = a.status;
+    g.grid = std::max(p.gram_ctas, std::min(p.nleaves, current_sms()));
     g.fold = a;
     return g;
 }
@@ -788,7 +801,10 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
                                               stream);
         if (st != TSQR_SUCCESS) return st;
     }
-    if ((p.gram_ctas ? gram_prepare((int)n, p.smem) : f64_prepare(p.smem)) != cudaSuccess)
+    const bool as_q = p.leaf == TSQR_LEAF_GRAM_Q;
+    if ((!p.gram_ctas ? f64_prepare(p.smem)
+         : as_q       ? gram_qr_prepare((int)n, p.smem)
+                      : gram_prepare((int)n, p.smem)) != cudaSuccess)
         return TSQR_ERR_CUDA;
     if (cudaMemsetAsync(a.counters, 0, w.cnt_words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
@@ -796,7 +812,7 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
     if (!p.gram_ctas)
         return f64_launch(a, p.warps, p.smem, stream) == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
     const GramArgs g = gram_args(p, w, a, base);
-    cudaError_t e = gram_launch(g, p.smem, stream);
+    cudaError_t e = as_q ? gram_qr_launch(g, p.smem, stream) : gram_launch(g, p.smem, stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         // a context that owns only part of the device: the plan's Householder reduction
         cudaGetLastError();
@@ -814,8 +830,8 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
 // plan's other fields are those of the reflectors that stand behind it), else plan_store's.
 // ms, against plan_store's: 4,194,304 x 32 1.02 / 24.4, 16,777,216 x 8 0.92 / 7.76, 100,003 x 32
 // 0.123 / 1.66, 10,000 x 16 0.064 / 0.38, 3,000 x 5 0.046 / 0.22.  A matrix left to the reflectors
-// pays for the sum: 4,194,304 x 32 24.65 / 24.36, and up to 16 columns for the 12-warp chunks the
-// single launch folds in (1,000,000 x 16 2.25 / 1.88).
+// pays for the sum, and up to 16 columns for passes that share the products' launch (one CTA an
+// SM): 4,194,304 x 32 24.6 / 24.4, 1,000,000 x 16 2.23 / 1.87, x 8 0.87 / 0.87, x 4 0.51 / 0.31.
 tsqr_status_t plan_qr(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSQR_ERR_CUDA;
@@ -1015,8 +1031,8 @@ tsqr_status_t run_qr(const double *A, int64_t m, int64_t n, int64_t lda, double 
         gq.form = g.p.Q;
         gq.verdict = g.p.verdict;
         gq.status = ws->status;
-        if (gram_prepare((int)n, p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
-        e = gram_launch(g, p.smem, stream);
+        if (gram_qr_prepare((int)n, p.smem) != cudaSuccess) return TSQR_ERR_CUDA;
+        e = gram_qr_launch(g, p.smem, stream);
     }
     if (e == cudaErrorCooperativeLaunchTooLarge) {  // (also a context that owns part of the device)
         cudaGetLastError();

@@ -154,6 +154,9 @@ __host__ __device__ inline SmemLayout smem_layout(int n, int hs, int ldS, int wa
     return smem_layout_s(n, ldS * n, warps);
 }
 
+// Shared memory of one of a CTA's leaves (groups of threads), a multiple of 16 bytes.
+__host__ __device__ inline int fold_group_doubles(const SmemLayout &L) { return (L.total + 1) & ~1; }
+
 // Packed upper triangle, row-major: row j holds R(j, j..n-1) at rowoff(j).
 __host__ __device__ inline int rowoff(int n, int j) { return j * n - (j * (j - 1)) / 2; }
 

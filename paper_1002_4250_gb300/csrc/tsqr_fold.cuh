@@ -19,10 +19,20 @@
 #include "tsqr_f64.cuh"
 #include "tsqr_internal.h"
 
-// Threads that run the fold and the tree: the CTA's, or fewer where a kernel lets the others
-// exit first (it defines this before including the header).
-#ifndef TSQR_FOLD_THREADS
+// Threads that run the fold and the tree of a leaf: the CTA's; or, where a kernel defines their
+// number before it includes this header, one of several groups of so many threads, each with a
+// leaf of its own, a named barrier and a part of the CTA's dynamic shared memory (threads past the
+// last group have left).  A constant: read from memory at run time it cost 7% (1,000,000 x 32).
+#ifdef TSQR_FOLD_THREADS
+#define TSQR_FOLD_TID (threadIdx.x % (TSQR_FOLD_THREADS))
+#define TSQR_FOLD_GROUP (threadIdx.x / (TSQR_FOLD_THREADS))
+#define TSQR_FOLD_SYNC() \
+    asm volatile("barrier.sync %0, %1;" ::"r"(1 + TSQR_FOLD_GROUP), "n"(TSQR_FOLD_THREADS) : "memory")
+#else
 #define TSQR_FOLD_THREADS blockDim.x
+#define TSQR_FOLD_TID threadIdx.x
+#define TSQR_FOLD_GROUP 0
+#define TSQR_FOLD_SYNC() __syncthreads()
 #endif
 
 namespace tsqr {
@@ -77,7 +87,7 @@ __device__ __forceinline__ void load_column(T *S, int ldS, int hs, const Chunk<T
     const Tin *src = c.src + (int64_t)col * c.lda;
     T *dst = S + (size_t)col * ldS;
     if constexpr (Copy<T, Tin>::kAsync) {
-        for (int i = threadIdx.x; i < hs; i += TSQR_FOLD_THREADS) {
+        for (int i = TSQR_FOLD_TID; i < hs; i += TSQR_FOLD_THREADS) {
             const bool ok = i < c.rows;
             if constexpr (sizeof(T) == 8)
                 cp_async8(dst + i, ok ? (const void *)(src + i) : (const void *)c.src, ok ? 8 : 0);
@@ -86,7 +96,7 @@ __device__ __forceinline__ void load_column(T *S, int ldS, int hs, const Chunk<T
         }
         cp_async_commit();
     } else {
-        for (int i = threadIdx.x; i < hs; i += TSQR_FOLD_THREADS)
+        for (int i = TSQR_FOLD_TID; i < hs; i += TSQR_FOLD_THREADS)
             dst[i] = (i < c.rows) ? (T)widen(src[i]) : (T)0;
     }
 }
@@ -488,8 +498,8 @@ __device__ __forceinline__ void fold_leaf(T *__restrict__ S, const int ldS, cons
                                           double *__restrict__ tot, double *__restrict__ npart,
                                           const int n, const Chunk<Tin> pf,
                                           const QChunk qc = QChunk{}) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int lane = TSQR_FOLD_TID & 31;
+    const int warp = TSQR_FOLD_TID >> 5;
     const int Wb = (TSQR_FOLD_THREADS >> 5) - 1;
     const bool reducer = (warp == Wb);
     const int Hw = hs / Wb;
@@ -545,7 +555,7 @@ __device__ __forceinline__ void fold_leaf(T *__restrict__ S, const int ldS, cons
             npart[warp * 32 + lane] = (double)(nacc + nacc2);
             for (int id = lane; id < 32 + U; id += 32) seg[id] = (T)0;
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
 
         Reflector h;
         if (reducer) {
@@ -564,7 +574,7 @@ __device__ __forceinline__ void fold_leaf(T *__restrict__ S, const int ldS, cons
             else
                 phase_b_plain<T, B>(lane, J, U, r, Hw, n, S, ldS, r0, Sj, SJ, fT, seg);
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
 
         // ---- reducer: dot products in a fixed order, row J of R, factors f[k] for k > J
         if (reducer) {
@@ -590,11 +600,11 @@ __device__ __forceinline__ void fold_leaf(T *__restrict__ S, const int ldS, cons
             __syncwarp();
             apply_reflector<T>(lane, n, J, h, Rp, f, dk, fT);
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
     }
     if constexpr (kStore) {
         if (!reducer) store_tail_rows(S, ldS, r0, r, lane, n - 1, qc);
-        __syncthreads();  // the prefetch below reuses column n-1
+        TSQR_FOLD_SYNC();  // the prefetch below reuses column n-1
     }
     if (Copy<T, Tin>::kAsync && pf.src) {
         for (int col = n - 2; col < n; ++col)
@@ -622,8 +632,8 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
                                            double *__restrict__ dk, const int n,
                                            double *nsc = nullptr,
                                            const bool worker_sums = true) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int lane = TSQR_FOLD_TID & 31;
+    const int warp = TSQR_FOLD_TID >> 5;
     const int Wp = (TSQR_FOLD_THREADS >> 5) - 1;  // worker warps 1..Wp
     const int ss = seg_stride(n);
     double *seg = seg_all + (warp > 0 ? warp - 1 : 0) * ss;
@@ -656,7 +666,7 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
         } else {
             for (int id = lane; id < 32 + U; id += 32) seg[id] = 0.0;
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
 
         Reflector hr;
         if (warp == 0) {
@@ -728,7 +738,7 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
                 dk[kc0 + rel] = d0 + d1;
             }
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
 
         if (warp == 0) {
             if (!worker_sums) {
@@ -754,14 +764,14 @@ __device__ __forceinline__ void fold_stack(double *__restrict__ S, const int ldS
             }
             apply_reflector(lane, n, J, hr, Rp, f, dk);
         }
-        __syncthreads();
+        TSQR_FOLD_SYNC();
     }
 }
 
 // Packed upper triangle (smem) -> column-major n x n (global), zeros below the diagonal.
 __device__ __forceinline__ void store_packed(const double *__restrict__ Rp, int n,
                                              double *__restrict__ dst, int64_t ld) {
-    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
+    for (int idx = TSQR_FOLD_TID; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         dst[row + (int64_t)col * ld] = (row <= col) ? Rp[rowoff(n, row) + col - row] : 0.0;
     }
@@ -770,7 +780,7 @@ __device__ __forceinline__ void store_packed(const double *__restrict__ Rp, int 
 // Column-major global (L2, bypassing L1) -> packed upper triangle in smem.
 __device__ __forceinline__ void load_packed_cg(const double *src, int64_t ld, int n,
                                                double *__restrict__ Rp) {
-    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
+    for (int idx = TSQR_FOLD_TID; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         if (row <= col) Rp[rowoff(n, row) + col - row] = __ldcg(src + row + (int64_t)col * ld);
     }
@@ -779,7 +789,7 @@ __device__ __forceinline__ void load_packed_cg(const double *src, int64_t ld, in
 // Column-major global -> S (upper triangle kept, strict lower part stored as zero).
 __device__ __forceinline__ void load_tri_cg(const double *src, int64_t ld, int n,
                                             double *__restrict__ S, int ldS) {
-    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
+    for (int idx = TSQR_FOLD_TID; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         S[row + col * ldS] = (row <= col) ? __ldcg(src + row + (int64_t)col * ld) : 0.0;
     }
@@ -790,7 +800,7 @@ __device__ __forceinline__ void store_normalized(const double *__restrict__ Rp, 
                                                  double *__restrict__ R, int64_t ldr,
                                                  int *status) {
     bool bad = false;
-    for (int idx = threadIdx.x; idx < n * n; idx += TSQR_FOLD_THREADS) {
+    for (int idx = TSQR_FOLD_TID; idx < n * n; idx += TSQR_FOLD_THREADS) {
         const int col = idx / n, row = idx - col * n;
         double v = 0.0;
         if (row <= col) {
@@ -838,7 +848,7 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
     for (;;) {
         if (cnt == 1) {
             if constexpr (kStore) {
-                for (int k2 = threadIdx.x; k2 < n; k2 += TSQR_FOLD_THREADS)
+                for (int k2 = TSQR_FOLD_TID; k2 < n; k2 += TSQR_FOLD_THREADS)
                     a.q.signs[k2] = (Rp[rowoff(n, k2)] < 0.0) ? -1.0 : 1.0;
             }
             store_normalized(Rp, n, a.R, a.ldr, a.status);
@@ -855,9 +865,9 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
         }
         store_packed(Rp, n, a.slots + (size_t)(off + t) * n * n, n);
         __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) flag[0] = atomicAdd(&a.counters[next_off + parent], 1u);
-        __syncthreads();
+        TSQR_FOLD_SYNC();
+        if (TSQR_FOLD_TID == 0) flag[0] = atomicAdd(&a.counters[next_off + parent], 1u);
+        TSQR_FOLD_SYNC();
         if (flag[0] + 1 < (unsigned)nchild) return;  // a later sibling combines
         __threadfence();
         // the last child to arrive stacks the children in index order: the first on top
@@ -865,7 +875,7 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
         for (int ch = 1; ch < nchild; ++ch)
             load_tri_cg(a.slots + (size_t)(off + first + ch) * n * n, n, n,
                         Sd + (size_t)(ch - 1) * n, ldSd);
-        __syncthreads();
+        TSQR_FOLD_SYNC();
         if constexpr (kStore) {
             const size_t id = (size_t)next_off + parent;
             const int ldv = (k - 1) * n;
@@ -874,7 +884,7 @@ __device__ __forceinline__ void climb_tree(const F64Args &a, double *Sd, const i
             // the node's tails: rows 0..(nchild-1) n - 1 of S (zero below each diagonal)
             double *dst = a.q.node_V + id * (size_t)ldv * n;
             const int rows = (nchild - 1) * n;
-            for (int idx = threadIdx.x; idx < rows * n; idx += TSQR_FOLD_THREADS) {
+            for (int idx = TSQR_FOLD_TID; idx < rows * n; idx += TSQR_FOLD_THREADS) {
                 const int col = idx / rows, row = idx - col * rows;
                 dst[row + (size_t)col * ldv] = Sd[row + (size_t)col * ldSd];
             }
@@ -901,9 +911,10 @@ template <typename T, typename Tin, int B, int V, bool kPipe, bool kStore = fals
 __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, const int ldSd,
                                               const int s_doubles, const int leaf,
                                               const int worker_sum_nodes = kWorkerSumNodes) {
-    extern __shared__ __align__(16) double smem[];
+    extern __shared__ __align__(16) double smem_all[];
     const int n = a.n;
     const SmemLayout L = smem_layout_s(n, s_doubles, TSQR_FOLD_THREADS >> 5);
+    double *const smem = smem_all + TSQR_FOLD_GROUP * fold_group_doubles(L);
     T *S = reinterpret_cast<T *>(smem + L.S);
     double *Sd = smem + L.S;
     double *Rp = smem + L.Rp;
@@ -918,7 +929,7 @@ __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, co
     double *npart = smem + L.npart;
     unsigned int *flag = reinterpret_cast<unsigned int *>(smem + L.scal);
 
-    for (int i = threadIdx.x; i < n * (n + 1) / 2; i += TSQR_FOLD_THREADS) Rp[i] = 0.0;
+    for (int i = TSQR_FOLD_TID; i < n * (n + 1) / 2; i += TSQR_FOLD_THREADS) Rp[i] = 0.0;
 
     // rows of this leaf, folded in chunks of h rows
     const int64_t u0 = ((int64_t)leaf * a.nunits) / a.nleaves;
@@ -933,7 +944,7 @@ __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, co
         first.rows = (int)((rend - rbeg < a.h) ? rend - rbeg : a.h);
         for (int col = 0; col < n; ++col) load_column(S, a.ldS, a.hs, first, col);
         cp_async_wait_all();
-        __syncthreads();
+        TSQR_FOLD_SYNC();
     }
     for (int64_t c = 0; c < nchunks; ++c) {
         Chunk<Tin> next;
@@ -957,11 +968,11 @@ __device__ __forceinline__ void leaf_tree_job(const F64Args &a, const Tin *A, co
                                                next, qc);
         if (next.src) {
             if constexpr (!Copy<T, Tin>::kAsync) {
-                __syncthreads();
+                TSQR_FOLD_SYNC();
                 for (int col = 0; col < n; ++col) load_column(S, a.ldS, a.hs, next, col);
             }
             cp_async_wait_all();
-            __syncthreads();
+            TSQR_FOLD_SYNC();
         }
     }
 

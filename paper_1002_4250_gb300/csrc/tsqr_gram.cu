@@ -1,83 +1,32 @@
 // Exact-Gram reduction on the tensor cores: the kernels (tsqr_gram.cuh has the method,
 // tsqr_gram_dev.cuh the device code).
-#include <cstring>
-
 #include "tsqr_gram.cuh"
-#define TSQR_FOLD_THREADS (32 * (kGramFoldWarps + 1))
-#include "tsqr_gram_dev.cuh"
+#define TSQR_FOLD_THREADS (32 * (kGramFoldR.warps + 1))
+#include "tsqr_gram_single.cuh"
 
 namespace tsqr {
 
 namespace {
-using namespace gram;
 
-constexpr long long kVerdictPolls = 1LL << 27;  // of at least 0.2 us each
-
-// The Householder reduction of the same CTA (12 bulk warps and the reducer; the other warps have
-// left), kept out of line: it runs only where the Gram sum cannot serve.
-__device__ __noinline__ void fold_job(const F64Args &f, const int leaf) {
-    leaf_tree_job<double, double, 2, 1, false>(f, f.A, f.ldS, f.ldS * f.n, leaf);
-}
-
-// The same keeping its reflectors (tsqr_qr).
-__device__ __noinline__ void fold_store_job(const F64Args &f, const int leaf) {
-    leaf_tree_job<double, double, 2, 1, false, true>(f, f.A, f.ldS, f.ldS * f.n, leaf);
-}
-
-// What bounds it: shared memory.  A 128-row round at 32 columns moves some 275 KB through it (A in
-// and out 64, its digits 64, the products' operands 147), 2.15k of the 3.2k cycles a round takes;
-// cutting alone is 1.2k, the products 0.8k.  Then the flush of every 1,024 rows' sums (7k cycles).
-// The Householder leaves it stands before are bound by FP64 arithmetic.  us: 4,194,304 x 32 10,103
-// before, 486 now (HBM's share 161); 16,777,216 x 8 2,697 / 399 (161); 10,000 x 16 198 / 38.9,
-// latency: the sums 14k cycles, the tree 9k, the root 25k.
-//
-// One FP64 matrix of at most 32 columns in one launch: CTA c sums slab c, the root factors, every
-// CTA waits for its verdict and runs its leaf of the Householder reduction where the Gram cannot
-// serve.  One CTA per SM, launched cooperatively.
-template <int NB>
-__global__ void __launch_bounds__(kGramThreads, 1)
-tsqr_gram_f64_kernel(const __grid_constant__ GramArgs a) {
-    extern __shared__ __align__(1024) double smem_d[];
-    unsigned char *smem = reinterpret_cast<unsigned char *>(smem_d);
-    const int tid = threadIdx.x, b = blockIdx.x;
-    const size_t slot_bytes = gram_slot_bytes(NB);
-    if (b < a.p.nslab) {
-        Cta c;
-        cta_begin(c, smem);
-        const bool root = item_of<NB, 0>(a.p, Cols{0, a.p.n, 0, 0}, 0, b, slot_bytes, c);
-        if (!c.ok && tid == 0) atomicOr(a.status, kStatusTimeoutBit);
-        cta_end(c);
-        if (root) {
-            const bool good = finish(a.p, slot_bytes, c.sm, c.stages);
-            __syncthreads();
-            if (tid == 0) {
-                __threadfence();
-                atomicExch(a.p.verdict, good ? 1u : 2u);
-            }
-            if (good) return;
-        }
+// tsqr_r's leaves: several a CTA hide each other's reflector chains and barriers, as two or three
+// CTAs an SM do for that reduction by itself.  Out of line: they run only where the Gram sum cannot
+// serve.  (A zero column, us, with one leaf of 12 warps a CTA / so: 10,000 x 16 249 / 180, 1,000,000 x
+// 32 3,202 / 2,939.)
+struct RLeaves {
+    static constexpr GramFold kShape = kGramFoldR;
+    template <int B>
+    static __device__ __noinline__ void fold(const F64Args &f, const int leaf) {
+        leaf_tree_job<double, double, B, 1, false>(f, f.A, f.ldS, f.ldS * f.n, leaf);
     }
-    // the verdict: 1, done; 2, the Householder reduction
-    Smem &sm = *reinterpret_cast<Smem *>(smem);
-    if (tid == 0) {
-        unsigned v = 0;
-        for (long long it = 0; it < kVerdictPolls; ++it) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.p.verdict) : "memory");
-            if (v) break;
-            __nanosleep(200);
-        }
-        sm.flag = (int)v;
-        if (!v) atomicOr(a.status, kStatusTimeoutBit);
+    static __device__ __forceinline__ void run(const F64Args &f, const int leaf) {
+        if (f.blk == 3)
+            fold<3>(f, leaf);
+        else if (f.blk == 2)
+            fold<2>(f, leaf);
+        else
+            fold<1>(f, leaf);
     }
-    __syncthreads();
-    const int v = sm.flag;
-    __syncthreads();
-    if (v != 2 || b >= a.fold.nleaves || tid >= TSQR_FOLD_THREADS) return;
-    if (a.fold.q.V)
-        fold_store_job(a.fold, b);
-    else
-        fold_job(a.fold, b);
-}
+};
 
 // A queue of work items (sets of columns over slabs of rows) of one matrix or many: the CTA that
 // completes a matrix's last set factors it.  Bound by the two-block sets, 3.9k cycles a 64-row round:
@@ -161,20 +110,6 @@ tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {
     cta_end(c);
 }
 
-typedef void (*GramKernel)(const GramArgs);
-struct Variant {
-    GramKernel fn;
-    size_t smem;
-    int kb_round;
-};
-template <int NB>
-Variant variant() {
-    using Sh = Shape<NB, 0>;
-    return Variant{tsqr_gram_f64_kernel<NB>, smem_bytes<Sh>(), Sh::kRoundKb};
-}
-Variant variant_for(int n) {
-    return n <= 8 ? variant<8>() : n <= 16 ? variant<16>() : n <= 24 ? variant<24>() : variant<32>();
-}
 constexpr size_t queue_smem() {
     size_t b = smem_bytes<Shape<8, 0>>();
     for (size_t o : {smem_bytes<Shape<16, 0>>(), smem_bytes<Shape<24, 0>>(),
@@ -190,28 +125,11 @@ static_assert(kHead + (kGramRootMaxN * (kGramRootMaxN + 1) / 2 + 3 * kGramRootMa
 
 }  // namespace
 
-int gram_round_rows(int n) { return 64 * variant_for(n).kb_round; }
-size_t gram_smem_bytes(int n) { return variant_for(n).smem; }
-
-cudaError_t gram_prepare(int n, size_t smem_bytes) {
-    return set_smem_attrs(variant_for(n).fn, smem_bytes);
-}
-
+int gram_round_rows(int n) { return 64 * variant_for<RLeaves>(n).kb_round; }
+size_t gram_smem_bytes(int n) { return variant_for<RLeaves>(n).smem; }
+cudaError_t gram_prepare(int n, size_t smem_bytes) { return single_prepare<RLeaves>(n, smem_bytes); }
 cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream) {
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(a.p.nslab > a.fold.nleaves ? a.p.nslab : a.fold.nleaves);
-    cfg.blockDim = dim3(kGramThreads);
-    cfg.dynamicSmemBytes = smem_bytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeCooperative;
-    at.val.cooperative = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    GramArgs args = a;
-    void *params[1] = {&args};
-    return cudaLaunchKernelExC(&cfg, (const void *)variant_for(a.p.n).fn, params);
+    return single_launch<RLeaves>(a, smem_bytes, stream);
 }
 
 cudaError_t gram_queue_launch(const GramQueueArgs &a, int grid, cudaStream_t stream) {

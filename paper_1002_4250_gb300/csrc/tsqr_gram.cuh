@@ -23,7 +23,16 @@ namespace tsqr {
 
 constexpr int kGramSlicers = 16;    // warps that cut entries into digits; one more multiplies
 constexpr int kGramThreads = 32 * (kGramSlicers + 1);
-constexpr int kGramFoldWarps = 12;  // bulk warps of the Householder reduction (and its reducer)
+// The Householder leaves behind the single launch: `groups` a CTA at a time, of `warps` bulk warps and
+// a reducer each.
+struct GramFold {
+    int warps, groups;
+};
+constexpr GramFold kGramFoldR{4, 3}, kGramFoldQ{12, 1};
+constexpr bool gram_fold_fits(const GramFold f) {
+    return 32 * (f.warps + 1) * f.groups <= kGramThreads && f.groups < 16;  // (named barriers)
+}
+static_assert(gram_fold_fits(kGramFoldR) && gram_fold_fits(kGramFoldQ), "the leaves' threads");
 constexpr int kGramMaxN = 32;       // one column block: tsqr_r's single launch
 constexpr int kGramRootMaxN = 128;  // widest matrix one CTA factors
 
@@ -65,7 +74,8 @@ __host__ __device__ inline int gram_guard(int64_t m) {
 struct GramArgs {          // tsqr_r's single launch: one problem of one column block
     GramProblem p;
     int *status;
-    F64Args fold;          // the Householder reduction (its A is FP64; nleaves <= grid)
+    int grid;              // CTAs, at least the Householder leaves over the groups of a CTA
+    F64Args fold;          // the Householder reduction (its A is FP64)
 };
 
 // Q = A R^-1 (tsqr_gram_q.cuh).  Rows of a tile: up to 16 columns, two or four 128-row blocks of A

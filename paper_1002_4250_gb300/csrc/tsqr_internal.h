@@ -45,6 +45,9 @@ int gram_round_rows(int n);
 size_t gram_smem_bytes(int n);
 cudaError_t gram_prepare(int n, size_t smem_bytes);
 cudaError_t gram_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream);
+// The same with tsqr_qr's Householder leaves behind the sum.
+cudaError_t gram_qr_prepare(int n, size_t smem_bytes);
+cudaError_t gram_qr_launch(const GramArgs &a, size_t smem_bytes, cudaStream_t stream);
 // A queue of column sets and slabs on `grid` CTAs (at most one per SM).
 struct GramQueueArgs;
 cudaError_t gram_queue_launch(const GramQueueArgs &a, int grid, cudaStream_t stream);

@@ -793,3 +793,21 @@ def test_chunks_behind_the_sum(T, n):
     for m in (10000, 100003):
         p = T.tsqr_resolve_plan(m, n)
         assert p.ctas >= min(0.8 * sms, m // (64 * p.warps))
+
+
+@pytest.mark.parametrize("m", [256, 300, 641, 1000, 5003, 60013, 400009])
+@pytest.mark.parametrize("n", [1, 2, 5, 8, 9, 16, 24, 32])
+def test_leaves_behind_the_sum(T, m, n):
+    """The Householder leaves of the single launch, three a CTA, at every block height (one, two and
+    three rows) and with fewer leaves than groups: the bytes of that reduction by itself."""
+    import torch
+    At = workloads.gaussian(m, n, seed=m % 89 + n)
+    At[n // 2] = 0.0
+    Ad = At.cuda().T
+    R = T.tsqr_r(Ad)
+    p = T.last_plan()
+    assert p.leaf == T.LEAF_GRAM and p.warps == 4 and T.tsqr_last_launch_count() == 1
+    ref = T.tsqr_r_ex(Ad, plan=T.make_plan("hybrid", tile_rows=p.tile_rows, ctas=p.ctas,
+                                           warps=p.warps, arity=p.arity))
+    assert torch.equal(R, ref)
+    assert T.tsqr_get_device_status() == T.SUCCESS
