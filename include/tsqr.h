@@ -244,8 +244,9 @@ tsqr_status_t tsqr_qr(const double *A, int64_t m, int64_t n, int64_t lda, double
  *   plan as for tsqr_qr (NULL = AUTO; a GRAM plan, as tsqr_r and this call report, is AUTO).
  * With few right-hand sides (k <= max(1, n / 4) and n + k <= TSQR_MAX_N) the augmented matrix
  * [A | B] is factorized instead (its R holds R and (Q^T B)(0:n, :) side by side; with the AUTO
- * plan by the exact Gram sum of [A | B], read where they are, and by the Householder reduction
- * of a copy where that cannot serve) and one triangular solve follows; R then equals tsqr_r's
+ * plan by the exact Gram sum of [A | B], read where they are and factored as far as A's columns, so
+ * that a B in A's range is served too, and by the Householder reduction of a copy where that
+ * cannot serve) and one triangular solve follows; R then equals tsqr_r's
  * up to rounding.  Otherwise the columns of B
  * go k_g = min(k, n) at a time (two launches per group after the factorization) and R is
  * tsqr_r_ex's bit for bit under the plan tsqr_last_plan reports (a Householder one).

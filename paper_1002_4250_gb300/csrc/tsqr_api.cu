@@ -676,11 +676,11 @@ GramLayout gram_layout(int64_t m, int64_t n, int sms) {
     }
     return w;
 }
-// The Gram sum of [A | B] (B: columns na .. n-1, or none) and its factor R in the workspace at
-// base; *verdict: the device word that tells the launches behind it whether R is there.
+// The Gram sum of [A | B] (B: columns na .. n-1, or none) and the first np rows of its factor R (the
+// others zero), workspace at base; *verdict: the device word that tells the launches behind it whether R is there.
 tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_t lda,
                            const double *B, int64_t ldb, int64_t na, int64_t m, int64_t n,
-                           void *base, double *R, int64_t ldr, int *status,
+                           int64_t np, void *base, double *R, int64_t ldr, int *status,
                            const unsigned int **verdict, int *launches, cudaStream_t stream) {
     if (cudaMemsetAsync(base, 0, w.words * sizeof(unsigned int), stream) != cudaSuccess)
         return TSQR_ERR_CUDA;
@@ -694,6 +694,7 @@ tsqr_status_t enqueue_gram(const GramLayout &w, int sms, const double *A, int64_
     q.one.m = m;
     q.one.n = (int)n;
     q.one.na = (int)na;
+    q.one.np = (int)np;
     q.one.nb = w.nb;
     q.one.nslab = w.nslab;
     q.one.nkb = (m + 63) / 64;
@@ -767,7 +768,7 @@ GramArgs gram_args(const F64Plan &p, const RLayout &w, const F64Args &a, void *b
     g.p.A = a.A;
     g.p.lda = a.lda;
     g.p.m = a.m;
-    g.p.n = g.p.na = a.n;
+    g.p.n = g.p.na = g.p.np = a.n;
     g.p.nb = 1;
     g.p.nslab = p.gram_ctas;
     g.p.nkb = (a.m + 63) / 64;
@@ -796,7 +797,7 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
     a.ldr = ldr;
     a.status = status;
     if (p.gram_queue) {
-        const tsqr_status_t st = enqueue_gram(w.g, sms, A, lda, nullptr, 0, n, m, n,
+        const tsqr_status_t st = enqueue_gram(w.g, sms, A, lda, nullptr, 0, n, m, n, n,
                                               (char *)base + w.gram_off, R, ldr, status, &a.skip, launches,
                                               stream);
         if (st != TSQR_SUCCESS) return st;
@@ -822,9 +823,10 @@ tsqr_status_t enqueue_r(const F64Plan &p, const RLayout &w, int sms, const doubl
     return e == cudaSuccess ? TSQR_SUCCESS : TSQR_ERR_CUDA;
 }
 
+// sums: the Gram sum first where it serves; rows: of R that are wanted (0: all).
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
                        int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream,
-                       bool sums = true);
+                       bool sums = true, int64_t rows = 0);
 
 // tsqr_qr's plan: the Gram factor and Q = A R^-1 where AUTO can take them (one column block; the
 // plan's other fields are those of the reflectors that stand behind it), else plan_store's.
@@ -1241,7 +1243,7 @@ tsqr_status_t run_lstsq_augmented(const double *A, int64_t m, int64_t n, int64_t
     double *Ra = (double *)(base + cnt_bytes + slot_bytes + aug_bytes);
     F64Args a = plan_args(p, aug, m, na, m);
     if (gram) {
-        st = enqueue_gram(gl, sms, A, lda, B, ldb, n, m, na, (char *)Ra + ra_bytes, Ra, na, ws->status,
+        st = enqueue_gram(gl, sms, A, lda, B, ldb, n, m, na, n, (char *)Ra + ra_bytes, Ra, na, ws->status,
                           &a.skip, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
         g_last_plan.leaf = TSQR_LEAF_GRAM;
@@ -1544,7 +1546,7 @@ struct CaqrPanel {
 
 tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, double *R,
                        int64_t ldr, int64_t nb, const tsqr_plan_t *over, cudaStream_t stream,
-                       const bool sums) {
+                       const bool sums, const int64_t rows) {
     g_last_launches = 0;
     g_last_plan = tsqr_plan_t{};
     int dev = 0;
@@ -1690,7 +1692,7 @@ tsqr_status_t run_caqr(const double *A, int64_t m, int64_t N, int64_t lda, doubl
     int launches = 0;
     const unsigned int *skip = nullptr;
     if (gram) {
-        st = enqueue_gram(gl, di.sms, A, lda, nullptr, 0, N, m, N, base + total, R, ldr, ws->status,
+        st = enqueue_gram(gl, di.sms, A, lda, nullptr, 0, N, m, N, rows ? rows : N, base + total, R, ldr, ws->status,
                           &skip, &launches, stream);
         if (st != TSQR_SUCCESS) return st;
     }
@@ -1795,7 +1797,7 @@ tsqr_status_t run_lstsq_panels(const double *A, int64_t m, int64_t n, int64_t ld
         st = TSQR_ERR_CUDA;
     int launches = 0;
     if (st == TSQR_SUCCESS) {
-        st = run_caqr(aug, m, na, m, Ra, na, kCaqrPanel, nullptr, stream);
+        st = run_caqr(aug, m, na, m, Ra, na, kCaqrPanel, nullptr, stream, true, n);
         launches = g_last_launches;
     }
     Workspace *ws = nullptr;
@@ -2039,7 +2041,7 @@ void plan_gram_batch(const void *const *ptrs, const int64_t *ms, const int32_t *
         GramProblem &g = (*probs)[i];
         g.A = (const double *)ptrs[i];
         g.lda = g.m = ms[i];
-        g.n = g.na = ns[i];
+        g.n = g.na = g.np = ns[i];
         g.nb = (ns[i] + 31) / 32;
         g.nkb = (ms[i] + 63) / 64;
         g.guard = gram_guard(ms[i]);

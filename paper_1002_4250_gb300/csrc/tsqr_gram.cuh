@@ -41,6 +41,7 @@ struct GramProblem {
     const double *A, *B;
     int64_t lda, ldb, m;
     int n, na;
+    int np;                // rows of R that are wanted: n, or na where [A | B] is a least-squares problem's
     int nb;                // column blocks; sets 0 .. nb-1 are a block against itself, then (0, 1),
                            // (0, 2), (1, 2), (0, 3), ...
     int nslab;             // slabs of rows: slab s holds 64-row blocks [s nkb / nslab, ...)

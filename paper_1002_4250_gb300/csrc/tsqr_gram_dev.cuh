@@ -822,17 +822,18 @@ __device__ __forceinline__ double r_entry(const i128 l, const u64 s, const int g
     return b ? round64(__umul64hi(top, s), b - 186 + g, l < 0) : 0.0;
 }
 
-// C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it.  rowv: 3 n
-// entries of scratch (the scaled pivots stay in the last n).  Thread k < n returns pivot k, scaled,
+// C: packed upper rows (row k at rowoff(n, k) - k + j); row k's l replaces it, k < np (the rows
+// below are not done: a right-hand side in the matrix's range has no pivot).  rowv: 3 n
+// entries of scratch (the scaled pivots stay in the last n).  Thread k < np returns pivot k, scaled,
 // and its shift.  Returns false if a pivot is too small (*low: zero on entry, then non-zero).
 //
-// A chain of n steps, each a reciprocal, a quotient and a multiplication deep.  The first n threads
+// A chain of np steps, each a reciprocal, a quotient and a multiplication deep.  The first n threads
 // hold column j = tid: row k's l are theirs, and while the others take row k off the rows below they
 // find the next pivot (from the diagonal as it was and l's own share) and its reciprocal.  Up to 32
 // columns the trailing matrix stays in registers.  (1,000 x 32, with what follows here: 53 us a call,
 // 72 with full products, the reciprocal in the chain and R in double-double.)
-static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int n, int *low,
-                                                 u128 &mine, int &myz) {
+static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int n, const int np,
+                                                 int *low, u128 &mine, int &myz) {
     const int tid = threadIdx.x, nt = kGramThreads, warp = tid >> 5, lane = tid & 31;
     constexpr i128 kLeast = (i128)1 << (122 - kPivotBits);
     Q128 *Lq = rowv, *Cp = rowv + n, *dv = rowv + 2 * n;
@@ -863,7 +864,7 @@ static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int 
         if (d0 < kLeast) return false;  // the same for every thread
         if (tid < n) pivot(d0);
     }
-    for (int k = 0; k < n; ++k) {
+    for (int k = 0; k < np; ++k) {
         Q128 *Ck = C + rowoff(n, k) - k;
         u128 lm = 0, cm = 0;  // |l| and |c| of the thread's column
         if (tid < n) {
@@ -883,7 +884,7 @@ static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int 
                 if (tid == k + 1) Lq[k] = pack(diag);
             }
         }
-        if (k + 1 == n) break;
+        if (k + 1 == np) break;
         __syncthreads();
         if (tid < n) {
             const i128 a = unpack(Lq[k + 1]), b = unpack(Cp[k + 1]);
@@ -919,20 +920,22 @@ static __device__ __noinline__ bool factor_chain(Q128 *C, Q128 *rowv, const int 
 
 // R from the chain's l and pivots: R(k, k) = sqrt(d_k) 2^-z_k, R(k, j) = l sqrt(d_k), g[j] the power
 // of two of column j; in integers to the last (the chip has two FP64 lanes an SM).
-static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int *g,
-                                                double *R, const int64_t ldr, int *low) {
+static __device__ __noinline__ bool factor_root(Q128 *C, Q128 *rowv, const int n, const int np,
+                                                const int *g, double *R, const int64_t ldr, int *low) {
     const int tid = threadIdx.x, nt = kGramThreads;
     Q128 *Lq = rowv;
     u128 mine;
     int myz;
-    if (!factor_chain(C, rowv, n, low, mine, myz)) return false;
+    if (!factor_chain(C, rowv, n, np, low, mine, myz)) return false;
     __syncthreads();
-    if (tid < n) Lq[tid] = Q128{sqrt64(mine), (u64)myz};
+    if (tid < np) Lq[tid] = Q128{sqrt64(mine), (u64)myz};
     __syncthreads();
     for (int o = tid; o < n * n; o += nt) {
         const int col = o / n, row = o - col * n;
         double v = 0.0;
-        if (row < col) {
+        if (row >= np) {
+            // (not done, not wanted)
+        } else if (row < col) {
             v = r_entry(unpack(C[rowoff(n, row) - row + col]), Lq[row].lo, g[col]);
         } else if (row == col) {
             v = round64(Lq[row].lo, g[col] - 64 - (int)Lq[row].hi, false);
@@ -1053,7 +1056,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
         const u64 dh = (u64)((u128)d >> 64);
         const int len = dh ? 128 - __clzll((long long)dh) : 64 - __clzll((long long)(u64)d);
         sm.E[tid] = d > 0 ? (122 - len) >> 1 : 0;  // shift of the column
-        if (!(d > 0)) sm.bad = 1;
+        if (!(d > 0) && tid < p.np) sm.bad = 1;
         sm.Dnew[tid] = 73 - sm.E[tid] + sm.D[tid] + kUnit + p.guard / 2;
     }
     __syncthreads();
@@ -1064,7 +1067,7 @@ static __device__ __noinline__ bool finish(const GramProblem &p, const size_t sl
         C[rowoff(n, i) - i + j] = pack(shift128(entry(i, j), sm.E[i] + sm.E[j]));
     }
     __syncthreads();
-    if (!factor_root(C, rowv, n, sm.Dnew, p.R, p.ldr, &sm.bad)) return false;
+    if (!factor_root(C, rowv, n, p.np, sm.Dnew, p.R, p.ldr, &sm.bad)) return false;
     if (p.Q) {
         invert_root(p, C, rowv + 2 * n, sm);
         __syncthreads();

@@ -53,7 +53,7 @@ __global__ void tsqr_gram_scale_kernel(const GramWideArgs a) {
     const int e = g > 0 ? (122 - len) >> 1 : 0;
     a.E[j] = e;
     a.g[j] = 73 - e + d + kUnit + p.guard / 2;
-    if (bad || d <= kLeastD || !(g > 0)) *a.bad = 1;
+    if (bad || d <= kLeastD || (!(g > 0) && j < p.np)) *a.bad = 1;
 }
 
 __global__ void tsqr_gram_fill_kernel(const GramWideArgs a) {
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kGramThreads) tsqr_gram_panel_kernel(const Gra
     __shared__ Q128 L[kBw * (kBw + 1) / 2], rowv[3 * kBw];
     __shared__ u64 rec[kBw];
     __shared__ int zs[kBw], low;
-    const int n = a.p.n, k0 = kb * kBw, w = min(kBw, n - k0);
+    const int n = a.p.n, k0 = kb * kBw, w = min(kBw, n - k0), wp = min(w, a.p.np - k0);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // one thread's read decides for the CTA: another CTA of this launch may be setting the word, and
     // threads that saw it would be missing from the barriers of those that did not
@@ -105,14 +105,15 @@ __global__ void __launch_bounds__(kGramThreads) tsqr_gram_panel_kernel(const Gra
     __syncthreads();
     u128 mine;
     int myz;
-    if (!factor_chain(L, rowv, w, &low, mine, myz)) {  // (the same for every thread of every CTA)
+    if (!factor_chain(L, rowv, w, wp, &low, mine, myz)) {  // (the same for every thread of every CTA)
         if (tid == 0) *a.bad = 1;
         return;
     }
-    const Q128 *piv = rowv + 2 * w;
-    if (tid < w) {
-        rec[tid] = recip60(mine);
-        zs[tid] = myz;
+    Q128 *piv = rowv + 2 * w;
+    if (tid < w) {  // (rows past wp go along as they are)
+        if (tid >= wp) piv[tid] = pack((i128)1 << 121);
+        rec[tid] = recip60(tid < wp ? mine : (u128)1 << 121);
+        zs[tid] = tid < wp ? myz : 0;
     }
     __syncthreads();
     if (blockIdx.x == 0) {
@@ -197,12 +198,12 @@ __global__ void tsqr_gram_write_kernel(const GramWideArgs a) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int tile = blockIdx.x; tile < nb * nb; tile += gridDim.x) {
         const int i0 = tile / nb * kBw, j0 = tile % nb * kBw;
-        if (ty == 0) sq[tx] = i0 <= j0 && i0 + tx < n ? sqrt64((u128)unpack(d[i0 + tx])) : 0;
+        if (ty == 0) sq[tx] = i0 <= j0 && i0 + tx < a.p.np ? sqrt64((u128)unpack(d[i0 + tx])) : 0;
         __syncthreads();
         for (int u = ty; u < kBw; u += 8) {
             const int i = i0 + u, j = j0 + tx;
             double v = 0.0;
-            if (i <= j && j < n) {
+            if (i <= j && j < n && i < a.p.np) {
                 // (a diagonal block's l are mirrored, see the panel kernel)
                 v = i == j ? round64(sq[u], a.g[j] - 64 - a.z[i], false)
                            : r_entry(unpack(i0 == j0 ? C[(int64_t)j * n + i] : C[(int64_t)i * n + j]),
@@ -222,18 +223,18 @@ __global__ void tsqr_gram_write_kernel(const GramWideArgs a) {
 }  // namespace
 
 int gram_wide_launch(const GramWideArgs &a, cudaStream_t stream) {
-    const int n = a.p.n, nb = (n + kBw - 1) / kBw;
+    const int n = a.p.n, nb = (n + kBw - 1) / kBw, done = (a.p.np + kBw - 1) / kBw;
     int launches = 0;
     tsqr_gram_scale_kernel<<<(n + 127) / 128, 128, 0, stream>>>(a);
     const int64_t fill = ((int64_t)n * n + 255) / 256;
     tsqr_gram_fill_kernel<<<(int)(fill < 4096 ? fill : 4096), 256, 0, stream>>>(a);
     launches += 2;
-    for (int kb = 0; kb < nb; ++kb) {
+    for (int kb = 0; kb < done; ++kb) {
         const int right = n - (kb + 1) * kBw;
         const int ctas = right > 0 ? (right + kGramThreads / 32 - 1) / (kGramThreads / 32) : 1;
         tsqr_gram_panel_kernel<<<ctas < 1024 ? ctas : 1024, kGramThreads, 0, stream>>>(a, kb);
         ++launches;
-        if (right <= 0) break;
+        if (kb + 1 == done) break;
         const int t = (right + kBw - 1) / kBw;
         tsqr_gram_update_kernel<<<t * (t + 1) / 2, 1024, 0, stream>>>(a, kb);
         ++launches;

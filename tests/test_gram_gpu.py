@@ -811,3 +811,42 @@ def test_leaves_behind_the_sum(T, m, n):
                                            warps=p.warps, arity=p.arity))
     assert torch.equal(R, ref)
     assert T.tsqr_get_device_status() == T.SUCCESS
+
+
+@pytest.mark.parametrize("m,n,k", [(9001, 8, 2), (20011, 31, 1), (20011, 32, 1), (20011, 33, 8),
+                                   (9001, 60, 5), (20011, 100, 25), (6007, 150, 40), (5003, 128, 33)])
+@pytest.mark.parametrize("kind", ["consistent", "one of them", "noisy", "tiny"])
+def test_regressions_need_only_the_pivots_of_the_matrix(oracle, T, m, n, k, kind):
+    """B in the range of A (whose residual has no pivot in the sum): served, X as close to the known
+    solution as for a noisy B, R the same bytes whatever B is.  B below the fixed point's range
+    goes to the Householder reduction."""
+    import torch
+    At = workloads.gaussian(m, n, seed=n)
+    X0 = torch.randn(n, k, generator=torch.Generator().manual_seed(3), dtype=torch.float64)
+    Bt = (At.T @ X0).T.contiguous()
+    if kind == "noisy":
+        Bt += workloads.gaussian(m, k, seed=5)
+    elif kind == "one of them":
+        Bt[1:] += workloads.gaussian(m, k, seed=5)[1:]
+    elif kind == "tiny":
+        Bt[0] *= 2.0 ** -430
+        X0[:, 0] *= 2.0 ** -430
+    T.tsqr_get_device_status()
+    X, R = T.tsqr_lstsq(At.cuda().T, Bt.cuda().T)
+    assert T.tsqr_get_device_status() == T.SUCCESS
+    A, B = oracle.from_torch_colmajor(At), oracle.from_torch_colmajor(Bt)
+    X, X0 = X.cpu().numpy(), X0.numpy()
+    kap = oracle.kappa_from_r(oracle.householder_r(A, nthreads=16))
+    c = max(50.0, 2.0 * np.sqrt(m * max(1.0, n / 32.0)))
+    for j in range(k):
+        ref = X0[:, j]
+        if kind == "noisy" or (kind == "one of them" and j > 0):
+            ref = oracle.lstsq(A, np.asfortranarray(B[:, j:j + 1]), nthreads=16)[:, 0]
+        res = np.linalg.norm(B[:, j] - A @ ref)
+        tol = c * (kap + kap ** 2 * res / (np.linalg.norm(A, 2) * np.linalg.norm(ref))) * U
+        assert np.linalg.norm(X[:, j] - ref) <= tol * np.linalg.norm(ref)
+    if kind != "tiny":
+        noisy = workloads.gaussian(m, k, seed=6)
+        assert torch.equal(T.tsqr_lstsq(At.cuda().T, noisy.cuda().T)[1], R)
+    if n + k <= 128:
+        _check(oracle, R, At)
