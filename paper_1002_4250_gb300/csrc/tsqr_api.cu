@@ -613,7 +613,7 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
     const GramFold shape = with_q ? kGramFoldQ : kGramFoldR;
     p->warps = shape.warps;
     const size_t budget = std::min(di.smem_block_optin, di.smem_sm - 1024) / shape.groups / 16 * 16;
-    int r = max_rows_per_lane_p(n, p->warps, budget, false);
+    const int rmax = max_rows_per_lane_p(n, p->warps, budget, false);
     auto usable = [&](const int rows) {
         // from three rows on a multiple of three: a lane's run of rows times an odd number of columns
         // then starts in another shared-memory bank than its neighbours' (us, 8 rows a lane / 6:
@@ -627,11 +627,19 @@ tsqr_status_t plan_r(int64_t m, int n, const tsqr_plan_t *over, F64Plan *p) {
                q_leaf_wy_smem_bytes(n, n, ld_for(hs, 1), true) <= di.smem_block_optin &&
                wy_smem_bytes(n, hs | 1) <= di.smem_block_optin;
     };
-    while (r > 0 && !usable(r)) --r;
-    // the shortest chunk that leaves every group one, where the matrix is short enough
+    // the height with the least work for the group that has most: its chunks, each some four rows a
+    // lane's worth of reflector chain besides (thin QR 1,000,000 x 5, us: 755 with 217 chunks of 4,608
+    // rows on 152 SMs, 625 with 435 of 2,304)
     const int64_t groups = (int64_t)di.sms * shape.groups;
-    for (int s = 2; s < r; ++s)
-        if (usable(s) && m <= 32 * s * p->warps * groups) r = s;
+    int r = 0;
+    int64_t least = 0;
+    for (int s = rmax > 1 ? 2 : 1; s <= rmax; ++s) {
+        const int64_t rows = 32LL * s * p->warps, cost = (m + rows * groups - 1) / (rows * groups) * (s + 4);
+        if (usable(s) && (r == 0 || cost < least)) {
+            r = s;
+            least = cost;
+        }
+    }
     tsqr_plan_t fold{TSQR_TREE_HYBRID, 0, (int32_t)groups, p->warps, 0, 0};
     const tsqr_status_t st = plan_with_r(m, n, &fold, false, r, di, p);
     if (st != TSQR_SUCCESS) return st;
