@@ -697,6 +697,7 @@ def bench_batched(dev, threads):
 KERNEL_SOURCES = ("paper_1002_4250_gb300/csrc/tsqr_gram.cu",
                   "paper_1002_4250_gb300/csrc/tsqr_gram.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_gram_dev.cuh",
+                  "paper_1002_4250_gb300/csrc/tsqr_gram_single.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_tc.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_fold.cuh",
                   "paper_1002_4250_gb300/csrc/tsqr_f64.cuh",

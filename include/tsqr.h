@@ -279,8 +279,8 @@ tsqr_status_t tsqr_lstsq(const double *A, int64_t m, int64_t n, int64_t lda, con
  * reflectors (8 m panel bytes) and small tree buffers, from the per-stream pool.  Launches:
  * (the exact Gram sum, AUTO plan and panel width, up to 2,048 columns and m >= max(256, 4 n): the
  * sum, and past 128 columns two per 32 columns and three more for its factor, after which the
- * panels' launches return at once unless it could not serve;) three per panel (the factorization, its chunks' compact WY factors and the update; two where
- * the blocked update does not fit) except the last (the factorization alone).  Returns
+ * panels' launches return at once unless it could not serve;) three per panel (the
+ * factorization, its chunks' compact WY factors and the update; two where the blocked update does not fit) except the last (the factorization alone).  Returns
  * TSQR_ERR_INVALID_ARG for bad sizes, TSQR_ERR_UNSUPPORTED for a panel above TSQR_MAX_N or a
  * plan tsqr_qr would refuse, TSQR_ERR_ALLOC when the workspace cannot be had. */
 tsqr_status_t tsqr_caqr_r(const double *A, int64_t m, int64_t n, int64_t lda, double *R,
@@ -429,8 +429,8 @@ void tsqr_release_workspace(void);
 /* Static description of a status code. */
 const char *tsqr_status_string(int32_t status);
 
-/* The plan of the factorization the last call on this host thread ran (the first panel's for
- * tsqr_caqr_r), in the form tsqr_r_ex accepts: passed back as a plan it gives the same
+/* The plan of the factorization the last call on this host thread ran (for tsqr_caqr_r the first
+ * panel's, also where the exact Gram sum came before the panels), in the form tsqr_r_ex accepts: passed back as a plan it gives the same
  * partition, kernels and bytes.  All fields zero when that call ran no factorization.
  *   out : host pointer, required.  Returns TSQR_ERR_INVALID_ARG when NULL. */
 tsqr_status_t tsqr_last_plan(tsqr_plan_t *out);

@@ -18,11 +18,11 @@ constexpr long long kVerdictPolls = 1LL << 27;  // of at least 0.2 us each
 // and out 64, its digits 64, the products' operands 147), 2.15k of the 3.2k cycles a round takes;
 // cutting alone is 1.2k, the products 0.8k.  Then the flush of every 1,024 rows' sums (7k cycles).
 // The Householder leaves it stands before are bound by FP64 arithmetic.  us: 4,194,304 x 32 10,103
-// before, 486 now (HBM's share 161); 16,777,216 x 8 2,697 / 399 (161); 10,000 x 16 198 / 38.9,
+// before, 482 now (HBM's share 161); 16,777,216 x 8 2,697 / 395 (161); 10,000 x 16 198 / 38.9,
 // latency: the sums 14k cycles, the tree 9k, the root 25k.
 //
 // One FP64 matrix of at most 32 columns in one launch: CTA c sums slab c, the root factors, every
-// CTA waits for its verdict and runs its leaf of the Householder reduction where the Gram cannot
+// CTA waits for its verdict and runs its leaves of the Householder reduction where the Gram cannot
 // serve.  One CTA per SM, launched cooperatively.
 template <int NB, typename Leaves>
 __global__ void __launch_bounds__(kGramThreads, 1)

@@ -943,16 +943,14 @@ tsqr_q_gram_kernel(const __grid_constant__ GramQArgs g, const __grid_constant__ 
         q_leaf_wy_call(a, blockIdx.x);
 }
 
-// R X = C for R upper triangular (n x n), C (n x k, leading dimension ldc): one warp per column,
-// rows last to first, each row's sum over the solved rows split across the lanes (a fixed
-// butterfly).  A zero or non-finite result is noted in the status word.
 // R X = C for n <= 32 T: one warp a column, row i of the running right-hand side in lane i % 32.
 // From the last row up, x_i goes to every lane by shuffles and is taken out of the rows above, the
 // next columns of R already on their way (their loads do not wait for x).  The quotient is a
 // product with the row's reciprocal (a division, some 375 cycles, would be most of a row's chain)
 // and its residual: x_i and the right-hand side are kept as a double and what its rounding left
 // out, so X carries the rounding of its last addition.  n = 32, one column: row sums with
-// divisions took 20 us.
+// divisions took 20 us.  (No reciprocal overflows: R's diagonal is zero or at least 2^-537, the root
+// of the least sum of squares.)  A non-finite result is noted in the status word.
 template <int T>
 __global__ void __launch_bounds__(256) tsqr_trsm_small_kernel(const double *R, int64_t ldr,
                                                               const double *C, int64_t ldc, double *X,
@@ -1013,6 +1011,9 @@ __global__ void __launch_bounds__(256) tsqr_trsm_small_kernel(const double *R, i
     if (bad && lane == 0 && status) atomicOr(status, kStatusNonfiniteBit);
 }
 
+// R X = C for R upper triangular (n x n), C (n x k, leading dimension ldc): one warp per column,
+// rows last to first, each row's sum over the solved rows split across the lanes (a fixed
+// butterfly).  A zero or non-finite result is noted in the status word.
 __global__ void __launch_bounds__(1024) tsqr_trsm_kernel(const double *R, int64_t ldr,
                                                          const double *C, int64_t ldc, double *X,
                                                          int64_t ldx, int n, int k, int *status) {
