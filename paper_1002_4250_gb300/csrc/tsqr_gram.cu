@@ -32,7 +32,7 @@ struct RLeaves {
 // completes a matrix's last set factors it.  Bound by the two-block sets, 3.9k cycles a 64-row round:
 // the digits of 64 columns 1.4k, 64 KB of operands read for each of eight products, the flush 0.9k
 // a round (one accumulator set, so every 1,024 rows).  us, Householder / here: 4,194,304 x 128 154,900 /
-// 7,190; 1,000,000 x 50 with an odd leading dimension (8-byte copies of every other column) 6,670 / 625;
+// 7,115; 1,000,000 x 50 with an odd leading dimension (8-byte copies of every other column) 6,670 / 625;
 // 512 problems 27,300 / 1,450.
 __global__ void __launch_bounds__(kGramThreads, 1)
 tsqr_gram_queue_f64_kernel(const __grid_constant__ GramQueueArgs a) {

@@ -3,7 +3,6 @@
 // fixed-point Cholesky factor of the whole.
 #pragma once
 
-#include <climits>
 #include <type_traits>
 
 #include "tsqr_fold.cuh"
@@ -90,7 +89,7 @@ struct alignas(16) Smem {   // beside the stages
     uint64_t drain;         // all tensor-core work so far is done
     uint32_t tmem;
     int flag, bad, item;
-    int above;              // the first round with an entry above its column's range
+    int above[2];           // a stage's round has an entry above its column's range
     int stop;               // the round that was not multiplied for it; -1: none
     int D[128], E[128], Dnew[128];
 };
@@ -323,7 +322,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     const uint64_t desc0 = tc::smem_desc(tc::smem_u32(c.stages), 16, 1024, tc::kSw128);
     const bool issuer = tid == kGramThreads - 32;  // the thread that issues the tensor-core work
     constexpr long long kPolls = 1LL << 22;
-    volatile int *const above = &sm.above, *const stop = &sm.stop;
+    volatile int *const above = sm.above, *const stop = &sm.stop;
     int blocks = 0;                 // 64-row blocks in the accumulators
     int used[2] = {0, 0};           // rounds given to each stage since the barriers' last start
     uint32_t drained = 0;           // completions of sm.drain since then
@@ -338,7 +337,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             tc::mbar_inval(&sm.drain);
             tc::mbar_init(&sm.drain, 1);
             tc::fence_mbar_init();
-            *above = INT_MAX;
+            above[0] = above[1] = 0;
             *stop = -1;
         }
         used[0] = used[1] = 0;
@@ -497,9 +496,9 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
     // Rounds run without a CTA barrier: a warp slices its task of a round into the round's stage as
     // soon as the tensor cores are done with the round before the last (free), and the last warp,
     // which slices nothing, issues a round's products once all have arrived (full).  A warp that meets an entry
-    // above its column's range leaves the round's number before it arrives (the least one stays); the
-    // last warp then issues nothing for that round and sets the stop, which every wait watches, and
-    // the whole CTA takes that round block by block.
+    // above its column's range says so of the round's stage before it arrives; the last warp then
+    // issues nothing for that round and sets the stop, which every wait watches, and the whole CTA
+    // takes that round block by block.
     restart_barriers();
 #pragma unroll 1
     for (int r = 0; r < Sh::kRaws; ++r) load_round(r);
@@ -522,7 +521,7 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
             if (go) {
                 int dmin = 2;
                 if (mine) slice8(raw_of(r), sm.D[lc], dmin, dst + b * Sh::kStage, step);
-                if (__any_sync(0xffffffffu, dmin < 2) && lane == 0) atomicMin(&sm.above, r);
+                if (__any_sync(0xffffffffu, dmin < 2) && lane == 0) above[b] = 1;
                 tc::fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&sm.full[b]);
@@ -530,10 +529,12 @@ __device__ __noinline__ void sum_rows(const GramProblem &p, const Cols cols, con
         } else {
             if (c.ok) c.ok = tc::mbar_wait(&sm.full[b], used[b] & 1, kPolls);
             __syncwarp();
-            // (one lane reads it for all: another warp may be saying so of the next round, which
-            // is not this one's to stop for: where the rounds break off decides where the sums are
-            // cut, and has to follow from the data alone)
-            go = __shfl_sync(0xffffffffu, lane == 0 ? *above : 0, 0) > r;
+            // (round r's word alone: another warp may be saying so of the next round, in the other
+            // stage, and where the rounds break off decides where the sums are cut, which has to
+            // follow from the data; no warp is in round r + 2 before round r is multiplied.  One
+            // word with the least round number, by shared-memory atomics: 7,203 us at 4,194,304 x
+            // 128, 7,115 so)
+            go = above[b] == 0;
             if (issuer) {
                 if (go) {
                     multiply(b, 0, Sh::kRoundKb);
